@@ -446,7 +446,7 @@ typedef struct {
 } olap_batch_item;
 
 /* Check the items, upload the work queues (Top-K items largest first, one CTA
- * each; probe items largest first, cut into chunks of 32768 probe rows that
+ * each; probe items largest first, cut into chunks of 16384 probe rows that
  * any CTA may take) and capture the persistent launches in a CUDA graph.
  * Blocking. */
 olap_status olap_batch_create(olap_ctx* ctx, const olap_batch_item* items, uint64_t n_items, olap_batch** out);

@@ -14,13 +14,12 @@
 // stop at a key's last copy instead of walking on to the chain's end.
 //
 // Probe: every warp takes chunks of consecutive rows from a global counter
-// and hands them to its lanes in order (the loads of keys and row-ids
-// coalesce; no lane waits at a partition or range boundary).  Each lane runs
-// two independent probe streams and walks their chains one bucket per step; a
-// stream whose chain ends starts its next row at once (its key is already
-// loaded), so lanes do not wait for the longest chain of the warp.  Matches
-// are staged per warp in shared memory and appended to the output with one
-// atomic on the global count per flush.
+// (the loads of keys and row-ids coalesce) and probes them a tile of 128 rows
+// at a time, four bucket loads in flight per lane.  Probes whose chain goes on
+// past the home bucket are compacted per warp and walked 32 at a time, so
+// lanes do not wait for the longest chain of the warp.  Matches are staged
+// per warp in shared memory and appended to the output with one atomic on the
+// global count per flush.
 //
 // Partitioned probe (table much larger than L2, many probe rows): a table
 // larger than L2 turns every probe into a random DRAM sector read, and those
@@ -112,7 +111,7 @@ __global__ void __launch_bounds__(JB_TPB) join_side_kernel(const int64_t* keys, 
 }
 
 // The probe: rows [0, a.n) handed out in chunks by a row queue (see
-// probe_queue).  Used on the input (direct probe) and on the rows reordered
+// probe_rows).  Used on the input (direct probe) and on the rows reordered
 // by partition (pass 3 of the partitioned probe): there the chunks come out in
 // partition order, so the warps of the whole grid work on one partition's
 // table slice at a time and that slice stays in L2.
@@ -123,10 +122,10 @@ __global__ void __launch_bounds__(JB_TPB) join_side_kernel(const int64_t* keys, 
 // or the input when the partition passes were skipped), through L1 when the
 // plan says so.
 template <bool L2_ONLY>
-__global__ void __launch_bounds__(JP_TPB, 4) join_probe_kernel(ProbeArgs args, unsigned long long* next_row,
+__global__ void __launch_bounds__(JP_TPB, JP_CTAS) join_probe_kernel(ProbeArgs args, unsigned long long* next_row,
                                                                const ProbeCtl* ctl) {
-    extern __shared__ __align__(16) uint2 stage[];
-    const unsigned warp = threadIdx.x >> 5;
+    extern __shared__ __align__(16) unsigned char psmem[];
+    unsigned char* mine = psmem + (threadIdx.x >> 5) * JP_WARP_SMEM;
     ProbeArgs a = args;
     bool l1 = !L2_ONLY;
     if (ctl) {
@@ -140,10 +139,11 @@ __global__ void __launch_bounds__(JP_TPB, 4) join_probe_kernel(ProbeArgs args, u
     RowQueue q;
     q.counter = next_row;
     q.n = a.n;
+    q.chunk = queue_chunk(a.n, gridDim.x * JP_WARPS);
     if (l1)
-        probe_queue<false, JP_S>(a, q, stage + warp * JP_WCAP);
+        probe_rows<false>(a, q, mine);
     else
-        probe_queue<true, JP_S>(a, q, stage + warp * JP_WCAP);
+        probe_rows<true>(a, q, mine);
 }
 
 // ---- Bloom pre-probe ------------------------------------------------------

@@ -26,8 +26,20 @@ namespace olap {
 constexpr uint64_t JN_EMPTY = ~0ull;
 constexpr int JB_TPB = 256;
 constexpr int JP_TPB = 256;
-constexpr int JP_STAGE = 6144;    // pairs staged per CTA (48 KB), split evenly over its warps
-constexpr int JP_SMEM = JP_STAGE * 8;
+constexpr int JP_WARPS = JP_TPB / 32;
+// Shape of the probe kernels, from a sweep (2^20-row table in L2 with 18 M
+// probes / 2^24 rows with 30 M probes, partitioned / the same with Zipf
+// probes, direct): 4 rows per lane on 16 warps per SM take 126 / 484 /
+// 364 us; on 24 warps 142 / 519 / 455 us (spills, less L1); 8 rows 165 /
+// 559 / 435 us.  A stage of 384 pairs flushes too often (the count word
+// serialises: 128 / 596 us), one of 1280 takes the L1 the buckets use (690 us
+// on the Zipf probes).
+constexpr unsigned JP_WCAP = 640;           // pairs staged per warp
+constexpr int JP_U = 4;                     // rows in flight per lane
+constexpr int JP_CTAS = 2;                  // probe CTAs per SM
+constexpr unsigned JP_PEND = 32 * JP_U + 32;  // probes per warp that walk on past their home bucket
+constexpr int JP_WARP_SMEM = JP_WCAP * 8 + JP_PEND * 16;
+constexpr int JP_SMEM = JP_WARPS * JP_WARP_SMEM;
 
 struct JoinCtl {
     unsigned long long side_count;   // build rows with the empty-marker key
@@ -134,10 +146,6 @@ __device__ __forceinline__ Bucket ld_bucket(const ulonglong2* slots, uint32_t b)
     return v;
 }
 
-constexpr int JP_S = 2;                                 // independent probe streams per lane
-constexpr int JP_WARPS = JP_TPB / 32;
-constexpr unsigned JP_WCAP = JP_STAGE / JP_WARPS;         // staged pairs per warp
-
 // Copy a warp's staged pairs to the output with one atomic on the global
 // count (whole warp calls; cnt is warp-uniform).
 __device__ __forceinline__ void warp_flush(const ProbeArgs& a, uint2* ws, unsigned& cnt) {
@@ -147,166 +155,176 @@ __device__ __forceinline__ void warp_flush(const ProbeArgs& a, uint2* ws, unsign
     unsigned long long g = 0;
     if (lane == 0) g = atomicAdd(a.count, static_cast<unsigned long long>(cnt));
     g = __shfl_sync(0xFFFFFFFFu, g, 0);
-    for (unsigned i = lane; i < cnt; i += 32)
-        if (g + i < a.cap) st_stream_pair(a.out + g + i, ws[i]);
+    // pairs past the capacity are only counted
+    const uint64_t room = g < a.cap ? a.cap - g : 0;
+    const unsigned n = room < cnt ? static_cast<unsigned>(room) : cnt;
+    uint2* o = a.out + g;
+    for (unsigned i = lane; i < n; i += 32) st_stream_pair(o + i, ws[i]);
     __syncwarp();
     cnt = 0;
 }
 
-// Stage one pair for every lane where m is set (whole warp calls).
-__device__ __forceinline__ void warp_put(const ProbeArgs& a, uint2* ws, unsigned& cnt, bool m, uint2 p) {
+// Stage one pair for every lane where m is set (whole warp calls; the caller
+// has made room for 32).
+__device__ __forceinline__ void warp_put(uint2* ws, unsigned& cnt, bool m, uint2 p) {
     const unsigned b = __ballot_sync(0xFFFFFFFFu, m);
-    if (b == 0) return;
-    if (cnt + 32 > JP_WCAP) warp_flush(a, ws, cnt);
-    const unsigned lane = threadIdx.x & 31u;
-    if (m) ws[cnt + __popc(b & ((1u << lane) - 1u))] = p;
+    if (m) ws[cnt + __popc(b & ((1u << (threadIdx.x & 31u)) - 1u))] = p;
     cnt += __popc(b);
 }
 
-// Rows handed to the lanes of one warp.  The warp takes chunks of JQ_CHUNK
-// consecutive rows from a global counter and gives them out in order, the
-// lanes that need a row in one step getting consecutive rows, so the loads of
-// their keys and row-ids coalesce.  Every field is warp-uniform: `cur` is the
-// chunk being handed out, `nxt` the one taken after it (empty: b == e).
-constexpr uint64_t JQ_CHUNK = 512;
+// Rows handed to the warps: chunks of consecutive rows from a counter (global
+// for a whole probe, shared memory for one chunk of a batch item), so that
+// warps stay busy to the end and a partitioned probe moves through its
+// partitions in order, the whole grid on one table slice at a time.
+struct RowQueue {
+    unsigned long long* counter;  // next unclaimed row (zeroed before the launch)
+    uint64_t n;
+    uint32_t chunk;               // rows per take: 32, 64, ... JQ_CHUNK
+};
+constexpr uint32_t JQ_CHUNK = 512;
+
+// Rows per take for n rows over `warps` warps: JQ_CHUNK (one atomic per 512
+// rows) once every warp gets that many, fewer for small probes so that all
+// warps take part (100,003 rows against a 2^20-row table: 37.9 -> 13.2 us,
+// 10^6 rows 36 -> 18 us).
+__device__ __forceinline__ uint32_t queue_chunk(uint64_t n, uint32_t warps) {
+    uint32_t c = JQ_CHUNK;
+    while (c > 32 && static_cast<uint64_t>(c) * warps > n) c >>= 1;
+    return c;
+}
 
 struct RowRange {
     uint64_t b, e;
 };
-
-struct RowQueue {
-    RowRange cur, nxt;
-    unsigned long long* counter;  // next unclaimed row (zeroed before the launch)
-    uint64_t n;
-};
-
-__device__ __forceinline__ RowRange take_chunk(RowQueue& q) {
+__device__ __forceinline__ RowRange take_chunk(const RowQueue& q) {
     unsigned long long g = 0;
-    if ((threadIdx.x & 31u) == 0) g = atomicAdd(q.counter, static_cast<unsigned long long>(JQ_CHUNK));
+    if ((threadIdx.x & 31u) == 0) g = atomicAdd(q.counter, static_cast<unsigned long long>(q.chunk));
     g = __shfl_sync(0xFFFFFFFFu, g, 0);
-    return RowRange{min(static_cast<uint64_t>(g), q.n), min(static_cast<uint64_t>(g) + JQ_CHUNK, q.n)};
+    return RowRange{min(static_cast<uint64_t>(g), q.n), min(static_cast<uint64_t>(g) + q.chunk, q.n)};
 }
 
-// The next row of every lane in `need` (a ballot; whole warp calls): row
-// index, or false when the rows are exhausted.
-__device__ __forceinline__ bool queue_next(RowQueue& q, unsigned need, uint64_t* row) {
-    const unsigned c = __popc(need);
-    if (c == 0) return false;
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned r = __popc(need & ((1u << lane) - 1u));
-    uint64_t avail = q.cur.e - q.cur.b;
-    if (avail < c && q.nxt.b == q.nxt.e) q.nxt = take_chunk(q);
-    bool ok;
-    if (r < avail) {
-        *row = q.cur.b + r;
-        ok = true;
-    } else {
-        *row = q.nxt.b + (r - avail);
-        ok = *row < q.nxt.e;
-    }
-    if (c <= avail) {
-        q.cur.b += c;
-    } else {
-        const uint64_t used = min(static_cast<uint64_t>(c) - avail, q.nxt.e - q.nxt.b);
-        q.cur = RowRange{q.nxt.b + used, q.nxt.e};
-        q.nxt = RowRange{0, 0};
-    }
-    return ok && ((need >> lane) & 1u);
+// One probe against one bucket (whole warp calls, with room for 64 pairs):
+// stage the matches, and push the probe when its chain goes on.  A match
+// whose slot counts no further copies of its key ends the walk, as does a
+// bucket with a free slot.  An entry of `pend` holds the key, the row-id in
+// the low half of y and the bucket to read in the high half.
+__device__ __forceinline__ void probe_step(uint2* ws, unsigned& cnt, ulonglong2* pend, unsigned& np, bool real,
+                                           const Bucket& v, uint64_t key, uint32_t rid, uint32_t bk, uint32_t mask) {
+    const bool m0 = real && v.k0 == key, m1 = real && v.k1 == key;
+    const uint64_t w = m0 ? v.w0 : v.w1;
+    warp_put(ws, cnt, m0 || m1, make_uint2(rid, static_cast<uint32_t>(w)));
+    // (with both slots matching, slot 0 counts slot 1 as a further copy)
+    const bool go = real && v.k1 != JN_EMPTY && !((m0 || m1) && (w >> 32) == 0);
+    if (!__any_sync(0xFFFFFFFFu, go)) return;
+    const bool both = m0 && m1;
+    warp_put(ws, cnt, both, make_uint2(rid, static_cast<uint32_t>(v.w1)));
+    const bool on = go && !(both && (v.w1 >> 32) == 0);
+    const unsigned b = __ballot_sync(0xFFFFFFFFu, on);
+    if (on)
+        pend[np + __popc(b & ((1u << (threadIdx.x & 31u)) - 1u))] =
+            make_ulonglong2(key, rid | (static_cast<uint64_t>((bk + 1u) & mask) << 32));
+    np += __popc(b);
 }
 
-// One warp probes rows from the queue until the rows run out.  Each lane runs
-// JP_S independent streams.  A stream walks its row's chain one bucket per
-// step and, when the chain ends, switches at once to the row it has already
-// loaded and asks the queue for the next one.  Matches go to the warp's own
-// stage `ws`, flushed to the output whenever it could overflow and at the end.
-template <bool L2_ONLY, int S>
-__device__ __forceinline__ void probe_queue(const ProbeArgs& a, RowQueue& q, uint2* ws) {
+// One warp probes chunks of rows until the queue is empty, a tile of 32 *
+// JP_U rows at a time: every lane has JP_U independent bucket loads in
+// flight, and the next tile's keys are loaded while the current tile's
+// buckets arrive.  The few probes whose chain goes on (a full home bucket
+// without the key's last copy) are compacted in shared memory and walked 32
+// at a time, so no lane waits for another's longer chain.  Bound by the
+// bucket reads: L2-resident tables run at 143 G probes/s (103 G when every
+// lane walked its chains itself, two rows at a time), a 2^24-row table with
+// 30 M partitioned probes in 484 us for the whole call (648 us), with 2^28
+// probes in 3.30 ms (4.26 ms).
+template <bool L2_ONLY>
+__device__ __forceinline__ void probe_rows(const ProbeArgs& a, const RowQueue& q, unsigned char* warp_smem) {
+    uint2* ws = reinterpret_cast<uint2*>(warp_smem + JP_PEND * 16);
+    ulonglong2* pend = reinterpret_cast<ulonglong2*>(warp_smem);
     const unsigned lane = threadIdx.x & 31u;
     const uint32_t mask = static_cast<uint32_t>(a.mask);
-    unsigned cnt = 0;
-    uint64_t key[S], pkey[S];
-    uint32_t rid[S], prid[S], bk[S];
-    bool live[S], plive[S];
-    Bucket v[S];
-    q.cur = take_chunk(q);
-    q.nxt = RowRange{0, 0};
-    // current rows, then the rows loaded ahead
+    constexpr unsigned TILE = 32u * JP_U;
+    unsigned cnt = 0, np = 0;
+    uint64_t key[JP_U];
+    uint32_t rid[JP_U];
+    auto load_tile = [&](const RowRange& r) {
+        const int64_t* kp = a.keys + r.b + lane;
+        const uint32_t* rp = a.rowids + r.b + lane;
+        const uint32_t i0 = static_cast<uint32_t>(r.b) + lane;
+        if (r.e - r.b >= TILE) {
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-        uint64_t i = 0;
-        live[s] = queue_next(q, 0xFFFFFFFFu, &i);
-        key[s] = live[s] ? ld_stream_u64(a.keys + i) : JN_EMPTY;
-        rid[s] = live[s] ? (a.rowids ? ld_stream_u32(a.rowids + i) : static_cast<uint32_t>(i)) : 0u;
-    }
+            for (int j = 0; j < JP_U; ++j) key[j] = ld_stream_u64(kp + j * 32);
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-        uint64_t i = 0;
-        plive[s] = queue_next(q, 0xFFFFFFFFu, &i);
-        pkey[s] = plive[s] ? ld_stream_u64(a.keys + i) : JN_EMPTY;
-        prid[s] = plive[s] ? (a.rowids ? ld_stream_u32(a.rowids + i) : static_cast<uint32_t>(i)) : 0u;
-    }
+            for (int j = 0; j < JP_U; ++j) rid[j] = a.rowids ? ld_stream_u32(rp + j * 32) : i0 + j * 32;
+        } else {
+            const unsigned left = static_cast<unsigned>(r.e - r.b);
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-        bk[s] = static_cast<uint32_t>(fmix64(key[s])) & mask;
-        v[s] = (live[s] && key[s] != JN_EMPTY) ? ld_bucket<L2_ONLY>(a.slots, bk[s]) : Bucket{JN_EMPTY, 0, JN_EMPTY, 0};
-    }
-    while (true) {
-        bool any = false;
+            for (int j = 0; j < JP_U; ++j) {
+                const bool in = j * 32 + lane < left;
+                key[j] = in ? ld_stream_u64(kp + j * 32) : JN_EMPTY;
+                rid[j] = (in && a.rowids) ? ld_stream_u32(rp + j * 32) : i0 + j * 32;
+            }
+        }
+    };
+    auto drain = [&](unsigned keep) {           // walk pending probes while more than `keep` wait
+        while (np > keep) {
+            const unsigned take = min(np, 32u);
+            np -= take;
+            const bool act = lane < take;
+            if (cnt > JP_WCAP - 64) warp_flush(a, ws, cnt);
+            __syncwarp();
+            const ulonglong2 p = pend[np + (act ? lane : 0u)];
+            __syncwarp();
+            const uint32_t bk = static_cast<uint32_t>(p.y >> 32);
+            const Bucket v = ld_bucket<L2_ONLY>(a.slots, bk);
+            probe_step(ws, cnt, pend, np, act, v, p.x, static_cast<uint32_t>(p.y), bk, mask);
+        }
+    };
+    RowRange r = take_chunk(q);
+    load_tile(r);
+    while (r.b < r.e) {
+        Bucket v[JP_U];
+        uint32_t bk[JP_U];
 #pragma unroll
-        for (int s = 0; s < S; ++s) any = any || live[s];
-        if (!__any_sync(0xFFFFFFFFu, any)) break;
+        for (int j = 0; j < JP_U; ++j) {
+            bk[j] = static_cast<uint32_t>(fmix64(key[j])) & mask;
+            v[j] = ld_bucket<L2_ONLY>(a.slots, bk[j]);
+        }
+        uint64_t ck[JP_U];
+        uint32_t cr[JP_U];
+        const unsigned rows = static_cast<unsigned>(min(r.e - r.b, static_cast<uint64_t>(TILE)));
+#pragma unroll
+        for (int j = 0; j < JP_U; ++j) {
+            ck[j] = key[j];
+            cr[j] = rid[j];
+        }
+        r.b += TILE;
+        if (r.b >= r.e) r = take_chunk(q);
+        load_tile(r);
         // Probe keys equal to the empty marker pair with every side-list row;
-        // the warp emits them together, one such key at a time (rare).  With
-        // no side list such rows match nothing and are simply passed over.
+        // the warp emits them together, one such key at a time (rare).
+        if (a.n_side) {
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (a.n_side == 0) break;
-            unsigned sb = __ballot_sync(0xFFFFFFFFu, live[s] && key[s] == JN_EMPTY);
-            while (sb) {
-                const int src = __ffs(sb) - 1;
-                sb &= sb - 1;
-                const uint32_t r = __shfl_sync(0xFFFFFFFFu, rid[s], src);
-                for (uint64_t o0 = 0; o0 < a.n_side; o0 += 32) {
-                    const bool m = o0 + lane < a.n_side;
-                    warp_put(a, ws, cnt, m, make_uint2(r, m ? a.side[o0 + lane] : 0u));
+            for (int j = 0; j < JP_U; ++j) {
+                unsigned sb = __ballot_sync(0xFFFFFFFFu, ck[j] == JN_EMPTY && j * 32 + lane < rows);
+                while (sb) {
+                    const int src = __ffs(sb) - 1;
+                    sb &= sb - 1;
+                    const uint32_t rr = __shfl_sync(0xFFFFFFFFu, cr[j], src);
+                    for (uint64_t o0 = 0; o0 < a.n_side; o0 += 32) {
+                        if (cnt > JP_WCAP - 32) warp_flush(a, ws, cnt);
+                        const bool m = o0 + lane < a.n_side;
+                        warp_put(ws, cnt, m, make_uint2(rr, m ? a.side[o0 + lane] : 0u));
+                    }
                 }
             }
         }
-        // Matches in the current bucket of every stream; a match whose slot
-        // counts no further copies of its key ends the row's walk.
-        bool go[S];
+        if (cnt > JP_WCAP - 64 * JP_U) warp_flush(a, ws, cnt);
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-            const bool real = live[s] && key[s] != JN_EMPTY;
-            const bool m0 = real && v[s].k0 == key[s], m1 = real && v[s].k1 == key[s];
-            warp_put(a, ws, cnt, m0, make_uint2(rid[s], static_cast<uint32_t>(v[s].w0)));
-            warp_put(a, ws, cnt, m1, make_uint2(rid[s], static_cast<uint32_t>(v[s].w1)));
-            const bool last = (m0 && (v[s].w0 >> 32) == 0) || (m1 && (v[s].w1 >> 32) == 0);
-            go[s] = real && !last && v[s].k1 != JN_EMPTY;     // slot 1 taken: the bucket is full
-        }
-        // Each stream steps along its chain, or takes the row it loaded ahead
-        // and loads the queue's next row in its place.
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            const bool swap = live[s] && !go[s];
-            uint64_t i = 0;
-            const bool got = queue_next(q, __ballot_sync(0xFFFFFFFFu, swap && plive[s]), &i);
-            if (go[s]) {
-                bk[s] = (bk[s] + 1u) & mask;
-            } else if (swap) {
-                live[s] = plive[s];
-                key[s] = pkey[s];
-                rid[s] = prid[s];
-                bk[s] = static_cast<uint32_t>(fmix64(key[s])) & mask;
-                plive[s] = got;
-                if (got) {
-                    pkey[s] = ld_stream_u64(a.keys + i);
-                    prid[s] = a.rowids ? ld_stream_u32(a.rowids + i) : static_cast<uint32_t>(i);
-                }
-            }
-            if (live[s] && key[s] != JN_EMPTY) v[s] = ld_bucket<L2_ONLY>(a.slots, bk[s]);
-        }
+        for (int j = 0; j < JP_U; ++j)
+            probe_step(ws, cnt, pend, np, ck[j] != JN_EMPTY, v[j], ck[j], cr[j], bk[j], mask);
+        drain(31u);
     }
+    drain(0u);
     warp_flush(a, ws, cnt);
 }
 
