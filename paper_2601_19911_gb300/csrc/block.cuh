@@ -64,26 +64,40 @@ struct Pick {
     unsigned long long in_b;
 };
 
+// The thread's bins, PICK_BINS / TPB of them in order, are in v.  Counts sum
+// to less than 2^32.  sc: 24 words of shared memory.
 template <int TPB>
-__device__ Pick pick_bucket(const unsigned* hist, unsigned long long need, unsigned long long* sc) {
-    constexpr int PER = PICK_BINS / TPB;
-    unsigned v[PER];
-    unsigned long long local = 0;
-    const volatile unsigned* h = hist;
+__device__ __forceinline__ Pick pick_loaded(const unsigned (&v)[PICK_BINS / TPB], unsigned long long need,
+                                            unsigned long long* sc) {
+    constexpr int PER = PICK_BINS / TPB, NW = TPB / 32;
+    unsigned* warp_sums = reinterpret_cast<unsigned*>(sc);      // NW <= 32 entries
+    unsigned* res = warp_sums + 32;                             // b, below, in_b
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    unsigned local = 0;
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        v[j] = h[threadIdx.x * PER + j];
-        local += v[j];
+    for (int j = 0; j < PER; ++j) local += v[j];
+    unsigned incl = local;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= static_cast<unsigned>(o)) incl += t;
     }
-    unsigned long long* warp_sums = sc;        // 16 entries
-    unsigned long long* total = sc + 16;
-    unsigned long long* res = sc + 17;         // b, below, in_b
-    const unsigned long long before = block_excl_scan<TPB>(local, warp_sums, total);
-    if (before < need && need <= before + local) {
-        unsigned long long run = before;
+    if (lane == 31) warp_sums[warp] = incl;
+    __syncthreads();
+    unsigned ws = lane < NW ? warp_sums[lane] : 0u;             // every warp scans the warps' sums
+    const unsigned mine = ws;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_up_sync(0xFFFFFFFFu, ws, o);
+        if (lane >= static_cast<unsigned>(o)) ws += t;
+    }
+    const unsigned before = __shfl_sync(0xFFFFFFFFu, ws - mine, warp) + incl - local;
+    const unsigned nd = static_cast<unsigned>(need);
+    if (before < nd && nd <= before + local) {
+        unsigned run = before;
 #pragma unroll
         for (int j = 0; j < PER; ++j) {
-            if (run < need && need <= run + v[j]) {
+            if (run < nd && nd <= run + v[j]) {
                 res[0] = threadIdx.x * PER + j;
                 res[1] = run;
                 res[2] = v[j];
@@ -92,9 +106,34 @@ __device__ Pick pick_bucket(const unsigned* hist, unsigned long long need, unsig
         }
     }
     __syncthreads();
-    Pick p{static_cast<unsigned>(res[0]), res[1], res[2]};
+    const Pick p{res[0], res[1], res[2]};
     __syncthreads();
     return p;
+}
+
+// The thread's share of a histogram in global memory, read past L1.
+template <int TPB>
+__device__ __forceinline__ void pick_load_global(const unsigned* hist, unsigned (&v)[PICK_BINS / TPB]) {
+    constexpr int PER = PICK_BINS / TPB;
+    static_assert(PER % 4 == 0, "16-byte loads");
+    const uint4* h = reinterpret_cast<const uint4*>(hist) + threadIdx.x * (PER / 4);
+#pragma unroll
+    for (int j = 0; j < PER / 4; ++j) {
+        const uint4 x = __ldcg(h + j);
+        v[4 * j] = x.x;
+        v[4 * j + 1] = x.y;
+        v[4 * j + 2] = x.z;
+        v[4 * j + 3] = x.w;
+    }
+}
+// A histogram in shared memory.
+template <int TPB>
+__device__ Pick pick_bucket(const unsigned* hist, unsigned long long need, unsigned long long* sc) {
+    constexpr int PER = PICK_BINS / TPB;
+    unsigned v[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) v[j] = hist[threadIdx.x * PER + j];
+    return pick_loaded<TPB>(v, need, sc);
 }
 
 // Bitonic sort of `count` entries in shared memory (room for the next power of two), ascending
@@ -192,6 +231,25 @@ __device__ __forceinline__ KeyLimit key_limit(uint64_t t, int kind, bool desc) {
         default: float_limit<uint32_t>(t32, desc, &k.m32, &k.c32); break;   // float32
     }
     return k;
+}
+// The same test as one comparison without the XOR: every limit above is x >= c
+// or x <= c on the key's bits read as a signed or an unsigned integer.
+enum KeyCmp { CMP_GE_U = 0, CMP_LE_U = 1, CMP_GE_S = 2, CMP_LE_S = 3 };
+template <typename U>
+__device__ __forceinline__ int key_cmp(U m, U c, U* lim) {
+    constexpr U SIGN = static_cast<U>(1) << (sizeof(U) * 8 - 1);
+    if (m == 0) { *lim = c; return CMP_GE_U; }
+    if (m == static_cast<U>(~static_cast<U>(0))) { *lim = static_cast<U>(~c); return CMP_LE_U; }
+    if (m == SIGN) { *lim = c ^ SIGN; return CMP_GE_S; }
+    *lim = static_cast<U>(~c) ^ SIGN;                 // x ^ ~SIGN is the complement of x ^ SIGN
+    return CMP_LE_S;
+}
+template <int MODE, typename U, typename S>
+__device__ __forceinline__ bool key_pass(U x, U c) {
+    if (MODE == CMP_GE_U) return x >= c;
+    if (MODE == CMP_LE_U) return x <= c;
+    if (MODE == CMP_GE_S) return static_cast<S>(x) >= static_cast<S>(c);
+    return static_cast<S>(x) <= static_cast<S>(c);
 }
 __device__ __forceinline__ bool pass64(uint64_t bits, const KeyLimit& k) { return (bits ^ k.m64) >= k.c64; }
 __device__ __forceinline__ bool pass32(uint32_t bits, const KeyLimit& k) { return (bits ^ k.m32) >= k.c32; }

@@ -105,68 +105,6 @@ __device__ __forceinline__ int prefix_cmp(uint64_t w0, uint64_t w1, uint64_t p0,
     return a < b ? -1 : (a > b ? 1 : 0);
 }
 
-// Fold (w0, w1) into running AND / OR words.
-__device__ __forceinline__ void and_or(uint64_t w0, uint64_t w1, uint64_t* ao) {
-    ao[0] &= w0;
-    ao[1] &= w1;
-    ao[2] |= w0;
-    ao[3] |= w1;
-}
-
-// Reduce the running AND / OR words over the CTA (warp shuffles, then the
-// warps' results in shared memory) and merge them into `dst` with four
-// atomics per CTA: same-address atomics serialise in L2, so one per warp
-// would cost thousands of serial updates over the grid.  Whole CTA calls.
-template <int TPB>
-__device__ __forceinline__ void and_or_merge(uint64_t* ao, unsigned long long* dst) {
-    __shared__ unsigned long long s_ao[TPB / 32][4];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        ao[0] &= __shfl_xor_sync(0xFFFFFFFFu, ao[0], o);
-        ao[1] &= __shfl_xor_sync(0xFFFFFFFFu, ao[1], o);
-        ao[2] |= __shfl_xor_sync(0xFFFFFFFFu, ao[2], o);
-        ao[3] |= __shfl_xor_sync(0xFFFFFFFFu, ao[3], o);
-    }
-    if ((threadIdx.x & 31u) == 0)
-        for (int j = 0; j < 4; ++j) s_ao[threadIdx.x >> 5][j] = ao[j];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint64_t r[4] = {~0ull, ~0ull, 0ull, 0ull};
-        for (int w = 0; w < TPB / 32; ++w) {
-            r[0] &= s_ao[w][0];
-            r[1] &= s_ao[w][1];
-            r[2] |= s_ao[w][2];
-            r[3] |= s_ao[w][3];
-        }
-        atomicAnd(dst + 0, static_cast<unsigned long long>(r[0]));
-        atomicAnd(dst + 1, static_cast<unsigned long long>(r[1]));
-        atomicOr(dst + 2, static_cast<unsigned long long>(r[2]));
-        atomicOr(dst + 3, static_cast<unsigned long long>(r[3]));
-    }
-    __syncthreads();
-}
-
-// First bit position (0 = MSB of w0) where the entries behind merged AND / OR
-// words differ; `total` when they agree everywhere.
-__device__ __forceinline__ int first_diff(const unsigned long long* ao, int total) {
-    const uint64_t d0 = __ldcg(ao + 0) ^ __ldcg(ao + 2), d1 = __ldcg(ao + 1) ^ __ldcg(ao + 3);
-    const int f = d0 ? __clzll(static_cast<long long>(d0)) : (d1 ? 64 + __clzll(static_cast<long long>(d1)) : 128);
-    return f < total ? f : total;
-}
-
-// Bits [lo, hi) of a 64-bit word counted from its MSB (0 <= lo <= hi <= 64).
-__device__ __forceinline__ uint64_t bit_range(int lo, int hi) {
-    if (hi <= lo) return 0ull;
-    const uint64_t ones = (hi - lo == 64) ? ~0ull : ((1ull << (hi - lo)) - 1ull);
-    return ones << (64 - hi);
-}
-
-// Copy bits [from, to) of (a0, a1) into (p0, p1), whose bits there are zero.
-__device__ __forceinline__ void prefix_copy(uint64_t& p0, uint64_t& p1, uint64_t a0, uint64_t a1, int from, int to) {
-    if (from < 64) p0 |= a0 & bit_range(from, to < 64 ? to : 64);
-    if (to > 64) p1 |= a1 & bit_range((from > 64 ? from : 64) - 64, to - 64);
-}
-
 // Set bits [L, L + d) of (p0, p1) to `digit`.
 __device__ __forceinline__ void prefix_set(uint64_t& p0, uint64_t& p1, int L, int d, uint32_t digit) {
     const uint64_t v = static_cast<uint64_t>(digit);
@@ -196,14 +134,16 @@ __device__ __forceinline__ int ld_volatile_i32(const int* p) {
     return *reinterpret_cast<const volatile int*>(p);
 }
 
-// Grid barrier for cooperative launches (all CTAs co-resident).  Arrival is an
-// atomic count; the last CTA to arrive resets it and bumps a generation word
-// the others wait on.  The wait is bounded: after WAIT_LIMIT_CYCLES the CTA
-// records OLAP_E_TIMEOUT in *err and leaves; callers test the return value
-// and stop.  The counter returns to zero after every completed barrier.
+// Grid barrier for cooperative launches (all CTAs co-resident).  `count`
+// starts every call at zero (the kernel before the cooperative one resets it)
+// and only grows: the b-th barrier of the launch is passed when it reaches b
+// times the grid, so an arrival is one fire-and-forget add and the last one
+// releases everybody with no reset and no second word.  The wait is bounded:
+// after WAIT_LIMIT_CYCLES the CTA records OLAP_E_TIMEOUT in *err and leaves;
+// callers test the return value and stop.
 struct GridBar {
     unsigned count;
-    unsigned gen;
+    unsigned pad0;
     unsigned prep;        // tickets of the Top-K prepare kernel's CTAs (a multiple of its grid between launches)
     unsigned pad;
 };
@@ -222,23 +162,24 @@ __device__ __forceinline__ bool wait_changed(const unsigned* word, unsigned old,
     return true;
 }
 
-__device__ __forceinline__ bool grid_sync(GridBar* bar, int* err) {
+__device__ __forceinline__ bool grid_sync(GridBar* bar, int* err, unsigned& target) {
+    target += gridDim.x;
     __syncthreads();
+    bool ok = true;
     if (threadIdx.x == 0) {
-        const unsigned nblocks = gridDim.x * gridDim.y * gridDim.z;
-        const unsigned g = ld_acquire_u32(&bar->gen);
-        __threadfence();
-        if (atomicAdd(&bar->count, 1u) == nblocks - 1) {
-            atomicExch(&bar->count, 0u);
-            __threadfence();
-            st_release_u32(&bar->gen, g + 1);
-        } else {
-            wait_changed(&bar->gen, g, err, WAIT_LIMIT_CYCLES);
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&bar->count) : "memory");
+        const long long t0 = clock64();
+        while (ld_acquire_u32(&bar->count) < target) {
+            if (clock64() - t0 > WAIT_LIMIT_CYCLES) {
+                atomicCAS(err, 0, static_cast<int>(OLAP_E_TIMEOUT));
+                ok = false;
+                break;
+            }
+            __nanosleep(20);
         }
         __threadfence();
     }
-    __syncthreads();
-    return ld_volatile_i32(err) == 0;
+    return __syncthreads_and(ok) != 0;
 }
 
 // ---------------------------------------------------------------------------

@@ -3,15 +3,14 @@
 // row pointers of the Top-K rows in order).
 //
 // Three launches on one stream:
-//   0. topk_prepare_kernel zeroes the control block and, when N > 2^21 and K
-//      is small against N, reads a stratified sample of 8192 keys (16 CTAs,
-//      one key per thread) and finds the rank word of the sample's r-th best
-//      entry by a radix select in the last CTA to finish; r is chosen so that,
-//      with high probability, at least K keys but not many more fall at or
-//      below it.
+//   0. topk_prepare_kernel zeroes the control block and, when N is large and
+//      K is small against N, reads a stratified sample of 8192 keys (16 CTAs,
+//      one key per thread) and finds the sample's r-th best entry by a radix
+//      select in the last CTA to finish; r is chosen so that, with high
+//      probability, at least K keys but not many more fall at or below it.
 //   1. topk_filter_regs_kernel (default) or topk_filter_bulk_kernel (TMA
 //      bulk copies into a shared-memory ring): the only full pass over the
-//      keys, run only when there is a sample.  16-byte streaming loads, one
+//      keys, run only when there is a sample.  32-byte streaming loads, one
 //      compare per key against the threshold in the key's own bit domain,
 //      and every key that passes is appended (per-warp staging, one global
 //      atomic per flush) to a candidate buffer with its row-id.
@@ -19,13 +18,13 @@
 //   meet at bounded grid barriers.  Its source is the candidate buffer when
 //   the sample worked (at least K candidates, no overflow) and the full
 //   input otherwise (no sample, or a misjudged one).
-//   2. Refine: radix passes of 12-bit digits over the (key, row-id) composite
-//      of the candidates (or the input): a shared-memory histogram with
-//      __match_any_sync aggregation, merged into a global histogram; every
-//      CTA then scans it and extends the same prefix, until the bucket that
-//      holds the K-th entry has at most 4096 entries.
-//   3. Split: entries below the prefix are selected; entries equal to it go
-//      to a small buffer that one CTA sorts to take the remaining count.
+//   2. Refine: every pass cuts the current interval of the composite (rank
+//      word, row-id) order into up to 4096 equal bins (a shared-memory
+//      histogram with __match_any_sync aggregation, merged into a global
+//      one); every CTA then scans it and goes on with the same bin, until the
+//      bin that holds the K-th entry has at most 4096 entries.
+//   3. Split: entries below the interval are selected; entries in it go to a
+//      small buffer that is ranked to take the remaining count.
 //   4. Sort the K survivors by (rank word, row-id) -- in shared memory when
 //      K <= 4096, else tile sorts plus merge-path rounds across the grid --
 //      and write keys (original bits, by the inverse transform) and row-ids.
@@ -40,6 +39,25 @@
 namespace olap {
 
 namespace {
+
+__device__ __forceinline__ unsigned long long gtimer() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+// Programmatic dependent launch.  Every kernel of a call is launched while
+// the one before it in the stream is still running, and waits here until that
+// one has finished and its writes are visible.  A kernel launched without the
+// attribute passes straight through.
+__device__ __forceinline__ void wait_prior_grid() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Lets the next kernel in the stream launch now (it still waits for this one
+// to finish before it reads anything this one or an earlier one writes).
+__device__ __forceinline__ void allow_next_grid() {
+    asm volatile("griddepcontrol.launch_dependents;" :::);
+}
 
 struct Elem {
     uint64_t r;
@@ -80,22 +98,133 @@ __device__ __forceinline__ void write_result(const TopkArgs& a, uint64_t i, uint
     a.out_rowids[i] = rid;
 }
 
+// An interval of the composite (rank word, row-id) order: the entries with
+// rlo <= r <= rhi when rlo < rhi (any row-id), else those with r == rlo and
+// ilo <= row-id <= ihi.  A refine pass cuts it into at most 2^digit equal bins.
+struct Range {
+    uint64_t rlo, rhi;
+    uint32_t ilo, ihi;
+};
+__device__ __forceinline__ uint32_t max_rowid(const TopkArgs& a) {
+    return a.rowids ? 0xFFFFFFFFu : static_cast<uint32_t>(a.n - 1);
+}
+// (a 4-byte key's rank words are multiples of 2^32)
+__device__ __forceinline__ uint64_t max_rank(const TopkArgs& a) { return a.w4 ? 0xFFFFFFFF00000000ull : ~0ull; }
+__device__ __forceinline__ bool range_point(const Range& g) { return g.rlo == g.rhi && g.ilo == g.ihi; }
+// -1 below the interval, 0 in it, 1 above.
+__device__ __forceinline__ int range_cmp(const Range& g, uint64_t r, uint32_t rid) {
+    if (r < g.rlo) return -1;
+    if (r > g.rhi) return 1;
+    if (g.rlo != g.rhi) return 0;
+    return rid < g.ilo ? -1 : (rid > g.ihi ? 1 : 0);
+}
+__device__ __forceinline__ int range_shift(const Range& g, int digit) {
+    const int bits = g.rlo != g.rhi ? 64 - __clzll(static_cast<long long>(g.rhi - g.rlo))
+                                    : 32 - __clz(static_cast<int>(g.ihi - g.ilo));
+    return bits > digit ? bits - digit : 0;
+}
+__device__ __forceinline__ unsigned range_bin(const Range& g, int sh, uint64_t r, uint32_t rid) {
+    return static_cast<unsigned>(g.rlo != g.rhi ? (r - g.rlo) >> sh : static_cast<uint64_t>((rid - g.ilo) >> sh));
+}
+// Bin b of the interval.
+__device__ __forceinline__ Range range_narrow(const TopkArgs& a, const Range& g, int sh, unsigned b) {
+    Range o = g;
+    const uint64_t w = (1ull << sh) - 1ull;
+    if (g.rlo != g.rhi) {
+        o.rlo = g.rlo + (static_cast<uint64_t>(b) << sh);
+        o.rhi = g.rhi - o.rlo < w ? g.rhi : o.rlo + w;
+        if (a.w4) {
+            o.rlo = (o.rlo + 0xFFFFFFFFull) & 0xFFFFFFFF00000000ull;
+            o.rhi &= 0xFFFFFFFF00000000ull;
+        }
+        o.ilo = 0;
+        o.ihi = max_rowid(a);
+    } else {
+        o.ilo = g.ilo + (b << sh);
+        o.ihi = g.ihi - o.ilo < w ? g.ihi : o.ilo + static_cast<uint32_t>(w);
+    }
+    return o;
+}
+// The interval spanned by folded minima and maxima (fold_add).
+__device__ __forceinline__ Range range_of(const TopkArgs& a, const unsigned long long* mm) {
+    Range o{__ldcg(mm + 0), __ldcg(mm + 1), 0u, max_rowid(a)};
+    if (o.rlo == o.rhi) {
+        o.ilo = static_cast<uint32_t>(__ldcg(mm + 2));
+        o.ihi = static_cast<uint32_t>(__ldcg(mm + 3));
+    }
+    return o;
+}
+
+// Minimum and maximum of rank words and of row-ids, folded per thread, then
+// over the CTA into four global words (one atomic each: same-address atomics
+// serialise in L2).
+struct Fold {
+    uint64_t rmin, rmax;
+    uint32_t imin, imax;
+};
+__device__ __forceinline__ Fold fold_none() { return Fold{~0ull, 0ull, ~0u, 0u}; }
+__device__ __forceinline__ void fold_add(Fold& f, uint64_t r, uint32_t rid) {
+    f.rmin = min(f.rmin, r);
+    f.rmax = max(f.rmax, r);
+    f.imin = min(f.imin, rid);
+    f.imax = max(f.imax, rid);
+}
+template <int TPB>
+__device__ __forceinline__ Fold fold_cta(Fold f) {            // thread 0 gets the CTA's fold
+    __shared__ Fold s_f[TPB / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        f.rmin = min(f.rmin, __shfl_xor_sync(0xFFFFFFFFu, f.rmin, o));
+        f.rmax = max(f.rmax, __shfl_xor_sync(0xFFFFFFFFu, f.rmax, o));
+    }
+    f.imin = __reduce_min_sync(0xFFFFFFFFu, f.imin);
+    f.imax = __reduce_max_sync(0xFFFFFFFFu, f.imax);
+    if ((threadIdx.x & 31u) == 0) s_f[threadIdx.x >> 5] = f;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < TPB / 32; ++w) {
+            f.rmin = min(f.rmin, s_f[w].rmin);
+            f.rmax = max(f.rmax, s_f[w].rmax);
+            f.imin = min(f.imin, s_f[w].imin);
+            f.imax = max(f.imax, s_f[w].imax);
+        }
+    __syncthreads();
+    return f;
+}
+template <int TPB>
+__device__ __forceinline__ void fold_merge(const Fold& mine, unsigned long long* dst) {
+    const Fold f = fold_cta<TPB>(mine);
+    if (threadIdx.x == 0 && f.rmin <= f.rmax) {
+        atomicMin(dst + 0, static_cast<unsigned long long>(f.rmin));
+        atomicMax(dst + 1, static_cast<unsigned long long>(f.rmax));
+        atomicMin(dst + 2, static_cast<unsigned long long>(f.imin));
+        atomicMax(dst + 3, static_cast<unsigned long long>(f.imax));
+    }
+}
+__device__ __forceinline__ void fold_reset(unsigned long long* mm) {
+    mm[0] = mm[2] = ~0ull;
+    mm[1] = mm[3] = 0ull;
+}
+
 // Prepare kernel: a threshold rank word for the streaming pass from a
 // stratified sample of TK_SAMPLE keys (sample j is key (j * n) / TK_SAMPLE +
 // (n / TK_SAMPLE) / 2).  The prepare CTAs load it together, one key per
 // thread, into a.samples -- from one SM, 8192 scattered loads wait on each
 // other's DRAM latency -- and the last CTA to finish runs this radix select
 // with a.digit-bit digits on the sample held in registers; it stops as soon as
-// the upper edge of the chosen bucket has between r and r + 8 samples at or
-// below it (any such threshold serves), which for spread-out keys is after the
-// first digit.
-__device__ uint64_t sample_threshold(const TopkArgs& a, unsigned* sh, unsigned long long* sc) {
+// the chosen bucket's upper edge has between r and r + 8 samples at or
+// below it, which for spread-out keys is after the first digit.  The
+// threshold is the largest of those samples.  With the smallest of them it
+// also fixes the interval of the select's fused first pass (see fuse_range):
+// four times their spread below the threshold, or the threshold alone when
+// they are all equal.
+__device__ void sample_threshold(const TopkArgs& a, unsigned* sh, unsigned long long* sc) {
     uint64_t s[TK_SPT];
 #pragma unroll
     for (int j = 0; j < TK_SPT; ++j) s[j] = __ldcg(a.samples + static_cast<uint64_t>(j) * TK_TPB + threadIdx.x);
     const int kb = a.w4 ? 32 : 64;
     const unsigned long long r = a.sample_rank;
-    uint64_t prefix = 0;
+    uint64_t prefix = 0, edge = 0;
     unsigned long long rem = r, cum = 0;
     for (int L = 0; L < kb; L += a.digit) {
         const int d = min(a.digit, kb - L);
@@ -111,9 +240,28 @@ __device__ uint64_t sample_threshold(const TopkArgs& a, unsigned* sh, unsigned l
         prefix |= static_cast<uint64_t>(pk.b) << (64 - L - d);
         rem -= pk.below;
         cum += pk.below;
-        if (cum + pk.in_b <= r + 8) return prefix | ((1ull << (64 - L - d)) - 1ull);
+        edge = prefix | ((1ull << (64 - L - d)) - 1ull);
+        if (cum + pk.in_b <= r + 8) break;
     }
-    return prefix;
+    __shared__ unsigned long long lo, hi;                    // of the few samples up to the edge
+    if (threadIdx.x == 0) {
+        lo = ~0ull;
+        hi = 0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < TK_SPT; ++j)
+        if (s[j] <= edge) {
+            atomicMin(&lo, static_cast<unsigned long long>(s[j]));
+            atomicMax(&hi, static_cast<unsigned long long>(s[j]));
+        }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const uint64_t t = hi, d = hi - lo;
+        a.ctl->thresh = t;
+        a.ctl->fbase = d >= t / 4 ? (d ? 0ull : t) : t - 4 * d;
+        a.ctl->ts[1] = gtimer();
+    }
 }
 
 // Hits of the streaming pass are staged per warp in shared memory and
@@ -134,41 +282,39 @@ __device__ __forceinline__ WarpStage warp_stage(unsigned char* base) {
     return WarpStage{reinterpret_cast<uint64_t*>(p), reinterpret_cast<uint32_t*>(p + WS_CAP * 8), 0u};
 }
 
-// The select's first radix pass, folded into the streaming filter (the
+// The select's first refine pass, folded into the streaming filter (the
 // register and two-column filters).  Every candidate already passes through
-// a warp stage; as it leaves, its digit at the first bit where candidates can
-// differ (just below the threshold's leading zeros, the select's first pass
-// position) is counted in a CTA histogram in shared memory, which the CTA adds
-// to the select's pass-0 histogram when it is done.  The select then starts
-// at the bucket pick, one pass over the candidates and one grid barrier
-// sooner.  (The pass's AND / OR fold, which lets a pass skip bits all its
-// entries share, is left to the select's later passes: four 64-bit shared
-// atomics per candidate slowed the streaming pass by 5-10 %.)
-__shared__ unsigned g_fuse_hist[TK_BINS];
+// a warp stage; as it leaves, its bin of the interval [fbase, threshold] is
+// counted in a CTA histogram in shared memory, which the CTA adds to the
+// select's pass-0 histogram when it is done.  The select then starts at the
+// bin pick, one pass over the candidates and one grid barrier sooner.  The
+// interval comes from the sampled keys at or below the threshold, so it fits
+// keys that cluster (doubles of one magnitude) and, when those samples are
+// all equal, bins the ties by row-id.  2^26 rows ordered by a 1024-value
+// column and a second one: one pass instead of three over the candidates, the
+// select 29 -> 11.6 us.  Candidates below the interval are counted in one
+// more word.
+__shared__ unsigned g_fuse_hist[TK_BINS + 1];
 
-// Bit position and width of the fused digit (those of the select's first pass).
-struct FuseDigit {
-    int L, d, kb;
+struct FuseRange {
+    Range g;
+    int sh;
 };
-__device__ __forceinline__ FuseDigit fuse_digit(const TopkArgs& a, uint64_t t) {
-    FuseDigit f;
-    f.kb = a.w4 ? 32 : 64;
-    const int lz = __clzll(static_cast<long long>(t));
-    f.L = lz < f.kb ? lz : f.kb;
-    f.d = min(a.digit, f.kb + 32 - f.L);
+__device__ __forceinline__ FuseRange fuse_range(const TopkArgs& a) {
+    FuseRange f;
+    f.g = Range{__ldcg(&a.ctl->fbase), __ldcg(&a.ctl->thresh), 0u, max_rowid(a)};
+    f.sh = range_shift(f.g, a.digit);
     return f;
 }
 
 template <int TPB>
 __device__ __forceinline__ void fuse_init() {
-    for (int b = threadIdx.x; b < TK_BINS; b += TPB) g_fuse_hist[b] = 0;
+    for (int b = threadIdx.x; b <= TK_BINS; b += TPB) g_fuse_hist[b] = 0;
     __syncthreads();
 }
 
-__device__ __forceinline__ void fuse_add(const FuseDigit& f, uint64_t r, uint32_t rid) {
-    uint64_t w0, w1;
-    comp_words(r, rid, f.kb, w0, w1);
-    atomicAdd(&g_fuse_hist[comp_digit(w0, w1, f.L, f.d)], 1u);
+__device__ __forceinline__ void fuse_add(const FuseRange& f, uint64_t r, uint32_t rid) {
+    atomicAdd(&g_fuse_hist[r < f.g.rlo ? TK_BINS : range_bin(f.g, f.sh, r, rid)], 1u);
 }
 
 // Whole CTA, after its last candidate: add the CTA's counts to the pass-0
@@ -178,20 +324,8 @@ __device__ __forceinline__ void fuse_merge(const TopkArgs& a) {
     __syncthreads();
     for (int b = threadIdx.x; b < TK_BINS; b += TPB)
         if (g_fuse_hist[b]) atomicAdd(&a.ghist[b], g_fuse_hist[b]);
-}
-
-// Programmatic dependent launch.  The filter and the select are launched
-// while the kernel before them in the stream is still running; they wait here
-// until it has finished and its writes are visible (measured, 2^28 int64
-// keys: 3 us less per call).  A kernel launched without the attribute passes
-// straight through.
-__device__ __forceinline__ void wait_prior_grid() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-// Lets the next kernel in the stream launch now (it still waits for this one
-// to finish before it reads anything).
-__device__ __forceinline__ void allow_next_grid() {
-    asm volatile("griddepcontrol.launch_dependents;" :::);
+    if (threadIdx.x == 0 && g_fuse_hist[TK_BINS])
+        atomicAdd(&a.ctl->flow, static_cast<unsigned long long>(g_fuse_hist[TK_BINS]));
 }
 
 // Move the warp's staged hits to the candidate buffer (all 32 lanes call).
@@ -214,18 +348,10 @@ __device__ __forceinline__ void stage_flush_plain(const TopkArgs& a, WarpStage& 
     ws.count = 0;
 }
 
-// The same, also counting the hits for the fused first pass.  Kept out of
-// line: it runs once per WS_CAP hits of a warp, and inlined into the
-// filter's unrolled loop it would cost the loop registers (occupancy).
-__device__ __forceinline__ void stage_flush_fused(const TopkArgs& a, const uint64_t* sr, const uint32_t* sidx,
-                                               unsigned count) {
-    __syncwarp();
-    const unsigned lane = threadIdx.x & 31u;
-    unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(&a.ctl->cand_count, static_cast<unsigned long long>(count));
-    base = __shfl_sync(0xFFFFFFFFu, base, 0);
-    const FuseDigit f = fuse_digit(a, __ldcg(&a.ctl->thresh));
-    for (unsigned j = lane; j < count; j += 32) {
+// The same, also counting the hits for the fused first pass.
+__device__ __forceinline__ void stage_write_fused(const TopkArgs& a, const FuseRange& f, const uint64_t* sr,
+                                                  const uint32_t* sidx, unsigned count, unsigned long long base) {
+    for (unsigned j = threadIdx.x & 31u; j < count; j += 32) {
         const unsigned long long pos = base + j;
         const uint32_t idx = sidx[j];
         const uint64_t r = sr[j];
@@ -236,6 +362,14 @@ __device__ __forceinline__ void stage_flush_fused(const TopkArgs& a, const uint6
         }
         fuse_add(f, r, rid);
     }
+}
+__device__ __forceinline__ void stage_flush_fused(const TopkArgs& a, const uint64_t* sr, const uint32_t* sidx,
+                                                  unsigned count) {
+    __syncwarp();
+    unsigned long long base = 0;
+    if ((threadIdx.x & 31u) == 0) base = atomicAdd(&a.ctl->cand_count, static_cast<unsigned long long>(count));
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    stage_write_fused(a, fuse_range(a), sr, sidx, count, base);
     __syncwarp();
 }
 
@@ -250,62 +384,78 @@ __device__ __forceinline__ void stage_flush(const TopkArgs& a, WarpStage& ws) {
     ws.count = 0;
 }
 
-// Test the VEC keys of one 16-byte vector (keys idx0 .. idx0 + VEC - 1)
-// against the threshold and stage the hits.  Called by all 32 lanes of a
-// warp together.
-template <bool W4, bool FUSE = false>
-__device__ __forceinline__ void filter_vector(const TopkArgs& a, const KeyLimit& lim, uint4 x, bool valid,
-                                              uint64_t idx0, WarpStage& ws) {
-    constexpr int VEC = W4 ? 4 : 2;
-    bool any;
-    if (W4) {
-        any = pass32(x.x, lim) | pass32(x.y, lim) | pass32(x.z, lim) | pass32(x.w, lim);
-    } else {
-        any = pass64(static_cast<uint64_t>(x.x) | (static_cast<uint64_t>(x.y) << 32), lim) |
-              pass64(static_cast<uint64_t>(x.z) | (static_cast<uint64_t>(x.w) << 32), lim);
-    }
-    if (!__any_sync(0xFFFFFFFFu, any && valid)) return;
-    unsigned hit = 0;
-    if (valid) {
-        if (W4) {
-            hit = (pass32(x.x, lim) ? 1u : 0u) | (pass32(x.y, lim) ? 2u : 0u) | (pass32(x.z, lim) ? 4u : 0u) |
-                  (pass32(x.w, lim) ? 8u : 0u);
-        } else {
-            hit = (pass64(static_cast<uint64_t>(x.x) | (static_cast<uint64_t>(x.y) << 32), lim) ? 1u : 0u) |
-                  (pass64(static_cast<uint64_t>(x.z) | (static_cast<uint64_t>(x.w) << 32), lim) ? 2u : 0u);
-        }
-    }
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned lt = (1u << lane) - 1u;
-    unsigned bal[VEC];
-    unsigned total = 0;
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) {
-        bal[e] = __ballot_sync(0xFFFFFFFFu, (hit >> e) & 1u);
-        total += __popc(bal[e]);
-    }
+// Stage the hits of a warp-vector: bit e of `hit` set for the lane's element e
+// of VEC, whose rank word is rank(e) and whose index is idx0 + e (all 32 lanes
+// call).  Most vectors that get here have one or two hits in all, so the
+// elements without any are skipped by one warp-wide OR.
+template <int VEC, bool FUSE, typename RankOf>
+__device__ __forceinline__ void stage_hits(const TopkArgs& a, unsigned hit, uint64_t idx0, WarpStage& ws, RankOf rank) {
+    const unsigned lt = (1u << (threadIdx.x & 31u)) - 1u;
+    const unsigned any = __reduce_or_sync(0xFFFFFFFFu, hit);
+    const unsigned total = __reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(__popc(hit)));
     if (ws.count + total > WS_CAP) stage_flush<FUSE>(a, ws);
     unsigned before = ws.count;
-    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
     for (int e = 0; e < VEC; ++e) {
-        if ((hit >> e) & 1u) {
-            const unsigned pos = before + __popc(bal[e] & lt);
-            uint64_t r;
-            if (W4) r = rank_key(w[e], a.kind, a.desc);
-            else r = rank_key(static_cast<uint64_t>(w[2 * e]) | (static_cast<uint64_t>(w[2 * e + 1]) << 32), a.kind, a.desc);
-            ws.r[pos] = r;
+        if (!((any >> e) & 1u)) continue;
+        const bool h = (hit >> e) & 1u;
+        const unsigned bal = __ballot_sync(0xFFFFFFFFu, h);
+        if (h) {
+            const unsigned pos = before + __popc(bal & lt);
+            ws.r[pos] = rank(e);
             ws.idx[pos] = static_cast<uint32_t>(idx0 + e);
         }
-        before += __popc(bal[e]);
+        before += __popc(bal);
     }
-    ws.count += total;
+    ws.count = before;
+}
+
+// Test the keys of one vector of NW 32-bit words (keys idx0 ...) against the
+// threshold and stage the hits.  Called by all 32 lanes of a warp together.
+template <bool W4, int NW, bool FUSE>
+__device__ __forceinline__ void filter_vector(const TopkArgs& a, const KeyLimit& lim, const uint32_t (&w)[NW],
+                                              bool valid, uint64_t idx0, WarpStage& ws) {
+    constexpr int VEC = W4 ? NW : NW / 2;
+    auto key = [&](int e) {
+        return W4 ? static_cast<uint64_t>(w[e]) : static_cast<uint64_t>(w[2 * e]) | (static_cast<uint64_t>(w[2 * e + 1]) << 32);
+    };
+    auto pass = [&](int e) { return W4 ? pass32(w[e], lim) : pass64(key(e), lim); };
+    bool any = false;
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) any = any | pass(e);
+    if (!__any_sync(0xFFFFFFFFu, any && valid)) return;
+    unsigned hit = 0;
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) hit |= (valid && pass(e)) ? (1u << e) : 0u;
+    stage_hits<VEC, FUSE>(a, hit, idx0, ws, [&](int e) { return rank_key(key(e), a.kind, a.desc); });
+}
+
+// One 32-byte streaming load (sm_100 and later): half as many load
+// instructions and votes per byte as 16-byte ones.  Read-only pass over 2^31
+// bytes, 64 bytes in flight per thread: 292.5 us, 315 us with 16-byte loads.
+__device__ __forceinline__ void ld_stream_32(const void* p, uint32_t (&w)[8]) {
+    uint64_t v[4];
+    asm volatile("ld.global.cs.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        w[2 * j] = static_cast<uint32_t>(v[j]);
+        w[2 * j + 1] = static_cast<uint32_t>(v[j] >> 32);
+    }
+}
+__device__ __forceinline__ void ld_stream_words(const void* p, uint32_t (&w)[8]) { ld_stream_32(p, w); }
+__device__ __forceinline__ void ld_stream_words(const void* p, uint32_t (&w)[4]) {
+    const uint4 v = ld_stream_v4(p);
+    w[0] = v.x;
+    w[1] = v.y;
+    w[2] = v.z;
+    w[3] = v.w;
 }
 
 // The unaligned head [0, head) and ragged tail [tail0, n) of the keys: at
-// most 2 * VEC - 2 keys, one per lane of warp 0 of CTA 0.
+// most 14 keys, one per lane of warp 0 of CTA 0.
 template <bool FUSE = false>
-__device__ __forceinline__ void filter_ends(const TopkArgs& a, uint64_t t, uint64_t head, uint64_t tail0) {
+__device__ __forceinline__ void filter_ends(const TopkArgs& a, uint64_t t, uint64_t head, uint64_t tail0,
+                                            WarpStage& ws) {
     if (blockIdx.x != 0 || threadIdx.x >= 32) return;
     const uint64_t rest = head + (a.n - tail0);
     const uint64_t j = threadIdx.x;
@@ -315,57 +465,154 @@ __device__ __forceinline__ void filter_ends(const TopkArgs& a, uint64_t t, uint6
         idx = j < head ? j : tail0 + (j - head);
         r = load_input(a, idx).r;
     }
-    const bool hit = valid && r <= t;
-    const unsigned bal = __ballot_sync(0xFFFFFFFFu, hit);
-    if (!bal) return;
-    unsigned long long base = 0;
-    if (threadIdx.x == 0) base = atomicAdd(&a.ctl->cand_count, static_cast<unsigned long long>(__popc(bal)));
-    base = __shfl_sync(0xFFFFFFFFu, base, 0);
-    if (hit) {
-        const unsigned long long pos = base + __popc(bal & ((1u << threadIdx.x) - 1u));
-        const uint32_t rid = a.rowids ? a.rowids[idx] : static_cast<uint32_t>(idx);
-        if (pos < a.cand_cap) {
-            a.cand_r[pos] = r;
-            a.cand_rid[pos] = rid;
-        }
-        if (FUSE) fuse_add(fuse_digit(a, t), r, rid);
+    stage_hits<1, FUSE>(a, valid && r <= t ? 1u : 0u, idx, ws, [&](int) { return r; });
+}
+
+// The last hits of all warps of the CTA, with one atomic on the global count
+// (one per warp is 4864 on one word at the end of the pass: 4 us).
+template <int TPB>
+__device__ __forceinline__ void cta_flush_fused(const TopkArgs& a, const WarpStage& ws) {
+    __shared__ unsigned cnts[TPB / 32];
+    __shared__ unsigned long long s_base;
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const FuseRange f = fuse_range(a);
+    if (lane == 0) cnts[warp] = ws.count;
+    __syncthreads();
+    unsigned before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < TPB / 32; ++w) {
+        if (w < static_cast<int>(warp)) before += cnts[w];
+        all += cnts[w];
     }
+    if (threadIdx.x == 0 && all) s_base = atomicAdd(&a.ctl->cand_count, static_cast<unsigned long long>(all));
+    __syncthreads();
+    if (all) stage_write_fused(a, f, ws.r, ws.idx, ws.count, s_base + before);
 }
 
 // Phase 1: the single streaming pass.  Appends (rank word, row-id) of every
-// key whose rank word is <= t; counts all of them.
-template <bool W4, int TPB>
-__device__ void filter_pass(const TopkArgs& a, uint64_t t, unsigned char* stage_smem) {
-    constexpr int W = W4 ? 4 : 8;
-    constexpr int VEC = 16 / W;
-    const uint64_t n = a.n;
-    const uintptr_t addr = reinterpret_cast<uintptr_t>(a.keys);
-    const uint64_t head0 = ((16 - (addr & 15)) & 15) / W;
-    const uint64_t head = head0 < n ? head0 : n;
-    const uint64_t nvec = (n - head) / VEC;
-    const uint64_t tail0 = head + nvec * VEC;
-    const unsigned char* vbase = static_cast<const unsigned char*>(a.keys) + head * W;
-    const KeyLimit lim = key_limit(t, a.kind, a.desc);
-    WarpStage ws = warp_stage(stage_smem);
-
-    const uint64_t per_block = static_cast<uint64_t>(TPB) * TK_UNROLL;
-    const uint64_t stride = per_block * gridDim.x;
-    for (uint64_t bb = per_block * blockIdx.x; bb < nvec; bb += stride) {
-        uint4 v[TK_UNROLL];
-#pragma unroll
-        for (int u = 0; u < TK_UNROLL; ++u) {
-            const uint64_t vi = bb + static_cast<uint64_t>(u) * TPB + threadIdx.x;
-            if (vi < nvec) v[u] = ld_stream_v4(vbase + vi * 16);
-            else v[u] = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
-        }
-#pragma unroll
-        for (int u = 0; u < TK_UNROLL; ++u) {
-            const uint64_t vi = bb + static_cast<uint64_t>(u) * TPB + threadIdx.x;
-            filter_vector<W4, true>(a, lim, v[u], vi < nvec, head + vi * VEC, ws);
-        }
+// key whose rank word is <= t; counts all of them.  Two 32-byte loads in
+// flight per thread, tested in one comparison per key and one vote per 64
+// bytes.  The first loads are issued before the threshold is known: the keys
+// are complete (the prepare kernel has waited for everything before it), so
+// only the threshold has to be waited for.  Bound by HBM: 2^28 int64 keys
+// 313 -> 303 us (7.1 TB/s); 2 * 10^7 float32 keys, with the final flush by
+// CTA, 24 -> 15 us of the kernel, most of it start and end.
+template <bool W4>
+struct FilterSpan {                            // the 32-byte vectors of the keys
+    static constexpr int W = W4 ? 4 : 8;
+    static constexpr int VEC = 32 / W;
+    uint64_t head, nvec, tail0;
+    const unsigned char* base;
+    __device__ explicit FilterSpan(const TopkArgs& a) {
+        const uint64_t head0 = ((32 - (reinterpret_cast<uintptr_t>(a.keys) & 31)) & 31) / W;
+        head = head0 < a.n ? head0 : a.n;
+        nvec = (a.n - head) / VEC;
+        tail0 = head + nvec * VEC;
+        base = static_cast<const unsigned char*>(a.keys) + head * W;
     }
-    stage_flush<true>(a, ws);
-    filter_ends<true>(a, t, head, tail0);
+};
+
+template <int TPB>
+__device__ __forceinline__ void filter_load(const unsigned char* base, uint64_t end, uint64_t bb,
+                                            uint32_t (&v)[TK_UNROLL][8]) {
+#pragma unroll
+    for (int u = 0; u < TK_UNROLL; ++u) {
+        const uint64_t vi = bb + static_cast<uint64_t>(u) * TPB + threadIdx.x;
+        ld_stream_words(base + (vi < end ? vi : 0) * 32, v[u]);
+    }
+}
+
+// The steps of a CTA: PER vectors each while whole rounds of the grid
+// remain; what is left after those is split evenly, so that no CTA has a
+// round more than another.
+struct FilterStep {
+    uint64_t bb, end;                          // vectors of the current step
+    uint64_t whole;                            // vectors of the whole rounds
+    __device__ void split(uint64_t nvec, uint64_t per) {      // after the last whole round
+        const uint64_t share = ((nvec - whole + gridDim.x - 1) / gridDim.x + 31) & ~31ull;
+        bb = min(nvec, whole + share * blockIdx.x);
+        end = min(nvec, bb + share);
+    }
+    __device__ void first(uint64_t nvec, uint64_t per) {
+        whole = nvec / (per * gridDim.x) * (per * gridDim.x);
+        bb = per * blockIdx.x;
+        end = bb + per;
+        if (bb >= whole) split(nvec, per);
+    }
+    __device__ void next(uint64_t nvec, uint64_t per) {
+        if (bb >= whole) {
+            bb = end;
+            return;
+        }
+        bb += per * gridDim.x;
+        end = bb + per;
+        if (bb >= whole) split(nvec, per);
+    }
+};
+
+template <bool W4, int TPB, int MODE>
+__device__ __forceinline__ void filter_loop(const TopkArgs& a, const FilterSpan<W4>& sp, uint64_t lim, FilterStep st,
+                                            uint32_t (&v)[TK_UNROLL][8], WarpStage& ws) {
+    constexpr int VEC = FilterSpan<W4>::VEC;
+    constexpr uint64_t PER = static_cast<uint64_t>(TPB) * TK_UNROLL;
+    auto key = [&](int u, int e) {
+        return W4 ? static_cast<uint64_t>(v[u][e])
+                  : static_cast<uint64_t>(v[u][2 * e]) | (static_cast<uint64_t>(v[u][2 * e + 1]) << 32);
+    };
+    auto pass = [&](int u, int e) {
+        return W4 ? key_pass<MODE, uint32_t, int32_t>(v[u][e], static_cast<uint32_t>(lim))
+                  : key_pass<MODE, uint64_t, int64_t>(key(u, e), lim);
+    };
+    while (st.bb < st.end) {
+        bool any = false;
+#pragma unroll
+        for (int u = 0; u < TK_UNROLL; ++u)
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) any = any | pass(u, e);
+        if (__any_sync(0xFFFFFFFFu, any)) {
+#pragma unroll
+            for (int u = 0; u < TK_UNROLL; ++u) {
+                const uint64_t vi = st.bb + static_cast<uint64_t>(u) * TPB + threadIdx.x;
+                unsigned hit = 0;
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) hit |= (vi < st.end && pass(u, e)) ? (1u << e) : 0u;
+                if (__any_sync(0xFFFFFFFFu, hit != 0))
+                    stage_hits<VEC, true>(a, hit, sp.head + vi * VEC, ws,
+                                          [&](int e) { return rank_key(key(u, e), a.kind, a.desc); });
+            }
+        }
+        st.next(sp.nvec, PER);
+        if (st.bb < st.end) filter_load<TPB>(sp.base, st.end, st.bb, v);
+    }
+}
+
+template <bool W4, int TPB>
+__device__ void filter_pass(const TopkArgs& a, unsigned char* stage_smem) {
+    const FilterSpan<W4> sp(a);
+    FilterStep st;
+    st.first(sp.nvec, static_cast<uint64_t>(TPB) * TK_UNROLL);
+    uint32_t v[TK_UNROLL][8];
+    if (st.bb < st.end) filter_load<TPB>(sp.base, st.end, st.bb, v);
+    wait_prior_grid();
+    allow_next_grid();
+    const uint64_t t = __ldcg(&a.ctl->thresh);
+    const KeyLimit kl = key_limit(t, a.kind, a.desc);
+    uint64_t lim;
+    int mode;
+    if (W4) {
+        uint32_t l32;
+        mode = key_cmp<uint32_t>(kl.m32, kl.c32, &l32);
+        lim = l32;
+    } else {
+        mode = key_cmp<uint64_t>(kl.m64, kl.c64, &lim);
+    }
+    WarpStage ws = warp_stage(stage_smem);
+    if (mode == CMP_GE_U) filter_loop<W4, TPB, CMP_GE_U>(a, sp, lim, st, v, ws);
+    else if (mode == CMP_LE_U) filter_loop<W4, TPB, CMP_LE_U>(a, sp, lim, st, v, ws);
+    else if (mode == CMP_GE_S) filter_loop<W4, TPB, CMP_GE_S>(a, sp, lim, st, v, ws);
+    else filter_loop<W4, TPB, CMP_LE_S>(a, sp, lim, st, v, ws);
+    filter_ends<true>(a, t, sp.head, sp.tail0, ws);
+    cta_flush_fused<TPB>(a, ws);
 }
 
 // The 32-bit order-preserving transform of one 4-byte key kind as two masks:
@@ -386,102 +633,76 @@ __device__ __forceinline__ uint32_t rank32(uint32_t b, Rank32 m) {
     return b ^ (static_cast<uint32_t>(static_cast<int32_t>(b) >> 31) & m.flip) ^ m.fixed;
 }
 
-// Stage the hits among the four rows of one 16-byte vector of each column.
-__device__ __forceinline__ void filter_vector_pair(const TopkArgs& a, uint64_t t, Rank32 m0, Rank32 m1, uint4 x0,
-                                                   uint4 x1, bool valid, uint64_t idx0, WarpStage& ws) {
-    const uint32_t c0[4] = {x0.x, x0.y, x0.z, x0.w}, c1[4] = {x1.x, x1.y, x1.z, x1.w};
-    uint64_t r[4];
-    unsigned hit = 0;
+// Phase 1 for a two-column key: both columns streamed with vector loads when
+// they share their alignment (a scalar head and tail around the vectors; 32
+// bytes of each column per load, 16 when they share only that), else row by
+// row; every row whose composite rank word is <= t is appended.
+template <int TPB, int NW>
+__device__ void filter_pass_pair_vec(const TopkArgs& a, uint64_t t, WarpStage& ws) {
+    constexpr int U = 8 / NW;                  // 32 bytes of each column in flight per thread
+    constexpr int VB = NW * 4;
+    const uint64_t n = a.n;
+    const Rank32 m0 = rank32_of(a.kind, a.desc), m1 = rank32_of(a.kind2, a.desc2);
+    const uint32_t t0 = static_cast<uint32_t>(t >> 32);
+    const uintptr_t a0 = reinterpret_cast<uintptr_t>(a.keys);
+    const uint64_t head0 = ((VB - (a0 & (VB - 1))) & (VB - 1)) / 4;
+    const uint64_t head = head0 < n ? head0 : n;
+    const uint64_t nvec = (n - head) / NW;
+    const uint64_t tail0 = head + nvec * NW;
+    const unsigned char* v0 = static_cast<const unsigned char*>(a.keys) + head * 4;
+    const unsigned char* v1 = static_cast<const unsigned char*>(a.keys2) + head * 4;
+    const uint64_t per_block = static_cast<uint64_t>(TPB) * U;
+    const uint64_t stride = per_block * gridDim.x;
+    for (uint64_t bb = per_block * blockIdx.x; bb < nvec; bb += stride) {
+        uint32_t x0[U][NW], x1[U][NW];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        r[e] = (static_cast<uint64_t>(rank32(c0[e], m0)) << 32) | rank32(c1[e], m1);
-        hit |= (valid && r[e] <= t) ? (1u << e) : 0u;
-    }
-    if (!__any_sync(0xFFFFFFFFu, hit != 0)) return;
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned lt = (1u << lane) - 1u;
-    unsigned bal[4];
-    unsigned total = 0;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        bal[e] = __ballot_sync(0xFFFFFFFFu, (hit >> e) & 1u);
-        total += __popc(bal[e]);
-    }
-    if (ws.count + total > WS_CAP) stage_flush<true>(a, ws);
-    unsigned before = ws.count;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        if ((hit >> e) & 1u) {
-            const unsigned pos = before + __popc(bal[e] & lt);
-            ws.r[pos] = r[e];
-            ws.idx[pos] = static_cast<uint32_t>(idx0 + e);
+        for (int u = 0; u < U; ++u) {
+            const uint64_t vi = bb + static_cast<uint64_t>(u) * TPB + threadIdx.x;
+            const uint64_t at = (vi < nvec ? vi : 0) * VB;
+            ld_stream_words(v0 + at, x0[u]);
+            ld_stream_words(v1 + at, x1[u]);
         }
-        before += __popc(bal[e]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint64_t vi = bb + static_cast<uint64_t>(u) * TPB + threadIdx.x;
+            auto rank = [&](int e) { return (static_cast<uint64_t>(rank32(x0[u][e], m0)) << 32) | rank32(x1[u][e], m1); };
+            // few rows pass on the first column alone, and those are tested whole
+            bool any = false;
+#pragma unroll
+            for (int e = 0; e < NW; ++e) any = any | (rank32(x0[u][e], m0) <= t0);
+            if (!__any_sync(0xFFFFFFFFu, any)) continue;
+            unsigned hit = 0;
+#pragma unroll
+            for (int e = 0; e < NW; ++e) hit |= (vi < nvec && rank(e) <= t) ? (1u << e) : 0u;
+            if (!__any_sync(0xFFFFFFFFu, hit != 0)) continue;
+            stage_hits<NW, true>(a, hit, head + vi * NW, ws, rank);
+        }
     }
-    ws.count += total;
+    filter_ends<true>(a, t, head, tail0, ws);
 }
-
-// Phase 1 for a two-column key: both columns streamed with 16-byte loads when
-// they share their alignment (a scalar head and tail around the vectors),
-// else row by row; every row whose composite rank word is <= t is appended.
-constexpr int TK_PAIR_UNROLL = 2;          // vector pairs (32 bytes) in flight per thread
 
 template <int TPB>
 __device__ void filter_pass_pair(const TopkArgs& a, uint64_t t, unsigned char* stage_smem) {
     const uint64_t n = a.n;
-    const Rank32 m0 = rank32_of(a.kind, a.desc), m1 = rank32_of(a.kind2, a.desc2);
-    const uintptr_t a0 = reinterpret_cast<uintptr_t>(a.keys), a1 = reinterpret_cast<uintptr_t>(a.keys2);
+    const uintptr_t off = reinterpret_cast<uintptr_t>(a.keys) ^ reinterpret_cast<uintptr_t>(a.keys2);
     WarpStage ws = warp_stage(stage_smem);
+    if ((off & 31) == 0) {
+        filter_pass_pair_vec<TPB, 8>(a, t, ws);
+    } else if ((off & 15) == 0) {
+        filter_pass_pair_vec<TPB, 4>(a, t, ws);
+    } else {
     const unsigned lane = threadIdx.x & 31u;
-    if (((a0 ^ a1) & 15) == 0) {
-        const uint64_t head0 = ((16 - (a0 & 15)) & 15) / 4;
-        const uint64_t head = head0 < n ? head0 : n;
-        const uint64_t nvec = (n - head) / 4;
-        const uint64_t tail0 = head + nvec * 4;
-        const unsigned char* v0 = static_cast<const unsigned char*>(a.keys) + head * 4;
-        const unsigned char* v1 = static_cast<const unsigned char*>(a.keys2) + head * 4;
-        const uint64_t per_block = static_cast<uint64_t>(TPB) * TK_PAIR_UNROLL;
-        const uint64_t stride = per_block * gridDim.x;
-        for (uint64_t bb = per_block * blockIdx.x; bb < nvec; bb += stride) {
-            uint4 x0[TK_PAIR_UNROLL], x1[TK_PAIR_UNROLL];
-#pragma unroll
-            for (int u = 0; u < TK_PAIR_UNROLL; ++u) {
-                const uint64_t vi = bb + static_cast<uint64_t>(u) * TPB + threadIdx.x;
-                if (vi < nvec) {
-                    x0[u] = ld_stream_v4(v0 + vi * 16);
-                    x1[u] = ld_stream_v4(v1 + vi * 16);
-                } else {
-                    x0[u] = x1[u] = make_uint4(0, 0, 0, 0);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < TK_PAIR_UNROLL; ++u) {
-                const uint64_t vi = bb + static_cast<uint64_t>(u) * TPB + threadIdx.x;
-                filter_vector_pair(a, t, m0, m1, x0[u], x1[u], vi < nvec, head + vi * 4, ws);
-            }
-        }
-        stage_flush<true>(a, ws);
-        filter_ends<true>(a, t, head, tail0);
-        return;
-    }
     const uint64_t stride = static_cast<uint64_t>(TPB) * gridDim.x;
-    const uint64_t lt = (1u << lane) - 1u;
     for (uint64_t wb = static_cast<uint64_t>(blockIdx.x) * TPB + (threadIdx.x & ~31u); wb < n; wb += stride) {
         const uint64_t i = wb + lane;
         uint64_t r = ~0ull;
         if (i < n) r = pair_rank(static_cast<const uint32_t*>(a.keys)[i], static_cast<const uint32_t*>(a.keys2)[i], a);
         const bool hit = i < n && r <= t;
-        const unsigned bal = __ballot_sync(0xFFFFFFFFu, hit);
-        if (!bal) continue;
-        if (ws.count + __popc(bal) > WS_CAP) stage_flush<true>(a, ws);
-        if (hit) {
-            const unsigned pos = ws.count + __popc(bal & static_cast<unsigned>(lt));
-            ws.r[pos] = r;
-            ws.idx[pos] = static_cast<uint32_t>(i);
-        }
-        ws.count += __popc(bal);
+        if (!__any_sync(0xFFFFFFFFu, hit)) continue;
+        stage_hits<1, true>(a, hit ? 1u : 0u, i, ws, [&](int) { return r; });
     }
-    stage_flush<true>(a, ws);
+    }
+    cta_flush_fused<TPB>(a, ws);
 }
 
 // Issue the bulk copy of the tile at byte offset `off` of the key body into
@@ -558,7 +779,8 @@ __device__ bool filter_pass_bulk(const TopkArgs& a, uint64_t t, unsigned char* s
             const bool valid = v < nv;
             uint4 x = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
             if (valid) x = ld_shared_v4(st + v * 16);
-            filter_vector<W4>(a, lim, x, valid, idx_base + static_cast<uint64_t>(v) * VEC, ws);
+            const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
+            filter_vector<W4, 4, false>(a, lim, xw, valid, idx_base + static_cast<uint64_t>(v) * VEC, ws);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);
@@ -577,6 +799,7 @@ __device__ bool filter_pass_bulk(const TopkArgs& a, uint64_t t, unsigned char* s
             par ^= 1u;
         }
     }
+    filter_ends(a, t, head, tail0, ws);
     stage_flush(a, ws);
     if (!__syncthreads_and(ok)) {
         // Let the copies this CTA issued land before leaving.  Only the last
@@ -591,82 +814,71 @@ __device__ bool filter_pass_bulk(const TopkArgs& a, uint64_t t, unsigned char* s
         __syncthreads();
         return false;
     }
-    filter_ends(a, t, head, tail0);
     return true;
 }
 
-__device__ __forceinline__ unsigned long long gtimer() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// One refine pass: histogram of digit [L, L+d) of the composites that match
-// the prefix, merged into `gh`, and the AND / OR of those composites merged
-// into `ao`.  `gz` and `az` (the buffers of the pass after next) are reset by
+// One refine pass: histogram of the bins of the entries in the interval,
+// merged into `gh`, and the minima and maxima of those entries merged into
+// `mm`.  `gz` and `mz` (the buffers of the pass after next) are reset by
 // CTA 0.
-__device__ void hist_pass(const TopkArgs& a, bool cand, uint64_t src_n, uint64_t p0, uint64_t p1,
-                          int L, int d, int kb, unsigned* gh, unsigned* gz, unsigned* sh, unsigned long long* ao,
-                          unsigned long long* az) {
+__device__ void hist_pass(const TopkArgs& a, bool cand, uint64_t src_n, const Range& g, int shift, unsigned* gh,
+                          unsigned* gz, unsigned* sh, unsigned long long* mm, unsigned long long* mz) {
     for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB) sh[b] = 0;
     if (blockIdx.x == 0) {
         for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB) gz[b] = 0;
-        if (threadIdx.x == 0) {
-            az[0] = az[1] = ~0ull;
-            az[2] = az[3] = 0ull;
-        }
+        if (threadIdx.x == 0) fold_reset(mz);
     }
     __syncthreads();
-    uint64_t acc[4] = {~0ull, ~0ull, 0ull, 0ull};
+    Fold acc = fold_none();
     const uint64_t stride = static_cast<uint64_t>(TK_TPB) * gridDim.x;
     const unsigned lane = threadIdx.x & 31u;
     for (uint64_t wb = static_cast<uint64_t>(blockIdx.x) * TK_TPB + (threadIdx.x & ~31u); wb < src_n;
          wb += stride) {
         const uint64_t i = wb + lane;
-        unsigned dig = 0xFFFFFFFFu;
+        unsigned bin = 0xFFFFFFFFu;
         if (i < src_n) {
             const Elem e = load_src(a, cand, i);
-            uint64_t w0, w1;
-            comp_words(e.r, e.rid, kb, w0, w1);
-            if (prefix_cmp(w0, w1, p0, p1, L) == 0) {
-                dig = comp_digit(w0, w1, L, d);
-                and_or(w0, w1, acc);
+            if (range_cmp(g, e.r, e.rid) == 0) {
+                bin = range_bin(g, shift, e.r, e.rid);
+                fold_add(acc, e.r, e.rid);
             }
         }
-        const unsigned peers = __match_any_sync(0xFFFFFFFFu, dig);
-        if (dig != 0xFFFFFFFFu && lane == static_cast<unsigned>(__ffs(peers) - 1))
-            atomicAdd(&sh[dig], static_cast<unsigned>(__popc(peers)));
+        const unsigned peers = __match_any_sync(0xFFFFFFFFu, bin);
+        if (bin != 0xFFFFFFFFu && lane == static_cast<unsigned>(__ffs(peers) - 1))
+            atomicAdd(&sh[bin], static_cast<unsigned>(__popc(peers)));
     }
-    and_or_merge<TK_TPB>(acc, ao);
+    fold_merge<TK_TPB>(acc, mm);
     for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB)
         if (sh[b]) atomicAdd(&gh[b], sh[b]);
 }
 
-// Split: entries below the prefix are selected (appended to out), entries
-// equal to it go to the small buffer, or straight to out when all of them
+// Split: entries below the interval are selected (appended to out), entries
+// in it go to the small buffer, or straight to out when all of them
 // (or any `krem` identical ones) are taken.
-// With FOLD, the AND / OR of the entries it writes to out (those below the
-// prefix, and with take_all the equal ones it keeps) is merged into
-// ctl->fin for the larger-K finish, which then needs no pass of its own.
+// With FOLD, the minima and maxima of the entries it writes to out (those
+// below the interval, and with take_all the ones in it that it keeps) are
+// merged into ctl->fin for the larger-K finish, which then needs no pass of
+// its own.  `nx` is the thread's first candidate on the candidate path; every
+// entry is loaded one step ahead.
 template <bool FOLD>
-__device__ void split_pass(const TopkArgs& a, bool cand, uint64_t src_n, uint64_t p0, uint64_t p1,
-                           int L, int kb, bool take_all, uint64_t krem) {
+__device__ void split_pass(const TopkArgs& a, bool cand, uint64_t src_n, const Range& g, bool take_all,
+                           uint64_t krem, Elem nx) {
     TopkCtl* ctl = a.ctl;
-    uint64_t acc[4] = {~0ull, ~0ull, 0ull, 0ull};
+    Fold acc = fold_none();
     const uint64_t stride = static_cast<uint64_t>(TK_TPB) * gridDim.x;
     const unsigned lane = threadIdx.x & 31u;
     const uint64_t eq_base = a.k - krem;
+    if (!cand) {
+        const uint64_t i0 = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x;
+        if (i0 < src_n) nx = load_src(a, cand, i0);
+    }
     for (uint64_t wb = static_cast<uint64_t>(blockIdx.x) * TK_TPB + (threadIdx.x & ~31u); wb < src_n;
          wb += stride) {
         const uint64_t i = wb + lane;
         int c = 1;
-        Elem e{0, 0};
-        uint64_t w0 = 0, w1 = 0;
-        if (i < src_n) {
-            e = load_src(a, cand, i);
-            comp_words(e.r, e.rid, kb, w0, w1);
-            c = prefix_cmp(w0, w1, p0, p1, L);
-        }
+        const Elem e = nx;
+        if (i < src_n) c = range_cmp(g, e.r, e.rid);
+        if (i + stride < src_n) nx = load_src(a, cand, i + stride);
         const unsigned lt = __ballot_sync(0xFFFFFFFFu, c < 0);
         const unsigned eq = __ballot_sync(0xFFFFFFFFu, c == 0);
         if (lt) {
@@ -677,7 +889,7 @@ __device__ void split_pass(const TopkArgs& a, bool cand, uint64_t src_n, uint64_
                 const uint64_t pos = base + __popc(lt & ((1u << lane) - 1u));
                 a.out_r0[pos] = e.r;
                 a.out_rid0[pos] = e.rid;
-                if (FOLD) and_or(w0, w1, acc);
+                if (FOLD) fold_add(acc, e.r, e.rid);
             }
         }
         if (eq) {
@@ -691,7 +903,7 @@ __device__ void split_pass(const TopkArgs& a, bool cand, uint64_t src_n, uint64_
                     if (pos < krem) {
                         a.out_r0[eq_base + pos] = e.r;
                         a.out_rid0[eq_base + pos] = e.rid;
-                        if (FOLD) and_or(w0, w1, acc);
+                        if (FOLD) fold_add(acc, e.r, e.rid);
                     }
                 } else if (pos < TK_SMALL) {
                     a.small_r[pos] = e.r;
@@ -700,7 +912,7 @@ __device__ void split_pass(const TopkArgs& a, bool cand, uint64_t src_n, uint64_
             }
         }
     }
-    if (FOLD) and_or_merge<TK_TPB>(acc, ctl->fin);
+    if (FOLD) fold_merge<TK_TPB>(acc, ctl->fin);
 }
 
 // Merge-path split: how many of the first `diag` outputs of the merge of
@@ -734,9 +946,11 @@ __global__ void __launch_bounds__(TK_TPB) topk_prepare_kernel(TopkArgs a) {
     __shared__ unsigned long long sc[24];
     __shared__ int last;
     TopkCtl* ctl = a.ctl;
+    wait_prior_grid();                    // the call before may still read the control block
     allow_next_grid();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctl->ts[0] = gtimer();
+        a.bar->count = 0;
         ctl->cand_count = 0;
         ctl->out_count = 0;
         ctl->eq_count = 0;
@@ -744,13 +958,9 @@ __global__ void __launch_bounds__(TK_TPB) topk_prepare_kernel(TopkArgs a) {
         ctl->err = 0;
         ctl->path = a.use_sample ? 1 : 0;
         ctl->passes = 0;
-        ctl->thresh = ~0ull;
-        for (int s = 0; s < 3; ++s) {
-            ctl->ao[s][0] = ctl->ao[s][1] = ~0ull;
-            ctl->ao[s][2] = ctl->ao[s][3] = 0ull;
-        }
-        ctl->fin[0] = ctl->fin[1] = ~0ull;
-        ctl->fin[2] = ctl->fin[3] = 0ull;
+        ctl->flow = 0;
+        for (int s = 0; s < 3; ++s) fold_reset(ctl->mm[s]);
+        fold_reset(ctl->fin);
     }
     for (int b = blockIdx.x * TK_TPB + threadIdx.x; b < 3 * TK_BINS; b += gridDim.x * TK_TPB) a.ghist[b] = 0;
     if (!a.use_sample) {
@@ -765,11 +975,7 @@ __global__ void __launch_bounds__(TK_TPB) topk_prepare_kernel(TopkArgs a) {
     __syncthreads();
     if (!last) return;
     __threadfence();
-    const uint64_t t = sample_threshold(a, sh, sc);
-    if (threadIdx.x == 0) {
-        ctl->thresh = t;
-        ctl->ts[1] = gtimer();
-    }
+    sample_threshold(a, sh, sc);
 }
 
 // Kernel 2 of 3 (sampled path only): the single streaming pass over the keys,
@@ -778,6 +984,7 @@ template <bool W4>
 __global__ void __launch_bounds__(TKF_TPB, 4) topk_filter_bulk_kernel(TopkArgs a) {
     extern __shared__ __align__(128) unsigned char fsmem[];
     wait_prior_grid();
+    allow_next_grid();
     const uint64_t t = __ldcg(&a.ctl->thresh);
     filter_pass_bulk<W4, TKF_TPB>(a, t, fsmem);
 }
@@ -788,9 +995,7 @@ template <bool W4, int TPB>
 __global__ void __launch_bounds__(TPB, 1024 / TPB) topk_filter_regs_kernel(TopkArgs a) {
     extern __shared__ __align__(16) unsigned char stage[];
     fuse_init<TPB>();
-    wait_prior_grid();
-    const uint64_t t = __ldcg(&a.ctl->thresh);
-    filter_pass<W4, TPB>(a, t, stage);
+    filter_pass<W4, TPB>(a, stage);
     fuse_merge<TPB>(a);
 }
 
@@ -800,6 +1005,7 @@ __global__ void __launch_bounds__(TPB, 1024 / TPB) topk_filter_pair_kernel(TopkA
     extern __shared__ __align__(16) unsigned char stage[];
     fuse_init<TPB>();
     wait_prior_grid();
+    allow_next_grid();
     const uint64_t t = __ldcg(&a.ctl->thresh);
     filter_pass_pair<TPB>(a, t, stage);
     fuse_merge<TPB>(a);
@@ -810,72 +1016,82 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long sc[24];
     TopkCtl* ctl = a.ctl;
-    const int kb = a.w4 ? 32 : 64;
-    const int TB = kb + 32;
     unsigned* sh = reinterpret_cast<unsigned*>(smem);
     uint64_t* sr = reinterpret_cast<uint64_t*>(smem);
     uint32_t* srid = reinterpret_cast<uint32_t*>(smem + TK_RANK_MAX * 8);
 
     wait_prior_grid();
+    allow_next_grid();
     const bool stamp = blockIdx.x == 0 && threadIdx.x == 0;
     if (stamp) ctl->ts[2] = gtimer();
+    unsigned bar_target = 0;                                 // of the grid barriers
     // Source of the selection: the candidates of the streaming pass when the
     // sample judged well (at least k of them, all stored), else the input.
     bool cand = false;
     uint64_t src_n = a.n;
+    uint64_t low = 0;                                        // candidates below the fused interval
+    FuseRange fr{};
+    unsigned hv0[TK_BINS / TK_TPB];                          // the thread's bins of the fused pass
+    Elem first{0, 0};                                        // the thread's first candidate
     if (a.use_sample) {
-        if (ld_volatile_i32(&ctl->err) != 0) return report(a);
+        // all that the first steps need, in one round trip to L2
+        const int err = __ldcg(&ctl->err);
         const uint64_t cnt = __ldcg(&ctl->cand_count);
+        fr = fuse_range(a);
+        low = __ldcg(&ctl->flow);
+        pick_load_global<TK_TPB>(a.ghist, hv0);
+        const uint64_t i0 = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x;
+        if (i0 < a.cand_cap) first = Elem{__ldcg(a.cand_r + i0), __ldcg(a.cand_rid + i0)};
+        if (err != 0) return report(a);
         cand = cnt >= a.k && cnt <= a.cand_cap;
         if (cand) src_n = cnt;
         if (stamp) ctl->path = cand ? 1 : 2;
     }
     const unsigned long long use_ts3 = stamp ? gtimer() : 0ull;
 
-    // Phase 2: radix refine of the (rank word, row-id) prefix.  Candidates are
-    // all at or below the threshold, so they share its leading zero bits: the
-    // refine starts below them.
-    uint64_t p0 = 0, p1 = 0, krem = a.k, bcnt = src_n;
-    int L = 0, pass = 0, npass = 0;
-    if (cand) {
-        const int lz = __clzll(static_cast<long long>(__ldcg(&ctl->thresh)));
-        L = lz < kb ? lz : kb;
-    }
+    // Phase 2: refine the interval that holds the K-th entry.  Candidates are
+    // all at or below the threshold.
+    Range g{0ull, cand ? fr.g.rhi : max_rank(a), 0u, max_rowid(a)};
+    uint64_t krem = a.k, bcnt = src_n;
+    int pass = 0, npass = 0;
     // With the filter's fused first pass, pass 0's histogram is ready on the
     // candidate path; on the fallback path it holds the filter's partial
     // counts, so the passes start at buffer 1 (clean) and pass 2 clears
     // buffer 0 before pass 3 uses it.
     bool ready = a.fuse && cand;
     if (a.fuse && !cand) pass = 1;
-    while (bcnt > TK_SMALL && L < TB && krem < bcnt) {
-        const int d = min(a.digit, TB - L);
-        unsigned* gh = a.ghist + (pass % 3) * TK_BINS;
-        unsigned* gz = a.ghist + ((pass + 1) % 3) * TK_BINS;
-        unsigned long long* ao = ctl->ao[pass % 3];
-        const bool fused_pass = ready;
-        if (!ready) {
-            hist_pass(a, cand, src_n, p0, p1, L, d, kb, gh, gz, sh, ao, ctl->ao[(pass + 1) % 3]);
-            if (!grid_sync(a.bar, &ctl->err)) return report(a);
+    if (ready && bcnt > TK_SMALL && krem < bcnt) {
+        if (low >= a.k) {
+            g.rhi = fr.g.rlo - 1;
+            if (a.w4) g.rhi &= 0xFFFFFFFF00000000ull;
+            bcnt = low;
+        } else {
+            const Pick pk = pick_loaded<TK_TPB>(hv0, a.k - low, sc);
+            krem = a.k - low - pk.below;
+            bcnt = pk.in_b;
+            g = range_narrow(a, fr.g, fr.sh, pk.b);
         }
         ready = false;
+        ++pass;
         ++npass;
-        const Pick pk = pick_bucket<TK_TPB>(gh, krem, sc);
-        // every matching entry in one bucket (the fused pass folds no AND / OR)
-        const bool whole = pk.below == 0 && pk.in_b == bcnt && !fused_pass;
+    }
+    while (bcnt > TK_SMALL && !range_point(g) && krem < bcnt) {
+        const int shift = range_shift(g, a.digit);
+        unsigned* gh = a.ghist + (pass % 3) * TK_BINS;
+        unsigned* gz = a.ghist + ((pass + 1) % 3) * TK_BINS;
+        unsigned long long* mm = ctl->mm[pass % 3];
+        hist_pass(a, cand, src_n, g, shift, gh, gz, sh, mm, ctl->mm[(pass + 1) % 3]);
+        if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
+        ++npass;
+        unsigned hv[TK_BINS / TK_TPB];
+        pick_load_global<TK_TPB>(gh, hv);
+        const Pick pk = pick_loaded<TK_TPB>(hv, krem, sc);
+        // every entry of the interval in one bin: go on with the interval that
+        // their minima and maxima span
+        const bool whole = pk.below == 0 && pk.in_b == bcnt;
         krem -= pk.below;
         bcnt = pk.in_b;
-        prefix_set(p0, p1, L, d, pk.b);
-        L += d;
-        if (whole) {
-            // The bucket holds exactly the entries the AND / OR saw: their
-            // common bits join the prefix and the next digit starts where
-            // they first differ.
-            const int f = first_diff(ao, TB);
-            if (f > L) {
-                prefix_copy(p0, p1, __ldcg(ao + 0), __ldcg(ao + 1), L, f);
-                L = f;
-            }
-        }
+        g = whole ? range_of(a, mm) : range_narrow(a, g, shift, pk.b);
         ++pass;
     }
     // The buffer at pass % 3 must be clean for the finish: when the fused
@@ -887,22 +1103,22 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
         ctl->ts[4] = gtimer();
     }
 
-    // Phase 3: split around the prefix.
-    const bool take_all = (krem == bcnt) || (L >= TB);
-    // the larger-K finish wants the AND / OR of the entries split writes out
+    // Phase 3: split around the interval.
+    const bool take_all = (krem == bcnt) || range_point(g);
+    // the larger-K finish wants the span of the entries split writes out
     const bool large = (take_all ? a.k : a.k - krem) + (take_all ? 0 : bcnt) > TK_RANK_MAX;
     if (large)
-        split_pass<true>(a, cand, src_n, p0, p1, L, kb, take_all, krem);
+        split_pass<true>(a, cand, src_n, g, take_all, krem, first);
     else
-        split_pass<false>(a, cand, src_n, p0, p1, L, kb, take_all, krem);
-    if (!grid_sync(a.bar, &ctl->err)) return report(a);
+        split_pass<false>(a, cand, src_n, g, take_all, krem, first);
+    if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
     if (stamp) ctl->ts[5] = gtimer();
 
     // Phase 4, survivors that fit one CTA's shared memory (every K <= 4096):
     // each warp of the grid takes survivors one at a time and computes its
     // final position as its rank -- the number of entries of its own set
     // that order before it (equal entries by position), so ranks are
-    // distinct.  The "below" entries (prefix < P) precede every bucket entry;
+    // distinct.  The "below" entries precede every bucket entry;
     // a bucket entry is kept when its rank within the bucket is below krem.
     {
         const uint64_t nb = take_all ? a.k : a.k - krem;     // out_r0[0, nb)
@@ -950,10 +1166,10 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
 
     // Phase 4, larger K.  (a) The bucket entries (ns <= 4096) are ranked by
     // the grid as above and the first krem written at their final positions.
-    // (b) The below entries are partitioned on the 12-bit digit at the refine
-    // start L0 -- a histogram, a scan, a scatter into out_r1 -- and every
-    // bucket of at most TK_SMALL entries is ranked in one CTA's shared memory
-    // and written at its final positions.  Skewed inputs with a larger bucket
+    // (b) The below entries are partitioned into the 4096 bins of the interval
+    // they span -- a histogram, a scan, a scatter into out_r1 -- and every
+    // bin of at most TK_SMALL entries is ranked in one CTA's shared memory
+    // and written at its final positions.  Skewed inputs with a larger bin
     // fall back to tile sorts and merge-path rounds.
     {
         const uint64_t nb = take_all ? a.k : a.k - krem;
@@ -981,12 +1197,11 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
             }
             __syncthreads();
         }
-        // (b) partition histogram of the below entries, on the digit that
-        // starts at the first bit where they differ (their AND / OR, folded
-        // by the split pass that wrote them), so that clustered keys and ties
-        // on the key spread over the buckets.
-        const int L0 = min(first_diff(ctl->fin, TB), TB - 1);
-        const int dp = min(a.digit, TB - L0);
+        // (b) partition histogram of the below entries over the interval they
+        // span (folded by the split pass that wrote them), so that clustered
+        // keys and ties on the key spread over the bins.
+        const Range pr = range_of(a, ctl->fin);
+        const int psh = range_shift(pr, a.digit);
         unsigned* ph = a.ghist + (pass % 3) * TK_BINS;          // clean (zeroed by the last pass or prepare)
         unsigned* pc = a.ghist + ((pass + 1) % 3) * TK_BINS;    // cursors, zeroed here
         for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB) sh[b] = 0;
@@ -997,11 +1212,7 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
         for (uint64_t wb = static_cast<uint64_t>(blockIdx.x) * TK_TPB + (threadIdx.x & ~31u); wb < nb; wb += gstride) {
             const uint64_t i = wb + lane;
             unsigned dig = 0xFFFFFFFFu;
-            if (i < nb) {
-                uint64_t w0, w1;
-                comp_words(__ldcg(a.out_r0 + i), __ldcg(a.out_rid0 + i), kb, w0, w1);
-                dig = comp_digit(w0, w1, L0, dp);
-            }
+            if (i < nb) dig = range_bin(pr, psh, __ldcg(a.out_r0 + i), __ldcg(a.out_rid0 + i));
             const unsigned peers = __match_any_sync(0xFFFFFFFFu, dig);
             if (dig != 0xFFFFFFFFu && lane == static_cast<unsigned>(__ffs(peers) - 1))
                 atomicAdd(&sh[dig], static_cast<unsigned>(__popc(peers)));
@@ -1009,7 +1220,7 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
         __syncthreads();
         for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB)
             if (sh[b]) atomicAdd(&ph[b], sh[b]);
-        if (!grid_sync(a.bar, &ctl->err)) return report(a);
+        if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
         // Scan of the partition histogram (every CTA), largest bucket.
         constexpr int PER = TK_BINS / TK_TPB;
         unsigned v[PER];
@@ -1039,14 +1250,12 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
             for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x; i < nb; i += gstride) {
                 const uint64_t er = __ldcg(a.out_r0 + i);
                 const uint32_t erid = __ldcg(a.out_rid0 + i);
-                uint64_t w0, w1;
-                comp_words(er, erid, kb, w0, w1);
-                const unsigned d = comp_digit(w0, w1, L0, dp);
+                const unsigned d = range_bin(pr, psh, er, erid);
                 const unsigned pos = off[d] + atomicAdd(&pc[d], 1u);
                 a.out_r1[pos] = er;
                 a.out_rid1[pos] = erid;
             }
-            if (!grid_sync(a.bar, &ctl->err)) return report(a);
+            if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
             // Buckets of at most 32 entries: one warp each, ranked in
             // registers (lane i holds entry i; the others come by shuffle).
             for (int b = gw; b < TK_BINS; b += nwarps) {
@@ -1138,7 +1347,7 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
         }
     }
     if (a.k <= TK_SMALL) return;
-    if (!grid_sync(a.bar, &ctl->err)) return report(a);
+    if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
 
     // K > 4096: sort tiles of TK_SMALL, then merge-path rounds.
     const uint64_t k = a.k;
@@ -1158,7 +1367,7 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
         }
         __syncthreads();
     }
-    if (!grid_sync(a.bar, &ctl->err)) return report(a);
+    if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
     uint64_t* src_r = a.out_r0;
     uint32_t* src_rid = a.out_rid0;
     uint64_t* dst_r = a.out_r1;
@@ -1197,7 +1406,7 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
                 }
             }
         }
-        if (!grid_sync(a.bar, &ctl->err)) return report(a);
+        if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
         uint64_t* tr = src_r; src_r = dst_r; dst_r = tr;
         uint32_t* ti = src_rid; src_rid = dst_rid; dst_rid = ti;
     }
@@ -1403,8 +1612,7 @@ cudaError_t topk_launch(const TopkArgs& args, const TopkGeom& geom, cudaStream_t
     a.fuse = a.use_sample && (a.pair || a.filter == TK_FILTER_REGS) ? 1 : 0;
     cudaError_t e;
     if (ev && (e = cudaEventRecord(ev[0], stream)) != cudaSuccess) return e;
-    topk_prepare_kernel<<<a.use_sample ? TK_PREP_CTAS : 1, TK_TPB, 0, stream>>>(a);
-    e = cudaGetLastError();
+    e = launch_kernel(topk_prepare_kernel, a.use_sample ? TK_PREP_CTAS : 1, TK_TPB, 0, stream, a, false);
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[1], stream)) != cudaSuccess) return e;
     if (a.use_sample) {

@@ -16,7 +16,7 @@ constexpr int TK_SMALL = 4096;            // entries one CTA sorts in shared mem
 constexpr int TK_SAMPLE = 8192;           // sample size of the threshold estimate
 constexpr int TK_SPT = TK_SAMPLE / TK_TPB;
 constexpr int TK_PREP_CTAS = TK_SAMPLE / TK_TPB;   // prepare CTAs on the sampled path: one key per thread
-constexpr int TK_UNROLL = 4;              // 16-byte loads in flight per thread (register filter)
+constexpr int TK_UNROLL = 2;              // 32-byte loads in flight per thread (register filter)
 constexpr uint64_t TK_DIRECT_N = 1ull << 21;   // at or below: no sample, refine the input
 constexpr int TK_RANK_MAX = 8192;         // survivors ranked in shared memory by the whole grid
 constexpr int TK_SORT_SMEM = TK_RANK_MAX * 12;  // select kernel shared bytes (ranking / sort tile / histogram)
@@ -39,6 +39,8 @@ enum TopkFilter { TK_FILTER_REGS = 0, TK_FILTER_BULK = 1 };
 struct TopkCtl {
     unsigned long long cand_count;   // filter: rank words <= threshold seen
     unsigned long long thresh;       // sample threshold (inclusive)
+    unsigned long long fbase;        // the fused first pass bins [fbase, thresh]
+    unsigned long long flow;         // candidates below fbase
     unsigned long long out_count;    // split: entries below the final prefix
     unsigned long long eq_count;     // split: prefix-equal entries taken wholesale
     unsigned long long small_count;  // split: prefix-equal entries kept for the finish
@@ -46,11 +48,10 @@ struct TopkCtl {
     int path;                        // 0 direct, 1 sampled candidates, 2 fallback
     int passes;                      // refine passes run
     int pad;
-    // AND and OR of the composite words (w0, w1) of the entries a refine pass
-    // saw (three slots, by pass), and of the selected entries before the
-    // finish partition: {and0, and1, or0, or1}.  Bits where AND == OR are
-    // common to all those entries.
-    unsigned long long ao[3][4];
+    // Minimum and maximum rank word, minimum and maximum row-id of the entries
+    // a refine pass saw (three slots, by pass), and of the selected entries
+    // before the finish partition.
+    unsigned long long mm[3][4];
     unsigned long long fin[4];
     // %globaltimer stamps: prepare start, prepare end (sample done), select
     // start (filter done), source decided, refine done, split done, end,
