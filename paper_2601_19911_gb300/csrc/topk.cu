@@ -858,8 +858,10 @@ __device__ void hist_pass(const TopkArgs& a, bool cand, uint64_t src_n, const Ra
 // With FOLD, the minima and maxima of the entries it writes to out (those
 // below the interval, and with take_all the ones in it that it keeps) are
 // merged into ctl->fin for the larger-K finish, which then needs no pass of
-// its own.  `nx` is the thread's first candidate on the candidate path; every
-// entry is loaded one step ahead.
+// its own, and the appends take one atomic per CTA and step (nearly every
+// warp has some: 9,000 atomics on two words for 293,000 candidates).  `nx` is
+// the thread's first candidate on the candidate path; every entry is loaded
+// one step ahead.
 template <bool FOLD>
 __device__ void split_pass(const TopkArgs& a, bool cand, uint64_t src_n, const Range& g, bool take_all,
                            uint64_t krem, Elem nx) {
@@ -872,47 +874,129 @@ __device__ void split_pass(const TopkArgs& a, bool cand, uint64_t src_n, const R
         const uint64_t i0 = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x;
         if (i0 < src_n) nx = load_src(a, cand, i0);
     }
-    for (uint64_t wb = static_cast<uint64_t>(blockIdx.x) * TK_TPB + (threadIdx.x & ~31u); wb < src_n;
-         wb += stride) {
-        const uint64_t i = wb + lane;
+    __shared__ unsigned s_lt[TK_TPB / 32], s_eq[TK_TPB / 32];
+    __shared__ unsigned long long s_base[2];
+    const unsigned warp = threadIdx.x >> 5;
+    unsigned long long* eq_ctr = take_all ? &ctl->eq_count : &ctl->small_count;
+    for (uint64_t cb = static_cast<uint64_t>(blockIdx.x) * TK_TPB; cb < src_n; cb += stride) {
+        const uint64_t i = cb + threadIdx.x;
         int c = 1;
         const Elem e = nx;
         if (i < src_n) c = range_cmp(g, e.r, e.rid);
         if (i + stride < src_n) nx = load_src(a, cand, i + stride);
         const unsigned lt = __ballot_sync(0xFFFFFFFFu, c < 0);
         const unsigned eq = __ballot_sync(0xFFFFFFFFu, c == 0);
-        if (lt) {
-            unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(&ctl->out_count, static_cast<unsigned long long>(__popc(lt)));
-            base = __shfl_sync(0xFFFFFFFFu, base, 0);
-            if (c < 0) {
-                const uint64_t pos = base + __popc(lt & ((1u << lane) - 1u));
-                a.out_r0[pos] = e.r;
-                a.out_rid0[pos] = e.rid;
-                if (FOLD) fold_add(acc, e.r, e.rid);
+        unsigned long long blt = 0, beq = 0;                 // the warp's first positions
+        if (FOLD) {
+            if (lane == 0) {
+                s_lt[warp] = __popc(lt);
+                s_eq[warp] = __popc(eq);
+            }
+            __syncthreads();
+            unsigned nlt = 0, neq = 0, all_lt = 0, all_eq = 0;
+#pragma unroll
+            for (unsigned w = 0; w < TK_TPB / 32; ++w) {
+                if (w == warp) {
+                    nlt = all_lt;
+                    neq = all_eq;
+                }
+                all_lt += s_lt[w];
+                all_eq += s_eq[w];
+            }
+            if (threadIdx.x == 0 && all_lt) s_base[0] = atomicAdd(&ctl->out_count, static_cast<unsigned long long>(all_lt));
+            if (threadIdx.x == 32 && all_eq) s_base[1] = atomicAdd(eq_ctr, static_cast<unsigned long long>(all_eq));
+            __syncthreads();
+            blt = s_base[0] + nlt;
+            beq = s_base[1] + neq;
+        } else {
+            if (lt) {
+                if (lane == 0) blt = atomicAdd(&ctl->out_count, static_cast<unsigned long long>(__popc(lt)));
+                blt = __shfl_sync(0xFFFFFFFFu, blt, 0);
+            }
+            if (eq) {
+                if (lane == 0) beq = atomicAdd(eq_ctr, static_cast<unsigned long long>(__popc(eq)));
+                beq = __shfl_sync(0xFFFFFFFFu, beq, 0);
             }
         }
-        if (eq) {
-            unsigned long long base = 0;
-            unsigned long long* ctr = take_all ? &ctl->eq_count : &ctl->small_count;
-            if (lane == 0) base = atomicAdd(ctr, static_cast<unsigned long long>(__popc(eq)));
-            base = __shfl_sync(0xFFFFFFFFu, base, 0);
-            if (c == 0) {
-                const uint64_t pos = base + __popc(eq & ((1u << lane) - 1u));
-                if (take_all) {
-                    if (pos < krem) {
-                        a.out_r0[eq_base + pos] = e.r;
-                        a.out_rid0[eq_base + pos] = e.rid;
-                        if (FOLD) fold_add(acc, e.r, e.rid);
-                    }
-                } else if (pos < TK_SMALL) {
-                    a.small_r[pos] = e.r;
-                    a.small_rid[pos] = e.rid;
+        if (c < 0) {
+            const uint64_t pos = blt + __popc(lt & ((1u << lane) - 1u));
+            a.out_r0[pos] = e.r;
+            a.out_rid0[pos] = e.rid;
+            if (FOLD) fold_add(acc, e.r, e.rid);
+        } else if (c == 0) {
+            const uint64_t pos = beq + __popc(eq & ((1u << lane) - 1u));
+            if (take_all) {
+                if (pos < krem) {
+                    a.out_r0[eq_base + pos] = e.r;
+                    a.out_rid0[eq_base + pos] = e.rid;
+                    if (FOLD) fold_add(acc, e.r, e.rid);
                 }
+            } else if (pos < TK_SMALL) {
+                a.small_r[pos] = e.r;
+                a.small_rid[pos] = e.rid;
             }
         }
     }
     if (FOLD) fold_merge<TK_TPB>(acc, ctl->fin);
+}
+
+// c -= 1 when entry j orders before entry e, or equals it and `ties`: the
+// borrow of the 96-bit difference, five adds and no branch.  (Written with
+// comparisons the compiler branches on the rank words, and lanes diverge on
+// every entry.)
+__device__ __forceinline__ void rank_count(unsigned& c, uint64_t jr, uint32_t jrid, uint64_t er, uint32_t erid,
+                                           bool ties) {
+    asm("{\n .reg .u32 t;\n"
+        " sub.cc.u32 t, 0, %6;\n"
+        " subc.cc.u32 t, %1, %2;\n"
+        " subc.cc.u32 t, %3, %4;\n"
+        " subc.cc.u32 t, %5, %7;\n"
+        " subc.u32 %0, %0, 0;\n}"
+        : "+r"(c)
+        : "r"(jrid), "r"(erid), "r"(static_cast<uint32_t>(jr)), "r"(static_cast<uint32_t>(er)),
+          "r"(static_cast<uint32_t>(jr >> 32)), "r"(ties ? 1u : 0u), "r"(static_cast<uint32_t>(er >> 32)));
+}
+
+// Entries of [lo, hi) in shared memory that order before entry e of them
+// (equal ones by position); whole warp calls and gets the count.
+__device__ __forceinline__ unsigned warp_rank_of(const uint64_t* sr, const uint32_t* srid, int lo, int hi, int e) {
+    const uint64_t er = sr[e];
+    const uint32_t erid = srid[e];
+    unsigned c = 0;
+#pragma unroll 4
+    for (int j = lo + static_cast<int>(threadIdx.x & 31u); j < hi; j += 32) rank_count(c, sr[j], srid[j], er, erid, j < e);
+    return __reduce_add_sync(0xFFFFFFFFu, 0u - c);
+}
+
+// Rank a bin of m <= 32 * Q entries in one warp's registers (a lane holds
+// entries lane, lane + 32, ...; the others come by shuffle) and write them
+// from position o on.
+template <int Q>
+__device__ __forceinline__ void warp_rank_bin(const TopkArgs& a, uint64_t o, unsigned m) {
+    const unsigned lane = threadIdx.x & 31u;
+    uint64_t er[Q];
+    uint32_t erid[Q];
+    unsigned c[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const unsigned i = q * 32u + lane;
+        er[q] = i < m ? __ldcg(a.out_r1 + o + i) : ~0ull;
+        erid[q] = i < m ? __ldcg(a.out_rid1 + o + i) : ~0u;
+        c[q] = 0;
+    }
+#pragma unroll
+    for (int p = 0; p < Q; ++p) {
+        const unsigned lim = m > p * 32u ? min(32u, m - p * 32u) : 0u;
+        for (unsigned j = 0; j < lim; ++j) {
+            const uint64_t jr = __shfl_sync(0xFFFFFFFFu, er[p], j);
+            const uint32_t jrid = __shfl_sync(0xFFFFFFFFu, erid[p], j);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) rank_count(c[q], jr, jrid, er[q], erid[q], p < q || (p == q && j < lane));
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+        if (q * 32u + lane < m) write_result(a, o + (0u - c[q]), er[q], erid[q]);
 }
 
 // Merge-path split: how many of the first `diag` outputs of the merge of
@@ -1140,19 +1224,10 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
             const int gw = static_cast<int>(blockIdx.x) * (TK_TPB / 32) + static_cast<int>(threadIdx.x >> 5);
             for (int e = gw; e < nbi + nsi; e += nwarps) {
                 const bool below = e < nbi;
-                const int lo = below ? 0 : nbi, hi = below ? nbi : nbi + nsi;
-                const uint64_t er = sr[e];
-                const uint32_t erid = srid[e];
-                unsigned c = 0;
-                for (int j = lo + static_cast<int>(lane); j < hi; j += 32) {
-                    const uint64_t jr = sr[j];
-                    const uint32_t jrid = srid[j];
-                    c += (jr < er || (jr == er && (jrid < erid || (jrid == erid && j < e)))) ? 1u : 0u;
-                }
-                c = __reduce_add_sync(0xFFFFFFFFu, c);
+                const unsigned c = warp_rank_of(sr, srid, below ? 0 : nbi, below ? nbi : nbi + nsi, e);
                 if (lane == 0) {
-                    if (below) write_result(a, c, er, erid);
-                    else if (c < krem) write_result(a, nb + c, er, erid);
+                    if (below) write_result(a, c, sr[e], srid[e]);
+                    else if (c < krem) write_result(a, nb + c, sr[e], srid[e]);
                 }
             }
             if (stamp) {
@@ -1166,11 +1241,16 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
 
     // Phase 4, larger K.  (a) The bucket entries (ns <= 4096) are ranked by
     // the grid as above and the first krem written at their final positions.
-    // (b) The below entries are partitioned into the 4096 bins of the interval
-    // they span -- a histogram, a scan, a scatter into out_r1 -- and every
-    // bin of at most TK_SMALL entries is ranked in one CTA's shared memory
-    // and written at its final positions.  Skewed inputs with a larger bin
-    // fall back to tile sorts and merge-path rounds.
+    // (b) The below entries are partitioned into bins -- a histogram, a scan,
+    // a scatter into out_r1 -- and every bin is ranked and written at its
+    // final positions.  The bins are first the 4096 equal ones of the interval
+    // the entries span; when one of those holds more than TK_SMALL (a few
+    // heavily tied keys), they are the gaps between 2047 of the entries, taken
+    // evenly and sorted, with the entries equal to one of those
+    // in bins of their own, which need no ranking: composites rarely tie, so
+    // any distribution of keys splits (10^8 int32 keys of 1024 values,
+    // K = 100,000: finish 222 -> 50 us).  More entries than such bins can
+    // take, or an unlucky choice, fall back to tile sorts and merge-path rounds.
     {
         const uint64_t nb = take_all ? a.k : a.k - krem;
         const int nsi = take_all ? 0 : static_cast<int>(bcnt);
@@ -1184,104 +1264,84 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
             }
             __syncthreads();
             for (int e = gw; e < nsi; e += nwarps) {
-                const uint64_t er = sr[e];
-                const uint32_t erid = srid[e];
-                unsigned c = 0;
-                for (int j = static_cast<int>(lane); j < nsi; j += 32) {
-                    const uint64_t jr = sr[j];
-                    const uint32_t jrid = srid[j];
-                    c += (jr < er || (jr == er && (jrid < erid || (jrid == erid && j < e)))) ? 1u : 0u;
-                }
-                c = __reduce_add_sync(0xFFFFFFFFu, c);
-                if (lane == 0 && c < krem) write_result(a, nb + c, er, erid);
+                const unsigned c = warp_rank_of(sr, srid, 0, nsi, e);
+                if (lane == 0 && c < krem) write_result(a, nb + c, sr[e], srid[e]);
             }
             __syncthreads();
         }
-        // (b) partition histogram of the below entries over the interval they
-        // span (folded by the split pass that wrote them), so that clustered
-        // keys and ties on the key spread over the bins.
-        const Range pr = range_of(a, ctl->fin);
-        const int psh = range_shift(pr, a.digit);
-        unsigned* ph = a.ghist + (pass % 3) * TK_BINS;          // clean (zeroed by the last pass or prepare)
-        unsigned* pc = a.ghist + ((pass + 1) % 3) * TK_BINS;    // cursors, zeroed here
-        for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB) sh[b] = 0;
-        if (blockIdx.x == 0)
-            for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB) pc[b] = 0;
-        __syncthreads();
-        const uint64_t gstride = static_cast<uint64_t>(TK_TPB) * gridDim.x;
-        for (uint64_t wb = static_cast<uint64_t>(blockIdx.x) * TK_TPB + (threadIdx.x & ~31u); wb < nb; wb += gstride) {
-            const uint64_t i = wb + lane;
-            unsigned dig = 0xFFFFFFFFu;
-            if (i < nb) dig = range_bin(pr, psh, __ldcg(a.out_r0 + i), __ldcg(a.out_rid0 + i));
-            const unsigned peers = __match_any_sync(0xFFFFFFFFu, dig);
-            if (dig != 0xFFFFFFFFu && lane == static_cast<unsigned>(__ffs(peers) - 1))
-                atomicAdd(&sh[dig], static_cast<unsigned>(__popc(peers)));
-        }
-        __syncthreads();
-        for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB)
-            if (sh[b]) atomicAdd(&ph[b], sh[b]);
-        if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
-        // Scan of the partition histogram (every CTA), largest bucket.
-        constexpr int PER = TK_BINS / TK_TPB;
-        unsigned v[PER];
-        unsigned long long local = 0;
-        unsigned mx = 0;
-        const volatile unsigned* hv = ph;
+        // One partition with the given bins: 1 done, 0 a bin too large, -1 a
+        // wait expired.  ph: clean; pc: zeroed here for the cursors; `pure`:
+        // odd bins hold identical entries.
+        auto partition = [&](auto bin, unsigned* ph, unsigned* pc, bool pure) -> int {
+            for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB) sh[b] = 0;
+            if (blockIdx.x == 0)
+                for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB) pc[b] = 0;
+            __syncthreads();
+            const uint64_t gstride = static_cast<uint64_t>(TK_TPB) * gridDim.x;
+            for (uint64_t wb = static_cast<uint64_t>(blockIdx.x) * TK_TPB + (threadIdx.x & ~31u); wb < nb;
+                 wb += gstride) {
+                const uint64_t i = wb + lane;
+                unsigned dig = 0xFFFFFFFFu;
+                if (i < nb) dig = bin(__ldcg(a.out_r0 + i), __ldcg(a.out_rid0 + i));
+                const unsigned peers = __match_any_sync(0xFFFFFFFFu, dig);
+                if (dig != 0xFFFFFFFFu && lane == static_cast<unsigned>(__ffs(peers) - 1))
+                    atomicAdd(&sh[dig], static_cast<unsigned>(__popc(peers)));
+            }
+            __syncthreads();
+            for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB)
+                if (sh[b]) atomicAdd(&ph[b], sh[b]);
+            if (!grid_sync(a.bar, &ctl->err, bar_target)) return -1;
+            // Scan of the partition histogram (every CTA), largest bin.
+            constexpr int PER = TK_BINS / TK_TPB;
+            unsigned v[PER];
+            unsigned long long local = 0;
+            unsigned mx = 0;
+            pick_load_global<TK_TPB>(ph, v);
 #pragma unroll
-        for (int j = 0; j < PER; ++j) {
-            v[j] = hv[threadIdx.x * PER + j];
-            local += v[j];
-            mx = max(mx, v[j]);
-        }
-        const unsigned long long before = block_excl_scan<TK_TPB>(local, reinterpret_cast<unsigned long long*>(sc),
-                                                          reinterpret_cast<unsigned long long*>(sc) + 16);
-        unsigned* off = sh;                                      // exclusive offsets per bucket
-        {
-            unsigned long long run = before;
+            for (int j = 0; j < PER; ++j) {
+                local += v[j];
+                if (!(pure && (j & 1))) mx = max(mx, v[j]);
+            }
+            unsigned* off = sh;                              // exclusive offsets per bin
+            unsigned long long run = block_excl_scan<TK_TPB>(local, sc, sc + 16);
 #pragma unroll
             for (int j = 0; j < PER; ++j) {
                 off[threadIdx.x * PER + j] = static_cast<unsigned>(run);
                 run += v[j];
             }
-        }
-        const bool fits = __syncthreads_and(mx <= static_cast<unsigned>(TK_SMALL));
-        if (fits) {
-            // Scatter the below entries into bucket order (out_r1).
+            if (!__syncthreads_and(mx <= static_cast<unsigned>(TK_SMALL))) return 0;
+            // Scatter the below entries into bin order (out_r1).
             for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x; i < nb; i += gstride) {
                 const uint64_t er = __ldcg(a.out_r0 + i);
                 const uint32_t erid = __ldcg(a.out_rid0 + i);
-                const unsigned d = range_bin(pr, psh, er, erid);
+                const unsigned d = bin(er, erid);
                 const unsigned pos = off[d] + atomicAdd(&pc[d], 1u);
                 a.out_r1[pos] = er;
                 a.out_rid1[pos] = erid;
             }
-            if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
-            // Buckets of at most 32 entries: one warp each, ranked in
-            // registers (lane i holds entry i; the others come by shuffle).
+            if (!grid_sync(a.bar, &ctl->err, bar_target)) return -1;
+            // Bins of at most 128 entries: one warp each, in registers.
+            auto size = [&](int b) { return (b + 1 < TK_BINS ? off[b + 1] : static_cast<unsigned>(nb)) - off[b]; };
             for (int b = gw; b < TK_BINS; b += nwarps) {
-                const unsigned m = hv[b];
-                if (m == 0 || m > 32) continue;
+                const unsigned m = size(b);
+                const bool same = pure && (b & 1);
+                if (m == 0 || (m > 128 && !same)) continue;
                 const unsigned o = off[b];
-                uint64_t er = 0;
-                uint32_t erid = 0;
-                if (lane < m) {
-                    er = __ldcg(a.out_r1 + o + lane);
-                    erid = __ldcg(a.out_rid1 + o + lane);
+                if (same) {
+                    for (unsigned i = lane; i < m; i += 32)
+                        write_result(a, o + i, __ldcg(a.out_r1 + o + i), __ldcg(a.out_rid1 + o + i));
+                    continue;
                 }
-                unsigned c = 0;
-                for (unsigned j = 0; j < m; ++j) {
-                    const uint64_t jr = __shfl_sync(0xFFFFFFFFu, er, j);
-                    const uint32_t jrid = __shfl_sync(0xFFFFFFFFu, erid, j);
-                    c += (jr < er || (jr == er && (jrid < erid || (jrid == erid && j < lane)))) ? 1u : 0u;
-                }
-                if (lane < m) write_result(a, o + c, er, erid);
+                if (m <= 32) warp_rank_bin<1>(a, o, m);
+                else if (m <= 64) warp_rank_bin<2>(a, o, m);
+                else warp_rank_bin<4>(a, o, m);
             }
-            // Larger buckets: one CTA each, ranked in shared memory.
+            // Larger bins: one CTA each, ranked in shared memory.
             uint64_t* br = reinterpret_cast<uint64_t*>(smem + TK_BINS * 4);
             uint32_t* brid = reinterpret_cast<uint32_t*>(smem + TK_BINS * 4 + TK_SMALL * 8);
             for (int b = blockIdx.x; b < TK_BINS; b += gridDim.x) {
-                const unsigned m = hv[b];
-                if (m <= 32) continue;
+                const unsigned m = size(b);
+                if (m <= 128 || (pure && (b & 1))) continue;
                 const unsigned o = off[b];
                 for (unsigned i = threadIdx.x; i < m; i += TK_TPB) {
                     br[i] = __ldcg(a.out_r1 + o + i);
@@ -1289,19 +1349,54 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
                 }
                 __syncthreads();
                 for (unsigned e = threadIdx.x >> 5; e < m; e += TK_TPB / 32) {
-                    const uint64_t er = br[e];
-                    const uint32_t erid = brid[e];
-                    unsigned c = 0;
-                    for (unsigned j = lane; j < m; j += 32) {
-                        const uint64_t jr = br[j];
-                        const uint32_t jrid = brid[j];
-                        c += (jr < er || (jr == er && (jrid < erid || (jrid == erid && j < e)))) ? 1u : 0u;
-                    }
-                    c = __reduce_add_sync(0xFFFFFFFFu, c);
-                    if (lane == 0) write_result(a, o + c, er, erid);
+                    const unsigned c = warp_rank_of(br, brid, 0, static_cast<int>(m), static_cast<int>(e));
+                    if (lane == 0) write_result(a, o + c, br[e], brid[e]);
                 }
                 __syncthreads();
             }
+            return 1;
+        };
+        unsigned* hb[3];                                     // the three histograms; hb[0] is clean
+        for (int j = 0; j < 3; ++j) hb[j] = a.ghist + ((pass + j) % 3) * TK_BINS;
+        const Range pr = range_of(a, ctl->fin);
+        const int psh = range_shift(pr, a.digit);
+        int done = partition([&](uint64_t r, uint32_t rid) { return range_bin(pr, psh, r, rid); }, hb[0], hb[1], false);
+        if (done == 0 && nb <= TK_SPLIT_MAX) {
+            uint64_t* pr_r = reinterpret_cast<uint64_t*>(smem + TK_BINS * 4 + TK_SMALL * 12);
+            uint32_t* pr_rid = reinterpret_cast<uint32_t*>(smem + TK_BINS * 4 + TK_SMALL * 12 + (TK_SPLITTERS + 1) * 8);
+            for (int j = threadIdx.x; j < TK_SPLITTERS; j += TK_TPB) {
+                const uint64_t i = static_cast<uint64_t>(j) * nb / TK_SPLITTERS;
+                pr_r[j] = __ldcg(a.out_r0 + i);
+                pr_rid[j] = __ldcg(a.out_rid0 + i);
+            }
+            __syncthreads();
+            // sorted by the grid: every warp ranks some (in one CTA a bitonic
+            // sort of 2047 takes 50 us), then every CTA reads them in order
+            for (int e = gw; e < TK_SPLITTERS; e += nwarps) {
+                const unsigned c = warp_rank_of(pr_r, pr_rid, 0, TK_SPLITTERS, e);
+                if (lane == 0) {
+                    a.split_r[c] = pr_r[e];
+                    a.split_rid[c] = pr_rid[e];
+                }
+            }
+            if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
+            for (int j = threadIdx.x; j < TK_SPLITTERS; j += TK_TPB) {
+                pr_r[j] = __ldcg(a.split_r + j);
+                pr_rid[j] = __ldcg(a.split_rid + j);
+            }
+            __syncthreads();
+            auto gap = [&](uint64_t r, uint32_t rid) {       // 2 * splitters below, + 1 when equal to the next
+                int lo = 0;
+#pragma unroll
+                for (int w = (TK_SPLITTERS + 1) / 2; w > 0; w >>= 1)
+                    if (elem_less(pr_r[lo + w - 1], pr_rid[lo + w - 1], r, rid)) lo += w;
+                const bool eq = lo < TK_SPLITTERS && pr_r[lo] == r && pr_rid[lo] == rid;
+                return static_cast<unsigned>(2 * lo + (eq ? 1 : 0));
+            };
+            done = partition(gap, hb[1], hb[2], true);
+        }
+        if (done < 0) return report(a);
+        if (done) {
             if (stamp) {
                 ctl->ts[7] = gtimer();
                 ctl->ts[8] = ctl->ts[7];
@@ -1310,8 +1405,8 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
             }
             return;
         }
-        // Skewed: the bucket entries are already written; sort the below
-        // entries with the merge path (k below plus krem written above).
+        // The bucket entries are already written; sort the below entries with
+        // the merge path (k below plus krem written above).
     }
 
     // Phase 4, fallback: CTA 0 finishes the bucket, then a grid merge sort.
@@ -1444,7 +1539,7 @@ size_t topk_scratch_bytes(const TopkPlan& p, uint64_t k) {
     b += up256(TK_SMALL * 8) + up256(TK_SMALL * 4);
     const uint64_t kk = std::max<uint64_t>(k, 1);
     b += up256(kk * 8) + up256(kk * 4);
-    if (k > TK_SMALL) b += up256(kk * 8) + up256(kk * 4);
+    if (k > TK_SMALL) b += up256(kk * 8) + up256(kk * 4) + up256(TK_SPLITTERS * 8) + up256(TK_SPLITTERS * 4);
     return b;
 }
 
@@ -1471,9 +1566,11 @@ void topk_carve(TopkArgs& a, const TopkPlan& p, void* base) {
     if (a.k > TK_SMALL) {
         a.out_r1 = static_cast<uint64_t*>(take(kk * 8));
         a.out_rid1 = static_cast<uint32_t*>(take(kk * 4));
+        a.split_r = static_cast<uint64_t*>(take(TK_SPLITTERS * 8));
+        a.split_rid = static_cast<uint32_t*>(take(TK_SPLITTERS * 4));
     } else {
-        a.out_r1 = nullptr;
-        a.out_rid1 = nullptr;
+        a.out_r1 = a.split_r = nullptr;
+        a.out_rid1 = a.split_rid = nullptr;
     }
     a.samples = p.use_sample ? static_cast<uint64_t*>(take(TK_SAMPLE * 8)) : nullptr;
     a.use_sample = p.use_sample;

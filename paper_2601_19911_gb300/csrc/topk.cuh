@@ -19,6 +19,8 @@ constexpr int TK_PREP_CTAS = TK_SAMPLE / TK_TPB;   // prepare CTAs on the sample
 constexpr int TK_UNROLL = 2;              // 32-byte loads in flight per thread (register filter)
 constexpr uint64_t TK_DIRECT_N = 1ull << 21;   // at or below: no sample, refine the input
 constexpr int TK_RANK_MAX = 8192;         // survivors ranked in shared memory by the whole grid
+constexpr int TK_SPLITTERS = 2047;        // splitters of the larger-K finish on tied keys (2^k - 1)
+constexpr uint64_t TK_SPLIT_MAX = 2048ull * 512;   // entries they may split (about 512 per gap)
 constexpr int TK_SORT_SMEM = TK_RANK_MAX * 12;  // select kernel shared bytes (ranking / sort tile / histogram)
 constexpr int TK_MAX_STAGES = 16;         // full + empty mbarrier pairs reserved after the ring
 constexpr int TK_SMEM_MAX = 227 * 1024;   // opt-in shared memory per CTA
@@ -86,6 +88,8 @@ struct TopkArgs {
     uint32_t* out_rid0;
     uint64_t* out_r1;                // k entries, merge ping-pong (k > TK_SMALL)
     uint32_t* out_rid1;
+    uint64_t* split_r;               // TK_SPLITTERS sorted splitters (k > TK_SMALL)
+    uint32_t* split_rid;
     uint64_t* samples;               // TK_SAMPLE rank words of the sample (sampled path)
     void* out_keys;                  // caller's outputs (device)
     uint32_t* out_rowids;
