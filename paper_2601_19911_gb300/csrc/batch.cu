@@ -9,12 +9,14 @@
 // into parts that run as items of their own; a second launch merges each
 // split item's parts.  Per item:
 //   * Top-K (K <= 4096): a stratified sample of 2048 keys gives a threshold
-//     rank word; one streaming pass appends the keys at or below it to the
-//     CTA's own candidate buffer (no global atomics); block-local radix passes
-//     over the candidates find the bucket of the K-th entry; the split puts
-//     the selected entries in shared memory, where they are sorted.  Small
-//     items (n <= 4096) are sorted whole; a misjudged sample falls back to
-//     radix passes over the item's keys.
+//     rank word and the spread below it; one streaming pass appends the keys
+//     at or below the threshold to the CTA's own candidate buffer (no global
+//     atomics); the candidates are counted in 4096 equal bins of that
+//     interval, and those of the bins up to the K-th entry's are put in bin
+//     order in shared memory and ranked within their bins.  Small items take
+//     all their keys as candidates.  Ties and outliers that crowd a bin go
+//     through block-local radix passes and a sort instead, a misjudged sample
+//     through radix passes over the item's keys.
 //   * probe: the probe loop of the join kernel over one chunk of at most
 //     BP_CHUNK probe rows of an item, handed to the CTA's warps by a row
 //     queue in shared memory; a large item is many chunks taken by many
@@ -41,16 +43,15 @@ constexpr int BT_SMALL = 4096;            // entries one sort handles
 constexpr int BT_SAMPLE = 2048;           // sample keys per item
 constexpr int BT_SPT = BT_SAMPLE / BT_TPB;
 constexpr uint32_t BT_CAND = 65536;       // candidate capacity per CTA
-constexpr int BT_WS = 128;                // staged hits per warp
 constexpr int BT_BINS = 4096;
-constexpr int BT_SMEM = 2 * BT_SMALL * 12; // two sort areas; also the histogram, stages, probe stage
+constexpr int BT_SMEM = 2 * BT_SMALL * 12; // two sort areas; also the histogram and the entries in bin order
 // Probe rows per work unit (4096 to 32768 run a batch of 128 probe items with
 // 18 M rows against a 2^20-row table in 257, 237, 229, 222 us; smaller units
 // balance a batch of few items better).
 constexpr uint64_t BP_CHUNK = 16384;
-constexpr uint64_t BT_SPLIT_N = 1ull << 19;  // smallest Top-K item that may be split into parts
-constexpr uint64_t BT_PART = 1ull << 18;     // smallest target rows per part (parts are balanced)
-static_assert((BT_TPB / 32) * BT_WS * 12 <= BT_SMEM, "warp stages must fit");
+constexpr uint64_t BT_SPLIT_N = 1ull << 17;  // smallest Top-K item that may be split into parts
+constexpr uint64_t BT_PART = 1ull << 16;     // smallest target rows per part (parts are balanced)
+static_assert(BT_BINS * 4 + BT_SMALL * 12 <= BT_SMEM, "bins and entries must fit");
 
 struct __align__(8) Item {
     int op;                      // OLAP_OP_TOPK / OLAP_OP_PROBE
@@ -101,6 +102,10 @@ __device__ __forceinline__ uint64_t item_rank(const Item& it, uint64_t i, uint32
     return r;
 }
 
+__device__ __forceinline__ uint32_t item_max_rowid(const Item& it) {
+    return it.rowids ? 0xFFFFFFFFu : static_cast<uint32_t>(it.rowid_base + it.n - 1);
+}
+
 __device__ __forceinline__ void put_result(const Item& it, uint64_t i, uint64_t r, uint32_t rid) {
     if (it.out_mode == ITEM_OUT_RANKS) {
         static_cast<uint64_t*>(it.out_keys)[i] = r;
@@ -118,10 +123,11 @@ __device__ __forceinline__ void put_result(const Item& it, uint64_t i, uint64_t 
     it.out_rowids[i] = rid;
 }
 
-// Threshold rank word from a stratified sample: radix select (digit bits) with the
-// early exit of the grid version (between r and r + 8 samples at or below).
-__device__ uint64_t cta_sample_threshold(const Item& it, unsigned r, unsigned* hist, unsigned long long* sc,
-                                         int digit) {
+// Interval [rlo, rhi] of rank words from a stratified sample: rhi is the
+// filter's threshold (radix select with the early exit of the grid version:
+// between r and r + 8 samples at or below it, the largest of those), rlo four
+// times their spread below it (rlo == rhi when they are all equal).
+__device__ Range cta_sample_range(const Item& it, unsigned r, unsigned* hist, unsigned long long* sc, int digit) {
     uint64_t s[BT_SPT];
 #pragma unroll
     for (int j = 0; j < BT_SPT; ++j) {
@@ -131,7 +137,7 @@ __device__ uint64_t cta_sample_threshold(const Item& it, unsigned r, unsigned* h
         s[j] = item_rank(it, pos, &rid);
     }
     const int kb = it.w4 ? 32 : 64;
-    uint64_t prefix = 0;
+    uint64_t prefix = 0, edge = 0;
     unsigned long long rem = r, cum = 0;
     for (int L = 0; L < kb; L += digit) {
         const int d = min(digit, kb - L);
@@ -147,108 +153,125 @@ __device__ uint64_t cta_sample_threshold(const Item& it, unsigned r, unsigned* h
         prefix |= static_cast<uint64_t>(pk.b) << (64 - L - d);
         rem -= pk.below;
         cum += pk.below;
-        if (cum + pk.in_b <= r + 8) return prefix | ((1ull << (64 - L - d)) - 1ull);
+        edge = prefix | ((1ull << (64 - L - d)) - 1ull);
+        if (cum + pk.in_b <= r + 8) break;
     }
-    return prefix;
+    if (threadIdx.x == 0) {
+        sc[0] = ~0ull;
+        sc[1] = 0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < BT_SPT; ++j)
+        if (s[j] <= edge) {
+            atomicMin(&sc[0], static_cast<unsigned long long>(s[j]));
+            atomicMax(&sc[1], static_cast<unsigned long long>(s[j]));
+        }
+    __syncthreads();
+    const uint64_t t = sc[1], d = t - sc[0];
+    __syncthreads();
+    return Range{d >= t / 4 ? (d ? 0ull : t) : t - 4 * d, t, 0u, item_max_rowid(it)};
 }
 
-// Move a warp's staged hits to the CTA's candidate buffer.
-__device__ __forceinline__ void cta_flush_stage(uint64_t* ws_r, uint32_t* ws_idx, unsigned& cnt, const Item& it,
-                                                uint64_t* cand_r, uint32_t* cand_rid, unsigned* s_cand) {
-    if (cnt == 0) return;
-    __syncwarp();
-    const unsigned lane = threadIdx.x & 31u;
-    unsigned base = 0;
-    if (lane == 0) base = atomicAdd(s_cand, cnt);
-    base = __shfl_sync(0xFFFFFFFFu, base, 0);
-    for (unsigned j = lane; j < cnt; j += 32) {
-        if (base + j < BT_CAND) {
-            const uint32_t idx = ws_idx[j];
-            cand_r[base + j] = ws_r[j];
-            cand_rid[base + j] = it.rowids ? it.rowids[idx] : static_cast<uint32_t>(it.rowid_base + idx);
+// The 4096 bins of the selection: equal parts of an interval, bin 0 also
+// holding what lies below it.
+struct CtaBins {
+    Range g;
+    int sh;
+    __device__ explicit CtaBins(const Range& r) : g(r), sh(range_shift(r, 12)) {
+        if (range_bin(g, sh, g.rhi, g.ihi) + 1 >= BT_BINS) ++sh;
+    }
+    __device__ unsigned operator()(uint64_t r, uint32_t rid) const {
+        return range_cmp(g, r, rid) < 0 ? 0u : 1u + range_bin(g, sh, r, rid);
+    }
+};
+// The streaming pass of one item by one CTA: 32-byte loads, one comparison
+// per key, one vote per 64 bytes and warp; the few hits append themselves to
+// the CTA's candidate buffer through a shared counter.
+template <bool W4, int MODE>
+__device__ __forceinline__ void cta_filter_loop(const Item& it, uint64_t lim, const unsigned char* base, uint64_t head,
+                                                uint64_t nvec, uint64_t* cand_r, uint32_t* cand_rid,
+                                                unsigned* s_cand) {
+    constexpr int VEC = W4 ? 8 : 4;
+    constexpr int U = 2;
+    for (uint64_t bb = 0; bb < nvec; bb += U * BT_TPB) {
+        uint32_t v[U][8];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint64_t vi = bb + static_cast<uint64_t>(u) * BT_TPB + threadIdx.x;
+            ld_stream_words(base + (vi < nvec ? vi : 0) * 32, v[u]);
+        }
+        auto key = [&](int u, int e) {
+            return W4 ? static_cast<uint64_t>(v[u][e])
+                      : static_cast<uint64_t>(v[u][2 * e]) | (static_cast<uint64_t>(v[u][2 * e + 1]) << 32);
+        };
+        auto pass = [&](int u, int e) {
+            return W4 ? key_pass<MODE, uint32_t, int32_t>(v[u][e], static_cast<uint32_t>(lim))
+                      : key_pass<MODE, uint64_t, int64_t>(key(u, e), lim);
+        };
+        bool any = false;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) any = any | pass(u, e);
+        if (!__any_sync(0xFFFFFFFFu, any)) continue;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint64_t vi = bb + static_cast<uint64_t>(u) * BT_TPB + threadIdx.x;
+            if (vi >= nvec) continue;
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+                if (!pass(u, e)) continue;
+                const unsigned pos = atomicAdd(s_cand, 1u);
+                if (pos >= BT_CAND) continue;
+                const uint64_t i = head + vi * VEC + e;
+                cand_r[pos] = rank_key(key(u, e), it.kind, it.desc);
+                cand_rid[pos] = it.rowids ? it.rowids[i] : static_cast<uint32_t>(it.rowid_base + i);
+            }
         }
     }
-    __syncwarp();
-    cnt = 0;
 }
 
-// Test one key (rank via the key-domain limit) and stage a hit; the whole
-// warp calls with its lanes' keys.
+// Returns the candidate count (which may exceed what the buffer holds).
 template <bool W4>
-__device__ __forceinline__ void cta_filter_key(const Item& it, const KeyLimit& lim, bool valid, uint64_t bits,
-                                               uint64_t idx, uint64_t* ws_r, uint32_t* ws_idx, unsigned& cnt,
-                                               uint64_t* cand_r, uint32_t* cand_rid, unsigned* s_cand) {
-    const bool hit = valid && (W4 ? pass32(static_cast<uint32_t>(bits), lim) : pass64(bits, lim));
-    const unsigned bal = __ballot_sync(0xFFFFFFFFu, hit);
-    if (!bal) return;
-    if (cnt + __popc(bal) > BT_WS) cta_flush_stage(ws_r, ws_idx, cnt, it, cand_r, cand_rid, s_cand);
-    const unsigned lane = threadIdx.x & 31u;
-    if (hit) {
-        const unsigned pos = cnt + __popc(bal & ((1u << lane) - 1u));
-        ws_r[pos] = rank_key(bits, it.kind, it.desc);
-        ws_idx[pos] = static_cast<uint32_t>(idx);
-    }
-    cnt += __popc(bal);
-}
-
-// The streaming pass of one item by one CTA.  Returns the candidate count.
-template <bool W4>
-__device__ unsigned cta_filter(const Item& it, uint64_t t, unsigned char* smem, uint64_t* cand_r,
-                               uint32_t* cand_rid, unsigned* s_cand) {
-    const KeyLimit lim = key_limit(t, it.kind, it.desc);
-    const unsigned w = threadIdx.x >> 5, lane = threadIdx.x & 31u;
-    uint64_t* ws_r = reinterpret_cast<uint64_t*>(smem + w * BT_WS * 12);
-    uint32_t* ws_idx = reinterpret_cast<uint32_t*>(smem + w * BT_WS * 12 + BT_WS * 8);
-    unsigned cnt = 0;
+__device__ unsigned cta_filter(const Item& it, uint64_t t, uint64_t* cand_r, uint32_t* cand_rid, unsigned* s_cand) {
+    const KeyLimit kl = key_limit(t, it.kind, it.desc);
     if (threadIdx.x == 0) *s_cand = 0;
     __syncthreads();
     constexpr int W = W4 ? 4 : 8;
     const uint64_t n = it.n;
-    const uintptr_t addr = reinterpret_cast<uintptr_t>(it.keys);
-    const uint64_t head0 = ((16 - (addr & 15)) & 15) / W;
+    const uint64_t head0 = ((32 - (reinterpret_cast<uintptr_t>(it.keys) & 31)) & 31) / W;
     const uint64_t head = head0 < n ? head0 : n;
-    constexpr uint64_t VEC = 16 / W;
+    constexpr uint64_t VEC = 32 / W;
     const uint64_t nvec = (n - head) / VEC;
     const uint64_t tail0 = head + nvec * VEC;
     const unsigned char* vbase = static_cast<const unsigned char*>(it.keys) + head * W;
-    // vectors: 4 in flight per thread
-    for (uint64_t bb = 0; bb < nvec; bb += 4 * BT_TPB) {
-        uint4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const uint64_t vi = bb + static_cast<uint64_t>(u) * BT_TPB + threadIdx.x;
-            v[u] = vi < nvec ? ld_stream_v4(vbase + vi * 16) : make_uint4(0, 0, 0, 0);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const uint64_t vi = bb + static_cast<uint64_t>(u) * BT_TPB + threadIdx.x;
-            const bool ok = vi < nvec;
-            const uint64_t i0 = head + vi * VEC;
-            if (W4) {
-                const uint32_t x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    cta_filter_key<W4>(it, lim, ok, x[e], i0 + e, ws_r, ws_idx, cnt, cand_r, cand_rid, s_cand);
-            } else {
-                cta_filter_key<W4>(it, lim, ok, static_cast<uint64_t>(v[u].x) | (static_cast<uint64_t>(v[u].y) << 32),
-                               i0, ws_r, ws_idx, cnt, cand_r, cand_rid, s_cand);
-                cta_filter_key<W4>(it, lim, ok, static_cast<uint64_t>(v[u].z) | (static_cast<uint64_t>(v[u].w) << 32),
-                               i0 + 1, ws_r, ws_idx, cnt, cand_r, cand_rid, s_cand);
+    uint64_t lim;
+    int mode;
+    if (W4) {
+        uint32_t l32;
+        mode = key_cmp<uint32_t>(kl.m32, kl.c32, &l32);
+        lim = l32;
+    } else {
+        mode = key_cmp<uint64_t>(kl.m64, kl.c64, &lim);
+    }
+    if (mode == CMP_GE_U) cta_filter_loop<W4, CMP_GE_U>(it, lim, vbase, head, nvec, cand_r, cand_rid, s_cand);
+    else if (mode == CMP_LE_U) cta_filter_loop<W4, CMP_LE_U>(it, lim, vbase, head, nvec, cand_r, cand_rid, s_cand);
+    else if (mode == CMP_GE_S) cta_filter_loop<W4, CMP_GE_S>(it, lim, vbase, head, nvec, cand_r, cand_rid, s_cand);
+    else cta_filter_loop<W4, CMP_LE_S>(it, lim, vbase, head, nvec, cand_r, cand_rid, s_cand);
+    // head and tail (at most 14 keys)
+    if (threadIdx.x < head + (n - tail0)) {
+        const uint64_t i = threadIdx.x < head ? threadIdx.x : tail0 + (threadIdx.x - head);
+        uint32_t rid;
+        const uint64_t r = item_rank(it, i, &rid);
+        if (r <= t) {
+            const unsigned pos = atomicAdd(s_cand, 1u);
+            if (pos < BT_CAND) {
+                cand_r[pos] = r;
+                cand_rid[pos] = rid;
             }
         }
     }
-    // head and tail (at most 2 * VEC - 2 keys) by warp 0
-    if (w == 0) {
-        const uint64_t rest = head + (n - tail0);
-        const bool ok = lane < rest;
-        uint64_t idx = 0, bits = 0;
-        if (ok) {
-            idx = lane < head ? lane : tail0 + (lane - head);
-            bits = W4 ? static_cast<const uint32_t*>(it.keys)[idx] : static_cast<const uint64_t*>(it.keys)[idx];
-        }
-        cta_filter_key<W4>(it, lim, ok, bits, idx, ws_r, ws_idx, cnt, cand_r, cand_rid, s_cand);
-    }
-    cta_flush_stage(ws_r, ws_idx, cnt, it, cand_r, cand_rid, s_cand);
     __syncthreads();
     return *reinterpret_cast<volatile unsigned*>(s_cand);
 }
@@ -263,6 +286,129 @@ __device__ __forceinline__ void src_get(const Item& it, bool cand, const uint64_
     }
 }
 
+// Select and sort at once: the bins (a histogram of the entries) up to the
+// one that reaches kk are scattered into bin order in shared memory, and
+// every entry finds its place within its bin, which holds a few.  False, with nothing written, when those bins hold more than BT_SMALL
+// entries or one of them more than BT_BIN_MAX (ties, outliers): the caller
+// then refines and sorts.  An item of 482,000 keys with K = 500 leaves about
+// 3,000 candidates, whose bitonic sort over 4096 slots takes 78 steps; with
+// the streaming pass above, the kernel went from 600 to 398 us (512 items,
+// 1.8 GB of keys).
+constexpr unsigned BT_BIN_MAX = 128;
+__device__ bool cta_bin_select(const Item& it, bool cand, const uint64_t* cand_r, const uint32_t* cand_rid,
+                               uint64_t src_n, uint64_t kk, const CtaBins& bin, unsigned char* smem,
+                               unsigned long long* sc) {
+    unsigned* off = reinterpret_cast<unsigned*>(smem);
+    uint64_t* sr = reinterpret_cast<uint64_t*>(smem + BT_BINS * 4);
+    uint32_t* srid = reinterpret_cast<uint32_t*>(smem + BT_BINS * 4 + BT_SMALL * 8);
+    constexpr int U = 2;                                   // entries loaded at a time: an L2 round trip each
+    for (int b = threadIdx.x; b < BT_BINS; b += BT_TPB) off[b] = 0;
+    __syncthreads();
+    for (uint64_t i0 = threadIdx.x; i0 < src_n; i0 += U * BT_TPB) {
+        uint64_t r[U];
+        uint32_t rid[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint64_t i = i0 + static_cast<uint64_t>(u) * BT_TPB;
+            if (i < src_n) src_get(it, cand, cand_r, cand_rid, i, r[u], rid[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i0 + static_cast<uint64_t>(u) * BT_TPB < src_n) atomicAdd(&off[bin(r[u], rid[u])], 1u);
+    }
+    __syncthreads();
+    constexpr int PER = BT_BINS / BT_TPB;
+    unsigned v[PER];
+    unsigned local = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        v[j] = off[threadIdx.x * PER + j];
+        local += v[j];
+    }
+    unsigned run = static_cast<unsigned>(block_excl_scan<BT_TPB>(local, sc, sc + 16));
+    // (the scan ends with a barrier: every bin has been read)
+    bool ok = true;
+    unsigned total = 0;                                    // through the bin that reaches kk, in one thread
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        if (run < kk) {                                    // one of the bins that are kept
+            if (v[j] > BT_BIN_MAX) ok = false;
+            if (run + v[j] >= kk) total = run + v[j];
+        }
+        off[threadIdx.x * PER + j] = run;
+        run += v[j];
+    }
+    if (total) sc[20] = total;
+    if (total > BT_SMALL) ok = false;
+    if (!__syncthreads_and(ok)) return false;
+    total = static_cast<unsigned>(sc[20]);
+    for (uint64_t i0 = threadIdx.x; i0 < src_n; i0 += U * BT_TPB) {
+        uint64_t r[U];
+        uint32_t rid[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint64_t i = i0 + static_cast<uint64_t>(u) * BT_TPB;
+            if (i < src_n) src_get(it, cand, cand_r, cand_rid, i, r[u], rid[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (i0 + static_cast<uint64_t>(u) * BT_TPB >= src_n) continue;
+            const unsigned b = bin(r[u], rid[u]);
+            if (off[b] >= total) continue;                 // (a kept bin's cursor passes `total` only when it is full)
+            const unsigned pos = atomicAdd(&off[b], 1u);
+            sr[pos] = r[u];
+            srid[pos] = rid[u];
+        }
+    }
+    __syncthreads();
+    // off[b] is now the end of bin b, and the start of the next
+    for (unsigned p = threadIdx.x; p < total; p += BT_TPB) {
+        const uint64_t r = sr[p];
+        const uint32_t rid = srid[p];
+        const unsigned b = bin(r, rid), lo = b ? off[b - 1] : 0u, hi = off[b];
+        unsigned c = 0;
+        for (unsigned j = lo; j < hi; ++j) rank_count(c, sr[j], srid[j], r, rid, j < p);
+        if (lo - c < kk) put_result(it, lo - c, r, rid);
+    }
+    return true;
+}
+
+// The interval that the entries of the item's input span.
+__device__ Range cta_input_range(const Item& it, unsigned long long* sc) {
+    uint64_t rmin = ~0ull, rmax = 0;
+    uint32_t imin = ~0u, imax = 0;
+    if (threadIdx.x == 0) {
+        sc[0] = sc[2] = ~0ull;
+        sc[1] = sc[3] = 0;
+    }
+    __syncthreads();
+    for (uint64_t i = threadIdx.x; i < it.n; i += BT_TPB) {
+        uint32_t rid;
+        const uint64_t r = item_rank(it, i, &rid);
+        rmin = min(rmin, r);
+        rmax = max(rmax, r);
+        imin = min(imin, rid);
+        imax = max(imax, rid);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        rmin = min(rmin, __shfl_xor_sync(0xFFFFFFFFu, rmin, o));
+        rmax = max(rmax, __shfl_xor_sync(0xFFFFFFFFu, rmax, o));
+    }
+    imin = __reduce_min_sync(0xFFFFFFFFu, imin);
+    imax = __reduce_max_sync(0xFFFFFFFFu, imax);
+    if ((threadIdx.x & 31u) == 0) {
+        atomicMin(&sc[0], static_cast<unsigned long long>(rmin));
+        atomicMax(&sc[1], static_cast<unsigned long long>(rmax));
+        atomicMin(&sc[2], static_cast<unsigned long long>(imin));
+        atomicMax(&sc[3], static_cast<unsigned long long>(imax));
+    }
+    __syncthreads();
+    const Range g{sc[0], sc[1], static_cast<uint32_t>(sc[2]), static_cast<uint32_t>(sc[3])};
+    __syncthreads();
+    return g;
+}
+
 // Top-K of one item by one CTA.
 __device__ void cta_topk(const Item& it, unsigned char* smem, uint64_t* cand_r, uint32_t* cand_rid,
                          unsigned long long* sc, unsigned* s_misc, int digit) {
@@ -275,7 +421,36 @@ __device__ void cta_topk(const Item& it, unsigned char* smem, uint64_t* cand_r, 
     uint64_t* sr = reinterpret_cast<uint64_t*>(smem);
     uint32_t* srid = reinterpret_cast<uint32_t*>(smem + 2 * BT_SMALL * 8);
     unsigned* hist = reinterpret_cast<unsigned*>(smem);
+    const int kb = it.w4 ? 32 : 64;
+    const int TB = kb + 32;
+    bool cand = false;
+    uint64_t src_n = n;
+    int L = 0;
+    Range g;
+    if (n > BT_SMALL && kk <= n / 16) {
+        const double lam = static_cast<double>(kk) * BT_SAMPLE / static_cast<double>(n);
+        unsigned r = static_cast<unsigned>(ceil(lam + 4.0 * sqrt(lam))) + 3u;
+        if (r > BT_SAMPLE) r = BT_SAMPLE;
+        g = cta_sample_range(it, r, hist, sc, digit);
+        const unsigned c = it.w4 ? cta_filter<true>(it, g.rhi, cand_r, cand_rid, &s_misc[0])
+                                  : cta_filter<false>(it, g.rhi, cand_r, cand_rid, &s_misc[0]);
+        if (c >= kk && c <= BT_CAND) {
+            cand = true;
+            src_n = c;
+            const int lz = __clzll(static_cast<long long>(g.rhi));
+            L = lz < kb ? lz : kb;
+        }
+    }
+    // (an input too small or a K too large for a sample: its own span; after a
+    // misjudged sample the refine below is as quick)
+    const bool small = n <= BT_SMALL || kk > n / 16;
+    if (small) g = cta_input_range(it, sc);
+    if ((cand || small) && cta_bin_select(it, cand, cand_r, cand_rid, src_n, kk, CtaBins(g), smem, sc)) {
+        if (threadIdx.x == 0) *it.count = kk;
+        return;
+    }
     if (n <= BT_SMALL) {
+        __syncthreads();
         for (uint64_t i = threadIdx.x; i < n; i += BT_TPB) sr[i] = item_rank(it, i, &srid[i]);
         __syncthreads();
         block_sort<BT_TPB>(sr, srid, static_cast<int>(n));
@@ -283,26 +458,7 @@ __device__ void cta_topk(const Item& it, unsigned char* smem, uint64_t* cand_r, 
         if (threadIdx.x == 0) *it.count = kk;
         return;
     }
-    const int kb = it.w4 ? 32 : 64;
-    const int TB = kb + 32;
-    bool cand = false;
-    uint64_t src_n = n;
-    int L = 0;
-    if (kk <= n / 16) {
-        const double lam = static_cast<double>(kk) * BT_SAMPLE / static_cast<double>(n);
-        unsigned r = static_cast<unsigned>(ceil(lam + 4.0 * sqrt(lam))) + 3u;
-        if (r > BT_SAMPLE) r = BT_SAMPLE;
-        const uint64_t t = cta_sample_threshold(it, r, hist, sc, digit);
-        __syncthreads();
-        const unsigned c = it.w4 ? cta_filter<true>(it, t, smem, cand_r, cand_rid, &s_misc[0])
-                                  : cta_filter<false>(it, t, smem, cand_r, cand_rid, &s_misc[0]);
-        if (c >= kk && c <= BT_CAND) {
-            cand = true;
-            src_n = c;
-            const int lz = __clzll(static_cast<long long>(t));
-            L = lz < kb ? lz : kb;
-        }
-    }
+    __syncthreads();
     // Block-local radix refine of the (rank word, row-id) prefix.
     uint64_t p0 = 0, p1 = 0, krem = kk, bcnt = src_n;
     const unsigned lane = threadIdx.x & 31u;
@@ -661,7 +817,9 @@ olap_status olap_batch_create(olap_ctx* ctx, const olap_batch_item* items, uint6
     // and a merge item selects the item's Top-K from the parts' results in a
     // second launch.  Measured on the 4096-query batch, where no item exceeds
     // the share, splitting every item above 2^19 keys was slower (8.0 against
-    // 6.3 ms): the parts' fixed costs outweigh a tail that is not there.
+    // 6.3 ms): the parts' fixed costs outweigh a tail that is not there.  A
+    // CTA streams at most 32 GB/s, so small batches gain from small parts (64
+    // items, 1.9 * 10^7 keys, parts from 2^18 or 2^16 rows: 239 or 147 us).
     const int topk_ctas_hint = ctx->sm_count * 2;
     double topk_bytes = 0.0;
     for (uint64_t i = 0; i < n_items; ++i)
