@@ -66,6 +66,7 @@ struct __align__(8) Item {
     uint32_t* out_rowids;
     const uint64_t* table;       // probe: buckets of 2 x 16-byte slots
     uint64_t mask;
+    uint64_t chain_mask;
     const uint32_t* side;
     uint64_t n_side;
     uint2* out_pairs;
@@ -632,6 +633,7 @@ __global__ void __launch_bounds__(JP_TPB, JP_CTAS) batch_probe_kernel(const Item
                 s_args.n = it.n;
                 s_args.slots = reinterpret_cast<const ulonglong2*>(it.table);
                 s_args.mask = it.mask;
+                s_args.chain_mask = it.chain_mask;
                 s_args.side = it.side;
                 s_args.n_side = it.n_side;
                 s_args.out = it.out_pairs;
@@ -790,6 +792,7 @@ olap_status olap_batch_create(olap_ctx* ctx, const olap_batch_item* items, uint6
             if (x.table->device != ctx->device) return fail(ctx, OLAP_E_INVALID, "batch item: table on another device");
             d.table = reinterpret_cast<const uint64_t*>(x.table->slots);
             d.mask = x.table->n_buckets - 1;
+            d.chain_mask = x.table->chain_mask;
             d.side = x.table->side;
             d.n_side = x.table->n_side;
             d.out_pairs = reinterpret_cast<uint2*>(x.out_pairs);

@@ -96,11 +96,13 @@ __device__ __forceinline__ void rank_count(unsigned& c, uint64_t jr, uint32_t jr
           "r"(static_cast<uint32_t>(jr >> 32)), "r"(ties ? 1u : 0u), "r"(static_cast<uint32_t>(er >> 32)));
 }
 
-// Block-wide exclusive scan over one value per thread (TPB threads, <= 1024).
+// Block-wide exclusive scan over one value per thread (TPB threads; warp_sums
+// holds a word per warp, and callers keep the total 16 words after it).
 template <int TPB>
 __device__ __forceinline__ unsigned long long block_excl_scan(unsigned long long v,
                                                               unsigned long long* warp_sums,
                                                               unsigned long long* total) {
+    static_assert(TPB <= 512, "16 warp sums");
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     unsigned long long incl = v;
 #pragma unroll

@@ -9,9 +9,14 @@
 // with all bits set; build rows carrying that key value live in a side list.
 // Hash: the 64-bit finalizer of MurmurHash3 (fmix64, A. Appleby).
 //
-// Build: one CAS pass, then a pass that records in every occupied slot how
-// many further copies of its key follow it along the chain, so a probe can
-// stop at a key's last copy instead of walking on to the chain's end.
+// Build: the rows are appended to the table blocks (1024 buckets) their home
+// buckets lie in, and every block is then built in one CTA's shared memory:
+// insertion, the count of further copies of its key along the chain in every
+// slot (so a probe can stop at a key's last copy instead of walking on to the
+// chain's end), and the block's part of the Bloom filter.  Chains wrap within
+// their block.  A block with more rows than slots (thousands of copies of one
+// key) sends the whole build to the general way: one CAS pass over the table,
+// a pass over its chains, and chains that wrap at the table's end.
 //
 // Probe: every warp takes chunks of consecutive rows from a global counter
 // (the loads of keys and row-ids coalesce) and probes them a tile of 128 rows
@@ -44,6 +49,251 @@ namespace olap {
 
 namespace {
 
+// Build, first pass: every row goes, as a 16-byte entry {key, row-id}, to the
+// next free places of its home bucket's block, in the memory that the block's
+// slots will take.  The places come from the block's cursor, which sits in the
+// block's last slot (zeroed before the launch).  A CTA takes a tile of rows,
+// counts them per block, takes the places of all its rows of a block with one
+// global atomic, puts the tile in block order in shared memory and writes it
+// out from there, so that the rows of a block are written side by side: a
+// lone 16-byte write costs the L2 a whole sector, and those are the bound
+// (2^24 rows: 712 us row by row, 330 us with the partition passes before this
+// one; 4 * 10^6 rows in one pass 62 us, two rows per block and tile).
+// The blocks of a tile span at most JS_BINS: all blocks of a small table, or,
+// for larger ones, those of the few partitions that the tile's rows are
+// already ordered by; a tile that spans more goes row by row.
+constexpr int JS_TPB = 512;
+constexpr int JS_PER = 8;
+constexpr int JS_TILE = JS_TPB * JS_PER;
+constexpr int JS_BINS = 4096;
+constexpr int JS_SMEM = JS_TILE * 12 + JS_BINS * 8;
+constexpr int JS_PARTS = 64;                                  // partitions of a larger build's rows
+static_assert(JS_TPB <= 512 && JS_TILE <= 65535, "scan words; ranks in 16 bits");
+
+__global__ void __launch_bounds__(JS_TPB, 2) join_block_scatter_kernel(const int64_t* keys, const uint32_t* rowids,
+                                                                       uint64_t n, int per, ulonglong2* slots,
+                                                                       uint64_t mask, int block_log, JoinCtl* ctl) {
+    extern __shared__ __align__(16) unsigned char ssmem[];
+    uint64_t* sk = reinterpret_cast<uint64_t*>(ssmem);                       // the tile in block order
+    uint32_t* sr = reinterpret_cast<uint32_t*>(ssmem + JS_TILE * 8);
+    unsigned* off = reinterpret_cast<unsigned*>(ssmem + JS_TILE * 12);       // rows per block, then first position
+    unsigned* base = off + JS_BINS;                                          // first place minus first position
+    __shared__ unsigned lo, hi;                                              // the tile's blocks
+    __shared__ unsigned long long sc[24];
+    const unsigned room = (2u << block_log) - 1u;             // entries a block may hold: one slot stays free
+    auto cursor = [&](uint64_t blk) {
+        return reinterpret_cast<unsigned*>(slots + (blk << (block_log + 1)) + room);
+    };
+    auto block_of = [&](uint64_t key) { return static_cast<unsigned>((fmix64(key) & mask) >> block_log); };
+    bool crowded = false;
+    unsigned side = 0;
+    auto put = [&](unsigned blk, unsigned pos, uint64_t key, uint32_t rid) {
+        if (pos < room) slots[(static_cast<uint64_t>(blk) << (block_log + 1)) + pos] = make_ulonglong2(key, rid);
+        else crowded = true;
+    };
+    const uint64_t tile = static_cast<uint64_t>(per) * JS_TPB;               // per <= JS_PER rows per thread
+    for (uint64_t t0 = blockIdx.x * tile; t0 < n; t0 += gridDim.x * tile) {
+        uint64_t key[JS_PER];
+        uint32_t rid[JS_PER];
+        unsigned at[JS_PER];                                  // block, then rank in its block | block << 16
+#pragma unroll
+        for (int j = 0; j < JS_PER; ++j) {
+            const uint64_t i = t0 + static_cast<uint64_t>(j) * JS_TPB + threadIdx.x;
+            const bool in = j < per && i < n;
+            key[j] = in ? ld_stream_u64(keys + i) : JN_EMPTY;
+            rid[j] = (in && rowids) ? ld_stream_u32(rowids + i) : static_cast<uint32_t>(i);
+            side += (in && key[j] == JN_EMPTY) ? 1u : 0u;
+        }
+        for (unsigned b = threadIdx.x; b < JS_BINS; b += JS_TPB) off[b] = 0;
+        if (threadIdx.x == 0) {
+            lo = ~0u;
+            hi = 0;
+        }
+        __syncthreads();
+        unsigned mn = ~0u, mx = 0;
+#pragma unroll
+        for (int j = 0; j < JS_PER; ++j) {
+            at[j] = block_of(key[j]);
+            if (key[j] != JN_EMPTY) {
+                mn = min(mn, at[j]);
+                mx = max(mx, at[j]);
+            }
+        }
+        mn = __reduce_min_sync(0xFFFFFFFFu, mn);
+        mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+        if ((threadIdx.x & 31u) == 0) {
+            atomicMin(&lo, mn);
+            atomicMax(&hi, mx);
+        }
+        __syncthreads();
+        const unsigned b0 = lo;
+        if (b0 != ~0u && hi - b0 < JS_BINS) {
+#pragma unroll
+            for (int j = 0; j < JS_PER; ++j)
+                if (key[j] != JN_EMPTY) at[j] = (at[j] - b0) | (atomicAdd(&off[at[j] - b0], 1u) << 16);
+            __syncthreads();
+            constexpr int PER = JS_BINS / JS_TPB;
+            unsigned c[PER];
+            unsigned total = 0;
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                c[q] = off[threadIdx.x * PER + q];
+                total += c[q];
+            }
+            unsigned run = static_cast<unsigned>(block_excl_scan<JS_TPB>(total, sc, sc + 16));
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const unsigned b = threadIdx.x * PER + q;
+                off[b] = run;
+                if (c[q]) base[b] = atomicAdd(cursor(static_cast<uint64_t>(b0) + b), c[q]) - run;
+                run += c[q];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < JS_PER; ++j)
+                if (key[j] != JN_EMPTY) {
+                    const unsigned p = off[at[j] & 0xFFFFu] + (at[j] >> 16);
+                    sk[p] = key[j];
+                    sr[p] = rid[j];
+                }
+            __syncthreads();
+            const unsigned len = static_cast<unsigned>(sc[16]);               // the scan's total
+            for (unsigned p = threadIdx.x; p < len; p += JS_TPB) {
+                const unsigned blk = block_of(sk[p]);
+                put(blk, base[blk - b0] + p, sk[p], sr[p]);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < JS_PER; ++j)
+                if (key[j] != JN_EMPTY) put(at[j], atomicAdd(cursor(at[j]), 1u), key[j], rid[j]);
+        }
+        __syncthreads();                                      // before the next tile clears the bins
+    }
+    if (crowded) ctl->crowded = 1;
+    side = __reduce_add_sync(0xFFFFFFFFu, side);
+    if ((threadIdx.x & 31u) == 0 && side) atomicAdd(&ctl->side_count, static_cast<unsigned long long>(side));
+}
+
+// Build, second pass: one block of the table at a time per CTA.  Its entries
+// are taken into registers, inserted in shared memory (first free slot at or
+// after the home bucket, slot 0 before slot 1, wrapping within the block),
+// counted along their chains, and the whole block is written over them: the
+// table is written once, in order, and needs no clearing.  A block keeps a
+// free slot, so every chain in it ends.  Bound by the instructions of the
+// insertion and by the writes.  With the passes before and the Bloom filter,
+// 4 * 10^6 rows take 148 us and 2^24 rows 705 us, where clearing the table, a
+// CAS and a chain walk per row and eight atomics on the filter took 364 and
+// 2352 us.
+constexpr uint64_t JS_PART_MIN_N = 1ull << 22;                // smaller builds go row by row
+constexpr int JT_TPB = 512;
+constexpr int JT_SLOTS = 2 * static_cast<int>(JT_BLOCK);
+constexpr int JT_PER = JT_SLOTS / JT_TPB;
+constexpr int JT_BLOOM_MAX = 256;                             // filter blocks per table block in shared memory
+constexpr int JT_SMEM = JT_SLOTS * 16 + JT_BLOOM_MAX * 32;
+
+__global__ void __launch_bounds__(JT_TPB, 3) join_block_build_kernel(ulonglong2* slots, uint64_t blocks, int block_log,
+                                                                     uint32_t* bloom, int per_log, JoinCtl* ctl) {
+    extern __shared__ __align__(16) unsigned char tsmem[];
+    uint64_t* sk = reinterpret_cast<uint64_t*>(tsmem);                       // keys of the block's slots
+    uint32_t* sr = reinterpret_cast<uint32_t*>(tsmem + JT_SLOTS * 8);        // their row-ids
+    uint32_t* sb = reinterpret_cast<uint32_t*>(tsmem + JT_SLOTS * 12);       // the block's filter words
+    __shared__ int copies;                                                   // some key of the block has several
+    if (ctl->crowded) return;                                                // (set by the pass before)
+    const unsigned bm = (1u << block_log) - 1u;
+    const unsigned nslots = 2u << block_log;
+    const unsigned nwords = bloom ? (BLOOM_WORDS << per_log) : 0u;
+    uint64_t k[JT_PER];
+    uint32_t r[JT_PER];
+    auto cursor = [&](uint64_t blk) {
+        return blk < blocks ? __ldcg(reinterpret_cast<const unsigned*>(slots + (blk + 1) * nslots - 1)) : 0u;
+    };
+    auto load = [&](uint64_t blk, unsigned cnt) {
+#pragma unroll
+        for (int j = 0; j < JT_PER; ++j) {
+            const unsigned i = static_cast<unsigned>(j) * JT_TPB + threadIdx.x;
+            k[j] = JN_EMPTY;
+            if (i < cnt) {
+                const ulonglong2 e = __ldcg(slots + blk * nslots + i);
+                k[j] = e.x;
+                r[j] = static_cast<uint32_t>(e.y);
+            }
+        }
+    };
+    uint64_t blk = blockIdx.x;
+    load(blk, cursor(blk));
+    unsigned next_cnt = cursor(blk + gridDim.x);
+    for (; blk < blocks; blk += gridDim.x) {
+        ulonglong2* mine = slots + blk * nslots;
+        for (unsigned i = threadIdx.x; i < nslots / 2; i += JT_TPB)
+            reinterpret_cast<ulonglong2*>(sk)[i] = make_ulonglong2(JN_EMPTY, JN_EMPTY);
+        for (unsigned i = threadIdx.x; i < nwords; i += JT_TPB) sb[i] = 0u;
+        if (threadIdx.x == 0) copies = 0;
+        __syncthreads();                                     // (every thread has its entries in registers)
+        bool met = false;                                    // a copy of a key of this thread on its way
+#pragma unroll
+        for (int j = 0; j < JT_PER; ++j) {
+            if (k[j] == JN_EMPTY) continue;
+            const uint64_t h = fmix64(k[j]);
+            unsigned at = 2u * (static_cast<unsigned>(h) & bm);
+            while (true) {
+                unsigned long long c = *reinterpret_cast<volatile unsigned long long*>(sk + at);
+                if (c == JN_EMPTY)
+                    c = atomicCAS(reinterpret_cast<unsigned long long*>(sk + at), JN_EMPTY,
+                                  static_cast<unsigned long long>(k[j]));
+                if (c == JN_EMPTY) break;
+                met = met || c == k[j];
+                at = (at + 1u) & (nslots - 1u);              // slot 1, then slot 0 of the next bucket
+            }
+            sr[at] = r[j];
+            if (nwords) {
+                // the lanes go through the words of their blocks in different
+                // orders: in the same order they would meet on four banks
+                uint32_t* fb = sb + (static_cast<unsigned>(h >> 40) & ((1u << per_log) - 1u)) * BLOOM_WORDS;
+                const uint64_t g = bloom_bits(h);
+#pragma unroll
+                for (unsigned v = 0; v < BLOOM_WORDS; ++v) {
+                    const int w = static_cast<int>((v + threadIdx.x) & (BLOOM_WORDS - 1));
+                    atomicOr(fb + w, bloom_bit(g, w));
+                }
+            }
+        }
+        if (met) copies = 1;
+        // the next block's entries, on their way while this block is finished
+        load(blk + gridDim.x, next_cnt);
+        next_cnt = cursor(blk + 2ull * gridDim.x);
+        __syncthreads();
+        // Of two copies of a key the one further along passed the other on
+        // its way, so a block where no thread met one has none to count.
+        const bool count = copies != 0;
+        for (unsigned b0 = threadIdx.x; b0 <= bm; b0 += JT_TPB) {            // a bucket at a time
+            const ulonglong2 kk = reinterpret_cast<const ulonglong2*>(sk)[b0];
+            const uint2 rr = reinterpret_cast<const uint2*>(sr)[b0];
+            uint32_t f0 = 0, f1 = 0;                                         // further copies
+            if (count) {
+                f0 = kk.x != JN_EMPTY && kk.y == kk.x ? 1u : 0u;
+                unsigned b = b0;
+                uint64_t k1 = kk.y;
+                while (k1 != JN_EMPTY) {                                     // bucket b full: the chain goes on
+                    b = (b + 1u) & bm;
+                    if (b == b0) break;                                      // (once round: a block keeps a free slot)
+                    const uint64_t k0 = sk[2 * b];
+                    k1 = sk[2 * b + 1];
+                    f0 += (k0 == kk.x) + (k1 == kk.x);
+                    f1 += (k0 == kk.y) + (k1 == kk.y);
+                }
+            }
+            const uint64_t w0 = kk.x == JN_EMPTY ? ~0ull : rr.x | (static_cast<uint64_t>(f0) << 32);
+            const uint64_t w1 = kk.y == JN_EMPTY ? ~0ull : rr.y | (static_cast<uint64_t>(f1) << 32);
+            asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(mine + 2 * b0), "l"(kk.x), "l"(w0), "l"(kk.y),
+                         "l"(w1)
+                         : "memory");
+        }
+        for (unsigned i = threadIdx.x; i < nwords; i += JT_TPB) bloom[blk * nwords + i] = sb[i];
+        __syncthreads();
+    }
+}
+
+// The general build, for tables whose blocks do not hold their rows.
 __global__ void __launch_bounds__(JB_TPB) join_build_kernel(const int64_t* keys, const uint32_t* rowids,
                                                             uint64_t n, ulonglong2* slots, uint64_t mask,
                                                             JoinCtl* ctl) {
@@ -152,13 +402,14 @@ __global__ void __launch_bounds__(JP_TPB, JP_CTAS) join_probe_kernel(ProbeArgs a
 // kept in the side list, is not entered: the pre-probe keeps such probe rows
 // whatever the filter says).
 __global__ void __launch_bounds__(JB_TPB) join_bloom_kernel(const int64_t* keys, uint64_t n, uint32_t* bloom,
-                                                            uint64_t bmask) {
+                                                            BloomView f) {
     const uint64_t stride = static_cast<uint64_t>(gridDim.x) * JB_TPB;
     for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * JB_TPB + threadIdx.x; i < n; i += stride) {
         const uint64_t key = static_cast<uint64_t>(keys[i]);
         if (key == JN_EMPTY) continue;
-        uint32_t* blk = bloom + bloom_block(key, bmask) * BLOOM_WORDS;
-        const uint64_t g = fmix64(~key);
+        const uint64_t h = fmix64(key);
+        uint32_t* blk = bloom + bloom_block(f, h) * BLOOM_WORDS;
+        const uint64_t g = bloom_bits(h);
 #pragma unroll
         for (int w = 0; w < BLOOM_WORDS; ++w) atomicOr(blk + w, bloom_bit(g, w));
     }
@@ -169,6 +420,7 @@ constexpr int PF_SAMPLE = 4096;                // probe keys tested to decide
 constexpr uint64_t PF_MIN_N = 1ull << 20;      // smaller probes skip the pre-probe (automatic mode)
 constexpr int PF_PER = 4;                      // keys per lane per step
 constexpr unsigned PF_WCAP = 256;              // rows staged per warp
+constexpr int PF_CTAS = 6;                     // pre-probe CTAs per SM
 
 constexpr int PLAN_SLOTS = 2 * PF_SAMPLE;      // fingerprint set of the sample (32 KB)
 constexpr int PLAN_CTAS = PF_SAMPLE / PF_TPB;  // one sampled key per thread
@@ -178,8 +430,7 @@ struct PlanArgs {
     const int64_t* keys;
     const uint32_t* rowids;
     uint64_t n;
-    const uint32_t* bloom;                     // NULL: no pre-probe stage
-    uint64_t bmask;
+    BloomView bloom;                           // bits NULL: no pre-probe stage
     int pf_mode;                               // 1 automatic, 2 forced (with a filter)
     int skew_check;
     int partitioned;
@@ -220,7 +471,7 @@ __global__ void __launch_bounds__(PF_TPB) join_probe_plan_kernel(PlanArgs a) {
     {
         const uint64_t j = static_cast<uint64_t>(blockIdx.x) * PF_TPB + threadIdx.x;     // < PF_SAMPLE
         const uint64_t key = static_cast<uint64_t>(a.keys[(j * a.n) / PF_SAMPLE]);
-        const bool kept = a.bloom ? (key == JN_EMPTY || bloom_maybe(a.bloom, a.bmask, key)) : true;
+        const bool kept = a.bloom.bits ? (key == JN_EMPTY || bloom_maybe(a.bloom, key)) : true;
         const uint32_t fp = static_cast<uint32_t>(fmix64(key) >> 32) & ~3u;
         a.sample[j] = fp | (kept ? 2u : 0u) | 1u;
         if (kept) atomicAdd(&kept_cta, 1u);
@@ -262,7 +513,7 @@ __global__ void __launch_bounds__(PF_TPB) join_probe_plan_kernel(PlanArgs a) {
     __syncthreads();
     if (threadIdx.x == 0) {
         const unsigned passes = atomicAdd(&a.counters[0], 0u);
-        const bool active = a.bloom && (a.pf_mode == 2 || passes * 10u <= static_cast<unsigned>(PF_SAMPLE) * 6u);
+        const bool active = a.bloom.bits && (a.pf_mode == 2 || passes * 10u <= static_cast<unsigned>(PF_SAMPLE) * 6u);
         const unsigned reach = active ? passes : static_cast<unsigned>(PF_SAMPLE);
         const unsigned rep = active ? dup_kept : dup_all;
         const bool direct = a.skew_check && reach >= 64u && rep * 5u >= reach;
@@ -282,10 +533,13 @@ __global__ void __launch_bounds__(PF_TPB) join_probe_plan_kernel(PlanArgs a) {
 // The pre-probe: one streaming pass over the probe rows that keeps the rows
 // whose key may be in the table (and every row with the empty-marker key),
 // appended with their row-ids through a per-warp stage, one atomic per flush.
-__global__ void __launch_bounds__(PF_TPB) join_prefilter_kernel(const int64_t* keys, const uint32_t* rowids,
-                                                                uint64_t n, const uint32_t* bloom, uint64_t bmask,
-                                                                ProbeCtl* ctl, int64_t* out_keys,
-                                                                uint32_t* out_rowids) {
+// Bound by the latency of the keys and of the random filter-block reads from
+// L2, so as many warps as fit: six CTAs per SM for four, 2^25 Zipf rows against
+// a 2^24-row table, a tenth kept, 249 -> 227 us for the whole probe.  (Loading
+// the next keys ahead costs the registers that hold the filter blocks: 268.)
+__global__ void __launch_bounds__(PF_TPB, PF_CTAS) join_prefilter_kernel(const int64_t* keys, const uint32_t* rowids,
+                                                                uint64_t n, BloomView bloom, ProbeCtl* ctl,
+                                                                int64_t* out_keys, uint32_t* out_rowids) {
     if (!ctl->active) return;
     __shared__ int64_t sk[PF_TPB / 32][PF_WCAP];
     __shared__ uint32_t sr[PF_TPB / 32][PF_WCAP];
@@ -319,7 +573,7 @@ __global__ void __launch_bounds__(PF_TPB) join_prefilter_kernel(const int64_t* k
 #pragma unroll
         for (int j = 0; j < PF_PER; ++j) {
             const uint64_t i = g * G + static_cast<uint64_t>(j) * 32 + lane;
-            const bool maybe = bloom_maybe(bloom, bmask, key[j]);
+            const bool maybe = bloom_maybe(bloom, key[j]);
             keep[j] = i < n && (key[j] == JN_EMPTY || maybe);
         }
 #pragma unroll
@@ -554,6 +808,30 @@ int probe_grid(int device) {
     return cached[device].load();
 }
 
+// Resident CTAs of the two block build kernels.
+int block_build_grid(int device, int* scatter) {
+    static std::atomic<int> cached[64] = {};                  // build | scatter << 16
+    if (device < 0 || device >= 64) return 0;
+    int c = cached[device].load();
+    if (!c) {
+        int sms = 0, per = 0, per_s = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+            cudaFuncSetAttribute(join_block_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, JT_SMEM) !=
+                cudaSuccess ||
+            cudaFuncSetAttribute(join_block_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, JS_SMEM) !=
+                cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, join_block_build_kernel, JT_TPB, JT_SMEM) !=
+                cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_s, join_block_scatter_kernel, JS_TPB, JS_SMEM) !=
+                cudaSuccess)
+            return 0;
+        c = sms * std::max(1, per) | (sms * std::max(1, per_s)) << 16;
+        cached[device].store(c);
+    }
+    *scatter = c >> 16;
+    return c & 0xFFFF;
+}
+
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
 // Grid of the two partition passes.  Both take the same one (the scatter
@@ -592,6 +870,19 @@ int probe_parts(const olap_ctx* ctx, const olap_join_table* t, uint64_t n) {
     return static_cast<int>(std::max<uint64_t>(parts, 1));
 }
 
+// log2 of a table block's buckets (smaller tables are one block) and of its
+// Bloom filter blocks.
+static int log2_of(uint64_t x) {
+    int l = 0;
+    while ((1ull << l) < x) ++l;
+    return l;
+}
+static int table_block_log(uint64_t n_buckets) { return std::min(JT_BLOCK_LOG, log2_of(n_buckets)); }
+static BloomView bloom_view(const olap_join_table* t) {
+    const int bl = table_block_log(t->n_buckets);
+    return BloomView{t->bloom, t->n_buckets - 1, bl, log2_of(t->bloom_blocks) - (log2_of(t->n_buckets) - bl)};
+}
+
 // Whether a probe of n rows against t runs the Bloom pre-probe stage (its
 // sample still decides on the device whether rows are dropped).
 bool probe_prefilter(const olap_ctx* ctx, const olap_join_table* t, uint64_t n) {
@@ -614,6 +905,26 @@ size_t probe_scratch_bytes(const olap_ctx* ctx, const olap_join_table* t, uint64
     const size_t pb = probe_part_bytes(ctx, n, probe_parts(ctx, t, n));
     if (!probe_prefilter(ctx, t, n)) return pb;
     return pb + align256(n * 8) + align256(n * 4);
+}
+
+// The partition passes over n rows by the top bits of their home bucket, in
+// the context's partition scratch (which holds probe_part_bytes).
+static PartArgs part_args(const olap_ctx* ctx, const int64_t* keys, const uint32_t* rowids, uint64_t n,
+                          uint64_t n_buckets, int parts, unsigned grid) {
+    unsigned char* m = static_cast<unsigned char*>(ctx->part);
+    PartArgs q{};
+    q.keys = keys;
+    q.rowids = rowids;
+    q.n = n;
+    q.mask = n_buckets - 1;
+    q.shift = 0;
+    while ((n_buckets >> q.shift) > static_cast<uint64_t>(parts)) ++q.shift;
+    q.parts = parts;
+    q.out_keys = reinterpret_cast<int64_t*>(m);
+    q.out_rowids = reinterpret_cast<uint32_t*>(m + align256(n * 8));
+    q.cnt = reinterpret_cast<unsigned long long*>(m + align256(n * 8) + align256(n * 4));
+    q.pstart = q.cnt + static_cast<uint64_t>(grid) * parts;
+    return q;
 }
 
 }  // namespace olap
@@ -641,6 +952,7 @@ olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t
     a.n = n;
     a.slots = t->slots;
     a.mask = t->n_buckets - 1;
+    a.chain_mask = t->chain_mask;
     a.side = t->side;
     a.n_side = t->n_side;
     a.out = reinterpret_cast<uint2*>(d_out);
@@ -668,21 +980,10 @@ olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t
             return fail(ctx, OLAP_E_INVALID, "probe pre-filter scratch too small");
     }
     if (parts > 1) {
-        unsigned char* m = static_cast<unsigned char*>(ctx->part);
         qgrid = static_cast<unsigned>(part_grid(ctx->device, ctx->sm_count));
         if (qgrid == 0) return fail(ctx, OLAP_E_CUDA, "partition kernel occupancy query failed");
-        q.keys = d_keys;
-        q.rowids = d_rowids;
-        q.n = n;
-        q.mask = a.mask;
-        q.shift = 0;
-        while ((t->n_buckets >> q.shift) > static_cast<uint64_t>(parts)) ++q.shift;
-        q.parts = parts;
-        q.out_keys = reinterpret_cast<int64_t*>(m);
-        q.out_rowids = reinterpret_cast<uint32_t*>(m + align256(n * 8));
-        q.cnt = reinterpret_cast<unsigned long long*>(m + align256(n * 8) + align256(n * 4));
-        q.pstart = q.cnt + static_cast<uint64_t>(qgrid) * parts;
-        if (q.pstart + parts + 1 > reinterpret_cast<unsigned long long*>(m + ctx->part_bytes))
+        q = part_args(ctx, d_keys, d_rowids, n, t->n_buckets, parts, qgrid);
+        if (q.pstart + parts + 1 > reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(ctx->part) + ctx->part_bytes))
             return fail(ctx, OLAP_E_INVALID, "probe partition scratch too small");
         q.pf = pf;
         q.pf_keys = pf_keys;
@@ -699,7 +1000,7 @@ olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t
     if ((e = cudaMemsetAsync(next_row, 0, sizeof(unsigned long long), s)) != cudaSuccess)
         return cuda_fail(ctx, e, "probe queue reset");
     ProbeArgs pa = a;
-    const uint64_t bmask = pre ? t->bloom_blocks - 1 : 0;
+    const BloomView bloom = pre ? bloom_view(t) : BloomView{nullptr, 0, 0, 0};
     if (pf) {
         const int pf_mode = pre ? (ctx->opts.join_prefilter == OLAP_PREFILTER_ON ? 2 : 1) : 0;
         const int skew_l1 = ctx->opts.join_bucket_loads == OLAP_LOADS_AUTO ? 1 : 0;
@@ -707,8 +1008,7 @@ olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t
         pl.keys = d_keys;
         pl.rowids = d_rowids;
         pl.n = n;
-        pl.bloom = pre ? t->bloom : nullptr;
-        pl.bmask = bmask;
+        pl.bloom = bloom;
         pl.pf_mode = pf_mode;
         pl.skew_check = skew_check ? 1 : 0;
         pl.partitioned = parts > 1 ? 1 : 0;
@@ -721,8 +1021,8 @@ olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t
         join_probe_plan_kernel<<<PLAN_CTAS, PF_TPB, 0, s>>>(pl);
     }
     if (pre)
-        join_prefilter_kernel<<<ctx->sm_count * 4, PF_TPB, 0, s>>>(d_keys, d_rowids, n, t->bloom, bmask, pf,
-                                                                   pf_keys, pf_rowids);
+        join_prefilter_kernel<<<ctx->sm_count * PF_CTAS, PF_TPB, 0, s>>>(d_keys, d_rowids, n, bloom, pf, pf_keys,
+                                                                   pf_rowids);
     if (parts > 1) {
         join_part_count_kernel<<<qgrid, JQ_TPB, 0, s>>>(q);
         join_part_scatter_kernel<<<qgrid, JQ_TPB, 0, s>>>(q);
@@ -774,7 +1074,9 @@ olap_status olap_join_build(olap_ctx* ctx, const int64_t* keys, const uint32_t* 
     const uint64_t l2 = ctx->l2_bytes ? ctx->l2_bytes : (64ull << 20);
     const bool with_bloom = n && (ctx->opts.join_prefilter == OLAP_PREFILTER_ON ||
                                   (ctx->opts.join_prefilter == OLAP_PREFILTER_AUTO && slot_bytes > l2 / 2));
-    const uint64_t bloom_blocks = with_bloom ? next_pow2((n + 15) / 16) : 0;
+    const int block_log = table_block_log(buckets);
+    const uint64_t blocks = buckets >> block_log;
+    const uint64_t bloom_blocks = with_bloom ? std::max(next_pow2((n + 15) / 16), blocks) : 0;
     const size_t bytes = slot_bytes + 256 + bloom_blocks * 32;
     if (!within_budget(ctx, bytes)) return fail(ctx, OLAP_E_NOMEM, "join table: device memory budget exceeded");
 
@@ -819,30 +1121,79 @@ olap_status olap_join_build(olap_ctx* ctx, const int64_t* keys, const uint32_t* 
         t->bloom = reinterpret_cast<uint32_t*>(static_cast<unsigned char*>(mem) + slot_bytes + 256);
         t->bloom_blocks = bloom_blocks;
     }
-    e = cudaMemsetAsync(mem, 0xFF, slot_bytes, ctx->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(jc, 0, sizeof(JoinCtl), ctx->stream);
-    if (e == cudaSuccess && bloom_blocks) e = cudaMemsetAsync(t->bloom, 0, bloom_blocks * 32, ctx->stream);
+    // Two passes over table blocks; the general build when there are no rows,
+    // when a block's filter does not fit in shared memory, or when a block
+    // turned out crowded.
+    const int grid = ctx->sm_count * 8;
+    const int per_log = bloom_blocks ? log2_of(bloom_blocks) - log2_of(blocks) : 0;
+    bool general = n == 0 || (1 << per_log) > JT_BLOOM_MAX;
+    JoinCtl hc{};
+    auto read_ctl = [&]() -> olap_status {
+        e = cudaMemcpyAsync(ctx->host_status, jc, sizeof(hc), cudaMemcpyDeviceToHost, ctx->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "join build");
+        std::memcpy(&hc, ctx->host_status, sizeof(hc));
+        return OLAP_OK;
+    };
+    e = cudaMemsetAsync(jc, 0, sizeof(JoinCtl), ctx->stream);
     if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "join table init"));
-    if (n) {
-        const int grid = ctx->sm_count * 8;
-        join_build_kernel<<<grid, JB_TPB, 0, ctx->stream>>>(dk, dr, n, t->slots, buckets - 1, jc);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "build launch"));
-        join_chain_kernel<<<grid, JB_TPB, 0, ctx->stream>>>(t->slots, buckets - 1);
+    if (!general) {
+        const size_t pitch = 32ull << block_log;
+        int sgrid = 0;
+        const int bgrid = block_build_grid(ctx->device, &sgrid);
+        if (bgrid <= 0) return bail(fail(ctx, OLAP_E_CUDA, "block build kernel set-up failed"));
+        // the blocks' cursors, in their last slots
+        e = cudaMemset2DAsync(static_cast<unsigned char*>(mem) + pitch - 16, pitch, 0, 16, blocks, ctx->stream);
+        if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "join table init"));
+        // More blocks than a tile counts: the rows are first ordered by the
+        // upper bits of their block (the probe's partition passes), when there
+        // is room for that; without it the first pass goes row by row.
+        const int64_t* bk = dk;
+        const uint32_t* br = dr;
+        if (blocks > static_cast<uint64_t>(JS_BINS) && n >= JS_PART_MIN_N) {
+            const unsigned pgrid = static_cast<unsigned>(part_grid(ctx->device, ctx->sm_count));
+            if (pgrid && ensure_part(ctx, probe_part_bytes(ctx, n, JS_PARTS)) == OLAP_OK) {
+                const PartArgs q = part_args(ctx, dk, dr, n, buckets, JS_PARTS, pgrid);
+                join_part_count_kernel<<<pgrid, JQ_TPB, 0, ctx->stream>>>(q);
+                join_part_scatter_kernel<<<pgrid, JQ_TPB, 0, ctx->stream>>>(q);
+                ctx->launches += 2;
+                bk = q.out_keys;
+                br = q.out_rowids;
+            }
+            ctx->last_error.clear();
+        }
+        const uint64_t threads = static_cast<uint64_t>(sgrid) * JS_TPB;
+        const int per = static_cast<int>(std::min<uint64_t>((n + threads - 1) / threads, JS_PER));
+        const uint64_t tiles = (n + static_cast<uint64_t>(per) * JS_TPB - 1) / (static_cast<uint64_t>(per) * JS_TPB);
+        join_block_scatter_kernel<<<static_cast<unsigned>(std::min<uint64_t>(tiles, sgrid)), JS_TPB, JS_SMEM,
+                                    ctx->stream>>>(bk, br, n, per, t->slots, buckets - 1, block_log, jc);
+        join_block_build_kernel<<<static_cast<unsigned>(std::min<uint64_t>(blocks, bgrid)), JT_TPB, JT_SMEM,
+                                  ctx->stream>>>(t->slots, blocks, block_log, t->bloom, per_log, jc);
         e = cudaGetLastError();
         if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "build launch"));
         ctx->launches += 2;
-        if (bloom_blocks) {
-            join_bloom_kernel<<<grid, JB_TPB, 0, ctx->stream>>>(dk, n, t->bloom, bloom_blocks - 1);
-            e = cudaGetLastError();
-            if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "bloom launch"));
-            ctx->launches += 1;
-        }
+        olap_status st = read_ctl();
+        if (st != OLAP_OK) return bail(st);
+        t->chain_mask = (1ull << block_log) - 1;
+        general = hc.crowded != 0;
     }
-    JoinCtl hc;
-    e = cudaMemcpyAsync(&hc, jc, sizeof(hc), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "join build"));
+    if (general) {
+        t->chain_mask = buckets - 1;
+        e = cudaMemsetAsync(mem, 0xFF, slot_bytes, ctx->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(jc, 0, sizeof(JoinCtl), ctx->stream);
+        if (e == cudaSuccess && bloom_blocks) e = cudaMemsetAsync(t->bloom, 0, bloom_blocks * 32, ctx->stream);
+        if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "join table init"));
+        if (n) {
+            join_build_kernel<<<grid, JB_TPB, 0, ctx->stream>>>(dk, dr, n, t->slots, buckets - 1, jc);
+            join_chain_kernel<<<grid, JB_TPB, 0, ctx->stream>>>(t->slots, buckets - 1);
+            if (bloom_blocks) join_bloom_kernel<<<grid, JB_TPB, 0, ctx->stream>>>(dk, n, t->bloom, bloom_view(t));
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "build launch"));
+            ctx->launches += bloom_blocks ? 3 : 2;
+        }
+        olap_status st = read_ctl();
+        if (st != OLAP_OK) return bail(st);
+    }
     if (hc.err) return bail(fail(ctx, static_cast<olap_status>(hc.err), "join build: table full"));
     if (hc.side_count) {
         e = cudaMalloc(reinterpret_cast<void**>(&t->side), hc.side_count * 4);

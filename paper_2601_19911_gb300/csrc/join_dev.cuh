@@ -19,6 +19,7 @@ struct olap_join_table {
     size_t bytes = 0;
     uint32_t* bloom = nullptr;        // blocked Bloom filter over the keys (NULL: none)
     uint64_t bloom_blocks = 0;        // 32-byte blocks, a power of two
+    uint64_t chain_mask = 0;          // chains wrap within this many buckets + 1 (see join_block_build_kernel)
 };
 
 namespace olap {
@@ -45,8 +46,12 @@ struct JoinCtl {
     unsigned long long side_count;   // build rows with the empty-marker key
     unsigned long long side_fill;
     int err;
-    int pad;
+    int crowded;                     // a table block got more rows than it has room for
 };
+
+// Blocks of the table that are built in one CTA's shared memory.
+constexpr int JT_BLOCK_LOG = 10;                       // 1024 buckets, 32 KB
+constexpr uint64_t JT_BLOCK = 1ull << JT_BLOCK_LOG;
 
 __device__ __forceinline__ uint64_t fmix64(uint64_t h) {
     h ^= h >> 33;
@@ -77,28 +82,40 @@ __device__ __forceinline__ void st_stream_pair(uint2* p, uint2 v) {
 // Blocked Bloom filter (Putze, Sanders & Singler, "Cache-, hash- and
 // space-efficient Bloom filters", WEA 2007): every key maps to one 32-byte
 // block (one sector, one load) and sets one bit in each of the block's eight
-// 32-bit words.  The block comes from bits 40..63 of fmix64(key), which the
-// table's bucket index (the low bits) does not use; the eight bit positions
-// come from 40 bits of a second hash, fmix64 of the complemented key.
+// 32-bit words.  The filter blocks of the keys of one table block lie
+// together, so that the CTA that builds the table block also fills them: the
+// upper bits of the filter block are the table block's, the lower ones bits
+// 40 and up of fmix64(key), which the table's bucket index (the low bits) does
+// not use.  The eight bit positions are the upper 40 bits of that hash times an
+// odd constant.
 constexpr int BLOOM_WORDS = 8;
 
-__device__ __forceinline__ uint64_t bloom_block(uint64_t key, uint64_t bmask) {
-    return (fmix64(key) >> 40) & bmask;
+struct BloomView {
+    const uint32_t* bits;             // NULL: no filter
+    uint64_t mask;                    // table buckets - 1
+    int block_log;                    // log2 buckets of a table block
+    int per_log;                      // log2 filter blocks per table block
+};
+__device__ __forceinline__ uint64_t bloom_block(const BloomView& f, uint64_t h) {
+    return (((h & f.mask) >> f.block_log) << f.per_log) | ((h >> 40) & ((1ull << f.per_log) - 1ull));
 }
+// The eight bit positions of a key with hash h, five bits each.
+__device__ __forceinline__ uint64_t bloom_bits(uint64_t h) { return (h * 0x9E3779B97F4A7C15ull) >> 24; }
 __device__ __forceinline__ uint32_t bloom_bit(uint64_t g, int w) {
     return 1u << static_cast<uint32_t>((g >> (5 * w)) & 31u);
 }
 // Whether `key` may be among the filter's keys (no false negatives).
-__device__ __forceinline__ bool bloom_maybe(const uint32_t* bloom, uint64_t bmask, uint64_t key) {
-    const ulonglong2* p = reinterpret_cast<const ulonglong2*>(bloom + bloom_block(key, bmask) * BLOOM_WORDS);
-    uint64_t a, b, c, d;
-    asm("ld.global.cg.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
-    const uint64_t g = fmix64(~key);
-    const uint64_t want01 = static_cast<uint64_t>(bloom_bit(g, 0)) | (static_cast<uint64_t>(bloom_bit(g, 1)) << 32);
-    const uint64_t want23 = static_cast<uint64_t>(bloom_bit(g, 2)) | (static_cast<uint64_t>(bloom_bit(g, 3)) << 32);
-    const uint64_t want45 = static_cast<uint64_t>(bloom_bit(g, 4)) | (static_cast<uint64_t>(bloom_bit(g, 5)) << 32);
-    const uint64_t want67 = static_cast<uint64_t>(bloom_bit(g, 6)) | (static_cast<uint64_t>(bloom_bit(g, 7)) << 32);
-    return (a & want01) == want01 && (b & want23) == want23 && (c & want45) == want45 && (d & want67) == want67;
+__device__ __forceinline__ bool bloom_maybe(const BloomView& f, uint64_t key) {
+    const uint64_t h = fmix64(key);
+    const ulonglong2* p = reinterpret_cast<const ulonglong2*>(f.bits + bloom_block(f, h) * BLOOM_WORDS);
+    uint64_t v[4];
+    asm("ld.global.cg.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p));
+    const uint64_t g = bloom_bits(h);
+    uint32_t missing = 0;
+#pragma unroll
+    for (int w = 0; w < BLOOM_WORDS; ++w)
+        missing |= bloom_bit(g, w) & ~static_cast<uint32_t>(v[w / 2] >> (32 * (w & 1)));
+    return missing == 0;
 }
 
 // Device-side plan of one probe, written by its sampling stage: whether the
@@ -121,6 +138,7 @@ struct ProbeArgs {
     uint64_t n;
     const ulonglong2* slots;
     uint64_t mask;
+    uint64_t chain_mask;
     const uint32_t* side;
     uint64_t n_side;
     uint2* out;
@@ -209,7 +227,7 @@ __device__ __forceinline__ RowRange take_chunk(const RowQueue& q) {
 // bucket with a free slot.  An entry of `pend` holds the key, the row-id in
 // the low half of y and the bucket to read in the high half.
 __device__ __forceinline__ void probe_step(uint2* ws, unsigned& cnt, ulonglong2* pend, unsigned& np, bool real,
-                                           const Bucket& v, uint64_t key, uint32_t rid, uint32_t bk, uint32_t mask) {
+                                           const Bucket& v, uint64_t key, uint32_t rid, uint32_t bk, uint32_t cmask) {
     const bool m0 = real && v.k0 == key, m1 = real && v.k1 == key;
     const uint64_t w = m0 ? v.w0 : v.w1;
     warp_put(ws, cnt, m0 || m1, make_uint2(rid, static_cast<uint32_t>(w)));
@@ -222,7 +240,7 @@ __device__ __forceinline__ void probe_step(uint2* ws, unsigned& cnt, ulonglong2*
     const unsigned b = __ballot_sync(0xFFFFFFFFu, on);
     if (on)
         pend[np + __popc(b & ((1u << (threadIdx.x & 31u)) - 1u))] =
-            make_ulonglong2(key, rid | (static_cast<uint64_t>((bk + 1u) & mask) << 32));
+            make_ulonglong2(key, rid | (static_cast<uint64_t>((bk & ~cmask) | ((bk + 1u) & cmask)) << 32));
     np += __popc(b);
 }
 
@@ -241,7 +259,7 @@ __device__ __forceinline__ void probe_rows(const ProbeArgs& a, const RowQueue& q
     uint2* ws = reinterpret_cast<uint2*>(warp_smem + JP_PEND * 16);
     ulonglong2* pend = reinterpret_cast<ulonglong2*>(warp_smem);
     const unsigned lane = threadIdx.x & 31u;
-    const uint32_t mask = static_cast<uint32_t>(a.mask);
+    const uint32_t mask = static_cast<uint32_t>(a.mask), cmask = static_cast<uint32_t>(a.chain_mask);
     constexpr unsigned TILE = 32u * JP_U;
     unsigned cnt = 0, np = 0;
     uint64_t key[JP_U];
@@ -276,7 +294,7 @@ __device__ __forceinline__ void probe_rows(const ProbeArgs& a, const RowQueue& q
             __syncwarp();
             const uint32_t bk = static_cast<uint32_t>(p.y >> 32);
             const Bucket v = ld_bucket<L2_ONLY>(a.slots, bk);
-            probe_step(ws, cnt, pend, np, act, v, p.x, static_cast<uint32_t>(p.y), bk, mask);
+            probe_step(ws, cnt, pend, np, act, v, p.x, static_cast<uint32_t>(p.y), bk, cmask);
         }
     };
     RowRange r = take_chunk(q);
@@ -321,7 +339,7 @@ __device__ __forceinline__ void probe_rows(const ProbeArgs& a, const RowQueue& q
         if (cnt > JP_WCAP - 64 * JP_U) warp_flush(a, ws, cnt);
 #pragma unroll
         for (int j = 0; j < JP_U; ++j)
-            probe_step(ws, cnt, pend, np, ck[j] != JN_EMPTY, v[j], ck[j], cr[j], bk[j], mask);
+            probe_step(ws, cnt, pend, np, ck[j] != JN_EMPTY, v[j], ck[j], cr[j], bk[j], cmask);
         drain(31u);
     }
     drain(0u);
