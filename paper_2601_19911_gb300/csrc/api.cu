@@ -290,13 +290,14 @@ static olap_status topk_enqueue(olap_ctx* ctx, const void* d_keys, olap_key_type
     ctx->last_topk_ctl = a.ctl;
     ctx->last_rowids_in_place = false;      // olap_topk sets it after this when it applies
     ctx->topk_timed = ctx->time_kernels;
-    ctx->topk_filtered = plan.use_sample;
+    ctx->topk_filtered = plan.use_sample == TK_SAMPLE_FILTER;
     cudaError_t e = topk_launch(a, ctx->topk_geom, stream, ctx->time_kernels ? ctx->kev : nullptr);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return cuda_fail(ctx, e, "Top-K launch");
     }
-    ctx->launches += plan.use_sample ? 3 : 2;           // prepare, [filter,] select
+    // the local kernel, or prepare, [filter,] select
+    ctx->launches += plan.local ? 1 : plan.use_sample == TK_SAMPLE_FILTER ? 3 : 2;
     if (ctl_out) *ctl_out = a.ctl;
     return OLAP_OK;
 }
@@ -515,7 +516,8 @@ olap_status olap_topk_rows(olap_ctx* ctx, const void* rows, olap_mem in_where, u
 // the copy carries the keys alone.  True, with *dr set to the row-ids'
 // device-accessible address, when that applies.
 static bool rowids_in_host(const uint32_t* rowids, olap_mem where, uint64_t n, uint64_t kk, const uint32_t** dr) {
-    if (!rowids || where != OLAP_MEM_HOST_PINNED || !topk_plan(n, kk).use_sample) return false;
+    if (!rowids || where != OLAP_MEM_HOST_PINNED || topk_plan(n, kk).use_sample != TK_SAMPLE_FILTER)
+        return false;
     void* mapped = nullptr;
     if (cudaHostGetDevicePointer(&mapped, const_cast<uint32_t*>(rowids), 0) != cudaSuccess || !mapped) {
         cudaGetLastError();

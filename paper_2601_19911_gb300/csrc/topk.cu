@@ -2,7 +2,8 @@
 // (Sec. III-A, "partial selection (or radix-based selection)", returning the
 // row pointers of the Top-K rows in order).
 //
-// Three launches on one stream:
+// A few thousand keys take one launch (topk_local_kernel).  Otherwise three
+// launches on one stream, the second one up to 2^21 keys part of the third:
 //   0. topk_prepare_kernel zeroes the control block and, when N is large and
 //      K is small against N, reads a stratified sample of 8192 keys (16 CTAs,
 //      one key per thread) and finds the sample's r-th best entry by a radix
@@ -250,13 +251,15 @@ struct WarpStage {
     uint64_t* r;          // WS_CAP rank words (shared)
     uint32_t* idx;        // WS_CAP key indices (shared)
     unsigned count;       // entries held (the same in every lane)
+    unsigned* hist;       // the CTA's histogram of the fused first pass (shared; NULL without one)
 };
 constexpr int WS_BYTES = WS_CAP * 12;
+constexpr int FUSE_BYTES = (TK_BINS + 4) * 4;     // the histogram, its count of entries below, 16-byte units
 
-__device__ __forceinline__ WarpStage warp_stage(unsigned char* base) {
+__device__ __forceinline__ WarpStage warp_stage(unsigned char* base, unsigned* hist) {
     const unsigned w = threadIdx.x >> 5;
     unsigned char* p = base + static_cast<size_t>(w) * WS_BYTES;
-    return WarpStage{reinterpret_cast<uint64_t*>(p), reinterpret_cast<uint32_t*>(p + WS_CAP * 8), 0u};
+    return WarpStage{reinterpret_cast<uint64_t*>(p), reinterpret_cast<uint32_t*>(p + WS_CAP * 8), 0u, hist};
 }
 
 // The select's first refine pass, folded into the streaming filter (the
@@ -271,7 +274,6 @@ __device__ __forceinline__ WarpStage warp_stage(unsigned char* base) {
 // column and a second one: one pass instead of three over the candidates, the
 // select 29 -> 11.6 us.  Candidates below the interval are counted in one
 // more word.
-__shared__ unsigned g_fuse_hist[TK_BINS + 1];
 
 struct FuseRange {
     Range g;
@@ -285,24 +287,23 @@ __device__ __forceinline__ FuseRange fuse_range(const TopkArgs& a) {
 }
 
 template <int TPB>
-__device__ __forceinline__ void fuse_init() {
-    for (int b = threadIdx.x; b <= TK_BINS; b += TPB) g_fuse_hist[b] = 0;
+__device__ __forceinline__ void fuse_init(unsigned* hist) {
+    for (int b = threadIdx.x; b <= TK_BINS; b += TPB) hist[b] = 0;
     __syncthreads();
 }
 
-__device__ __forceinline__ void fuse_add(const FuseRange& f, uint64_t r, uint32_t rid) {
-    atomicAdd(&g_fuse_hist[r < f.g.rlo ? TK_BINS : range_bin(f.g, f.sh, r, rid)], 1u);
+__device__ __forceinline__ void fuse_add(unsigned* hist, const FuseRange& f, uint64_t r, uint32_t rid) {
+    atomicAdd(&hist[r < f.g.rlo ? TK_BINS : range_bin(f.g, f.sh, r, rid)], 1u);
 }
 
 // Whole CTA, after its last candidate: add the CTA's counts to the pass-0
 // histogram (non-zero bins only).
 template <int TPB>
-__device__ __forceinline__ void fuse_merge(const TopkArgs& a) {
+__device__ __forceinline__ void fuse_merge(const TopkArgs& a, const unsigned* hist) {
     __syncthreads();
     for (int b = threadIdx.x; b < TK_BINS; b += TPB)
-        if (g_fuse_hist[b]) atomicAdd(&a.ghist[b], g_fuse_hist[b]);
-    if (threadIdx.x == 0 && g_fuse_hist[TK_BINS])
-        atomicAdd(&a.ctl->flow, static_cast<unsigned long long>(g_fuse_hist[TK_BINS]));
+        if (hist[b]) atomicAdd(&a.ghist[b], hist[b]);
+    if (threadIdx.x == 0 && hist[TK_BINS]) atomicAdd(&a.ctl->flow, static_cast<unsigned long long>(hist[TK_BINS]));
 }
 
 // Move the warp's staged hits to the candidate buffer (all 32 lanes call).
@@ -326,27 +327,26 @@ __device__ __forceinline__ void stage_flush_plain(const TopkArgs& a, WarpStage& 
 }
 
 // The same, also counting the hits for the fused first pass.
-__device__ __forceinline__ void stage_write_fused(const TopkArgs& a, const FuseRange& f, const uint64_t* sr,
-                                                  const uint32_t* sidx, unsigned count, unsigned long long base) {
-    for (unsigned j = threadIdx.x & 31u; j < count; j += 32) {
+__device__ __forceinline__ void stage_write_fused(const TopkArgs& a, const FuseRange& f, const WarpStage& ws,
+                                                  unsigned long long base) {
+    for (unsigned j = threadIdx.x & 31u; j < ws.count; j += 32) {
         const unsigned long long pos = base + j;
-        const uint32_t idx = sidx[j];
-        const uint64_t r = sr[j];
+        const uint32_t idx = ws.idx[j];
+        const uint64_t r = ws.r[j];
         const uint32_t rid = a.rowids ? a.rowids[idx] : idx;
         if (pos < a.cand_cap) {
             a.cand_r[pos] = r;
             a.cand_rid[pos] = rid;
         }
-        fuse_add(f, r, rid);
+        fuse_add(ws.hist, f, r, rid);
     }
 }
-__device__ __forceinline__ void stage_flush_fused(const TopkArgs& a, const uint64_t* sr, const uint32_t* sidx,
-                                                  unsigned count) {
+__device__ __forceinline__ void stage_flush_fused(const TopkArgs& a, const WarpStage& ws) {
     __syncwarp();
     unsigned long long base = 0;
-    if ((threadIdx.x & 31u) == 0) base = atomicAdd(&a.ctl->cand_count, static_cast<unsigned long long>(count));
+    if ((threadIdx.x & 31u) == 0) base = atomicAdd(&a.ctl->cand_count, static_cast<unsigned long long>(ws.count));
     base = __shfl_sync(0xFFFFFFFFu, base, 0);
-    stage_write_fused(a, fuse_range(a), sr, sidx, count, base);
+    stage_write_fused(a, fuse_range(a), ws, base);
     __syncwarp();
 }
 
@@ -357,7 +357,7 @@ __device__ __forceinline__ void stage_flush(const TopkArgs& a, WarpStage& ws) {
         return;
     }
     if (ws.count == 0) return;
-    stage_flush_fused(a, ws.r, ws.idx, ws.count);
+    stage_flush_fused(a, ws);
     ws.count = 0;
 }
 
@@ -442,7 +442,7 @@ __device__ __forceinline__ void cta_flush_fused(const TopkArgs& a, const WarpSta
     }
     if (threadIdx.x == 0 && all) s_base = atomicAdd(&a.ctl->cand_count, static_cast<unsigned long long>(all));
     __syncthreads();
-    if (all) stage_write_fused(a, f, ws.r, ws.idx, ws.count, s_base + before);
+    if (all) stage_write_fused(a, f, ws, s_base + before);
 }
 
 // Phase 1: the single streaming pass.  Appends (rank word, row-id) of every
@@ -543,7 +543,9 @@ __device__ __forceinline__ void filter_loop(const TopkArgs& a, const FilterSpan<
 }
 
 template <bool W4, int TPB>
-__device__ void filter_pass(const TopkArgs& a, unsigned char* stage_smem) {
+__device__ __forceinline__ void filter_pass(const TopkArgs& a, unsigned char* fsm) {
+    unsigned* hist = reinterpret_cast<unsigned*>(fsm);
+    fuse_init<TPB>(hist);
     const FilterSpan<W4> sp(a);
     FilterStep st;
     st.first(sp.nvec, static_cast<uint64_t>(TPB) * TK_UNROLL);
@@ -562,13 +564,14 @@ __device__ void filter_pass(const TopkArgs& a, unsigned char* stage_smem) {
     } else {
         mode = key_cmp<uint64_t>(kl.m64, kl.c64, &lim);
     }
-    WarpStage ws = warp_stage(stage_smem);
+    WarpStage ws = warp_stage(fsm + FUSE_BYTES, hist);
     if (mode == CMP_GE_U) filter_loop<W4, TPB, CMP_GE_U>(a, sp, lim, st, v, ws);
     else if (mode == CMP_LE_U) filter_loop<W4, TPB, CMP_LE_U>(a, sp, lim, st, v, ws);
     else if (mode == CMP_GE_S) filter_loop<W4, TPB, CMP_GE_S>(a, sp, lim, st, v, ws);
     else filter_loop<W4, TPB, CMP_LE_S>(a, sp, lim, st, v, ws);
     filter_ends<true>(a, t, sp.head, sp.tail0, ws);
     cta_flush_fused<TPB>(a, ws);
+    fuse_merge<TPB>(a, hist);
 }
 
 // The 32-bit order-preserving transform of one 4-byte key kind as two masks:
@@ -638,10 +641,15 @@ __device__ void filter_pass_pair_vec(const TopkArgs& a, uint64_t t, WarpStage& w
 }
 
 template <int TPB>
-__device__ void filter_pass_pair(const TopkArgs& a, uint64_t t, unsigned char* stage_smem) {
+__device__ __forceinline__ void filter_pass_pair(const TopkArgs& a, unsigned char* fsm) {
+    unsigned* hist = reinterpret_cast<unsigned*>(fsm);
+    fuse_init<TPB>(hist);
+    wait_prior_grid();
+    allow_next_grid();
+    const uint64_t t = __ldcg(&a.ctl->thresh);
     const uint64_t n = a.n;
     const uintptr_t off = reinterpret_cast<uintptr_t>(a.keys) ^ reinterpret_cast<uintptr_t>(a.keys2);
-    WarpStage ws = warp_stage(stage_smem);
+    WarpStage ws = warp_stage(fsm + FUSE_BYTES, hist);
     if ((off & 31) == 0) {
         filter_pass_pair_vec<TPB, 8>(a, t, ws);
     } else if ((off & 15) == 0) {
@@ -659,6 +667,7 @@ __device__ void filter_pass_pair(const TopkArgs& a, uint64_t t, unsigned char* s
     }
     }
     cta_flush_fused<TPB>(a, ws);
+    fuse_merge<TPB>(a, hist);
 }
 
 // Issue the bulk copy of the tile at byte offset `off` of the key body into
@@ -698,7 +707,7 @@ __device__ bool filter_pass_bulk(const TopkArgs& a, uint64_t t, unsigned char* s
     const KeyLimit lim = key_limit(t, a.kind, a.desc);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(tile) * stages);
     uint64_t* empty = full + TK_MAX_STAGES;
-    WarpStage ws = warp_stage(reinterpret_cast<unsigned char*>(empty + TK_MAX_STAGES));
+    WarpStage ws = warp_stage(reinterpret_cast<unsigned char*>(empty + TK_MAX_STAGES), nullptr);
     const uint64_t step = static_cast<uint64_t>(gridDim.x) * tile;       // bytes between my tiles
 
     if (threadIdx.x == 0) {
@@ -1012,29 +1021,29 @@ __global__ void __launch_bounds__(TKF_TPB, 4) topk_filter_bulk_kernel(TopkArgs a
     filter_pass_bulk<W4, TKF_TPB>(a, t, fsmem);
 }
 
-// Kernel 2 of 3, register-load flavour (TPB threads; the per-warp stages are
-// dynamic shared memory, (TPB / 32) * WS_BYTES).
+// Kernel 2 of 3, register-load flavour (TPB threads; dynamic shared memory:
+// the fused pass's histogram and the per-warp stages).
 template <bool W4, int TPB>
 __global__ void __launch_bounds__(TPB, 1024 / TPB) topk_filter_regs_kernel(TopkArgs a) {
-    extern __shared__ __align__(16) unsigned char stage[];
-    fuse_init<TPB>();
-    filter_pass<W4, TPB>(a, stage);
-    fuse_merge<TPB>(a);
+    extern __shared__ __align__(16) unsigned char fsm[];
+    filter_pass<W4, TPB>(a, fsm);
 }
 
 // Kernel 2 of 3 for a two-column key (register loads of both columns).
 template <int TPB>
 __global__ void __launch_bounds__(TPB, 1024 / TPB) topk_filter_pair_kernel(TopkArgs a) {
-    extern __shared__ __align__(16) unsigned char stage[];
-    fuse_init<TPB>();
-    wait_prior_grid();
-    allow_next_grid();
-    const uint64_t t = __ldcg(&a.ctl->thresh);
-    filter_pass_pair<TPB>(a, t, stage);
-    fuse_merge<TPB>(a);
+    extern __shared__ __align__(16) unsigned char fsm[];
+    filter_pass_pair<TPB>(a, fsm);
 }
 
-// Kernel 3 of 3 (cooperative): refine, split, finish and sort.
+// Kernel 3 of 3 (cooperative): refine, split, finish and sort.  For inputs of
+// at most TK_DIRECT_N keys with a sample it also makes the streaming pass (a
+// filter kernel of its own costs a launch and its end more than a few
+// megabytes take to read), and a grid barrier stands where the filter kernel
+// ended: 2^20 float64 keys, K = 100, 29 us with refine passes over the input,
+// 23 us so.
+enum SelectFilter { SEL_NONE = 0, SEL_W8 = 1, SEL_W4 = 2, SEL_PAIR = 3 };
+template <int FILTER>
 __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long sc[24];
@@ -1043,11 +1052,18 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
     uint64_t* sr = reinterpret_cast<uint64_t*>(smem);
     uint32_t* srid = reinterpret_cast<uint32_t*>(smem + TK_RANK_MAX * 8);
 
-    wait_prior_grid();
-    allow_next_grid();
+    unsigned bar_target = 0;                                 // of the grid barriers
+    if (FILTER == SEL_NONE) {
+        wait_prior_grid();
+        allow_next_grid();
+    } else {
+        if (FILTER == SEL_W8) filter_pass<false, TK_TPB>(a, smem);
+        if (FILTER == SEL_W4) filter_pass<true, TK_TPB>(a, smem);
+        if (FILTER == SEL_PAIR) filter_pass_pair<TK_TPB>(a, smem);
+        if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
+    }
     const bool stamp = blockIdx.x == 0 && threadIdx.x == 0;
     if (stamp) ctl->ts[2] = gtimer();
-    unsigned bar_target = 0;                                 // of the grid barriers
     // Source of the selection: the candidates of the streaming pass when the
     // sample judged well (at least k of them, all stored), else the input.
     bool cand = false;
@@ -1449,16 +1465,162 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
     if (gtid == 0) ctl->ts[6] = gtimer();
 }
 
+// The whole Top-K of a small input, in one launch without a control block or
+// a grid barrier: every CTA loads all n keys into shared memory, finds the
+// interval of the K-th entry by refine passes of its own over them (the same
+// in every CTA), lists the entries below it and in it, and ranks the entries
+// whose index falls to it among those.  Bound by latency: the loads, three
+// barriers a pass, and a launch less than the general path's two (TK_LOCAL_N
+// has both sides).
+__global__ void __launch_bounds__(TKL_TPB, 1) topk_local_kernel(TopkArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned* hist = reinterpret_cast<unsigned*>(smem);                      // then the two lists
+    uint16_t* list = reinterpret_cast<uint16_t*>(smem);                      // below from the front, the rest after
+    uint64_t* sr = reinterpret_cast<uint64_t*>(smem + TK_BINS * 4);
+    uint32_t* srid = reinterpret_cast<uint32_t*>(smem + TK_BINS * 4 + a.n * 8);
+    __shared__ unsigned long long sc[24];
+    __shared__ unsigned long long mm[4];
+    __shared__ unsigned n_below, n_eq;
+    const int n = static_cast<int>(a.n);
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    wait_prior_grid();
+    allow_next_grid();
+    unsigned long long t0 = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) t0 = gtimer();
+    auto span = [&](const Fold& mine) {                      // minima and maxima over the CTA, in mm
+        if (threadIdx.x == 0) fold_reset(mm);
+        __syncthreads();
+        Fold f = mine;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            f.rmin = min(f.rmin, __shfl_xor_sync(0xFFFFFFFFu, f.rmin, o));
+            f.rmax = max(f.rmax, __shfl_xor_sync(0xFFFFFFFFu, f.rmax, o));
+        }
+        f.imin = __reduce_min_sync(0xFFFFFFFFu, f.imin);
+        f.imax = __reduce_max_sync(0xFFFFFFFFu, f.imax);
+        if (lane == 0 && f.rmin <= f.rmax) {
+            atomicMin(&mm[0], static_cast<unsigned long long>(f.rmin));
+            atomicMax(&mm[1], static_cast<unsigned long long>(f.rmax));
+            atomicMin(&mm[2], static_cast<unsigned long long>(f.imin));
+            atomicMax(&mm[3], static_cast<unsigned long long>(f.imax));
+        }
+        __syncthreads();
+        Range g{mm[0], mm[1], 0u, max_rowid(a)};
+        if (g.rlo == g.rhi) {
+            g.ilo = static_cast<uint32_t>(mm[2]);
+            g.ihi = static_cast<uint32_t>(mm[3]);
+        }
+        __syncthreads();
+        return g;
+    };
+    Fold all = fold_none();
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += TKL_TPB) {
+        const Elem e = load_input(a, i);
+        sr[i] = e.r;
+        srid[i] = e.rid;
+        fold_add(all, e.r, e.rid);
+    }
+    Range g = span(all);
+    uint64_t krem = a.k, bcnt = a.n;
+    // Down to a bin that costs less to rank than another pass.
+    while (bcnt > 64 && !range_point(g) && krem < bcnt) {
+        const int shift = range_shift(g, TK_DIG);
+        for (int b = threadIdx.x; b < TK_BINS; b += TKL_TPB) hist[b] = 0;
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += TKL_TPB) {
+            const uint64_t r = sr[i];
+            const uint32_t rid = srid[i];
+            if (range_cmp(g, r, rid) == 0) atomicAdd(&hist[range_bin(g, shift, r, rid)], 1u);
+        }
+        __syncthreads();
+        const Pick pk = pick_bucket<TKL_TPB>(hist, krem, sc);
+        const bool whole = pk.below == 0 && pk.in_b == bcnt;
+        krem -= pk.below;
+        bcnt = pk.in_b;
+        if (whole) {
+            Fold f = fold_none();
+            for (int i = threadIdx.x; i < n; i += TKL_TPB)
+                if (range_cmp(g, sr[i], srid[i]) == 0) fold_add(f, sr[i], srid[i]);
+            const Range narrow = span(f);
+            // (an interval that does not shrink is cut like any other)
+            const bool same = narrow.rlo == g.rlo && narrow.rhi == g.rhi && narrow.ilo == g.ilo && narrow.ihi == g.ihi;
+            g = same ? range_narrow(a, g, shift, pk.b) : narrow;
+        } else {
+            g = range_narrow(a, g, shift, pk.b);
+        }
+    }
+    // The lists: fewer than K entries below the interval, and in it at most 64
+    // or, when all of it is taken, the rest of the K.  Identical entries (one
+    // key and row-id) are not ranked: krem copies are written.
+    const bool point = range_point(g);
+    const unsigned nb = static_cast<unsigned>(a.k - krem);
+    if (threadIdx.x == 0) n_below = n_eq = 0;
+    __syncthreads();                                         // (the histogram has been read)
+    for (int i = threadIdx.x; i < n; i += TKL_TPB) {
+        const int c = range_cmp(g, sr[i], srid[i]);
+        if (c < 0) list[atomicAdd(&n_below, 1u)] = static_cast<uint16_t>(i);
+        else if (c == 0 && !point) list[nb + atomicAdd(&n_eq, 1u)] = static_cast<uint16_t>(i);
+    }
+    if (point && blockIdx.x == 0)
+        for (unsigned t = threadIdx.x; t < krem; t += TKL_TPB) write_result(a, nb + t, g.rlo, g.ilo);
+    __syncthreads();
+    const unsigned total = static_cast<unsigned>(bcnt);
+    const int last = point ? -1 : 0;                         // range_cmp of the entries to rank
+    // entry i falls to warp i mod (warps of the grid)
+    const int nw = static_cast<int>(gridDim.x) * (TKL_TPB / 32);
+    const int gw = static_cast<int>(warp * gridDim.x + blockIdx.x);
+    for (int base = gw; base < n; base += 32 * nw) {
+        const int i = base + nw * static_cast<int>(lane);
+        const int c = i < n ? range_cmp(g, sr[i], srid[i]) : 1;
+        unsigned todo = __ballot_sync(0xFFFFFFFFu, c <= last);
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const int e = base + nw * src;
+            const bool below = __shfl_sync(0xFFFFFFFFu, c, src) < 0;
+            const uint64_t er = sr[e];
+            const uint32_t erid = srid[e];
+            unsigned cnt = 0;
+            const uint16_t* l = below ? list : list + nb;
+            const unsigned len = below ? nb : total;
+            for (unsigned j = lane; j < len; j += 32) {
+                const int x = l[j];
+                rank_count(cnt, sr[x], srid[x], er, erid, x < e);
+            }
+            const unsigned rank = __reduce_add_sync(0xFFFFFFFFu, 0u - cnt);
+            if (lane == 0) {
+                if (below) write_result(a, rank, er, erid);
+                else if (rank < krem) write_result(a, nb + rank, er, erid);
+            }
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const unsigned long long t1 = gtimer();
+        a.ctl->err = 0;
+        a.ctl->path = 0;
+        a.ctl->passes = 0;
+        a.ctl->cand_count = 0;
+        for (int j = 0; j < 6; ++j) a.ctl->ts[j] = t0;
+        for (int j = 6; j < 9; ++j) a.ctl->ts[j] = t1;
+        if (a.dev_status) *a.dev_status = OLAP_OK;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Host side.
 // ---------------------------------------------------------------------------
 TopkPlan topk_plan(uint64_t n, uint64_t k) {
-    TopkPlan p{0, 0, 0};
-    if (n > TK_DIRECT_N && k <= n / 256) {
+    TopkPlan p{0, 0, 0, 0};
+    if (n <= TK_LOCAL_N && k <= TK_LOCAL_K && n * k <= TK_LOCAL_NK) {
+        p.local = 1;
+        return p;
+    }
+    if (n > TK_SAMPLE_N && k <= n / 256) {
         const double lam = static_cast<double>(k) * TK_SAMPLE / static_cast<double>(n);
         double r = std::ceil(lam + 4.0 * std::sqrt(lam)) + 3.0;
         if (r > TK_SAMPLE) r = TK_SAMPLE;
-        p.use_sample = 1;
+        p.use_sample = n > TK_DIRECT_N ? TK_SAMPLE_FILTER : TK_SAMPLE_INLINE;
         p.sample_rank = static_cast<unsigned>(r);
         const uint64_t stratum = (n + TK_SAMPLE - 1) / TK_SAMPLE;
         uint64_t cap = 2 * (static_cast<uint64_t>(r) + 8) * stratum;
@@ -1512,6 +1674,7 @@ void topk_carve(TopkArgs& a, const TopkPlan& p, void* base) {
         a.out_rid1 = a.split_rid = nullptr;
     }
     a.samples = p.use_sample ? static_cast<uint64_t*>(take(TK_SAMPLE * 8)) : nullptr;
+    a.local = p.local;
     a.use_sample = p.use_sample;
     a.sample_rank = p.sample_rank;
     a.filter = TK_FILTER_BULK;
@@ -1521,6 +1684,10 @@ void topk_carve(TopkArgs& a, const TopkPlan& p, void* base) {
 // g_attr_lock, by the first thread that needs the kernels' attributes there.
 static std::atomic<int> g_smem_limit[64] = {};
 static std::mutex g_attr_lock;
+
+// Dynamic shared memory of a register filter with tpb threads.
+static int regs_smem(int tpb) { return FUSE_BYTES + tpb / 32 * WS_BYTES; }
+static_assert(FUSE_BYTES + TK_TPB / 32 * WS_BYTES <= TK_SORT_SMEM, "the select's own streaming pass");
 
 static bool set_kernel_attrs(int device) {
     if (g_smem_limit[device].load()) return true;
@@ -1533,33 +1700,27 @@ static bool set_kernel_attrs(int device) {
         cudaFuncGetAttributes(&fa, topk_filter_bulk_kernel<false>) != cudaSuccess)
         return false;
     const int lim = std::min<int>(optin - static_cast<int>(fa.sharedSizeBytes) - 256, TK_SMEM_MAX);
-    if (cudaFuncSetAttribute(topk_filter_bulk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             lim) != cudaSuccess ||
-        cudaFuncSetAttribute(topk_filter_bulk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             lim) != cudaSuccess ||
-        // the register filters' stages are dynamic, next to the fused pass's
-        // static histogram: above 48 KB together, so every variant opts in
-        cudaFuncSetAttribute(topk_filter_regs_kernel<false, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             8 * WS_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(topk_filter_regs_kernel<true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             8 * WS_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(topk_filter_pair_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             8 * WS_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(topk_filter_regs_kernel<false, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             16 * WS_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(topk_filter_regs_kernel<true, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             16 * WS_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(topk_filter_pair_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             16 * WS_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(topk_filter_regs_kernel<false, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             32 * WS_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(topk_filter_regs_kernel<true, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             32 * WS_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(topk_filter_pair_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             32 * WS_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(topk_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             TK_SORT_SMEM) != cudaSuccess)
-        return false;
+    bool ok = true;
+    auto opt_in = [&](auto fn, int bytes) {
+        ok = ok && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+    };
+    opt_in(topk_filter_bulk_kernel<false>, lim);
+    opt_in(topk_filter_bulk_kernel<true>, lim);
+    opt_in(topk_filter_regs_kernel<false, 256>, regs_smem(256));
+    opt_in(topk_filter_regs_kernel<true, 256>, regs_smem(256));
+    opt_in(topk_filter_pair_kernel<256>, regs_smem(256));
+    opt_in(topk_filter_regs_kernel<false, 512>, regs_smem(512));
+    opt_in(topk_filter_regs_kernel<true, 512>, regs_smem(512));
+    opt_in(topk_filter_pair_kernel<512>, regs_smem(512));
+    opt_in(topk_filter_regs_kernel<false, 1024>, regs_smem(1024));
+    opt_in(topk_filter_regs_kernel<true, 1024>, regs_smem(1024));
+    opt_in(topk_filter_pair_kernel<1024>, regs_smem(1024));
+    opt_in(topk_local_kernel, TKL_SMEM_MAX);
+    opt_in(topk_select_kernel<SEL_NONE>, TK_SORT_SMEM);
+    opt_in(topk_select_kernel<SEL_W8>, TK_SORT_SMEM);
+    opt_in(topk_select_kernel<SEL_W4>, TK_SORT_SMEM);
+    opt_in(topk_select_kernel<SEL_PAIR>, TK_SORT_SMEM);
+    if (!ok) return false;
     g_smem_limit[device].store(lim);
     return true;
 }
@@ -1588,7 +1749,7 @@ bool topk_geometry(int device, int tile_bytes, int stages, int ctas_per_sm, int 
     if (per_sm < 1) return false;
     g.filter_grid = sms * per_sm;
     cudaError_t oe;
-    const size_t rs = static_cast<size_t>(g.regs_tpb / 32) * WS_BYTES;
+    const size_t rs = static_cast<size_t>(regs_smem(g.regs_tpb));
     if (g.regs_tpb == 256)
         oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, topk_filter_regs_kernel<false, 256>, 256, rs);
     else if (g.regs_tpb == 512)
@@ -1598,14 +1759,20 @@ bool topk_geometry(int device, int tile_bytes, int stages, int ctas_per_sm, int 
     if (oe != cudaSuccess) return false;
     g.regs_grid = sms * std::max(1, std::min(per_sm, 2048 / g.regs_tpb));
     // Cooperative select kernel: every CTA resident, two per SM at most.
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, topk_select_kernel, TK_TPB, TK_SORT_SMEM) !=
-        cudaSuccess)
-        return false;
+    per_sm = 2;
+    auto fits = [&](auto fn) {
+        int per = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, TK_TPB, TK_SORT_SMEM) != cudaSuccess) per = 0;
+        per_sm = std::min(per_sm, per);
+    };
+    fits(topk_select_kernel<SEL_NONE>);
+    fits(topk_select_kernel<SEL_W8>);
+    fits(topk_select_kernel<SEL_W4>);
+    fits(topk_select_kernel<SEL_PAIR>);
     // Two CTAs per SM for the select in general; one per SM when it reads a
     // candidate list and finishes a small K: its grid barriers then dominate,
     // and half the arrivals take less time (measured, 2^28 keys, K = 1000:
     // select 22.6 -> 19.9 us; at K = 10^5 the merge-path finish wants both).
-    per_sm = std::min(per_sm, 2);
     if (per_sm < 1) return false;
     g.grid = sms * per_sm;
     g.grid_small = sms;
@@ -1645,16 +1812,30 @@ cudaError_t topk_launch(const TopkArgs& args, const TopkGeom& geom, cudaStream_t
     if (a.digit == 0) a.digit = TK_DIG;
     if (a.digit < TK_DIG_MIN || a.digit > TK_DIG) return cudaErrorInvalidValue;
     // the register and two-column filters fold the select's first pass
-    a.fuse = a.use_sample && (a.pair || a.filter == TK_FILTER_REGS) ? 1 : 0;
+    a.fuse = a.use_sample == TK_SAMPLE_INLINE ||
+                     (a.use_sample == TK_SAMPLE_FILTER && (a.pair || a.filter == TK_FILTER_REGS))
+                 ? 1
+                 : 0;
     cudaError_t e;
     if (ev && (e = cudaEventRecord(ev[0], stream)) != cudaSuccess) return e;
+    if (a.local) {
+        if (ev && ((e = cudaEventRecord(ev[1], stream)) != cudaSuccess ||
+                   (e = cudaEventRecord(ev[2], stream)) != cudaSuccess))
+            return e;
+        // a CTA for every 8 results: each reads the whole input, and ranking
+        // is what they share
+        const unsigned g = static_cast<unsigned>(std::min<uint64_t>(geom.grid_small, (a.k + 7) / 8));
+        e = launch_kernel(topk_local_kernel, g, TKL_TPB, TK_BINS * 4 + a.n * 12, stream, a, false);
+        if (e != cudaSuccess || !ev) return e;
+        return cudaEventRecord(ev[3], stream);
+    }
     e = launch_kernel(topk_prepare_kernel, a.use_sample ? TK_PREP_CTAS : 1, TK_TPB, 0, stream, a, false);
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[1], stream)) != cudaSuccess) return e;
-    if (a.use_sample) {
+    if (a.use_sample == TK_SAMPLE_FILTER) {
         void (*fn)(TopkArgs) = nullptr;
         unsigned grid = static_cast<unsigned>(geom.regs_grid), block = static_cast<unsigned>(geom.regs_tpb);
-        size_t smem = static_cast<size_t>(geom.regs_tpb / 32) * WS_BYTES;
+        size_t smem = static_cast<size_t>(regs_smem(geom.regs_tpb));
         if (a.pair) {
             fn = geom.regs_tpb == 256    ? topk_filter_pair_kernel<256>
                  : geom.regs_tpb == 1024 ? topk_filter_pair_kernel<1024>
@@ -1675,10 +1856,12 @@ cudaError_t topk_launch(const TopkArgs& args, const TopkGeom& geom, cudaStream_t
         if ((e = launch_kernel(fn, grid, block, smem, stream, a, false)) != cudaSuccess) return e;
     }
     if (ev && (e = cudaEventRecord(ev[2], stream)) != cudaSuccess) return e;
-    // (the direct path keeps both CTAs per SM: at 2^20 keys one per SM was
-    // measured slower, 0.051 against 0.049 ms)
+    // (the direct path keeps both CTAs per SM: its passes read the input)
     const int sgrid = (a.use_sample && a.k <= static_cast<uint64_t>(TK_SMALL)) ? geom.grid_small : geom.grid;
-    e = launch_kernel(topk_select_kernel, static_cast<unsigned>(sgrid), TK_TPB, TK_SORT_SMEM, stream, a, true);
+    void (*sel)(TopkArgs) = topk_select_kernel<SEL_NONE>;
+    if (a.use_sample == TK_SAMPLE_INLINE)
+        sel = a.pair ? topk_select_kernel<SEL_PAIR> : a.w4 ? topk_select_kernel<SEL_W4> : topk_select_kernel<SEL_W8>;
+    e = launch_kernel(sel, static_cast<unsigned>(sgrid), TK_TPB, TK_SORT_SMEM, stream, a, true);
     if (e != cudaSuccess || !ev) return e;
     return cudaEventRecord(ev[3], stream);
 }

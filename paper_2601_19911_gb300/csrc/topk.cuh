@@ -17,7 +17,25 @@ constexpr int TK_SAMPLE = 8192;           // sample size of the threshold estima
 constexpr int TK_SPT = TK_SAMPLE / TK_TPB;
 constexpr int TK_PREP_CTAS = TK_SAMPLE / TK_TPB;   // prepare CTAs on the sampled path: one key per thread
 constexpr int TK_UNROLL = 2;              // 32-byte loads in flight per thread (register filter)
-constexpr uint64_t TK_DIRECT_N = 1ull << 21;   // at or below: no sample, refine the input
+constexpr uint64_t TK_DIRECT_N = 1ull << 21;   // at or below: no filter kernel of its own
+// At or below: no sample, refine the input (float64 keys, K = 100, general path:
+// 2^18 keys 21 against 22.5 us, 400,000 both 22.6, 2^19 24.6 against 22.5, 2^20
+// 29 against 23-25).
+constexpr uint64_t TK_SAMPLE_N = 3ull << 17;
+// Few keys: every CTA holds the whole input in shared memory and works without
+// the others (topk_local_kernel), up to TK_LOCAL_N keys, K = TK_LOCAL_K and
+// n * K = TK_LOCAL_NK.  Device time against the general path, float64 keys:
+// 1000 keys 4.5 against 7-9 us, 5000 keys 7.6 against 11.6, 10,007 keys 11 (K
+// = 10) and 15 (K = 1000) against 12 and 16; past the line it loses: 16,000
+// keys with K = 4000 37 against 25 us, 16,384 with K = 100 15 against 14.
+constexpr uint64_t TK_LOCAL_N = 3ull << 12;
+constexpr uint64_t TK_LOCAL_K = 4096;
+constexpr uint64_t TK_LOCAL_NK = 1ull << 24;
+constexpr int TKL_TPB = 1024;
+constexpr int TKL_SMEM_MAX = TK_BINS * 4 + static_cast<int>(TK_LOCAL_N) * 12;
+// Whether and where the sampled streaming pass runs: in a kernel of its own, or
+// at the start of the select kernel.
+enum { TK_SAMPLE_NONE = 0, TK_SAMPLE_FILTER = 1, TK_SAMPLE_INLINE = 2 };
 constexpr int TK_RANK_MAX = 8192;         // survivors ranked in shared memory by the whole grid
 constexpr int TK_SPLITTERS = 2047;        // splitters of the larger-K finish on tied keys (2^k - 1)
 constexpr uint64_t TK_SPLIT_MAX = 2048ull * 512;   // entries they may split (about 512 per gap)
@@ -69,7 +87,8 @@ struct TopkArgs {
     int kind;                        // olap_key_type
     int w4;                          // 4-byte keys (float32, int32, uint32)
     int desc;
-    int use_sample;
+    int local;                       // topk_local_kernel
+    int use_sample;                  // TK_SAMPLE_NONE, _FILTER or _INLINE
     unsigned sample_rank;            // 1-based rank of the threshold in the sample
     int filter;                      // TopkFilter
     int fuse;                        // the filter folds the select's first radix pass (set at launch)
@@ -106,6 +125,7 @@ struct TopkArgs {
 
 // Plan of one Top-K call: which path and how much scratch it needs.
 struct TopkPlan {
+    int local;                       // topk_local_kernel
     int use_sample;
     unsigned sample_rank;
     uint64_t cand_cap;
