@@ -365,15 +365,23 @@ __global__ void __launch_bounds__(JB_TPB) join_side_kernel(const int64_t* keys, 
 // by partition (pass 3 of the partitioned probe): there the chunks come out in
 // partition order, so the warps of the whole grid work on one partition's
 // table slice at a time and that slice stays in L2.
+// The last CTA to finish returns the row counter and its ticket to zero for the
+// next probe of the context, and for a blocking call writes the pair count to
+// the host and clears it as well, so that such a call is its kernels and one
+// wait (three small memsets and a copy before).
 // `args` holds the rows as launched (the probe's input, or its partitioned
 // rows).  The device-side plan (ctl, when non-NULL) may change that: with the
 // Bloom pre-probe active the row count is the number of rows it kept, and
 // with `redirect` the rows are read from where the plan says (the kept rows,
 // or the input when the partition passes were skipped), through L1 when the
 // plan says so.
+struct ProbeDone {
+    unsigned* ticket;                          // CTAs done; zero between probes
+    unsigned long long* host_count;            // page-locked host word of a blocking call, else NULL
+};
 template <bool L2_ONLY>
 __global__ void __launch_bounds__(JP_TPB, JP_CTAS) join_probe_kernel(ProbeArgs args, unsigned long long* next_row,
-                                                               const ProbeCtl* ctl) {
+                                                                     const ProbeCtl* ctl, ProbeDone done) {
     extern __shared__ __align__(16) unsigned char psmem[];
     unsigned char* mine = psmem + (threadIdx.x >> 5) * JP_WARP_SMEM;
     ProbeArgs a = args;
@@ -394,6 +402,19 @@ __global__ void __launch_bounds__(JP_TPB, JP_CTAS) join_probe_kernel(ProbeArgs a
         probe_rows<false>(a, q, mine);
     else
         probe_rows<true>(a, q, mine);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(done.ticket, 1u) == gridDim.x - 1) {
+            __threadfence();
+            *done.ticket = 0;
+            *next_row = 0;
+            if (done.host_count) {
+                *done.host_count = __ldcg(a.count);
+                *a.count = 0;
+            }
+        }
+    }
 }
 
 // ---- Bloom pre-probe ------------------------------------------------------
@@ -934,10 +955,18 @@ using namespace olap;
 
 namespace {
 
+// With host_count the count word is the context's own (zero between probes),
+// and the probe leaves the count in *host_count; else the count goes to d_count.
 olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t* d_keys, const uint32_t* d_rowids,
-                          uint64_t n, olap_pair* d_out, uint64_t capacity, uint64_t* d_count, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(d_count, 0, sizeof(uint64_t), s);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "probe count reset");
+                          uint64_t n, olap_pair* d_out, uint64_t capacity, uint64_t* d_count, uint64_t* host_count,
+                          cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (host_count) {
+        *host_count = 0;
+        d_count = static_cast<uint64_t*>(ctx->aux);
+    } else if ((e = cudaMemsetAsync(d_count, 0, sizeof(uint64_t), s)) != cudaSuccess) {
+        return cuda_fail(ctx, e, "probe count reset");
+    }
     if (n == 0) {
         ctx->last_probe_parts = 1;
         ctx->last_probe_n = 0;
@@ -997,8 +1026,7 @@ olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t
         return cuda_fail(ctx, e, "timing event");
     // the row queue's counter, in the context's small device area
     unsigned long long* next_row = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(ctx->aux) + 256);
-    if ((e = cudaMemsetAsync(next_row, 0, sizeof(unsigned long long), s)) != cudaSuccess)
-        return cuda_fail(ctx, e, "probe queue reset");
+    const ProbeDone done{reinterpret_cast<unsigned*>(next_row + 1), reinterpret_cast<unsigned long long*>(host_count)};
     ProbeArgs pa = a;
     const BloomView bloom = pre ? bloom_view(t) : BloomView{nullptr, 0, 0, 0};
     if (pf) {
@@ -1030,9 +1058,9 @@ olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t
         pa.rowids = q.out_rowids;
     }
     if (ctx->opts.join_bucket_loads == OLAP_LOADS_L1)
-        join_probe_kernel<false><<<grid, JP_TPB, JP_SMEM, s>>>(pa, next_row, pf);
+        join_probe_kernel<false><<<grid, JP_TPB, JP_SMEM, s>>>(pa, next_row, pf, done);
     else
-        join_probe_kernel<true><<<grid, JP_TPB, JP_SMEM, s>>>(pa, next_row, pf);
+        join_probe_kernel<true><<<grid, JP_TPB, JP_SMEM, s>>>(pa, next_row, pf, done);
     e = cudaGetLastError();
     // [plan,] [filter,] [count, scatter,] probe
     if (e == cudaSuccess) ctx->launches += (pf ? 1 : 0) + (pre ? 1 : 0) + (parts > 1 ? 2 : 0) + 1;
@@ -1231,7 +1259,7 @@ olap_status olap_join_probe_async(olap_ctx* ctx, const olap_join_table* table, c
     if (capacity && !d_out) return fail(ctx, OLAP_E_INVALID, "out is NULL");
     if (!d_rowids && n > (1ull << 32)) return fail(ctx, OLAP_E_INVALID, "implicit row-ids need n <= 2^32");
     cudaStream_t s = stream ? static_cast<cudaStream_t>(stream) : ctx->stream;
-    return probe_enqueue(ctx, table, d_keys, d_rowids, n, d_out, capacity, d_count, s);
+    return probe_enqueue(ctx, table, d_keys, d_rowids, n, d_out, capacity, d_count, nullptr, s);
 }
 
 olap_status olap_join_probe(olap_ctx* ctx, const olap_join_table* table, const int64_t* keys,
@@ -1269,25 +1297,17 @@ olap_status olap_join_probe(olap_ctx* ctx, const olap_join_table* table, const i
         }
     }
     olap_pair* dout = out;
-    // Device count word: a small slot at the end of the output staging area
-    // (host outputs) or of the context scratch (device outputs).
-    uint64_t* dcount = nullptr;
     if (out_where != OLAP_MEM_DEVICE) {
-        const size_t ob = (capacity * 8 + 255) & ~static_cast<size_t>(255);
-        st = ensure_dev_out(ctx, ob + 256);
+        st = ensure_dev_out(ctx, capacity * 8);
         if (st != OLAP_OK) return st;
         dout = static_cast<olap_pair*>(ctx->dev_out);
-        dcount = reinterpret_cast<uint64_t*>(static_cast<unsigned char*>(ctx->dev_out) + ob);
-    } else {
-        dcount = static_cast<uint64_t*>(ctx->aux);
     }
-    st = probe_enqueue(ctx, table, dk, dr, n, dout, capacity, dcount, ctx->stream);
+    uint64_t* hcount = reinterpret_cast<uint64_t*>(ctx->host_status + 8);
+    st = probe_enqueue(ctx, table, dk, dr, n, dout, capacity, nullptr, hcount, ctx->stream);
     if (st != OLAP_OK) return st;
-    uint64_t cnt = 0;
-    e = cudaMemcpyAsync(ctx->host_status + 8, dcount, sizeof(uint64_t), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "join probe");
-    std::memcpy(&cnt, ctx->host_status + 8, sizeof(cnt));
+    const uint64_t cnt = *reinterpret_cast<volatile uint64_t*>(hcount);
     *out_count = cnt;
     if (cnt > capacity) return fail(ctx, OLAP_E_OVERFLOW, "join probe: output capacity too small");
     if (out_where != OLAP_MEM_DEVICE && cnt) {
