@@ -1131,7 +1131,8 @@ olap_status olap_join_build(olap_ctx* ctx, const int64_t* keys, const uint32_t* 
     t->n_build = n;
     t->load = load;
     void* mem = nullptr;
-    e = cudaMalloc(&mem, bytes);
+    const bool keep = ctx->opts.mem_budget_bytes == 0;
+    e = keep ? devmem::take(ctx->device, &mem, bytes, &t->cap) : devmem::alloc(ctx->device, &mem, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         delete t;
@@ -1141,6 +1142,7 @@ olap_status olap_join_build(olap_ctx* ctx, const int64_t* keys, const uint32_t* 
     t->bytes = bytes;
     JoinCtl* jc = reinterpret_cast<JoinCtl*>(static_cast<unsigned char*>(mem) + slot_bytes);
     auto bail = [&](olap_status st) {
+        cudaStreamSynchronize(ctx->stream);                  // launched passes may still write it
         cudaFree(mem);
         delete t;
         return st;
@@ -1224,7 +1226,7 @@ olap_status olap_join_build(olap_ctx* ctx, const int64_t* keys, const uint32_t* 
     }
     if (hc.err) return bail(fail(ctx, static_cast<olap_status>(hc.err), "join build: table full"));
     if (hc.side_count) {
-        e = cudaMalloc(reinterpret_cast<void**>(&t->side), hc.side_count * 4);
+        e = devmem::alloc(ctx->device, reinterpret_cast<void**>(&t->side), hc.side_count * 4);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return bail(cuda_fail(ctx, e, "join side list allocation"));
@@ -1372,7 +1374,8 @@ void olap_join_free(olap_join_table* t) {
     cudaGetDevice(&cur);
     cudaSetDevice(t->device);
     cudaDeviceSynchronize();
-    if (t->slots) cudaFree(t->slots);
+    if (t->slots && t->cap) devmem::give(t->device, t->slots, t->cap);
+    else if (t->slots) cudaFree(t->slots);
     if (t->side) cudaFree(t->side);
     t->slots = nullptr;
     t->side = nullptr;

@@ -17,6 +17,7 @@ struct olap_join_table {
     uint64_t n_build = 0;
     double load = 0.0;
     size_t bytes = 0;
+    size_t cap = 0;                   // size of its memory when that may be kept for another table, else 0
     uint32_t* bloom = nullptr;        // blocked Bloom filter over the keys (NULL: none)
     uint64_t bloom_blocks = 0;        // 32-byte blocks, a power of two
     uint64_t chain_mask = 0;          // chains wrap within this many buckets + 1 (see join_block_build_kernel)

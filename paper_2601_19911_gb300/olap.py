@@ -283,9 +283,15 @@ _EXTRA_BINDERS = []
 # Buffer marshalling
 # ---------------------------------------------------------------------------
 
+_torch_mod = None
+
+
 def _torch():
-    import torch  # noqa: WPS433 (torch is only plumbing: memory and streams)
-    return torch
+    global _torch_mod
+    if _torch_mod is None:
+        import torch  # noqa: WPS433 (torch is only plumbing: memory and streams)
+        _torch_mod = torch
+    return _torch_mod
 
 
 def mem_kind(buf) -> int:
@@ -322,23 +328,31 @@ def _check_rowids(rowids, where: int, n: int) -> None:
         raise ValueError(f"{numel(rowids)} row-ids for {n} keys")
 
 
+def _cut(buf, cnt: int):
+    """The first cnt entries (the buffer itself when it holds just those)."""
+    return buf if buf.shape[0] == cnt else buf[:cnt]
+
+
 def _check_count(got: int, want: int) -> None:
     if got != want:
         raise RuntimeError(f"the library returned {got} results where {want} were due")
 
 
+_KIND_OF = {np.dtype(npdt): kind for kind, npdt in KEY_NUMPY.items()}   # torch's dtypes join on first use
+
+
 def key_type_of(buf) -> int:
     dt = buf.dtype
-    if isinstance(buf, np.ndarray):
-        for kind, npdt in KEY_NUMPY.items():
-            if dt == npdt:
-                return kind
-    else:
+    kind = _KIND_OF.get(dt)
+    if kind is not None:
+        return kind
+    if not isinstance(buf, np.ndarray):
         torch = _torch()
         names = {KEY_I64: "int64", KEY_F32: "float32", KEY_F64: "float64", KEY_U64: "uint64",
                  KEY_I32: "int32", KEY_U32: "uint32"}
         for kind, nm in names.items():
             if getattr(torch, nm, None) is not None and dt == getattr(torch, nm):
+                _KIND_OF[dt] = kind
                 return kind
     raise TypeError(f"keys must be int64, float32, float64, uint64, int32 or uint32, got {dt}")
 
@@ -371,11 +385,13 @@ class Context:
         if st != OK:
             raise OlapError(st, "olap_ctx_create failed (no usable CUDA device?)")
         self.h = h
+        self._stream = None            # the context's stream, looked up once
 
     def close(self):
         if getattr(self, "h", None):
             self.lib.olap_ctx_destroy(self.h)
             self.h = None
+            self._stream = None
 
     def __del__(self):
         try:
@@ -410,12 +426,19 @@ class Context:
         tensor that torch is still writing would otherwise be read early, and
         one that torch is still clearing (a count, a status word) could be
         cleared after the library wrote it."""
-        if not force and not any(b is not None and mem_kind(b) == MEM_DEVICE for b in bufs
-                                 if not isinstance(b, np.ndarray)):
-            return
+        if not force:
+            for b in bufs:
+                if b is not None and not isinstance(b, np.ndarray) and b.is_cuda:
+                    break
+            else:
+                return
         torch = _torch()
         cur = torch.cuda.current_stream()
-        target = self.stream if stream is None else int(stream)
+        if self._stream is None:
+            self._stream = self.lib.olap_ctx_stream(self.h)
+            if self._stream is None:             # a closed context: the call itself is refused
+                return
+        target = self._stream if stream is None else int(stream)
         # nothing to wait for when torch's stream has finished its work (a
         # host-side query; a wait on the GPU costs the call a few us)
         if target != cur.cuda_stream and not cur.query():
@@ -442,7 +465,7 @@ class Context:
                                 ptr(out_keys), ptr(out_rowids), ow, ctypes.byref(got))
         self.check(st)
         _check_count(got.value, cnt)
-        return out_keys[:cnt], out_rowids[:cnt]
+        return _cut(out_keys, cnt), _cut(out_rowids, cnt)
 
     def topk_pair(self, keys0, order0: int, keys1, order1: int, k: int, rowids=None, out_keys0=None,
                   out_keys1=None, out_rowids=None):
@@ -468,7 +491,7 @@ class Context:
                                      mem_kind(out_keys0), ctypes.byref(got))
         self.check(st)
         _check_count(got.value, cnt)
-        return out_keys0[:cnt], out_keys1[:cnt], out_rowids[:cnt]
+        return _cut(out_keys0, cnt), _cut(out_keys1, cnt), _cut(out_rowids, cnt)
 
     def topk_rows(self, rows, row_bytes: int, key_offset: int, key_type: int, k: int, order: int = DESC,
                   out_rows=None, out_rowids=None):
