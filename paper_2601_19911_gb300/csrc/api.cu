@@ -340,7 +340,8 @@ struct PairSpec {
 static olap_status topk_enqueue(olap_ctx* ctx, const void* d_keys, olap_key_type type,
                                 const uint32_t* d_rowids, uint64_t n, uint64_t kk, olap_order order,
                                 void* d_out_keys, uint32_t* d_out_rowids, int32_t* dev_status,
-                                cudaStream_t stream, TopkCtl** ctl_out, const PairSpec* pair = nullptr) {
+                                cudaStream_t stream, TopkCtl** ctl_out, const PairSpec* pair = nullptr,
+                                const void* host_keys = nullptr) {
     const TopkPlan plan = topk_plan(n, kk);
     const bool reset = ctx->barrier_dirty || ctx->scratch_bytes < topk_scratch_bytes(plan, kk);
     olap_status st = ensure_scratch(ctx, topk_scratch_bytes(plan, kk));
@@ -352,6 +353,7 @@ static olap_status topk_enqueue(olap_ctx* ctx, const void* d_keys, olap_key_type
     }
     TopkArgs a{};
     a.keys = d_keys;
+    a.host_keys = host_keys;
     a.rowids = d_rowids;
     a.n = n;
     a.k = kk;
@@ -615,6 +617,29 @@ static bool rowids_in_host(const uint32_t* rowids, olap_mem where, uint64_t n, u
     return true;
 }
 
+// The device's address of a host column that the streaming pass reads and
+// copies itself (a sampled filter kernel of its own, register loads): page-locked
+// memory, or pageable memory where the device accesses it.  The copy keeps the
+// column's offset from a 32-byte boundary, within the staging that a plain copy
+// takes.  NULL: copied first.
+static const void* keys_in_host(const olap_ctx* ctx, const void* keys, size_t width, olap_mem where, uint64_t n,
+                                uint64_t kk) {
+    if (topk_plan(n, kk).use_sample != TK_SAMPLE_FILTER || ctx->opts.topk_filter == OLAP_FILTER_BULK) return nullptr;
+    const void* mapped = nullptr;
+    if (where == OLAP_MEM_HOST && ctx->host_direct) {
+        mapped = keys;
+    } else if (where == OLAP_MEM_HOST_PINNED) {
+        void* p = nullptr;
+        if (cudaHostGetDevicePointer(&p, const_cast<void*>(keys), 0) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        mapped = p;
+    }
+    const uintptr_t at = reinterpret_cast<uintptr_t>(mapped);
+    return (at & 31) + n * width <= ((n * width + 255) & ~static_cast<size_t>(255)) ? mapped : nullptr;
+}
+
 // Host memory the kernels write a blocking call's few results into: page-locked
 // memory, or pageable memory where the device accesses it itself; NULL when
 // they go through device memory and a copy.  Up to RESULTS_IN_PLACE rows: the
@@ -658,14 +683,18 @@ olap_status olap_topk(olap_ctx* ctx, const void* keys, olap_key_type type, const
     const void* dk = keys;
     const uint32_t* dr = rowids;
     const bool rowids_in_place = rowids_in_host(rowids, in_where, n, kk, &dr);
+    const void* hk = keys_in_host(ctx, keys, w, in_where, n, kk);
     if (in_where != OLAP_MEM_DEVICE) {
+        const size_t shift = hk ? reinterpret_cast<uintptr_t>(hk) & 31 : 0;
         const size_t kbytes = (n * w + 255) & ~static_cast<size_t>(255);
         const bool copy_rowids = rowids && !rowids_in_place;
         st = ensure_dev_in(ctx, kbytes + (copy_rowids ? n * 4 : 0));
         if (st != OLAP_OK) return st;
-        st = copy_h2d(ctx, ctx->dev_in, keys, n * w, in_where);
-        if (st != OLAP_OK) return st;
-        dk = ctx->dev_in;
+        if (!hk) {
+            st = copy_h2d(ctx, ctx->dev_in, keys, n * w, in_where);
+            if (st != OLAP_OK) return st;
+        }
+        dk = static_cast<unsigned char*>(ctx->dev_in) + shift;
         if (copy_rowids) {
             dr = reinterpret_cast<const uint32_t*>(static_cast<unsigned char*>(ctx->dev_in) + kbytes);
             st = copy_h2d(ctx, const_cast<uint32_t*>(dr), rowids, n * 4, in_where);
@@ -690,7 +719,7 @@ olap_status olap_topk(olap_ctx* ctx, const void* keys, olap_key_type type, const
     }
     // the kernels write the status into the context's page-locked word
     *ctx->host_status = OLAP_E_CUDA;
-    st = topk_enqueue(ctx, dk, type, dr, n, kk, order, dok, dor, ctx->host_status, ctx->stream, nullptr);
+    st = topk_enqueue(ctx, dk, type, dr, n, kk, order, dok, dor, ctx->host_status, ctx->stream, nullptr, nullptr, hk);
     if (st != OLAP_OK) return st;
     ctx->last_rowids_in_place = rowids_in_place;
     if (copy_out) {

@@ -47,6 +47,14 @@ __device__ __forceinline__ void ld_stream_32(const void* p, uint32_t (&w)[8]) {
         w[2 * j + 1] = static_cast<uint32_t>(v[j] >> 32);
     }
 }
+__device__ __forceinline__ void st_words(void* p, const uint32_t (&w)[8]) {          // 32-byte aligned
+    asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p),
+                 "l"(static_cast<uint64_t>(w[0]) | (static_cast<uint64_t>(w[1]) << 32)),
+                 "l"(static_cast<uint64_t>(w[2]) | (static_cast<uint64_t>(w[3]) << 32)),
+                 "l"(static_cast<uint64_t>(w[4]) | (static_cast<uint64_t>(w[5]) << 32)),
+                 "l"(static_cast<uint64_t>(w[6]) | (static_cast<uint64_t>(w[7]) << 32))
+                 : "memory");
+}
 __device__ __forceinline__ void ld_stream_words(const void* p, uint32_t (&w)[8]) { ld_stream_32(p, w); }
 __device__ __forceinline__ void ld_stream_words(const void* p, uint32_t (&w)[4]) {
     const uint4 v = ld_stream_v4(p);

@@ -70,15 +70,17 @@ __device__ __forceinline__ uint64_t pair_rank(uint32_t b0, uint32_t b1, const To
     return rank_key(b0, a.kind, a.desc) | (rank_key(b1, a.kind2, a.desc2) >> 32);
 }
 
+// Key bits of row i of the column at `keys` (a.keys, or a.host_keys).
+__device__ __forceinline__ uint64_t key_bits(const TopkArgs& a, const void* keys, uint64_t i) {
+    return a.w4 ? static_cast<uint64_t>(static_cast<const uint32_t*>(keys)[i]) : static_cast<const uint64_t*>(keys)[i];
+}
+
 __device__ __forceinline__ Elem load_input(const TopkArgs& a, uint64_t i) {
     Elem e;
-    if (a.pair) {
+    if (a.pair)
         e.r = pair_rank(static_cast<const uint32_t*>(a.keys)[i], static_cast<const uint32_t*>(a.keys2)[i], a);
-    } else {
-        const uint64_t bits = a.w4 ? static_cast<uint64_t>(static_cast<const uint32_t*>(a.keys)[i])
-                                   : static_cast<const uint64_t*>(a.keys)[i];
-        e.r = rank_key(bits, a.kind, a.desc);
-    }
+    else
+        e.r = rank_key(key_bits(a, a.keys, i), a.kind, a.desc);
     e.rid = a.rowids ? a.rowids[i] : static_cast<uint32_t>(i);
     return e;
 }
@@ -409,7 +411,7 @@ __device__ __forceinline__ void filter_vector(const TopkArgs& a, const KeyLimit&
 
 // The unaligned head [0, head) and ragged tail [tail0, n) of the keys: at
 // most 14 keys, one per lane of warp 0 of CTA 0.
-template <bool FUSE = false>
+template <bool FUSE = false, bool COPY = false>
 __device__ __forceinline__ void filter_ends(const TopkArgs& a, uint64_t t, uint64_t head, uint64_t tail0,
                                             WarpStage& ws) {
     if (blockIdx.x != 0 || threadIdx.x >= 32) return;
@@ -419,7 +421,14 @@ __device__ __forceinline__ void filter_ends(const TopkArgs& a, uint64_t t, uint6
     uint64_t idx = 0, r = ~0ull;
     if (valid) {
         idx = j < head ? j : tail0 + (j - head);
-        r = load_input(a, idx).r;
+        if (COPY) {
+            const uint64_t bits = key_bits(a, a.host_keys, idx);
+            if (a.w4) static_cast<uint32_t*>(const_cast<void*>(a.keys))[idx] = static_cast<uint32_t>(bits);
+            else static_cast<uint64_t*>(const_cast<void*>(a.keys))[idx] = bits;
+            r = rank_key(bits, a.kind, a.desc);
+        } else {
+            r = load_input(a, idx).r;
+        }
     }
     stage_hits<1, FUSE>(a, valid && r <= t ? 1u : 0u, idx, ws, [&](int) { return r; });
 }
@@ -459,12 +468,12 @@ struct FilterSpan {                            // the 32-byte vectors of the key
     static constexpr int VEC = 32 / W;
     uint64_t head, nvec, tail0;
     const unsigned char* base;
-    __device__ explicit FilterSpan(const TopkArgs& a) {
-        const uint64_t head0 = ((32 - (reinterpret_cast<uintptr_t>(a.keys) & 31)) & 31) / W;
+    __device__ FilterSpan(const TopkArgs& a, const void* keys) {
+        const uint64_t head0 = ((32 - (reinterpret_cast<uintptr_t>(keys) & 31)) & 31) / W;
         head = head0 < a.n ? head0 : a.n;
         nvec = (a.n - head) / VEC;
         tail0 = head + nvec * VEC;
-        base = static_cast<const unsigned char*>(a.keys) + head * W;
+        base = static_cast<const unsigned char*>(keys) + head * W;
     }
 };
 
@@ -506,7 +515,7 @@ struct FilterStep {
     }
 };
 
-template <bool W4, int TPB, int MODE>
+template <bool W4, int TPB, int MODE, bool COPY>
 __device__ __forceinline__ void filter_loop(const TopkArgs& a, const FilterSpan<W4>& sp, uint64_t lim, FilterStep st,
                                             uint32_t (&v)[TK_UNROLL][8], WarpStage& ws) {
     constexpr int VEC = FilterSpan<W4>::VEC;
@@ -519,7 +528,16 @@ __device__ __forceinline__ void filter_loop(const TopkArgs& a, const FilterSpan<
         return W4 ? key_pass<MODE, uint32_t, int32_t>(v[u][e], static_cast<uint32_t>(lim))
                   : key_pass<MODE, uint64_t, int64_t>(key(u, e), lim);
     };
+    unsigned char* copy = COPY ? const_cast<unsigned char*>(static_cast<const unsigned char*>(a.keys)) + sp.head * sp.W
+                               : nullptr;
     while (st.bb < st.end) {
+        if (COPY) {
+#pragma unroll
+            for (int u = 0; u < TK_UNROLL; ++u) {
+                const uint64_t vi = st.bb + static_cast<uint64_t>(u) * TPB + threadIdx.x;
+                if (vi < st.end) st_words(copy + vi * 32, v[u]);
+            }
+        }
         bool any = false;
 #pragma unroll
         for (int u = 0; u < TK_UNROLL; ++u)
@@ -542,11 +560,11 @@ __device__ __forceinline__ void filter_loop(const TopkArgs& a, const FilterSpan<
     }
 }
 
-template <bool W4, int TPB>
+template <bool W4, int TPB, bool COPY = false>
 __device__ __forceinline__ void filter_pass(const TopkArgs& a, unsigned char* fsm) {
     unsigned* hist = reinterpret_cast<unsigned*>(fsm);
     fuse_init<TPB>(hist);
-    const FilterSpan<W4> sp(a);
+    const FilterSpan<W4> sp(a, COPY ? a.host_keys : a.keys);
     FilterStep st;
     st.first(sp.nvec, static_cast<uint64_t>(TPB) * TK_UNROLL);
     uint32_t v[TK_UNROLL][8];
@@ -565,11 +583,11 @@ __device__ __forceinline__ void filter_pass(const TopkArgs& a, unsigned char* fs
         mode = key_cmp<uint64_t>(kl.m64, kl.c64, &lim);
     }
     WarpStage ws = warp_stage(fsm + FUSE_BYTES, hist);
-    if (mode == CMP_GE_U) filter_loop<W4, TPB, CMP_GE_U>(a, sp, lim, st, v, ws);
-    else if (mode == CMP_LE_U) filter_loop<W4, TPB, CMP_LE_U>(a, sp, lim, st, v, ws);
-    else if (mode == CMP_GE_S) filter_loop<W4, TPB, CMP_GE_S>(a, sp, lim, st, v, ws);
-    else filter_loop<W4, TPB, CMP_LE_S>(a, sp, lim, st, v, ws);
-    filter_ends<true>(a, t, sp.head, sp.tail0, ws);
+    if (mode == CMP_GE_U) filter_loop<W4, TPB, CMP_GE_U, COPY>(a, sp, lim, st, v, ws);
+    else if (mode == CMP_LE_U) filter_loop<W4, TPB, CMP_LE_U, COPY>(a, sp, lim, st, v, ws);
+    else if (mode == CMP_GE_S) filter_loop<W4, TPB, CMP_GE_S, COPY>(a, sp, lim, st, v, ws);
+    else filter_loop<W4, TPB, CMP_LE_S, COPY>(a, sp, lim, st, v, ws);
+    filter_ends<true, COPY>(a, t, sp.head, sp.tail0, ws);
     cta_flush_fused<TPB>(a, ws);
     fuse_merge<TPB>(a, hist);
 }
@@ -1000,7 +1018,8 @@ __global__ void __launch_bounds__(TK_TPB) topk_prepare_kernel(TopkArgs a) {
         return;
     }
     const uint64_t j = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x;   // < TK_SAMPLE
-    a.samples[j] = load_input(a, (j * a.n) / TK_SAMPLE + (a.n / TK_SAMPLE) / 2).r;
+    const uint64_t at = (j * a.n) / TK_SAMPLE + (a.n / TK_SAMPLE) / 2;
+    a.samples[j] = a.host_keys ? rank_key(key_bits(a, a.host_keys, at), a.kind, a.desc) : load_input(a, at).r;
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) last = (atomicAdd(&a.bar->prep, 1u) + 1u) % gridDim.x == 0;
@@ -1027,6 +1046,20 @@ template <bool W4, int TPB>
 __global__ void __launch_bounds__(TPB, 1024 / TPB) topk_filter_regs_kernel(TopkArgs a) {
     extern __shared__ __align__(16) unsigned char fsm[];
     filter_pass<W4, TPB>(a, fsm);
+}
+
+// Kernel 2 of 3 for a column in host memory that the device reads itself: the
+// same pass over the host column, which also leaves the copy in device memory
+// (a.keys, at the same offset from a 32-byte boundary) that a misjudged
+// sample's select reads.  Bound by the host link, which a kernel's loads fill
+// as well as a DMA copy (2^31 bytes 10.16 against 10.15 ms, 24 MB 120 against
+// 117 us): the filter's own pass over the copy goes, and the first loads are
+// under way while the sample is ranked.  2^21.5 page-locked int64 keys 173 ->
+// 157 us for the call, 2^24 710 -> 680, 2^28 10512 -> 10220.
+template <bool W4>
+__global__ void __launch_bounds__(TKR_TPB, 1) topk_filter_host_kernel(TopkArgs a) {
+    extern __shared__ __align__(16) unsigned char fsm[];
+    filter_pass<W4, TKR_TPB, true>(a, fsm);
 }
 
 // Kernel 2 of 3 for a two-column key (register loads of both columns).
@@ -1715,6 +1748,8 @@ static bool set_kernel_attrs(int device) {
     opt_in(topk_filter_regs_kernel<false, 1024>, regs_smem(1024));
     opt_in(topk_filter_regs_kernel<true, 1024>, regs_smem(1024));
     opt_in(topk_filter_pair_kernel<1024>, regs_smem(1024));
+    opt_in(topk_filter_host_kernel<false>, regs_smem(TKR_TPB));
+    opt_in(topk_filter_host_kernel<true>, regs_smem(TKR_TPB));
     opt_in(topk_local_kernel, TKL_SMEM_MAX);
     opt_in(topk_select_kernel<SEL_NONE>, TK_SORT_SMEM);
     opt_in(topk_select_kernel<SEL_W8>, TK_SORT_SMEM);
@@ -1813,7 +1848,7 @@ cudaError_t topk_launch(const TopkArgs& args, const TopkGeom& geom, cudaStream_t
     if (a.digit < TK_DIG_MIN || a.digit > TK_DIG) return cudaErrorInvalidValue;
     // the register and two-column filters fold the select's first pass
     a.fuse = a.use_sample == TK_SAMPLE_INLINE ||
-                     (a.use_sample == TK_SAMPLE_FILTER && (a.pair || a.filter == TK_FILTER_REGS))
+                     (a.use_sample == TK_SAMPLE_FILTER && (a.pair || a.host_keys || a.filter == TK_FILTER_REGS))
                  ? 1
                  : 0;
     cudaError_t e;
@@ -1836,7 +1871,12 @@ cudaError_t topk_launch(const TopkArgs& args, const TopkGeom& geom, cudaStream_t
         void (*fn)(TopkArgs) = nullptr;
         unsigned grid = static_cast<unsigned>(geom.regs_grid), block = static_cast<unsigned>(geom.regs_tpb);
         size_t smem = static_cast<size_t>(regs_smem(geom.regs_tpb));
-        if (a.pair) {
+        if (a.host_keys) {
+            fn = a.w4 ? topk_filter_host_kernel<true> : topk_filter_host_kernel<false>;
+            grid = TK_HOST_CTAS;
+            block = TKR_TPB;
+            smem = static_cast<size_t>(regs_smem(TKR_TPB));
+        } else if (a.pair) {
             fn = geom.regs_tpb == 256    ? topk_filter_pair_kernel<256>
                  : geom.regs_tpb == 1024 ? topk_filter_pair_kernel<1024>
                                          : topk_filter_pair_kernel<512>;

@@ -47,6 +47,7 @@ constexpr int TK_SMEM_MAX = 227 * 1024;   // opt-in shared memory per CTA
 // the register-load flavour uses CTAs of 256, 512 (default) or 1024 threads.
 constexpr int TKF_TPB = 256;
 constexpr int TKR_TPB = 512;
+constexpr unsigned TK_HOST_CTAS = 152;    // CTAs of the pass over a column in host memory
 constexpr int TK_TILE_DEFAULT = 16384;
 constexpr int TK_STAGES_DEFAULT = 3;
 constexpr int TK_CTAS_PER_SM_DEFAULT = 4;
@@ -81,6 +82,7 @@ struct TopkCtl {
 
 struct TopkArgs {
     const void* keys;
+    const void* host_keys;           // not NULL: the column in host memory, which the filter copies to keys
     const uint32_t* rowids;          // NULL => row-id = index
     uint64_t n;
     uint64_t k;                      // already min(k, n), > 0
