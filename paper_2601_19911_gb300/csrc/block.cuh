@@ -47,7 +47,21 @@ __device__ __forceinline__ void ld_stream_32(const void* p, uint32_t (&w)[8]) {
         w[2 * j + 1] = static_cast<uint32_t>(v[j] >> 32);
     }
 }
-__device__ __forceinline__ void st_words(void* p, const uint32_t (&w)[8]) {          // 32-byte aligned
+// Programmatic dependent launch.  Every kernel of a call is launched while
+// the one before it in the stream is still running, and waits here until that
+// one has finished and its writes are visible.  A kernel launched without the
+// attribute passes straight through.
+__device__ __forceinline__ void wait_prior_grid() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Lets the next kernel in the stream launch now (it still waits for this one
+// to finish before it reads anything this one or an earlier one writes).
+__device__ __forceinline__ void allow_next_grid() {
+    asm volatile("griddepcontrol.launch_dependents;" :::);
+}
+
+// A 32-byte store (of the vector ld_stream_words loads); p 32-byte aligned.
+__device__ __forceinline__ void st_words(void* p, const uint32_t (&w)[8]) {
     asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p),
                  "l"(static_cast<uint64_t>(w[0]) | (static_cast<uint64_t>(w[1]) << 32)),
                  "l"(static_cast<uint64_t>(w[2]) | (static_cast<uint64_t>(w[3]) << 32)),

@@ -386,6 +386,7 @@ __global__ void __launch_bounds__(JP_TPB, JP_CTAS) join_probe_kernel(ProbeArgs a
     unsigned char* mine = psmem + (threadIdx.x >> 5) * JP_WARP_SMEM;
     ProbeArgs a = args;
     bool l1 = !L2_ONLY;
+    wait_prior_grid();
     if (ctl) {
         if (ctl->active) a.n = ctl->count;
         if (ctl->redirect) {
@@ -444,7 +445,8 @@ constexpr unsigned PF_WCAP = 256;              // rows staged per warp
 constexpr int PF_CTAS = 6;                     // pre-probe CTAs per SM
 
 constexpr int PLAN_SLOTS = 2 * PF_SAMPLE;      // fingerprint set of the sample (32 KB)
-constexpr int PLAN_CTAS = PF_SAMPLE / PF_TPB;  // one sampled key per thread
+constexpr int PLAN_CTAS = 16;
+constexpr int PLAN_TPB = 1024;                 // the first PF_SAMPLE / PLAN_CTAS threads load the CTA's sample
 
 // The plan kernel's inputs, and its state in the context's device area.
 struct PlanArgs {
@@ -466,7 +468,8 @@ struct PlanArgs {
 // The probe's plan, decided on the device from a stratified sample of
 // PF_SAMPLE probe keys (n >= PF_SAMPLE; fewer rows are each taken once or
 // more).  PLAN_CTAS CTAs load the sample, one key per thread (from one SM,
-// 4096 scattered loads wait on each other's latency: 38 us), test it
+// 4096 scattered loads wait on each other's latency: 38 us; the other threads
+// of a CTA only help the last one decide: 12.5 -> 8.5 us), test it
 // against the Bloom filter and store one packed word per key: a 30-bit
 // fingerprint of the key, bit 1 = kept by the filter, bit 0 = 1.  The last
 // CTA to finish decides.  With a Bloom filter (pf_mode 1 = automatic,
@@ -483,19 +486,22 @@ struct PlanArgs {
 // not direct, as launched), else the kept rows (pf_keys, pf_rowids) when the
 // pre-probe runs, else the input; a direct probe reads buckets through L1
 // when `skew_l1`.  It also clears the counters for the next call.
-__global__ void __launch_bounds__(PF_TPB) join_probe_plan_kernel(PlanArgs a) {
+__global__ void __launch_bounds__(PLAN_TPB) join_probe_plan_kernel(PlanArgs a) {
+    allow_next_grid();
     __shared__ uint32_t fset[PLAN_SLOTS];
     __shared__ unsigned kept_cta, dup_all, dup_kept;
     __shared__ bool last;
     if (threadIdx.x == 0) kept_cta = 0;
     __syncthreads();
-    {
-        const uint64_t j = static_cast<uint64_t>(blockIdx.x) * PF_TPB + threadIdx.x;     // < PF_SAMPLE
+    constexpr int PER_CTA = PF_SAMPLE / PLAN_CTAS;
+    if (threadIdx.x < PER_CTA) {
+        const uint64_t j = static_cast<uint64_t>(blockIdx.x) * PER_CTA + threadIdx.x;
         const uint64_t key = static_cast<uint64_t>(a.keys[(j * a.n) / PF_SAMPLE]);
         const bool kept = a.bloom.bits ? (key == JN_EMPTY || bloom_maybe(a.bloom, key)) : true;
         const uint32_t fp = static_cast<uint32_t>(fmix64(key) >> 32) & ~3u;
         a.sample[j] = fp | (kept ? 2u : 0u) | 1u;
-        if (kept) atomicAdd(&kept_cta, 1u);
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, kept);
+        if ((threadIdx.x & 31u) == 0) atomicAdd(&kept_cta, static_cast<unsigned>(__popc(m)));
     }
     __threadfence();
     __syncthreads();
@@ -506,12 +512,12 @@ __global__ void __launch_bounds__(PF_TPB) join_probe_plan_kernel(PlanArgs a) {
     __syncthreads();
     if (!last) return;
     __threadfence();
-    for (int j = threadIdx.x; j < PLAN_SLOTS; j += PF_TPB) fset[j] = 0u;
+    for (int j = threadIdx.x; j < PLAN_SLOTS; j += PLAN_TPB) fset[j] = 0u;
     if (threadIdx.x == 0) dup_all = dup_kept = 0;
     __syncthreads();
     unsigned m_dup = 0, m_dup_kept = 0;
     if (a.skew_check) {
-        for (int j = threadIdx.x; j < PF_SAMPLE; j += PF_TPB) {
+        for (int j = threadIdx.x; j < PF_SAMPLE; j += PLAN_TPB) {
             const uint32_t w = __ldcg(a.sample + j);
             const uint32_t fp = w & ~2u;                 // the fingerprint, with the set's non-zero bit
             uint32_t slot = (fp >> 2) & (PLAN_SLOTS - 1);
@@ -529,8 +535,12 @@ __global__ void __launch_bounds__(PF_TPB) join_probe_plan_kernel(PlanArgs a) {
             m_dup_kept += (dup && (w & 2u)) ? 1u : 0u;
         }
     }
-    atomicAdd(&dup_all, m_dup);
-    atomicAdd(&dup_kept, m_dup_kept);
+    m_dup = __reduce_add_sync(0xFFFFFFFFu, m_dup);
+    m_dup_kept = __reduce_add_sync(0xFFFFFFFFu, m_dup_kept);
+    if ((threadIdx.x & 31u) == 0) {
+        atomicAdd(&dup_all, m_dup);
+        atomicAdd(&dup_kept, m_dup_kept);
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         const unsigned passes = atomicAdd(&a.counters[0], 0u);
@@ -561,6 +571,8 @@ __global__ void __launch_bounds__(PF_TPB) join_probe_plan_kernel(PlanArgs a) {
 __global__ void __launch_bounds__(PF_TPB, PF_CTAS) join_prefilter_kernel(const int64_t* keys, const uint32_t* rowids,
                                                                 uint64_t n, BloomView bloom, ProbeCtl* ctl,
                                                                 int64_t* out_keys, uint32_t* out_rowids) {
+    wait_prior_grid();
+    allow_next_grid();
     if (!ctl->active) return;
     __shared__ int64_t sk[PF_TPB / 32][PF_WCAP];
     __shared__ uint32_t sr[PF_TPB / 32][PF_WCAP];
@@ -615,8 +627,8 @@ __global__ void __launch_bounds__(PF_TPB, PF_CTAS) join_prefilter_kernel(const i
 
 // ---- partitioned probe ------------------------------------------------------
 
-constexpr int JQ_TPB = 256;
-constexpr int JQ_PER = 8;                      // probe rows per thread per tile
+constexpr int JQ_TPB = 320;
+constexpr int JQ_PER = 7;                      // probe rows per thread per tile
 constexpr int JQ_TILE = JQ_TPB * JQ_PER;       // rows per tile
 constexpr int JQ_PMAX = 256;                   // most partitions
 constexpr int JQ_CTAS_PER_SM = 4;              // grid of the two partition passes
@@ -629,8 +641,9 @@ struct PartArgs {
     uint64_t mask;                             // buckets - 1
     int shift;                                 // partition = home bucket >> shift
     int parts;
-    unsigned long long* cnt;                   // [gridDim.x][parts] rows per CTA and partition
-    unsigned long long* pstart;                // [parts + 1] partition offsets (written by CTA 0)
+    unsigned long long* counts;                // [parts] rows of each partition; zero between calls
+    unsigned long long* next;                  // [parts] next output row of each partition
+    unsigned* ticket;                          // CTAs that have counted; zero between calls
     int64_t* out_keys;
     uint32_t* out_rowids;
     const ProbeCtl* pf;                        // non-NULL: the device-side plan (pre-probe, direct)
@@ -654,151 +667,187 @@ __device__ __forceinline__ unsigned part_of(uint64_t key, const PartArgs& a) {
     return static_cast<unsigned>((fmix64(key) & a.mask) >> a.shift);
 }
 
-// Pass 1: rows of each partition in the tiles of this CTA (tiles blockIdx.x,
-// blockIdx.x + gridDim.x, ...).
+// The keys of the tile at t0, thread by thread (zeros past the end).
+__device__ __forceinline__ void part_load(const PartArgs& a, uint64_t t0, uint64_t (&k)[JQ_PER]) {
+    const int64_t* p = a.keys + t0 + threadIdx.x;
+    if (t0 + JQ_TILE <= a.n) {
+#pragma unroll
+        for (int j = 0; j < JQ_PER; ++j) k[j] = ld_stream_u64(p + j * JQ_TPB);
+    } else {
+#pragma unroll
+        for (int j = 0; j < JQ_PER; ++j)
+            k[j] = t0 + static_cast<uint64_t>(j) * JQ_TPB + threadIdx.x < a.n ? ld_stream_u64(p + j * JQ_TPB) : 0ull;
+    }
+}
+
+// Exclusive sum over a warp's lanes.
+__device__ __forceinline__ unsigned warp_excl_scan(unsigned x, unsigned lane) {
+    unsigned incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= static_cast<unsigned>(o)) incl += v;
+    }
+    return incl - x;
+}
+
+// Pass 1: rows of each partition; the last CTA to finish turns the totals into
+// the partitions' first output rows.  As many CTAs as fit: it waits for its
+// loads (3*10^7 rows 43 us, 5.6 TB/s).
 __global__ void __launch_bounds__(JQ_TPB) join_part_count_kernel(PartArgs args) {
+    wait_prior_grid();
+    allow_next_grid();
     if (args.pf && args.pf->direct) return;
     const PartArgs a = part_source(args);
     __shared__ unsigned h[JQ_PMAX];
     for (int p = threadIdx.x; p < a.parts; p += JQ_TPB) h[p] = 0;
     __syncthreads();
-    for (uint64_t t0 = static_cast<uint64_t>(blockIdx.x) * JQ_TILE; t0 < a.n;
-         t0 += static_cast<uint64_t>(gridDim.x) * JQ_TILE) {
+    const uint64_t stride = static_cast<uint64_t>(gridDim.x) * JQ_TILE;
+    for (uint64_t t0 = static_cast<uint64_t>(blockIdx.x) * JQ_TILE; t0 < a.n; t0 += stride) {
         uint64_t k[JQ_PER];
+        part_load(a, t0, k);
+        const unsigned len = static_cast<unsigned>(min(static_cast<uint64_t>(JQ_TILE), a.n - t0));
 #pragma unroll
-        for (int j = 0; j < JQ_PER; ++j) {
-            const uint64_t idx = t0 + static_cast<uint64_t>(j) * JQ_TPB + threadIdx.x;
-            k[j] = idx < a.n ? ld_stream_u64(a.keys + idx) : 0ull;
-        }
-#pragma unroll
-        for (int j = 0; j < JQ_PER; ++j) {
-            const uint64_t idx = t0 + static_cast<uint64_t>(j) * JQ_TPB + threadIdx.x;
-            if (idx < a.n) atomicAdd(&h[part_of(k[j], a)], 1u);
-        }
+        for (int j = 0; j < JQ_PER; ++j)
+            if (j * JQ_TPB + threadIdx.x < len) atomicAdd(&h[part_of(k[j], a)], 1u);
     }
     __syncthreads();
-    for (int p = threadIdx.x; p < a.parts; p += JQ_TPB)
-        a.cnt[static_cast<uint64_t>(blockIdx.x) * a.parts + p] = h[p];
-}
-
-// Pass 2: the same tiles again; each row goes to its partition at this CTA's
-// running offset (partition start + rows of that partition in lower CTAs +
-// rows already placed), reordered in shared memory so the writes of a
-// partition's run are contiguous.  The keys of the CTA's next tile are loaded
-// while the current one is reordered.  Three CTA barriers per tile: the
-// per-tile counts alternate between two arrays (the next tile's is zeroed
-// while this one is scanned), one warp scans them, and the next tile cannot
-// overwrite the reorder buffer before every thread has passed its first
-// barrier, which it reaches only after writing this tile out.
-__global__ void __launch_bounds__(JQ_TPB) join_part_scatter_kernel(PartArgs args) {
-    if (args.pf && args.pf->direct) return;
-    const PartArgs a = part_source(args);
-    __shared__ unsigned h[2][JQ_PMAX];
-    __shared__ unsigned off[JQ_PMAX];
-    __shared__ unsigned long long base[JQ_PMAX];
-    __shared__ unsigned long long tbase[JQ_PMAX];
+    const int p = threadIdx.x;
+    if (p < a.parts && h[p]) atomicAdd(&a.counts[p], static_cast<unsigned long long>(h[p]));
     __shared__ unsigned long long wsum[JQ_TPB / 32];
     __shared__ unsigned long long total;
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (p == 0) last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const unsigned long long c = p < a.parts ? __ldcg(a.counts + p) : 0ull;
+    const unsigned long long start = block_excl_scan<JQ_TPB>(c, wsum, &total);
+    if (p < a.parts) {
+        a.next[p] = start;
+        a.counts[p] = 0;
+    }
+    if (p == 0) *a.ticket = 0;
+}
+
+// Pass 2: each row to its partition, a tile at a time, reordered in shared
+// memory so that the tile's rows of a partition are one contiguous run, at a
+// place taken from the partition's cursor.  All CTAs append at the same few
+// places (one per partition), so the runs' ragged ends meet in L2 and DRAM
+// sees whole pages; rows of a partition keep no order.  The keys of the CTA's
+// next tile are loaded while the current one is reordered.  A shared atomic
+// per row gives its rank in the tile; then every warp scans the tile's counts
+// for itself (NP partitions a lane, for up to 32 * NP) and takes the runs'
+// starts from its lanes, so a tile needs two CTA barriers: counts complete,
+// and reordered.  The counts alternate between two arrays (the other one is
+// zeroed between the barriers), and the next tile cannot overwrite the reorder
+// buffer before every thread has passed its first barrier, which it reaches
+// only after writing this tile out.  Bound by shared memory: the scattered
+// stores of the reorder and the atomics collide in its banks (L1 at 75 %).
+// 3*10^7 rows into 32 partitions: 128 us, 163 with a region of its own for
+// every CTA, one scanning warp and three barriers; the whole probe of a
+// 2^24-row table 477 -> 437 us, 8*10^6 rows against 4*10^6 175 -> 139.  (Ranks
+// by ballots instead of shared atomics: 557.)  Tiles of 320 x 7 rows, four
+// CTAs: 256 x 8 444, 384 x 6 453, 512 x 6 464.
+template <int NP>
+__global__ void __launch_bounds__(JQ_TPB, JQ_CTAS_PER_SM) join_part_scatter_kernel(PartArgs args) {
+    wait_prior_grid();
+    allow_next_grid();
+    if (args.pf && args.pf->direct) return;
+    const PartArgs a = part_source(args);
+    constexpr int WIDTH = 32 * NP;
+    __shared__ unsigned h[2][WIDTH];
+    __shared__ unsigned long long tbase[WIDTH];          // output row of the tile's run, less its start
     __shared__ int64_t sk[JQ_TILE];
     __shared__ uint32_t sr[JQ_TILE];
     __shared__ uint8_t sp[JQ_TILE];
-    const int p = threadIdx.x;
-    const int P = a.parts;
-    {
-        unsigned long long below = 0, all = 0;
-        if (p < P) {
-            for (unsigned c = 0; c < gridDim.x; ++c) {
-                const unsigned long long v = a.cnt[static_cast<uint64_t>(c) * P + p];
-                all += v;
-                if (c < blockIdx.x) below += v;
-            }
-        }
-        const unsigned long long start = block_excl_scan<JQ_TPB>(all, wsum, &total);
-        if (p < P) {
-            base[p] = start + below;
-            h[0][p] = 0;
-        }
-        if (blockIdx.x == 0 && p < P) a.pstart[p] = start;
-        if (blockIdx.x == 0 && p == 0) a.pstart[P] = total;
-    }
+    if (threadIdx.x < WIDTH) h[0][threadIdx.x] = 0;
     __syncthreads();
     const unsigned lane = threadIdx.x & 31u;
-    const int PP = (P + 31) / 32;                      // partitions per lane of the scanning warp
     const uint64_t stride = static_cast<uint64_t>(gridDim.x) * JQ_TILE;
     uint64_t kc[JQ_PER];
     const uint64_t first = static_cast<uint64_t>(blockIdx.x) * JQ_TILE;
-#pragma unroll
-    for (int j = 0; j < JQ_PER; ++j) {
-        const uint64_t idx = first + static_cast<uint64_t>(j) * JQ_TPB + threadIdx.x;
-        kc[j] = idx < a.n ? ld_stream_u64(a.keys + idx) : 0ull;
-    }
+    if (first < a.n) part_load(a, first, kc);
     int cur = 0;
     for (uint64_t t0 = first; t0 < a.n; t0 += stride, cur ^= 1) {
         uint64_t kn[JQ_PER];
-#pragma unroll
-        for (int j = 0; j < JQ_PER; ++j) {
-            const uint64_t idx = t0 + stride + static_cast<uint64_t>(j) * JQ_TPB + threadIdx.x;
-            kn[j] = idx < a.n ? ld_stream_u64(a.keys + idx) : 0ull;
-        }
-        unsigned* hc = h[cur];
+        if (t0 + stride < a.n) part_load(a, t0 + stride, kn);
+        const unsigned len = static_cast<unsigned>(min(static_cast<uint64_t>(JQ_TILE), a.n - t0));
         unsigned pr[JQ_PER];                   // partition | rank in the tile << 8
 #pragma unroll
         for (int j = 0; j < JQ_PER; ++j) {
-            const uint64_t idx = t0 + static_cast<uint64_t>(j) * JQ_TPB + threadIdx.x;
             const unsigned q = part_of(kc[j], a);
-            pr[j] = idx < a.n ? (q | (atomicAdd(&hc[q], 1u) << 8)) : 0u;
+            pr[j] = j * JQ_TPB + threadIdx.x < len ? (q | (atomicAdd(&h[cur][q], 1u) << 8)) : 0u;
         }
         __syncthreads();
-        if (threadIdx.x < 32) {
-            // the tile's run starts (exclusive scan of its counts), the
-            // partitions' output positions, and the other count array zeroed
-            unsigned run = 0;
-            for (int i = 0; i < PP; ++i) {
-                const int q = static_cast<int>(lane) * PP + i;
-                if (q < P) run += hc[q];
-            }
-            unsigned incl = run;
+        // partitions lane + 32 * i: where their runs start in the tile
+        unsigned off[NP], below = 0;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                if (lane >= static_cast<unsigned>(o)) incl += v;
-            }
-            unsigned at = incl - run;
-            for (int i = 0; i < PP; ++i) {
-                const int q = static_cast<int>(lane) * PP + i;
-                if (q < P) {
-                    const unsigned c = hc[q];
-                    off[q] = at;
-                    tbase[q] = base[q];
-                    base[q] += c;
-                    h[cur ^ 1][q] = 0;
-                    at += c;
-                }
+        for (int i = 0; i < NP; ++i) {
+            const unsigned c = h[cur][lane + 32 * i];
+            off[i] = below + warp_excl_scan(c, lane);
+            if (i + 1 < NP) below = __shfl_sync(0xFFFFFFFFu, off[i] + c, 31);
+            if (threadIdx.x < 32) {
+                if (c) tbase[lane + 32 * i] = atomicAdd(&a.next[lane + 32 * i], static_cast<unsigned long long>(c)) - off[i];
+                h[cur ^ 1][lane + 32 * i] = 0;
             }
         }
-        __syncthreads();
 #pragma unroll
         for (int j = 0; j < JQ_PER; ++j) {
-            const uint64_t idx = t0 + static_cast<uint64_t>(j) * JQ_TPB + threadIdx.x;
-            if (idx < a.n) {
-                const unsigned q = pr[j] & 0xFFu;
-                const unsigned pos = off[q] + (pr[j] >> 8);
+            const unsigned i = j * JQ_TPB + threadIdx.x;
+            const unsigned q = pr[j] & 0xFFu;
+            unsigned pos = __shfl_sync(0xFFFFFFFFu, off[0], q & 31u);
+#pragma unroll
+            for (int b = 1; b < NP; ++b) {
+                const unsigned v = __shfl_sync(0xFFFFFFFFu, off[b], q & 31u);
+                if (q >> 5 == static_cast<unsigned>(b)) pos = v;
+            }
+            pos += pr[j] >> 8;
+            if (i < len) {
                 sk[pos] = static_cast<int64_t>(kc[j]);
-                sr[pos] = a.rowids ? ld_stream_u32(a.rowids + idx) : static_cast<uint32_t>(idx);
+                sr[pos] = a.rowids ? ld_stream_u32(a.rowids + t0 + i) : static_cast<uint32_t>(t0 + i);
                 sp[pos] = static_cast<uint8_t>(q);
             }
         }
         __syncthreads();
-        const unsigned len = static_cast<unsigned>(min(static_cast<uint64_t>(JQ_TILE), a.n - t0));
-        for (unsigned i = threadIdx.x; i < len; i += JQ_TPB) {
-            const unsigned q = sp[i];
-            const unsigned long long dst = tbase[q] + (i - off[q]);
-            a.out_keys[dst] = sk[i];
-            a.out_rowids[dst] = sr[i];
+#pragma unroll
+        for (int j = 0; j < JQ_PER; ++j) {
+            const unsigned i = j * JQ_TPB + threadIdx.x;
+            if (i < len) {
+                const unsigned long long dst = tbase[sp[i]] + i;
+                a.out_keys[dst] = sk[i];
+                a.out_rowids[dst] = sr[i];
+            }
         }
 #pragma unroll
         for (int j = 0; j < JQ_PER; ++j) kc[j] = kn[j];
     }
+}
+
+// The scatter pass for a number of partitions.
+void (*part_scatter(int parts))(PartArgs) {
+    return parts <= 32 ? join_part_scatter_kernel<1> : parts <= 64 ? join_part_scatter_kernel<2> : join_part_scatter_kernel<8>;
+}
+
+// A launch of the probe's chain; `after`: with programmatic stream
+// serialisation, behind a kernel of the same chain (it waits for the whole of
+// that kernel in wait_prior_grid, and only its launch overlaps).  Errors are
+// left to cudaGetLastError.
+template <typename... P>
+void launch_after(void (*fn)(P...), unsigned grid, int block, size_t smem, cudaStream_t s, bool after, P... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(static_cast<unsigned>(block));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = after ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, fn, args...);
 }
 
 uint64_t next_pow2(uint64_t x) {
@@ -855,20 +904,28 @@ int block_build_grid(int device, int* scatter) {
 
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
-// Grid of the two partition passes.  Both take the same one (the scatter
-// reads the count pass's per-CTA counts), at most JQ_CTAS_PER_SM per SM and no
-// more than the heavier scatter kernel keeps resident: every CTA owns a fixed
-// set of tiles, so CTAs beyond one wave would run their whole share late.
-int part_grid(int device, int sms) {
-    static std::atomic<int> cached[64] = {};
-    if (device < 0 || device >= 64) return 0;
-    if (const int c = cached[device].load()) return c;
-    int per_s = 0, per_c = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_s, join_part_scatter_kernel, JQ_TPB, 0) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_c, join_part_count_kernel, JQ_TPB, 0) != cudaSuccess)
-        return 0;
-    cached[device].store(sms * std::max(1, std::min(JQ_CTAS_PER_SM, std::min(per_s, per_c))));
-    return cached[device].load();
+// Grids of the two partition passes: the CTAs that stay resident.
+struct PartGrids {
+    unsigned count, scatter;
+};
+PartGrids part_grids(int device, int sms) {
+    static std::atomic<int> cached[64] = {};                  // per SM: count | scatter << 16
+    if (device < 0 || device >= 64) return {0, 0};
+    int c = cached[device].load();
+    if (!c) {
+        int per_c = 0, per_s = JQ_CTAS_PER_SM;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_c, join_part_count_kernel, JQ_TPB, 0) != cudaSuccess)
+            return {0, 0};
+        for (int parts : {32, 64, JQ_PMAX}) {
+            int p = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, part_scatter(parts), JQ_TPB, 0) != cudaSuccess)
+                return {0, 0};
+            per_s = std::min(per_s, p);
+        }
+        c = std::max(1, per_c) | std::max(1, per_s) << 16;
+        cached[device].store(c);
+    }
+    return {static_cast<unsigned>(sms * (c & 0xFFFF)), static_cast<unsigned>(sms * (c >> 16))};
 }
 
 }  // namespace
@@ -912,18 +969,13 @@ bool probe_prefilter(const olap_ctx* ctx, const olap_join_table* t, uint64_t n) 
     return opt == OLAP_PREFILTER_ON || (opt == OLAP_PREFILTER_AUTO && n >= PF_MIN_N);
 }
 
-// Partition scratch: [partitioned keys | row-ids | count matrix | partition
-// starts]; then, with the pre-probe, [kept keys | kept row-ids].  The probe's
-// device-side plan lives in the context's small device area.
-size_t probe_part_bytes(const olap_ctx* ctx, uint64_t n, int parts) {
-    if (parts <= 1) return 0;
-    // room for the largest grid the partition passes can take
-    const uint64_t grid = static_cast<uint64_t>(ctx->sm_count) * JQ_CTAS_PER_SM;
-    return align256(n * 8) + align256(n * 4) + align256(grid * parts * 8) + align256((parts + 1) * 8);
-}
+// Partition scratch: [partitioned keys | row-ids]; then, with the pre-probe,
+// [kept keys | kept row-ids].  The probe's device-side plan and the partitions'
+// counts live in the context's small device area.
+size_t probe_part_bytes(uint64_t n, int parts) { return parts <= 1 ? 0 : align256(n * 8) + align256(n * 4); }
 
 size_t probe_scratch_bytes(const olap_ctx* ctx, const olap_join_table* t, uint64_t n) {
-    const size_t pb = probe_part_bytes(ctx, n, probe_parts(ctx, t, n));
+    const size_t pb = probe_part_bytes(n, probe_parts(ctx, t, n));
     if (!probe_prefilter(ctx, t, n)) return pb;
     return pb + align256(n * 8) + align256(n * 4);
 }
@@ -931,7 +983,7 @@ size_t probe_scratch_bytes(const olap_ctx* ctx, const olap_join_table* t, uint64
 // The partition passes over n rows by the top bits of their home bucket, in
 // the context's partition scratch (which holds probe_part_bytes).
 static PartArgs part_args(const olap_ctx* ctx, const int64_t* keys, const uint32_t* rowids, uint64_t n,
-                          uint64_t n_buckets, int parts, unsigned grid) {
+                          uint64_t n_buckets, int parts) {
     unsigned char* m = static_cast<unsigned char*>(ctx->part);
     PartArgs q{};
     q.keys = keys;
@@ -943,8 +995,10 @@ static PartArgs part_args(const olap_ctx* ctx, const int64_t* keys, const uint32
     q.parts = parts;
     q.out_keys = reinterpret_cast<int64_t*>(m);
     q.out_rowids = reinterpret_cast<uint32_t*>(m + align256(n * 8));
-    q.cnt = reinterpret_cast<unsigned long long*>(m + align256(n * 8) + align256(n * 4));
-    q.pstart = q.cnt + static_cast<uint64_t>(grid) * parts;
+    unsigned char* aux = static_cast<unsigned char*>(ctx->aux) + 4096;
+    q.counts = reinterpret_cast<unsigned long long*>(aux);
+    q.next = q.counts + JQ_PMAX;
+    q.ticket = reinterpret_cast<unsigned*>(q.next + JQ_PMAX);
     return q;
 }
 
@@ -992,7 +1046,7 @@ olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t
     // the sample may still turn an automatically partitioned probe direct
     const bool skew_check = parts > 1 && ctx->opts.join_partitions == 0;
     PartArgs q{};
-    unsigned qgrid = 0;
+    PartGrids qg{};
     ProbeCtl* pf = nullptr;
     int64_t* pf_keys = nullptr;
     uint32_t* pf_rowids = nullptr;
@@ -1002,17 +1056,17 @@ olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t
     }
     if (pre || skew_check) pf = reinterpret_cast<ProbeCtl*>(static_cast<unsigned char*>(ctx->aux) + 1024);
     if (pre) {
-        unsigned char* m = static_cast<unsigned char*>(ctx->part) + probe_part_bytes(ctx, n, parts);
+        unsigned char* m = static_cast<unsigned char*>(ctx->part) + probe_part_bytes(n, parts);
         pf_keys = reinterpret_cast<int64_t*>(m);
         pf_rowids = reinterpret_cast<uint32_t*>(m + align256(n * 8));
         if (m + align256(n * 8) + align256(n * 4) > static_cast<unsigned char*>(ctx->part) + ctx->part_bytes)
             return fail(ctx, OLAP_E_INVALID, "probe pre-filter scratch too small");
     }
     if (parts > 1) {
-        qgrid = static_cast<unsigned>(part_grid(ctx->device, ctx->sm_count));
-        if (qgrid == 0) return fail(ctx, OLAP_E_CUDA, "partition kernel occupancy query failed");
-        q = part_args(ctx, d_keys, d_rowids, n, t->n_buckets, parts, qgrid);
-        if (q.pstart + parts + 1 > reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(ctx->part) + ctx->part_bytes))
+        qg = part_grids(ctx->device, ctx->sm_count);
+        if (qg.count == 0) return fail(ctx, OLAP_E_CUDA, "partition kernel occupancy query failed");
+        q = part_args(ctx, d_keys, d_rowids, n, t->n_buckets, parts);
+        if (probe_part_bytes(n, parts) > ctx->part_bytes)
             return fail(ctx, OLAP_E_INVALID, "probe partition scratch too small");
         q.pf = pf;
         q.pf_keys = pf_keys;
@@ -1046,21 +1100,25 @@ olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t
         pl.sample = reinterpret_cast<uint32_t*>(static_cast<unsigned char*>(ctx->aux) + 16384);
         pl.counters = reinterpret_cast<unsigned*>(static_cast<unsigned char*>(ctx->aux) + 1536);
         pl.ctl = pf;
-        join_probe_plan_kernel<<<PLAN_CTAS, PF_TPB, 0, s>>>(pl);
+        join_probe_plan_kernel<<<PLAN_CTAS, PLAN_TPB, 0, s>>>(pl);
     }
     if (pre)
-        join_prefilter_kernel<<<ctx->sm_count * PF_CTAS, PF_TPB, 0, s>>>(d_keys, d_rowids, n, bloom, pf, pf_keys,
-                                                                   pf_rowids);
+        launch_after(join_prefilter_kernel, static_cast<unsigned>(ctx->sm_count * PF_CTAS), PF_TPB, 0, s, true, d_keys,
+                     d_rowids, n, bloom, static_cast<ProbeCtl*>(pf), pf_keys, pf_rowids);
     if (parts > 1) {
-        join_part_count_kernel<<<qgrid, JQ_TPB, 0, s>>>(q);
-        join_part_scatter_kernel<<<qgrid, JQ_TPB, 0, s>>>(q);
+        // (the first kernel of the chain follows whatever the stream holds)
+        launch_after(join_part_count_kernel, qg.count, JQ_TPB, 0, s, pf != nullptr, q);
+        launch_after(part_scatter(parts), qg.scatter, JQ_TPB, 0, s, true, q);
         pa.keys = q.out_keys;
         pa.rowids = q.out_rowids;
     }
+    const bool after = pf || parts > 1;
     if (ctx->opts.join_bucket_loads == OLAP_LOADS_L1)
-        join_probe_kernel<false><<<grid, JP_TPB, JP_SMEM, s>>>(pa, next_row, pf, done);
+        launch_after(join_probe_kernel<false>, static_cast<unsigned>(grid), JP_TPB, JP_SMEM, s, after, pa, next_row,
+                     static_cast<const ProbeCtl*>(pf), done);
     else
-        join_probe_kernel<true><<<grid, JP_TPB, JP_SMEM, s>>>(pa, next_row, pf, done);
+        launch_after(join_probe_kernel<true>, static_cast<unsigned>(grid), JP_TPB, JP_SMEM, s, after, pa, next_row,
+                     static_cast<const ProbeCtl*>(pf), done);
     e = cudaGetLastError();
     // [plan,] [filter,] [count, scatter,] probe
     if (e == cudaSuccess) ctx->launches += (pf ? 1 : 0) + (pre ? 1 : 0) + (parts > 1 ? 2 : 0) + 1;
@@ -1181,11 +1239,11 @@ olap_status olap_join_build(olap_ctx* ctx, const int64_t* keys, const uint32_t* 
         const int64_t* bk = dk;
         const uint32_t* br = dr;
         if (blocks > static_cast<uint64_t>(JS_BINS) && n >= JS_PART_MIN_N) {
-            const unsigned pgrid = static_cast<unsigned>(part_grid(ctx->device, ctx->sm_count));
-            if (pgrid && ensure_part(ctx, probe_part_bytes(ctx, n, JS_PARTS)) == OLAP_OK) {
-                const PartArgs q = part_args(ctx, dk, dr, n, buckets, JS_PARTS, pgrid);
-                join_part_count_kernel<<<pgrid, JQ_TPB, 0, ctx->stream>>>(q);
-                join_part_scatter_kernel<<<pgrid, JQ_TPB, 0, ctx->stream>>>(q);
+            const PartGrids pg = part_grids(ctx->device, ctx->sm_count);
+            if (pg.count && ensure_part(ctx, probe_part_bytes(n, JS_PARTS)) == OLAP_OK) {
+                const PartArgs q = part_args(ctx, dk, dr, n, buckets, JS_PARTS);
+                launch_after(join_part_count_kernel, pg.count, JQ_TPB, 0, ctx->stream, false, q);
+                launch_after(part_scatter(JS_PARTS), pg.scatter, JQ_TPB, 0, ctx->stream, true, q);
                 ctx->launches += 2;
                 bk = q.out_keys;
                 br = q.out_rowids;

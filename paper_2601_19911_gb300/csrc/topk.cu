@@ -47,19 +47,6 @@ __device__ __forceinline__ unsigned long long gtimer() {
     return t;
 }
 
-// Programmatic dependent launch.  Every kernel of a call is launched while
-// the one before it in the stream is still running, and waits here until that
-// one has finished and its writes are visible.  A kernel launched without the
-// attribute passes straight through.
-__device__ __forceinline__ void wait_prior_grid() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-// Lets the next kernel in the stream launch now (it still waits for this one
-// to finish before it reads anything this one or an earlier one writes).
-__device__ __forceinline__ void allow_next_grid() {
-    asm volatile("griddepcontrol.launch_dependents;" :::);
-}
-
 struct Elem {
     uint64_t r;
     uint32_t rid;
