@@ -440,9 +440,9 @@ __global__ void __launch_bounds__(JB_TPB) join_bloom_kernel(const int64_t* keys,
 constexpr int PF_TPB = 256;
 constexpr int PF_SAMPLE = 4096;                // probe keys tested to decide
 constexpr uint64_t PF_MIN_N = 1ull << 20;      // smaller probes skip the pre-probe (automatic mode)
-constexpr int PF_PER = 4;                      // keys per lane per step
+constexpr int PF_PER = 6;                      // keys per lane per step
 constexpr unsigned PF_WCAP = 256;              // rows staged per warp
-constexpr int PF_CTAS = 6;                     // pre-probe CTAs per SM
+constexpr int PF_CTAS = 4;                     // pre-probe CTAs per SM
 
 constexpr int PLAN_SLOTS = 2 * PF_SAMPLE;      // fingerprint set of the sample (32 KB)
 constexpr int PLAN_CTAS = 16;
@@ -456,6 +456,7 @@ struct PlanArgs {
     BloomView bloom;                           // bits NULL: no pre-probe stage
     int pf_mode;                               // 1 automatic, 2 forced (with a filter)
     int skew_check;
+    uint64_t min_rows;                         // with skew_check: fewer rows than this are not worth partitioning
     int partitioned;
     int skew_l1;
     const int64_t* pf_keys;
@@ -481,7 +482,8 @@ struct PlanArgs {
 // few hot buckets, which stay in cache, while the partition passes would
 // cost two more passes over the rows.  Repeats are found in a shared-memory
 // fingerprint set; a fingerprint collision counts as a repeat (about 2^-7
-// of one per sample).  The last CTA zeroes the kept-row count and tells the
+// of one per sample).  It skips them as well when the pre-probe leaves fewer
+// than `min_rows` (2^25 uniform rows against 2^24, a tenth kept: 278 -> 252 us).  The last CTA zeroes the kept-row count and tells the
 // probe kernel where its rows are: the partitioned rows (`partitioned` and
 // not direct, as launched), else the kept rows (pf_keys, pf_rowids) when the
 // pre-probe runs, else the input; a direct probe reads buckets through L1
@@ -547,7 +549,9 @@ __global__ void __launch_bounds__(PLAN_TPB) join_probe_plan_kernel(PlanArgs a) {
         const bool active = a.bloom.bits && (a.pf_mode == 2 || passes * 10u <= static_cast<unsigned>(PF_SAMPLE) * 6u);
         const unsigned reach = active ? passes : static_cast<unsigned>(PF_SAMPLE);
         const unsigned rep = active ? dup_kept : dup_all;
-        const bool direct = a.skew_check && reach >= 64u && rep * 5u >= reach;
+        const bool skewed = a.skew_check && reach >= 64u && rep * 5u >= reach;
+        const bool few = a.skew_check && active && a.n * passes < a.min_rows * PF_SAMPLE;
+        const bool direct = skewed || few;
         ProbeCtl* ctl = a.ctl;
         ctl->active = active ? 1 : 0;
         ctl->direct = direct ? 1 : 0;
@@ -555,7 +559,7 @@ __global__ void __launch_bounds__(PLAN_TPB) join_probe_plan_kernel(PlanArgs a) {
         ctl->redirect = (!a.partitioned || direct) ? 1 : 0;
         ctl->keys = active ? a.pf_keys : a.keys;
         ctl->rowids = active ? a.pf_rowids : a.rowids;
-        ctl->l1 = (direct && a.skew_l1) ? 1 : 0;
+        ctl->l1 = (skewed && a.skew_l1) ? 1 : 0;
         a.counters[0] = 0;
         a.counters[1] = 0;
     }
@@ -564,10 +568,12 @@ __global__ void __launch_bounds__(PLAN_TPB) join_probe_plan_kernel(PlanArgs a) {
 // The pre-probe: one streaming pass over the probe rows that keeps the rows
 // whose key may be in the table (and every row with the empty-marker key),
 // appended with their row-ids through a per-warp stage, one atomic per flush.
-// Bound by the latency of the keys and of the random filter-block reads from
-// L2, so as many warps as fit: six CTAs per SM for four, 2^25 Zipf rows against
-// a 2^24-row table, a tenth kept, 249 -> 227 us for the whole probe.  (Loading
-// the next keys ahead costs the registers that hold the filter blocks: 268.)
+// Bound by the random filter-block reads from L2 (2.4*10^11 a second), the
+// more of which a lane has in flight the better: six keys a lane and four CTAs
+// per SM (eight keys, or five CTAs of five: the same; six of four: 3-5 %
+// slower).  The kept rows' row-ids are all loaded before the first is staged.
+// Whole probes against a 2^24-row table, a tenth kept: 2^25 Zipf rows with
+// row-ids 236 -> 208 us, uniform 296 -> 248 (without partition passes after it).
 __global__ void __launch_bounds__(PF_TPB, PF_CTAS) join_prefilter_kernel(const int64_t* keys, const uint32_t* rowids,
                                                                 uint64_t n, BloomView bloom, ProbeCtl* ctl,
                                                                 int64_t* out_keys, uint32_t* out_rowids) {
@@ -597,29 +603,38 @@ __global__ void __launch_bounds__(PF_TPB, PF_CTAS) join_prefilter_kernel(const i
     const uint64_t nw = static_cast<uint64_t>(gridDim.x) * (PF_TPB / 32);
     for (uint64_t g = static_cast<uint64_t>(blockIdx.x) * (PF_TPB / 32) + warp; g < groups; g += nw) {
         uint64_t key[PF_PER];
-        bool keep[PF_PER];
+        const uint64_t i0 = g * G + lane;
+        const unsigned len = static_cast<unsigned>(min(G, n - g * G));
+        const int64_t* kp = keys + i0;
+        if (len == G) {
+#pragma unroll
+            for (int j = 0; j < PF_PER; ++j) key[j] = ld_stream_u64(kp + j * 32);
+        } else {
+#pragma unroll
+            for (int j = 0; j < PF_PER; ++j) key[j] = j * 32 + lane < len ? ld_stream_u64(kp + j * 32) : 0ull;
+        }
+        unsigned kept[PF_PER];                 // the warp's rows kept of step j
 #pragma unroll
         for (int j = 0; j < PF_PER; ++j) {
-            const uint64_t i = g * G + static_cast<uint64_t>(j) * 32 + lane;
-            key[j] = i < n ? ld_stream_u64(keys + i) : 0ull;
+            const bool maybe = bloom_maybe(bloom, key[j]) || key[j] == JN_EMPTY;
+            kept[j] = __ballot_sync(0xFFFFFFFFu, maybe && j * 32 + lane < len);
+        }
+        uint32_t rid[PF_PER];                  // all of the kept rows' row-ids in flight before the first is staged
+#pragma unroll
+        for (int j = 0; j < PF_PER; ++j) {
+            rid[j] = static_cast<uint32_t>(i0 + j * 32);
+            if (rowids && ((kept[j] >> lane) & 1u)) rid[j] = ld_stream_u32(rowids + i0 + j * 32);
         }
 #pragma unroll
         for (int j = 0; j < PF_PER; ++j) {
-            const uint64_t i = g * G + static_cast<uint64_t>(j) * 32 + lane;
-            const bool maybe = bloom_maybe(bloom, key[j]);
-            keep[j] = i < n && (key[j] == JN_EMPTY || maybe);
-        }
-#pragma unroll
-        for (int j = 0; j < PF_PER; ++j) {
-            const uint64_t i = g * G + static_cast<uint64_t>(j) * 32 + lane;
-            const unsigned b = __ballot_sync(0xFFFFFFFFu, keep[j]);
+            if (kept[j] == 0) continue;
             if (cnt + 32 > PF_WCAP) flush();
-            if (keep[j]) {
-                const unsigned pos = cnt + __popc(b & ((1u << lane) - 1u));
+            if ((kept[j] >> lane) & 1u) {
+                const unsigned pos = cnt + __popc(kept[j] & ((1u << lane) - 1u));
                 wk[pos] = static_cast<int64_t>(key[j]);
-                wr[pos] = rowids ? ld_stream_u32(rowids + i) : static_cast<uint32_t>(i);
+                wr[pos] = rid[j];
             }
-            cnt += __popc(b);
+            cnt += __popc(kept[j]);
         }
     }
     flush();
@@ -930,6 +945,10 @@ PartGrids part_grids(int device, int sms) {
 
 }  // namespace
 
+// Rows from which on the partition passes may pay: a quarter of the table's
+// buckets (the plan kernel tests the rows its pre-probe leaves against it).
+static uint64_t part_min_rows(const olap_join_table* t) { return t->n_buckets / 4; }
+
 // Partitions the probe of `n` rows against `t` uses (1 = direct probe).
 int probe_parts(const olap_ctx* ctx, const olap_join_table* t, uint64_t n) {
     const int opt = ctx->opts.join_partitions;
@@ -939,9 +958,8 @@ int probe_parts(const olap_ctx* ctx, const olap_join_table* t, uint64_t n) {
     } else if (opt == 0) {
         const uint64_t tb = t->n_buckets * 32;
         const uint64_t l2 = ctx->l2_bytes ? ctx->l2_bytes : (64ull << 20);
-        // worth it when the table is well above L2 and the probe side reads
-        // at least a quarter as many buckets as the table has
-        if (tb > l2 / 2 && n >= t->n_buckets / 4) parts = next_pow2((tb + l2 / 4 - 1) / (l2 / 4));
+        // worth it when the table is well above L2 and there are rows enough
+        if (tb > l2 / 2 && n >= part_min_rows(t)) parts = next_pow2((tb + l2 / 4 - 1) / (l2 / 4));
     }
     parts = std::min<uint64_t>(parts, static_cast<uint64_t>(JQ_PMAX));
     parts = std::min<uint64_t>(parts, t->n_buckets);
@@ -1093,6 +1111,7 @@ olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t
         pl.bloom = bloom;
         pl.pf_mode = pf_mode;
         pl.skew_check = skew_check ? 1 : 0;
+        pl.min_rows = part_min_rows(t);
         pl.partitioned = parts > 1 ? 1 : 0;
         pl.skew_l1 = skew_l1;
         pl.pf_keys = pf_keys;

@@ -111,12 +111,18 @@ __device__ __forceinline__ bool bloom_maybe(const BloomView& f, uint64_t key) {
     const ulonglong2* p = reinterpret_cast<const ulonglong2*>(f.bits + bloom_block(f, h) * BLOOM_WORDS);
     uint64_t v[4];
     asm("ld.global.cg.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p));
+    // bit s of word w, for all words at once: every word rotated by its five
+    // bits (the shift itself drops the higher ones), the low bits combined
     const uint64_t g = bloom_bits(h);
-    uint32_t missing = 0;
+    const uint32_t lo = static_cast<uint32_t>(g), hi = static_cast<uint32_t>(g >> 32);
+    uint32_t all = 1u;
 #pragma unroll
-    for (int w = 0; w < BLOOM_WORDS; ++w)
-        missing |= bloom_bit(g, w) & ~static_cast<uint32_t>(v[w / 2] >> (32 * (w & 1)));
-    return missing == 0;
+    for (int w = 0; w < BLOOM_WORDS; ++w) {
+        const uint32_t x = static_cast<uint32_t>(v[w / 2] >> (32 * (w & 1)));
+        const uint32_t at = 5 * w < 28 ? lo >> (5 * w) : 5 * w < 32 ? __funnelshift_r(lo, hi, 5 * w) : hi >> (5 * w - 32);
+        all &= __funnelshift_r(x, x, at);
+    }
+    return all != 0;
 }
 
 // Device-side plan of one probe, written by its sampling stage: whether the

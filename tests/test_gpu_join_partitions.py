@@ -59,3 +59,24 @@ def test_one_partition(ctxs, parts):
             got = c.join_probe(t, torch.from_numpy(keys).cuda(), out=out)
             np.testing.assert_array_equal(packed(got.cpu().numpy().view(np.uint32)), oracle.join(bk, keys))
     t.free()
+
+
+@pytest.mark.parametrize("hit", [0.02, 0.5])
+def test_pre_probe_leaves_few_rows(hit):
+    """Rows enough to partition, but the pre-probe leaves fewer (0.02) or still
+    enough of them (0.5; a quarter of 2^23 buckets is 2.1 * 10^6 rows)."""
+    c = olap.Context(0)
+    b = datagen.join_build(1 << 22, "unique", seed=8)
+    t = c.join_build(torch.from_numpy(b.keys).cuda())
+    n = 5_000_011
+    assert c.join_probe_partitions(t, n) > 1
+    p = datagen.join_probe(n, b, hit, "uniform", seed=8)
+    want = oracle.join(b.keys, p.keys)
+    out = torch.empty((want.shape[0], 2), dtype=torch.int32, device="cuda")
+    for _ in range(2):
+        got = c.join_probe(t, torch.from_numpy(p.keys).cuda(), out=out)
+        info = c.join_probe_info()
+        assert info["prefiltered"] and (info["parts"] == 1) == (hit < 0.1)
+        np.testing.assert_array_equal(packed(got.cpu().numpy().view(np.uint32)), want)
+    t.free()
+    c.close()
