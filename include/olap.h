@@ -103,9 +103,10 @@ typedef struct {
     int topk_digit_bits;        /* radix digit width of the Top-K selects (8..12; 0 => 12), also
                                    for batches created on this context */
     int host_access;            /* olap_host_access: how pageable host memory is copied */
-    int batch_overlap;          /* batches: 0 => the Top-K and probe kernels run one after the
-                                   other, 1 => side by side (two branches of the graph); each
-                                   already fills the GPU, and side by side measured no faster */
+    int batch_overlap;          /* batches: 0 => the probe kernel runs behind the Top-K kernel,
+                                   taking over its CTAs' places as they leave, 1 => side by
+                                   side (two branches of the graph), which is slower: each
+                                   already fills the GPU */
     int batch_topk_ctas_per_sm; /* batches: resident Top-K CTAs per SM (1 or 2; 0 => 2) */
     int join_prefilter;         /* olap_prefilter: Bloom pre-probe of the join (Sec. III-B) */
     int staging_threads;        /* host threads that copy pageable data into and out of the

@@ -60,6 +60,24 @@ __device__ __forceinline__ void allow_next_grid() {
     asm volatile("griddepcontrol.launch_dependents;" :::);
 }
 
+// A launch in a chain of kernels; `after`: with programmatic stream
+// serialisation behind the kernel before it.  Errors are left to
+// cudaGetLastError.
+template <typename... P>
+inline void launch_after(void (*fn)(P...), unsigned grid, int block, size_t smem, cudaStream_t s, bool after, P... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(static_cast<unsigned>(block));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = after ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, fn, args...);
+}
+
 // A 32-byte store (of the vector ld_stream_words loads); p 32-byte aligned.
 __device__ __forceinline__ void st_words(void* p, const uint32_t (&w)[8]) {
     asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p),

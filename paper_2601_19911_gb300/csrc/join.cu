@@ -846,25 +846,6 @@ void (*part_scatter(int parts))(PartArgs) {
     return parts <= 32 ? join_part_scatter_kernel<1> : parts <= 64 ? join_part_scatter_kernel<2> : join_part_scatter_kernel<8>;
 }
 
-// A launch of the probe's chain; `after`: with programmatic stream
-// serialisation, behind a kernel of the same chain (it waits for the whole of
-// that kernel in wait_prior_grid, and only its launch overlaps).  Errors are
-// left to cudaGetLastError.
-template <typename... P>
-void launch_after(void (*fn)(P...), unsigned grid, int block, size_t smem, cudaStream_t s, bool after, P... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(static_cast<unsigned>(block));
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = after ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, fn, args...);
-}
-
 uint64_t next_pow2(uint64_t x) {
     uint64_t p = 1;
     while (p < x) p <<= 1;
