@@ -600,6 +600,20 @@ olap_status olap_topk_rows(olap_ctx* ctx, const void* rows, olap_mem in_where, u
     return OLAP_OK;
 }
 
+// The device's address of `bytes` of page-locked host memory, NULL unless all
+// of them are mapped.
+static void* mapped_host(const void* host, size_t bytes) {
+    void *first = nullptr, *last = nullptr;
+    unsigned char* h = static_cast<unsigned char*>(const_cast<void*>(host));
+    if (cudaHostGetDevicePointer(&first, h, 0) != cudaSuccess ||
+        cudaHostGetDevicePointer(&last, h + bytes - 1, 0) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return static_cast<unsigned char*>(last) - static_cast<unsigned char*>(first) == static_cast<ptrdiff_t>(bytes - 1)
+               ? first : nullptr;
+}
+
 // On the sampled path only the candidates' row-ids are ever read (as the
 // filter stages them), so row-ids in page-locked host memory can stay there:
 // the kernels read those few in place over the host link (NVLink-C2C), and
@@ -608,11 +622,8 @@ olap_status olap_topk_rows(olap_ctx* ctx, const void* rows, olap_mem in_where, u
 static bool rowids_in_host(const uint32_t* rowids, olap_mem where, uint64_t n, uint64_t kk, const uint32_t** dr) {
     if (!rowids || where != OLAP_MEM_HOST_PINNED || topk_plan(n, kk).use_sample != TK_SAMPLE_FILTER)
         return false;
-    void* mapped = nullptr;
-    if (cudaHostGetDevicePointer(&mapped, const_cast<uint32_t*>(rowids), 0) != cudaSuccess || !mapped) {
-        cudaGetLastError();
-        return false;
-    }
+    void* mapped = mapped_host(rowids, n * 4);
+    if (!mapped) return false;
     *dr = static_cast<const uint32_t*>(mapped);
     return true;
 }
@@ -629,12 +640,7 @@ static const void* keys_in_host(const olap_ctx* ctx, const void* keys, size_t wi
     if (where == OLAP_MEM_HOST && ctx->host_direct) {
         mapped = keys;
     } else if (where == OLAP_MEM_HOST_PINNED) {
-        void* p = nullptr;
-        if (cudaHostGetDevicePointer(&p, const_cast<void*>(keys), 0) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        mapped = p;
+        mapped = mapped_host(keys, n * width);
     }
     const uintptr_t at = reinterpret_cast<uintptr_t>(mapped);
     return (at & 31) + n * width <= ((n * width + 255) & ~static_cast<size_t>(255)) ? mapped : nullptr;
@@ -651,13 +657,7 @@ constexpr uint64_t RESULTS_IN_PLACE = 4096;
 static void* results_in_place(const olap_ctx* ctx, void* host, olap_mem where, uint64_t kk, size_t width) {
     if (kk > RESULTS_IN_PLACE || reinterpret_cast<uintptr_t>(host) % width) return nullptr;
     if (where == OLAP_MEM_HOST) return ctx->host_direct ? host : nullptr;
-    if (where != OLAP_MEM_HOST_PINNED) return nullptr;
-    void* mapped = nullptr;
-    if (cudaHostGetDevicePointer(&mapped, host, 0) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    return mapped;
+    return where == OLAP_MEM_HOST_PINNED ? mapped_host(host, kk * width) : nullptr;
 }
 
 olap_status olap_topk(olap_ctx* ctx, const void* keys, olap_key_type type, const uint32_t* rowids,
