@@ -2,6 +2,7 @@
 no trace in a table's contents, the amount kept is bounded, contexts with a
 budget take no part, threads share it safely, and it is given back with the
 last context."""
+import gc
 import threading
 
 import numpy as np
@@ -29,9 +30,11 @@ def _free_bytes():
 
 
 def test_reuse_bounds_and_return():
-    torch.zeros(1, device="cuda")
+    gc.collect()
+    torch.cuda.empty_cache()                   # what other tests left cached is not counted
     with olap.Context(0) as warm:
         _join(warm, 1000, 1)
+    torch.cuda.empty_cache()
     before = _free_bytes()
     with olap.Context(0) as ctx:
         for i, n in enumerate((200_000, 190_000, 1000, 200_000, 150_000, 300_000)):     # larger, smaller, reused
