@@ -1346,18 +1346,19 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
             }
             __syncthreads();
             // sorted by the grid: every warp ranks some (in one CTA a bitonic
-            // sort of 2047 takes 50 us), then every CTA reads them in order
+            // sort of 2047 takes 50 us), in out_r1, which is free until the entries
+            // are scattered; every CTA has read them in order before that
             for (int e = gw; e < TK_SPLITTERS; e += nwarps) {
                 const unsigned c = warp_rank_of(pr_r, pr_rid, 0, TK_SPLITTERS, e);
                 if (lane == 0) {
-                    a.split_r[c] = pr_r[e];
-                    a.split_rid[c] = pr_rid[e];
+                    a.out_r1[c] = pr_r[e];
+                    a.out_rid1[c] = pr_rid[e];
                 }
             }
             if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
             for (int j = threadIdx.x; j < TK_SPLITTERS; j += TK_TPB) {
-                pr_r[j] = __ldcg(a.split_r + j);
-                pr_rid[j] = __ldcg(a.split_rid + j);
+                pr_r[j] = __ldcg(a.out_r1 + j);
+                pr_rid[j] = __ldcg(a.out_rid1 + j);
             }
             __syncthreads();
             auto gap = [&](uint64_t r, uint32_t rid) {       // 2 * splitters below, + 1 when equal to the next
@@ -1660,7 +1661,7 @@ size_t topk_scratch_bytes(const TopkPlan& p, uint64_t k) {
     b += up256(TK_SMALL * 8) + up256(TK_SMALL * 4);
     const uint64_t kk = std::max<uint64_t>(k, 1);
     b += up256(kk * 8) + up256(kk * 4);
-    if (k > TK_SMALL) b += up256(kk * 8) + up256(kk * 4) + up256(TK_SPLITTERS * 8) + up256(TK_SPLITTERS * 4);
+    if (k > TK_SMALL) b += up256(kk * 8) + up256(kk * 4);
     return b;
 }
 
@@ -1687,11 +1688,9 @@ void topk_carve(TopkArgs& a, const TopkPlan& p, void* base) {
     if (a.k > TK_SMALL) {
         a.out_r1 = static_cast<uint64_t*>(take(kk * 8));
         a.out_rid1 = static_cast<uint32_t*>(take(kk * 4));
-        a.split_r = static_cast<uint64_t*>(take(TK_SPLITTERS * 8));
-        a.split_rid = static_cast<uint32_t*>(take(TK_SPLITTERS * 4));
     } else {
-        a.out_r1 = a.split_r = nullptr;
-        a.out_rid1 = a.split_rid = nullptr;
+        a.out_r1 = nullptr;
+        a.out_rid1 = nullptr;
     }
     a.samples = p.use_sample ? static_cast<uint64_t*>(take(TK_SAMPLE * 8)) : nullptr;
     a.local = p.local;

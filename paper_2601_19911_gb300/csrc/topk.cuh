@@ -38,6 +38,7 @@ constexpr int TKL_SMEM_MAX = TK_BINS * 4 + static_cast<int>(TK_LOCAL_N) * 12;
 enum { TK_SAMPLE_NONE = 0, TK_SAMPLE_FILTER = 1, TK_SAMPLE_INLINE = 2 };
 constexpr int TK_RANK_MAX = 8192;         // survivors ranked in shared memory by the whole grid
 constexpr int TK_SPLITTERS = 2047;        // splitters of the larger-K finish on tied keys (2^k - 1)
+static_assert(TK_SPLITTERS <= TK_SMALL, "the splitters fit where K > TK_SMALL entries do");
 constexpr uint64_t TK_SPLIT_MAX = 2048ull * 512;   // entries they may split (about 512 per gap)
 constexpr int TK_SORT_SMEM = TK_RANK_MAX * 12;  // select kernel shared bytes (ranking / sort tile / histogram)
 constexpr int TK_MAX_STAGES = 16;         // full + empty mbarrier pairs reserved after the ring
@@ -52,8 +53,8 @@ constexpr int TK_TILE_DEFAULT = 16384;
 constexpr int TK_STAGES_DEFAULT = 3;
 constexpr int TK_CTAS_PER_SM_DEFAULT = 4;
 
-// Filter flavours: 16-byte register loads, or bulk copies through a ring of
-// shared-memory stages (the default).
+// Filter flavours: 32-byte register loads (the default), or bulk copies through
+// a ring of shared-memory stages.
 enum TopkFilter { TK_FILTER_REGS = 0, TK_FILTER_BULK = 1 };
 
 // Device control block, zeroed by CTA 0 at the start of every launch.
@@ -109,8 +110,6 @@ struct TopkArgs {
     uint32_t* out_rid0;
     uint64_t* out_r1;                // k entries, merge ping-pong (k > TK_SMALL)
     uint32_t* out_rid1;
-    uint64_t* split_r;               // TK_SPLITTERS sorted splitters (k > TK_SMALL)
-    uint32_t* split_rid;
     uint64_t* samples;               // TK_SAMPLE rank words of the sample (sampled path)
     void* out_keys;                  // caller's outputs (device)
     uint32_t* out_rowids;
