@@ -145,7 +145,7 @@ typedef enum {
     OLAP_LOADS_L2_ONLY = 2      /* bypass L1 (ld.global.cg): no L1 line fills for 32-byte reads */
 } olap_loads;
 
-/* Streaming-pass flavour of Top-K: 16-byte register loads (the default), or
+/* Streaming-pass flavour of Top-K: 32-byte register loads (the default), or
  * bulk asynchronous copies (TMA engine) through a ring of shared-memory
  * stages. */
 typedef enum { OLAP_FILTER_AUTO = 0, OLAP_FILTER_BULK = 1, OLAP_FILTER_REGS = 2 } olap_filter;
@@ -194,7 +194,11 @@ olap_status olap_selftest_wait(olap_ctx* ctx, uint64_t limit_cycles, int32_t* ou
  * With row-ids in page-locked host memory and the sampled path (n > 2^21,
  * k <= n / 256), the row-ids are not copied: the kernels read the
  * candidates' row-ids in place over the host link (olap_topk_info_last
- * reports it); the keys are copied as usual.
+ * reports it).  On that path, with register loads, keys in host memory that
+ * the device can access are read over the link by the streaming pass itself,
+ * which leaves their copy on the device; otherwise they are copied first.
+ * Results of up to 4096 rows are written to host memory by the kernels where
+ * the device can access it.
  * The result is bit-exact: it equals a stable sort by (key, row-id) cut at k.
  * ------------------------------------------------------------------------ */
 olap_status olap_topk(olap_ctx* ctx, const void* keys, olap_key_type type, const uint32_t* rowids,
@@ -229,9 +233,9 @@ olap_status olap_topk_async(olap_ctx* ctx, const void* d_keys, olap_key_type typ
                             void* stream);
 
 /* What the last Top-K on this context did (diagnostics; blocks until the
- * context's stream is idle).  path: 0 = radix refine over the input (small n
- * or large k), 1 = sampled threshold + one streaming pass + refine over the
- * candidates, 2 = sample misjudged, refine over the input.  phase_ns:
+ * context's stream is idle).  path: 0 = no sample (small n, ranked or refined
+ * over the input; or large k), 1 = sampled threshold + one streaming pass +
+ * refine over the candidates, 2 = sample misjudged, refine over the input.  phase_ns:
  * sample, filter, refine, split, finish/sort, total, and within finish the
  * small-bucket sort and the survivor sort (device %globaltimer).
  * rowids_in_place: 1 when the call (a blocking olap_topk or olap_topk_pair
@@ -339,14 +343,17 @@ olap_status olap_topk_rows(olap_ctx* ctx, const void* rows, olap_mem in_where, u
  *
  * The table is an open-addressing table of 16-byte slots {int64 key, uint32
  * row-id, uint32 count of further copies of the key along its chain}, two
- * slots per 32-byte bucket, with linear probing over buckets (a bucket with a
- * free slot ends every chain; a probe also stops at its key's last copy).
+ * slots per 32-byte bucket, with linear probing over buckets, wrapping inside
+ * blocks of 1024 buckets (over the whole table when a block would overflow); a
+ * bucket with a free slot ends every chain, and a probe also stops at its
+ * key's last copy.
  * Capacity is the power of two of buckets that keeps n / (2 * buckets) at or
  * below the load factor.  Build rows whose key equals the table's empty
  * marker (all bits set, i.e. -1) are kept in a side list, so every int64 key
  * value joins correctly.  A table far above L2 also carries a blocked Bloom
  * filter for the pre-probe (see olap_prefilter).  The table stays resident on
- * the device until olap_join_free; it may be probed any number of times, from
+ * the device until olap_join_free (which may keep the memory for later
+ * builds, at most 2 GiB per device); it may be probed any number of times, from
  * any context on the same device.
  *
  * Result: every (probe row-id, build row-id) pair whose keys are equal, as a
@@ -391,7 +398,8 @@ olap_status olap_join_probe_async(olap_ctx* ctx, const olap_join_table* table, c
  * when they repeat (a skewed stream: at least a fifth of the sampled keys
  * that reach the probe equal an earlier one), the partition kernels return at
  * once and the probe reads its rows directly, its bucket reads through L1
- * unless join_bucket_loads says otherwise; olap_join_probe_info_last reports
+ * unless join_bucket_loads says otherwise; likewise (through L2) when the
+ * pre-probe leaves fewer rows than a quarter of the table's buckets; olap_join_probe_info_last reports
  * what ran.  Host arithmetic only; OLAP_E_INVALID for a NULL or freed table
  * or a NULL *parts. */
 olap_status olap_join_probe_partitions(olap_ctx* ctx, const olap_join_table* table, uint64_t n, int* parts);
