@@ -21,7 +21,8 @@
 //     BP_CHUNK probe rows of an item, handed to the CTA's warps by a row
 //     queue in shared memory; a large item is many chunks taken by many
 //     CTAs, all appending to the item's own count word, which a reset kernel
-//     zeroes before the probe queue starts.
+//     zeroes first.  The probe kernel launches behind the Top-K kernel and
+//     takes the places of its CTAs as they leave.
 // Descriptors are checked on the device; a bad one gets OLAP_E_DEVICE in its
 // status word and is skipped.
 #include <algorithm>

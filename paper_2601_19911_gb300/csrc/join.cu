@@ -30,9 +30,9 @@
 // larger than L2 turns every probe into a random DRAM sector read, and those
 // run at a small fraction of the streaming rate.  Instead the probe rows are
 // first radix-partitioned by the top bits of their home bucket into P
-// partitions (a counting pass and a scatter pass, both streaming, with the
-// same CTA-to-tile assignment so every CTA's output ranges come from the
-// count matrix without global atomics).  The probe then takes the reordered
+// partitions (a counting pass and a scatter pass, both streaming; the scatter
+// appends a tile's rows of a partition as one run at the partition's cursor).
+// The probe then takes the reordered
 // rows chunk by chunk in partition order, so the whole grid works on one
 // 1/P slice of the table at a time, sized to stay resident in L2: the table
 // is read from DRAM about once.

@@ -26,9 +26,12 @@
 //      bin that holds the K-th entry has at most 4096 entries.
 //   3. Split: entries below the interval are selected; entries in it go to a
 //      small buffer that is ranked to take the remaining count.
-//   4. Sort the K survivors by (rank word, row-id) -- in shared memory when
-//      K <= 4096, else tile sorts plus merge-path rounds across the grid --
+//   4. Put the K survivors in (rank word, row-id) order -- by counting smaller
+//      entries when K <= 4096; else spread over 4096 equal bins of their
+//      interval (or between 2047 sorted splitters when those crowd) and ranked
+//      within their bin; tile sorts plus merge-path rounds when both fail --
 //      and write keys (original bits, by the inverse transform) and row-ids.
+// A column in host memory is read by the pass itself (topk_filter_host_kernel).
 #include <algorithm>
 #include <atomic>
 #include <cmath>
