@@ -66,10 +66,13 @@ struct olap_ctx {
     void* rows_buf = nullptr;
     size_t rows_buf_bytes = 0;
 
-    // Partitioned-probe scratch (grow-only): partitioned keys, row-ids and
-    // the per-CTA partition counts.
+    // Partitioned-probe scratch (grow-only): partitioned keys and row-ids.
     void* part = nullptr;
     size_t part_bytes = 0;
+    // The same for a large build, which must neither move the probes' scratch
+    // (captured probes hold its address) nor write into a queued probe's rows.
+    void* build_part = nullptr;
+    size_t build_part_bytes = 0;
     uint64_t l2_bytes = 0;            // device L2 size
     bool host_direct = false;         // copy pageable host memory with a kernel (no CPU staging)
 
@@ -102,6 +105,7 @@ olap_status ensure_dev_in(olap_ctx* ctx, size_t bytes);
 olap_status ensure_dev_out(olap_ctx* ctx, size_t bytes);
 olap_status ensure_pinned(olap_ctx* ctx);
 olap_status ensure_part(olap_ctx* ctx, size_t bytes);
+olap_status ensure_build_part(olap_ctx* ctx, size_t bytes);
 
 // Device memory of freed join tables, kept for the next table of about the
 // same size: a table's cudaMalloc and cudaFree take 370 us at 134 MB, twice

@@ -979,11 +979,13 @@ size_t probe_scratch_bytes(const olap_ctx* ctx, const olap_join_table* t, uint64
     return pb + align256(n * 8) + align256(n * 4);
 }
 
-// The partition passes over n rows by the top bits of their home bucket, in
-// the context's partition scratch (which holds probe_part_bytes).
-static PartArgs part_args(const olap_ctx* ctx, const int64_t* keys, const uint32_t* rowids, uint64_t n,
+// The partition passes over n rows by the top bits of their home bucket, into
+// `rows` (probe_part_bytes), with PART_COUNT_BYTES at `counts`, zero before the
+// first call.
+constexpr size_t PART_COUNT_BYTES = 2 * JQ_PMAX * 8 + 256;
+static PartArgs part_args(void* rows, void* counts, const int64_t* keys, const uint32_t* rowids, uint64_t n,
                           uint64_t n_buckets, int parts) {
-    unsigned char* m = static_cast<unsigned char*>(ctx->part);
+    unsigned char* m = static_cast<unsigned char*>(rows);
     PartArgs q{};
     q.keys = keys;
     q.rowids = rowids;
@@ -994,8 +996,7 @@ static PartArgs part_args(const olap_ctx* ctx, const int64_t* keys, const uint32
     q.parts = parts;
     q.out_keys = reinterpret_cast<int64_t*>(m);
     q.out_rowids = reinterpret_cast<uint32_t*>(m + align256(n * 8));
-    unsigned char* aux = static_cast<unsigned char*>(ctx->aux) + 4096;
-    q.counts = reinterpret_cast<unsigned long long*>(aux);
+    q.counts = static_cast<unsigned long long*>(counts);
     q.next = q.counts + JQ_PMAX;
     q.ticket = reinterpret_cast<unsigned*>(q.next + JQ_PMAX);
     return q;
@@ -1064,7 +1065,7 @@ olap_status probe_enqueue(olap_ctx* ctx, const olap_join_table* t, const int64_t
     if (parts > 1) {
         qg = part_grids(ctx->device, ctx->sm_count);
         if (qg.count == 0) return fail(ctx, OLAP_E_CUDA, "partition kernel occupancy query failed");
-        q = part_args(ctx, d_keys, d_rowids, n, t->n_buckets, parts);
+        q = part_args(ctx->part, static_cast<unsigned char*>(ctx->aux) + 4096, d_keys, d_rowids, n, t->n_buckets, parts);
         if (probe_part_bytes(n, parts) > ctx->part_bytes)
             return fail(ctx, OLAP_E_INVALID, "probe partition scratch too small");
         q.pf = pf;
@@ -1240,8 +1241,12 @@ olap_status olap_join_build(olap_ctx* ctx, const int64_t* keys, const uint32_t* 
         const uint32_t* br = dr;
         if (blocks > static_cast<uint64_t>(JS_BINS) && n >= JS_PART_MIN_N) {
             const PartGrids pg = part_grids(ctx->device, ctx->sm_count);
-            if (pg.count && ensure_part(ctx, probe_part_bytes(n, JS_PARTS)) == OLAP_OK) {
-                const PartArgs q = part_args(ctx, dk, dr, n, buckets, JS_PARTS);
+            const size_t pb = probe_part_bytes(n, JS_PARTS);
+            if (pg.count && ensure_build_part(ctx, pb + PART_COUNT_BYTES) == OLAP_OK) {
+                void* counts = static_cast<unsigned char*>(ctx->build_part) + pb;
+                e = cudaMemsetAsync(counts, 0, PART_COUNT_BYTES, ctx->stream);
+                if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "partition counts"));
+                const PartArgs q = part_args(ctx->build_part, counts, dk, dr, n, buckets, JS_PARTS);
                 launch_after(join_part_count_kernel, pg.count, JQ_TPB, 0, ctx->stream, false, q);
                 launch_after(part_scatter(JS_PARTS), pg.scatter, JQ_TPB, 0, ctx->stream, true, q);
                 ctx->launches += 2;

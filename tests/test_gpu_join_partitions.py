@@ -80,3 +80,30 @@ def test_pre_probe_leaves_few_rows(hit):
         np.testing.assert_array_equal(packed(got.cpu().numpy().view(np.uint32)), want)
     t.free()
     c.close()
+
+
+def test_large_build_between_replays_of_a_captured_probe(ctxs):
+    """A large build orders its rows in scratch of its own: the scratch that a
+    captured probe uses neither moves nor changes."""
+    c = ctxs[32]
+    b = datagen.join_build(20_000, "unique", seed=4)
+    t = c.join_build(torch.from_numpy(b.keys).cuda())
+    p = datagen.join_probe(100_003, b, 0.5, "uniform", seed=4)
+    want = oracle.join(b.keys, p.keys)
+    dk = torch.from_numpy(p.keys).cuda()
+    out = torch.empty((want.shape[0], 2), dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int64, device="cuda")
+    c.join_probe_async(t, dk, out, want.shape[0], cnt)
+    c.sync()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        c.join_probe_async(t, dk, out, want.shape[0], cnt, stream=torch.cuda.current_stream().cuda_stream)
+    keys = torch.randint(-(1 << 62), 1 << 62, ((1 << 23) + 11,), device="cuda")
+    for _ in range(2):
+        c.join_build(keys).free()
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert int(cnt.item()) == want.shape[0]
+        np.testing.assert_array_equal(packed(out.cpu().numpy().view(np.uint32)), want)
+    t.free()
