@@ -199,6 +199,8 @@ olap_status olap_selftest_wait(olap_ctx* ctx, uint64_t limit_cycles, int32_t* ou
  * which leaves their copy on the device; otherwise they are copied first.
  * Results of up to 4096 rows are written to host memory by the kernels where
  * the device can access it.
+ * Outputs may lie over the call's own keys and row-ids (each output apart from
+ * the others): results are written after the last read of the input.
  * The result is bit-exact: it equals a stable sort by (key, row-id) cut at k.
  * ------------------------------------------------------------------------ */
 olap_status olap_topk(olap_ctx* ctx, const void* keys, olap_key_type type, const uint32_t* rowids,

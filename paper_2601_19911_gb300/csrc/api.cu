@@ -346,15 +346,6 @@ static olap_status topk_enqueue(olap_ctx* ctx, const void* d_keys, olap_key_type
                                 void* d_out_keys, uint32_t* d_out_rowids, int32_t* dev_status,
                                 cudaStream_t stream, TopkCtl** ctl_out, const PairSpec* pair = nullptr,
                                 const void* host_keys = nullptr) {
-    const TopkPlan plan = topk_plan(n, kk);
-    const bool reset = ctx->barrier_dirty || ctx->scratch_bytes < topk_scratch_bytes(plan, kk);
-    olap_status st = ensure_scratch(ctx, topk_scratch_bytes(plan, kk));
-    if (st != OLAP_OK) return st;
-    if (reset && stream != ctx->stream) {
-        // The barrier reset ran on the context stream; order the launch after it.
-        cudaError_t e = cudaStreamSynchronize(ctx->stream);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "barrier reset wait");
-    }
     TopkArgs a{};
     a.keys = d_keys;
     a.host_keys = host_keys;
@@ -364,7 +355,6 @@ static olap_status topk_enqueue(olap_ctx* ctx, const void* d_keys, olap_key_type
     a.kind = type;
     a.w4 = key_bytes(type) == 4;
     a.desc = order == OLAP_DESC;
-    topk_carve(a, plan, ctx->scratch);
     a.out_keys = d_out_keys;
     a.out_rowids = d_out_rowids;
     a.dev_status = dev_status;
@@ -376,6 +366,16 @@ static olap_status topk_enqueue(olap_ctx* ctx, const void* d_keys, olap_key_type
         a.desc2 = pair->order == OLAP_DESC;
         a.out_keys2 = pair->out_keys;
     }
+    const TopkPlan plan = topk_plan_call(a);
+    const bool reset = ctx->barrier_dirty || ctx->scratch_bytes < topk_scratch_bytes(plan, kk);
+    olap_status st = ensure_scratch(ctx, topk_scratch_bytes(plan, kk));
+    if (st != OLAP_OK) return st;
+    if (reset && stream != ctx->stream) {
+        // The barrier reset ran on the context stream; order the launch after it.
+        cudaError_t e = cudaStreamSynchronize(ctx->stream);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "barrier reset wait");
+    }
+    topk_carve(a, plan, ctx->scratch);
     a.filter = ctx->opts.topk_filter == OLAP_FILTER_BULK ? TK_FILTER_BULK : TK_FILTER_REGS;
     a.digit = ctx->opts.topk_digit_bits ? ctx->opts.topk_digit_bits : TK_DIG;
     ctx->last_topk_ctl = a.ctl;

@@ -102,8 +102,6 @@ extern "C" olap_status olap_topk_noalloc(const void* d_keys, olap_key_type type,
     olap_status st = setup_device(dev, &ds);
     if (st != OLAP_OK) return st;
 
-    const olap::TopkPlan plan = olap::topk_plan(n, kk);
-    if (olap::topk_scratch_bytes(plan, kk) > NOALLOC_BYTES) return OLAP_E_INVALID;
     olap::TopkArgs a{};
     a.keys = d_keys;
     a.rowids = d_rowids;
@@ -112,11 +110,13 @@ extern "C" olap_status olap_topk_noalloc(const void* d_keys, olap_key_type type,
     a.kind = type;
     a.w4 = olap::key_bytes(type) == 4;
     a.desc = order == OLAP_DESC;
-    olap::topk_carve(a, plan, ds.scratch);
-    a.filter = olap::TK_FILTER_REGS;
     a.out_keys = d_out_keys;
     a.out_rowids = d_out_rowids;
     a.dev_status = dev_status;
+    const olap::TopkPlan plan = olap::topk_plan_call(a);
+    if (olap::topk_scratch_bytes(plan, kk) > NOALLOC_BYTES) return OLAP_E_INVALID;
+    olap::topk_carve(a, plan, ds.scratch);
+    a.filter = olap::TK_FILTER_REGS;
     // The grid barrier must start at zero; an earlier call that gave up on a
     // wait may have left it mid-count.
     if (cudaMemsetAsync(a.bar, 0, sizeof(olap::GridBar), s) != cudaSuccess) {

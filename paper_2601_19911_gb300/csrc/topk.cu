@@ -1663,6 +1663,24 @@ TopkPlan topk_plan(uint64_t n, uint64_t k) {
     return p;
 }
 
+TopkPlan topk_plan_call(const TopkArgs& a) {
+    TopkPlan p = topk_plan(a.n, a.k);
+    if (!p.local) return p;
+    const size_t wide = a.pair || a.w4 ? 4 : 8;
+    struct Span {
+        const void* p;
+        size_t bytes;
+    };
+    const Span in[] = {{a.keys, a.n * wide}, {a.keys2, a.n * 4}, {a.rowids, a.n * 4}};
+    const Span out[] = {{a.out_keys, a.k * wide}, {a.out_keys2, a.k * 4}, {a.out_rowids, a.k * 4}, {a.dev_status, 4}};
+    for (const Span& i : in)
+        for (const Span& o : out) {
+            const uintptr_t x = reinterpret_cast<uintptr_t>(i.p), y = reinterpret_cast<uintptr_t>(o.p);
+            if (x && y && x < y + o.bytes && y < x + i.bytes) p.local = 0;
+        }
+    return p;
+}
+
 static size_t up256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
 size_t topk_scratch_bytes(const TopkPlan& p, uint64_t k) {

@@ -132,6 +132,12 @@ struct TopkPlan {
     uint64_t cand_cap;
 };
 TopkPlan topk_plan(uint64_t n, uint64_t k);
+// The plan of a call whose columns, sizes and outputs are in `args`: as above,
+// but not topk_local_kernel when an output lies over an input.  Its CTAs write
+// while others may still load; every other path writes its results behind a
+// grid barrier that follows the last read of the input, so results may take
+// the place of the keys or row-ids they come from.  Needs the same scratch.
+TopkPlan topk_plan_call(const TopkArgs& args);
 
 // Bytes of device scratch a call with this plan needs (all buffers above).
 size_t topk_scratch_bytes(const TopkPlan& p, uint64_t k);
