@@ -834,91 +834,146 @@ __device__ void hist_pass(const TopkArgs& a, bool cand, uint64_t src_n, const Ra
 }
 
 // Split: entries below the interval are selected (appended to out), entries
-// in it go to the small buffer, or straight to out when all of them
-// (or any `krem` identical ones) are taken.
-// With FOLD, the minima and maxima of the entries it writes to out (those
-// below the interval, and with take_all the ones in it that it keeps) are
-// merged into ctl->fin for the larger-K finish, which then needs no pass of
-// its own, and the appends take one atomic per CTA and step (nearly every
-// warp has some: 9,000 atomics on two words for 293,000 candidates).  `nx` is
-// the thread's first candidate on the candidate path; every entry is loaded
-// one step ahead.
-template <bool FOLD>
+// in it go to the small buffer, or to out when all of them (or any `krem`
+// identical ones) are taken.  Every entry is loaded one step ahead; `nx` is
+// the thread's first candidate on the candidate path.
 __device__ void split_pass(const TopkArgs& a, bool cand, uint64_t src_n, const Range& g, bool take_all,
                            uint64_t krem, Elem nx) {
     TopkCtl* ctl = a.ctl;
-    Fold acc = fold_none();
     const uint64_t stride = static_cast<uint64_t>(TK_TPB) * gridDim.x;
     const unsigned lane = threadIdx.x & 31u;
     const uint64_t eq_base = a.k - krem;
-    if (!cand) {
-        const uint64_t i0 = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x;
-        if (i0 < src_n) nx = load_src(a, cand, i0);
-    }
-    __shared__ unsigned s_lt[TK_TPB / 32], s_eq[TK_TPB / 32];
-    __shared__ unsigned long long s_base[2];
-    const unsigned warp = threadIdx.x >> 5;
     unsigned long long* eq_ctr = take_all ? &ctl->eq_count : &ctl->small_count;
-    for (uint64_t cb = static_cast<uint64_t>(blockIdx.x) * TK_TPB; cb < src_n; cb += stride) {
-        const uint64_t i = cb + threadIdx.x;
+    const uint64_t i0 = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x;
+    if (!cand && i0 < src_n) nx = load_src(a, cand, i0);
+    for (uint64_t wb = i0 - lane; wb < src_n; wb += stride) {
+        const uint64_t i = wb + lane;
         int c = 1;
         const Elem e = nx;
         if (i < src_n) c = range_cmp(g, e.r, e.rid);
         if (i + stride < src_n) nx = load_src(a, cand, i + stride);
         const unsigned lt = __ballot_sync(0xFFFFFFFFu, c < 0);
         const unsigned eq = __ballot_sync(0xFFFFFFFFu, c == 0);
-        unsigned long long blt = 0, beq = 0;                 // the warp's first positions
-        if (FOLD) {
-            if (lane == 0) {
-                s_lt[warp] = __popc(lt);
-                s_eq[warp] = __popc(eq);
-            }
-            __syncthreads();
-            unsigned nlt = 0, neq = 0, all_lt = 0, all_eq = 0;
-#pragma unroll
-            for (unsigned w = 0; w < TK_TPB / 32; ++w) {
-                if (w == warp) {
-                    nlt = all_lt;
-                    neq = all_eq;
-                }
-                all_lt += s_lt[w];
-                all_eq += s_eq[w];
-            }
-            if (threadIdx.x == 0 && all_lt) s_base[0] = atomicAdd(&ctl->out_count, static_cast<unsigned long long>(all_lt));
-            if (threadIdx.x == 32 && all_eq) s_base[1] = atomicAdd(eq_ctr, static_cast<unsigned long long>(all_eq));
-            __syncthreads();
-            blt = s_base[0] + nlt;
-            beq = s_base[1] + neq;
-        } else {
-            if (lt) {
-                if (lane == 0) blt = atomicAdd(&ctl->out_count, static_cast<unsigned long long>(__popc(lt)));
-                blt = __shfl_sync(0xFFFFFFFFu, blt, 0);
-            }
-            if (eq) {
-                if (lane == 0) beq = atomicAdd(eq_ctr, static_cast<unsigned long long>(__popc(eq)));
-                beq = __shfl_sync(0xFFFFFFFFu, beq, 0);
+        if (lt) {
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(&ctl->out_count, static_cast<unsigned long long>(__popc(lt)));
+            base = __shfl_sync(0xFFFFFFFFu, base, 0);
+            if (c < 0) {
+                const uint64_t pos = base + __popc(lt & ((1u << lane) - 1u));
+                a.out_r0[pos] = e.r;
+                a.out_rid0[pos] = e.rid;
             }
         }
-        if (c < 0) {
-            const uint64_t pos = blt + __popc(lt & ((1u << lane) - 1u));
-            a.out_r0[pos] = e.r;
-            a.out_rid0[pos] = e.rid;
-            if (FOLD) fold_add(acc, e.r, e.rid);
-        } else if (c == 0) {
-            const uint64_t pos = beq + __popc(eq & ((1u << lane) - 1u));
-            if (take_all) {
-                if (pos < krem) {
-                    a.out_r0[eq_base + pos] = e.r;
-                    a.out_rid0[eq_base + pos] = e.rid;
-                    if (FOLD) fold_add(acc, e.r, e.rid);
+        if (eq) {
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(eq_ctr, static_cast<unsigned long long>(__popc(eq)));
+            base = __shfl_sync(0xFFFFFFFFu, base, 0);
+            if (c == 0) {
+                const uint64_t pos = base + __popc(eq & ((1u << lane) - 1u));
+                if (take_all) {
+                    if (pos < krem) {
+                        a.out_r0[eq_base + pos] = e.r;
+                        a.out_rid0[eq_base + pos] = e.rid;
+                    }
+                } else if (pos < TK_SMALL) {
+                    a.small_r[pos] = e.r;
+                    a.small_rid[pos] = e.rid;
                 }
-            } else if (pos < TK_SMALL) {
-                a.small_r[pos] = e.r;
-                a.small_rid[pos] = e.rid;
             }
         }
     }
-    if (FOLD) fold_merge<TK_TPB>(acc, ctl->fin);
+}
+
+// The same for the larger-K finish, which also wants the minima and maxima of
+// the entries in out (merged into ctl->fin, so that it needs no pass of its
+// own).  Nearly every warp has some of those, and an atomic each on one word
+// is what such a pass then waits for (2^24 keys, K = 100,000: 97 us; with one
+// atomic per CTA and step, between two barriers, 199).  So a warp stages its
+// entries for out in shared memory and takes their places SPLIT_CAP at a time.
+// SPLIT_U loads are in flight per thread.
+constexpr int SPLIT_CAP = 256;
+constexpr int SPLIT_U = 4;
+static_assert(TK_TPB / 32 * SPLIT_CAP * 12 <= TK_SORT_SMEM, "the warps' stages");
+static_assert(SPLIT_U * 32 <= SPLIT_CAP, "a step's entries fit an empty stage");
+__device__ void split_pass_large(const TopkArgs& a, bool cand, uint64_t src_n, const Range& g, bool take_all,
+                                 uint64_t krem, bool whole, unsigned char* smem) {
+    TopkCtl* ctl = a.ctl;
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, lt_mask = (1u << lane) - 1u;
+    uint64_t* wr = reinterpret_cast<uint64_t*>(smem + warp * (SPLIT_CAP * 12));
+    uint32_t* wrid = reinterpret_cast<uint32_t*>(wr + SPLIT_CAP);
+    unsigned cnt = 0;                                        // staged entries of the warp
+    Fold acc = fold_none();
+    const uint64_t stride = static_cast<uint64_t>(TK_TPB) * gridDim.x;
+    const uint64_t eq_base = a.k - krem;
+    unsigned long long* eq_ctr = take_all ? &ctl->eq_count : &ctl->small_count;
+    const int last = whole ? 0 : -1;                         // range_cmp of the entries that all go to out
+    auto write = [&](unsigned long long base) {
+        __syncwarp();
+        for (unsigned j = lane; j < cnt; j += 32) {
+            a.out_r0[base + j] = wr[j];
+            a.out_rid0[base + j] = wrid[j];
+        }
+        __syncwarp();
+    };
+    for (uint64_t wb = static_cast<uint64_t>(blockIdx.x) * TK_TPB + (threadIdx.x & ~31u); wb < src_n;
+         wb += SPLIT_U * stride) {
+        Elem e[SPLIT_U];
+#pragma unroll
+        for (int u = 0; u < SPLIT_U; ++u) {
+            const uint64_t i = wb + lane + u * stride;
+            if (i < src_n) e[u] = load_src(a, cand, i);
+        }
+        if (cnt + SPLIT_U * 32 > SPLIT_CAP) {
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(&ctl->out_count, static_cast<unsigned long long>(cnt));
+            write(__shfl_sync(0xFFFFFFFFu, base, 0));
+            cnt = 0;
+        }
+#pragma unroll
+        for (int u = 0; u < SPLIT_U; ++u) {
+            const uint64_t i = wb + lane + u * stride;
+            const int c = i < src_n ? range_cmp(g, e[u].r, e[u].rid) : 1;
+            const unsigned lt = __ballot_sync(0xFFFFFFFFu, c <= last);
+            if (c <= last) {
+                const unsigned pos = cnt + __popc(lt & lt_mask);
+                wr[pos] = e[u].r;
+                wrid[pos] = e[u].rid;
+                fold_add(acc, e[u].r, e[u].rid);
+            }
+            cnt += __popc(lt);
+            const unsigned eq = __ballot_sync(0xFFFFFFFFu, c == 0 && last < 0);
+            if (!eq) continue;
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(eq_ctr, static_cast<unsigned long long>(__popc(eq)));
+            base = __shfl_sync(0xFFFFFFFFu, base, 0);
+            if (c != 0) continue;
+            const uint64_t pos = base + __popc(eq & lt_mask);
+            if (take_all) {
+                if (pos < krem) {
+                    a.out_r0[eq_base + pos] = e[u].r;
+                    a.out_rid0[eq_base + pos] = e[u].rid;
+                    fold_add(acc, e[u].r, e[u].rid);
+                }
+            } else if (pos < TK_SMALL) {
+                a.small_r[pos] = e[u].r;
+                a.small_rid[pos] = e[u].rid;
+            }
+        }
+    }
+    // what is left of all warps, with one atomic
+    __shared__ unsigned s_cnt[TK_TPB / 32];
+    __shared__ unsigned long long s_base;
+    if (lane == 0) s_cnt[warp] = cnt;
+    __syncthreads();
+    unsigned before = 0, all = 0;
+    for (unsigned w = 0; w < TK_TPB / 32; ++w) {
+        if (w < warp) before += s_cnt[w];
+        all += s_cnt[w];
+    }
+    if (threadIdx.x == 0 && all) s_base = atomicAdd(&ctl->out_count, static_cast<unsigned long long>(all));
+    __syncthreads();
+    if (all) write(s_base + before);
+    fold_merge<TK_TPB>(acc, ctl->fin);
 }
 
 // Entries of [lo, hi) in shared memory that order before entry e of them
@@ -1178,9 +1233,9 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
     // the larger-K finish wants the span of the entries split writes out
     const bool large = (take_all ? a.k : a.k - krem) + (take_all ? 0 : bcnt) > TK_RANK_MAX;
     if (large)
-        split_pass<true>(a, cand, src_n, g, take_all, krem, first);
+        split_pass_large(a, cand, src_n, g, take_all, krem, krem == bcnt, smem);
     else
-        split_pass<false>(a, cand, src_n, g, take_all, krem, first);
+        split_pass(a, cand, src_n, g, take_all, krem, first);
     if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
     if (stamp) ctl->ts[5] = gtimer();
 
