@@ -1350,7 +1350,7 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
                 off[threadIdx.x * PER + j] = static_cast<unsigned>(run);
                 run += v[j];
             }
-            if (!__syncthreads_and(mx <= static_cast<unsigned>(TK_SMALL))) return 0;
+            if (!__syncthreads_and(mx <= static_cast<unsigned>(TK_BIN_MAX))) return 0;
             // Scatter the below entries into bin order (out_r1).
             for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x; i < nb; i += gstride) {
                 const uint64_t er = __ldcg(a.out_r0 + i);
@@ -1362,36 +1362,48 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
             }
             if (!grid_sync(a.bar, &ctl->err, bar_target)) return -1;
             // Bins of at most 128 entries: one warp each, in registers.
+            // (`pure`: pairs of bins, so that the warps and CTAs share the even
+            // ones evenly; grids are even)
             auto size = [&](int b) { return (b + 1 < TK_BINS ? off[b + 1] : static_cast<unsigned>(nb)) - off[b]; };
-            for (int b = gw; b < TK_BINS; b += nwarps) {
-                const unsigned m = size(b);
-                const bool same = pure && (b & 1);
-                if (m == 0 || (m > 128 && !same)) continue;
-                const unsigned o = off[b];
-                if (same) {
-                    for (unsigned i = lane; i < m; i += 32)
+            const int each = pure ? 2 : 1;
+            for (int b = gw * each; b < TK_BINS; b += nwarps * each) {
+                if (pure) {                                  // the identical entries after bin b
+                    const unsigned o = off[b + 1], same = size(b + 1);
+                    for (unsigned i = lane; i < same; i += 32)
                         write_result(a, o + i, __ldcg(a.out_r1 + o + i), __ldcg(a.out_rid1 + o + i));
-                    continue;
                 }
+                const unsigned m = size(b), o = off[b];
+                if (m == 0 || m > 128) continue;
                 if (m <= 32) warp_rank_bin<1>(a, o, m);
                 else if (m <= 64) warp_rank_bin<2>(a, o, m);
                 else warp_rank_bin<4>(a, o, m);
             }
-            // Larger bins: one CTA each, ranked in shared memory.
+            // Larger bins: one CTA each, in shared memory, one or two threads
+            // an entry that go through the bin together (a warp an entry, as
+            // for the small buffer, spends most of its time on the sums: 2^24
+            // uniform int64 keys, K = 10^6 the call 647 -> 522 us).
             uint64_t* br = reinterpret_cast<uint64_t*>(smem + TK_BINS * 4);
             uint32_t* brid = reinterpret_cast<uint32_t*>(smem + TK_BINS * 4 + TK_SMALL * 8);
-            for (int b = blockIdx.x; b < TK_BINS; b += gridDim.x) {
+            for (int b = static_cast<int>(blockIdx.x) * each; b < TK_BINS; b += static_cast<int>(gridDim.x) * each) {
                 const unsigned m = size(b);
-                if (m <= 128 || (pure && (b & 1))) continue;
+                if (m <= 128) continue;
                 const unsigned o = off[b];
                 for (unsigned i = threadIdx.x; i < m; i += TK_TPB) {
                     br[i] = __ldcg(a.out_r1 + o + i);
                     brid[i] = __ldcg(a.out_rid1 + o + i);
                 }
                 __syncthreads();
-                for (unsigned e = threadIdx.x >> 5; e < m; e += TK_TPB / 32) {
-                    const unsigned c = warp_rank_of(br, brid, 0, static_cast<int>(m), static_cast<int>(e));
-                    if (lane == 0) write_result(a, o + c, br[e], brid[e]);
+                const unsigned two = m <= TK_TPB / 2 ? 1u : 0u;
+                for (unsigned e0 = 0; e0 < m; e0 += TK_TPB >> two) {
+                    const unsigned e = e0 + (threadIdx.x >> two);
+                    const unsigned at = e < m ? e : 0u;
+                    const uint64_t er = br[at];
+                    const uint32_t erid = brid[at];
+                    unsigned c = 0;
+#pragma unroll 4
+                    for (unsigned j = threadIdx.x & two; j < m; j += 1u + two) rank_count(c, br[j], brid[j], er, erid, j < at);
+                    if (two) c += __shfl_xor_sync(0xFFFFFFFFu, c, 1);
+                    if (e < m && !(threadIdx.x & two)) write_result(a, o + (0u - c), er, erid);
                 }
                 __syncthreads();
             }

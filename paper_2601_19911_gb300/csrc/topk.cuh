@@ -39,7 +39,14 @@ enum { TK_SAMPLE_NONE = 0, TK_SAMPLE_FILTER = 1, TK_SAMPLE_INLINE = 2 };
 constexpr int TK_RANK_MAX = 8192;         // survivors ranked in shared memory by the whole grid
 constexpr int TK_SPLITTERS = 2047;        // splitters of the larger-K finish on tied keys (2^k - 1)
 static_assert(TK_SPLITTERS <= TK_SMALL, "the splitters fit where K > TK_SMALL entries do");
-constexpr uint64_t TK_SPLIT_MAX = 2048ull * 512;   // entries they may split (about 512 per gap)
+// Entries they may split, about 128 per gap, which a warp ranks in registers
+// (tied int64 keys, K = 250,000: the call 332 us, 452 with tile sorts and merges;
+// 2 * 10^6 tied float32 keys, K = 400,000: 443 us by splitters, 326 by merges).
+constexpr uint64_t TK_SPLIT_MAX = 2048ull * 128;
+// Entries of a bin that the larger-K finish ranks in one CTA; a larger one makes
+// that CTA the last by far (2^26 normal int64 keys, K = 10^6, bins up to 4096:
+// the finish 1100 us, tile sorts and merges instead 370).
+constexpr int TK_BIN_MAX = 2048;
 constexpr int TK_SORT_SMEM = TK_RANK_MAX * 12;  // select kernel shared bytes (ranking / sort tile / histogram)
 constexpr int TK_MAX_STAGES = 16;         // full + empty mbarrier pairs reserved after the ring
 constexpr int TK_SMEM_MAX = 227 * 1024;   // opt-in shared memory per CTA
