@@ -213,18 +213,35 @@ __device__ void sample_threshold(const TopkArgs& a, unsigned* sh, unsigned long 
         edge = prefix | ((1ull << (64 - L - d)) - 1ull);
         if (cum + pk.in_b <= r + 8) break;
     }
-    __shared__ unsigned long long lo, hi;                    // of the few samples up to the edge
+    // The filter may be launched now (the other CTAs are gone), not before: its
+    // first loads, 20 MB over the GPU, keep this CTA's own loads and
+    // instruction fetches waiting (2^26 float32 keys: 14 us for the sample
+    // with the filter launched at its start, 7 so).
+    allow_next_grid();
+    __shared__ unsigned long long lo, hi;                    // of the samples up to the edge, mostly few
     if (threadIdx.x == 0) {
         lo = ~0ull;
         hi = 0;
     }
     __syncthreads();
+    uint64_t mn = ~0ull, mx = 0;
 #pragma unroll
     for (int j = 0; j < TK_SPT; ++j)
         if (s[j] <= edge) {
-            atomicMin(&lo, static_cast<unsigned long long>(s[j]));
-            atomicMax(&hi, static_cast<unsigned long long>(s[j]));
+            mn = min(mn, s[j]);
+            mx = max(mx, s[j]);
         }
+    if (__any_sync(0xFFFFFFFFu, mn <= mx)) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            mn = min(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, o));
+            mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+        }
+        if ((threadIdx.x & 31u) == 0) {
+            atomicMin(&lo, static_cast<unsigned long long>(mn));
+            atomicMax(&hi, static_cast<unsigned long long>(mx));
+        }
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         const uint64_t t = hi, d = hi - lo;
@@ -1050,7 +1067,6 @@ __global__ void __launch_bounds__(TK_TPB) topk_prepare_kernel(TopkArgs a) {
     __shared__ int last;
     TopkCtl* ctl = a.ctl;
     wait_prior_grid();                    // the call before may still read the control block
-    allow_next_grid();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctl->ts[0] = gtimer();
         a.bar->count = 0;
@@ -1067,6 +1083,7 @@ __global__ void __launch_bounds__(TK_TPB) topk_prepare_kernel(TopkArgs a) {
     }
     for (int b = blockIdx.x * TK_TPB + threadIdx.x; b < 3 * TK_BINS; b += gridDim.x * TK_TPB) a.ghist[b] = 0;
     if (!a.use_sample) {
+        allow_next_grid();
         if (threadIdx.x == 0) ctl->ts[1] = gtimer();
         return;
     }
