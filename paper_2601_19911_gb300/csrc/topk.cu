@@ -255,20 +255,37 @@ __device__ void sample_threshold(const TopkArgs& a, unsigned* sh, unsigned long 
 // flushed to the global candidate buffer WS_CAP at a time: one atomic on the
 // global count per flush instead of one per warp-vector with a hit (a single
 // global counter hit by every SM serialises in L2), and coalesced writes.
+struct FuseRange {
+    Range g;
+    int sh;
+};
+__device__ __forceinline__ FuseRange fuse_range(const TopkArgs& a) {
+    FuseRange f;
+    f.g = Range{__ldcg(&a.ctl->fbase), __ldcg(&a.ctl->thresh), 0u, max_rowid(a)};
+    f.sh = range_shift(f.g, a.digit);
+    return f;
+}
+
 constexpr int WS_CAP = 256;
 struct WarpStage {
-    uint64_t* r;          // WS_CAP rank words (shared)
+    uint64_t* w;          // WS_CAP words (shared): the keys' bits, or the rank words of two-column keys
     uint32_t* idx;        // WS_CAP key indices (shared)
     unsigned count;       // entries held (the same in every lane)
     unsigned* hist;       // the CTA's histogram of the fused first pass (shared; NULL without one)
+    const FuseRange* fr;  // its interval (shared)
 };
 constexpr int WS_BYTES = WS_CAP * 12;
+// Rank word of a staged word.  (Ranked as they leave the stage, in one loop, not
+// as they enter it, in one of the filter's 16 unrolled places.)
+__device__ __forceinline__ uint64_t staged_rank(const TopkArgs& a, uint64_t w) {
+    return a.pair ? w : rank_key(w, a.kind, a.desc);
+}
 constexpr int FUSE_BYTES = (TK_BINS + 4) * 4;     // the histogram, its count of entries below, 16-byte units
 
-__device__ __forceinline__ WarpStage warp_stage(unsigned char* base, unsigned* hist) {
+__device__ __forceinline__ WarpStage warp_stage(unsigned char* base, unsigned* hist, const FuseRange* fr) {
     const unsigned w = threadIdx.x >> 5;
     unsigned char* p = base + static_cast<size_t>(w) * WS_BYTES;
-    return WarpStage{reinterpret_cast<uint64_t*>(p), reinterpret_cast<uint32_t*>(p + WS_CAP * 8), 0u, hist};
+    return WarpStage{reinterpret_cast<uint64_t*>(p), reinterpret_cast<uint32_t*>(p + WS_CAP * 8), 0u, hist, fr};
 }
 
 // The select's first refine pass, folded into the streaming filter (the
@@ -283,17 +300,6 @@ __device__ __forceinline__ WarpStage warp_stage(unsigned char* base, unsigned* h
 // column and a second one: one pass instead of three over the candidates, the
 // select 29 -> 11.6 us.  Candidates below the interval are counted in one
 // more word.
-
-struct FuseRange {
-    Range g;
-    int sh;
-};
-__device__ __forceinline__ FuseRange fuse_range(const TopkArgs& a) {
-    FuseRange f;
-    f.g = Range{__ldcg(&a.ctl->fbase), __ldcg(&a.ctl->thresh), 0u, max_rowid(a)};
-    f.sh = range_shift(f.g, a.digit);
-    return f;
-}
 
 template <int TPB>
 __device__ __forceinline__ void fuse_init(unsigned* hist) {
@@ -327,7 +333,7 @@ __device__ __forceinline__ void stage_flush_plain(const TopkArgs& a, WarpStage& 
         const unsigned long long pos = base + j;
         if (pos < a.cand_cap) {
             const uint32_t idx = ws.idx[j];
-            a.cand_r[pos] = ws.r[j];
+            a.cand_r[pos] = staged_rank(a, ws.w[j]);
             a.cand_rid[pos] = a.rowids ? a.rowids[idx] : idx;
         }
     }
@@ -336,12 +342,12 @@ __device__ __forceinline__ void stage_flush_plain(const TopkArgs& a, WarpStage& 
 }
 
 // The same, also counting the hits for the fused first pass.
-__device__ __forceinline__ void stage_write_fused(const TopkArgs& a, const FuseRange& f, const WarpStage& ws,
-                                                  unsigned long long base) {
+__device__ __forceinline__ void stage_write_fused(const TopkArgs& a, const WarpStage& ws, unsigned long long base) {
+    const FuseRange f = *ws.fr;
     for (unsigned j = threadIdx.x & 31u; j < ws.count; j += 32) {
         const unsigned long long pos = base + j;
         const uint32_t idx = ws.idx[j];
-        const uint64_t r = ws.r[j];
+        const uint64_t r = staged_rank(a, ws.w[j]);
         const uint32_t rid = a.rowids ? a.rowids[idx] : idx;
         if (pos < a.cand_cap) {
             a.cand_r[pos] = r;
@@ -355,7 +361,7 @@ __device__ __forceinline__ void stage_flush_fused(const TopkArgs& a, const WarpS
     unsigned long long base = 0;
     if ((threadIdx.x & 31u) == 0) base = atomicAdd(&a.ctl->cand_count, static_cast<unsigned long long>(ws.count));
     base = __shfl_sync(0xFFFFFFFFu, base, 0);
-    stage_write_fused(a, fuse_range(a), ws, base);
+    stage_write_fused(a, ws, base);
     __syncwarp();
 }
 
@@ -371,11 +377,11 @@ __device__ __forceinline__ void stage_flush(const TopkArgs& a, WarpStage& ws) {
 }
 
 // Stage the hits of a warp-vector: bit e of `hit` set for the lane's element e
-// of VEC, whose rank word is rank(e) and whose index is idx0 + e (all 32 lanes
-// call).  Most vectors that get here have one or two hits in all, so the
+// of VEC, whose word to stage is word(e) and whose index is idx0 + e (all 32
+// lanes call).  Most vectors that get here have one or two hits in all, so the
 // elements without any are skipped by one warp-wide OR.
-template <int VEC, bool FUSE, typename RankOf>
-__device__ __forceinline__ void stage_hits(const TopkArgs& a, unsigned hit, uint64_t idx0, WarpStage& ws, RankOf rank) {
+template <int VEC, bool FUSE, typename WordOf>
+__device__ __forceinline__ void stage_hits(const TopkArgs& a, unsigned hit, uint64_t idx0, WarpStage& ws, WordOf word) {
     const unsigned lt = (1u << (threadIdx.x & 31u)) - 1u;
     const unsigned any = __reduce_or_sync(0xFFFFFFFFu, hit);
     const unsigned total = __reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(__popc(hit)));
@@ -388,7 +394,7 @@ __device__ __forceinline__ void stage_hits(const TopkArgs& a, unsigned hit, uint
         const unsigned bal = __ballot_sync(0xFFFFFFFFu, h);
         if (h) {
             const unsigned pos = before + __popc(bal & lt);
-            ws.r[pos] = rank(e);
+            ws.w[pos] = word(e);
             ws.idx[pos] = static_cast<uint32_t>(idx0 + e);
         }
         before += __popc(bal);
@@ -413,7 +419,7 @@ __device__ __forceinline__ void filter_vector(const TopkArgs& a, const KeyLimit&
     unsigned hit = 0;
 #pragma unroll
     for (int e = 0; e < VEC; ++e) hit |= (valid && pass(e)) ? (1u << e) : 0u;
-    stage_hits<VEC, FUSE>(a, hit, idx0, ws, [&](int e) { return rank_key(key(e), a.kind, a.desc); });
+    stage_hits<VEC, FUSE>(a, hit, idx0, ws, key);
 }
 
 // The unaligned head [0, head) and ragged tail [tail0, n) of the keys: at
@@ -425,19 +431,19 @@ __device__ __forceinline__ void filter_ends(const TopkArgs& a, uint64_t t, uint6
     const uint64_t rest = head + (a.n - tail0);
     const uint64_t j = threadIdx.x;
     const bool valid = j < rest;
-    uint64_t idx = 0, r = ~0ull;
+    uint64_t idx = 0, r = ~0ull, word = 0;
     if (valid) {
         idx = j < head ? j : tail0 + (j - head);
-        if (COPY) {
-            const uint64_t bits = key_bits(a, a.host_keys, idx);
-            if (a.w4) static_cast<uint32_t*>(const_cast<void*>(a.keys))[idx] = static_cast<uint32_t>(bits);
-            else static_cast<uint64_t*>(const_cast<void*>(a.keys))[idx] = bits;
-            r = rank_key(bits, a.kind, a.desc);
+        if (a.pair) {
+            word = r = load_input(a, idx).r;
         } else {
-            r = load_input(a, idx).r;
+            word = key_bits(a, COPY ? a.host_keys : a.keys, idx);
+            r = rank_key(word, a.kind, a.desc);
+            if (COPY && a.w4) static_cast<uint32_t*>(const_cast<void*>(a.keys))[idx] = static_cast<uint32_t>(word);
+            else if (COPY) static_cast<uint64_t*>(const_cast<void*>(a.keys))[idx] = word;
         }
     }
-    stage_hits<1, FUSE>(a, valid && r <= t ? 1u : 0u, idx, ws, [&](int) { return r; });
+    stage_hits<1, FUSE>(a, valid && r <= t ? 1u : 0u, idx, ws, [&](int) { return word; });
 }
 
 // The last hits of all warps of the CTA, with one atomic on the global count
@@ -447,7 +453,6 @@ __device__ __forceinline__ void cta_flush_fused(const TopkArgs& a, const WarpSta
     __shared__ unsigned cnts[TPB / 32];
     __shared__ unsigned long long s_base;
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const FuseRange f = fuse_range(a);
     if (lane == 0) cnts[warp] = ws.count;
     __syncthreads();
     unsigned before = 0, all = 0;
@@ -458,7 +463,7 @@ __device__ __forceinline__ void cta_flush_fused(const TopkArgs& a, const WarpSta
     }
     if (threadIdx.x == 0 && all) s_base = atomicAdd(&a.ctl->cand_count, static_cast<unsigned long long>(all));
     __syncthreads();
-    if (all) stage_write_fused(a, f, ws, s_base + before);
+    if (all) stage_write_fused(a, ws, s_base + before);
 }
 
 // Phase 1: the single streaming pass.  Appends (rank word, row-id) of every
@@ -558,8 +563,7 @@ __device__ __forceinline__ void filter_loop(const TopkArgs& a, const FilterSpan<
 #pragma unroll
                 for (int e = 0; e < VEC; ++e) hit |= (vi < st.end && pass(u, e)) ? (1u << e) : 0u;
                 if (__any_sync(0xFFFFFFFFu, hit != 0))
-                    stage_hits<VEC, true>(a, hit, sp.head + vi * VEC, ws,
-                                          [&](int e) { return rank_key(key(u, e), a.kind, a.desc); });
+                    stage_hits<VEC, true>(a, hit, sp.head + vi * VEC, ws, [&](int e) { return key(u, e); });
             }
         }
         st.next(sp.nvec, PER);
@@ -570,6 +574,7 @@ __device__ __forceinline__ void filter_loop(const TopkArgs& a, const FilterSpan<
 template <bool W4, int TPB, bool COPY = false>
 __device__ __forceinline__ void filter_pass(const TopkArgs& a, unsigned char* fsm) {
     unsigned* hist = reinterpret_cast<unsigned*>(fsm);
+    __shared__ FuseRange s_fr;
     fuse_init<TPB>(hist);
     const FilterSpan<W4> sp(a, COPY ? a.host_keys : a.keys);
     FilterStep st;
@@ -578,7 +583,9 @@ __device__ __forceinline__ void filter_pass(const TopkArgs& a, unsigned char* fs
     if (st.bb < st.end) filter_load<TPB>(sp.base, st.end, st.bb, v);
     wait_prior_grid();
     allow_next_grid();
-    const uint64_t t = __ldcg(&a.ctl->thresh);
+    if (threadIdx.x == 0) s_fr = fuse_range(a);
+    __syncthreads();
+    const uint64_t t = s_fr.g.rhi;
     const KeyLimit kl = key_limit(t, a.kind, a.desc);
     uint64_t lim;
     int mode;
@@ -589,7 +596,7 @@ __device__ __forceinline__ void filter_pass(const TopkArgs& a, unsigned char* fs
     } else {
         mode = key_cmp<uint64_t>(kl.m64, kl.c64, &lim);
     }
-    WarpStage ws = warp_stage(fsm + FUSE_BYTES, hist);
+    WarpStage ws = warp_stage(fsm + FUSE_BYTES, hist, &s_fr);
     if (mode == CMP_GE_U) filter_loop<W4, TPB, CMP_GE_U, COPY>(a, sp, lim, st, v, ws);
     else if (mode == CMP_LE_U) filter_loop<W4, TPB, CMP_LE_U, COPY>(a, sp, lim, st, v, ws);
     else if (mode == CMP_GE_S) filter_loop<W4, TPB, CMP_GE_S, COPY>(a, sp, lim, st, v, ws);
@@ -676,13 +683,16 @@ __device__ void filter_pass_pair_vec(const TopkArgs& a, uint64_t t, WarpStage& w
 template <int TPB>
 __device__ __forceinline__ void filter_pass_pair(const TopkArgs& a, unsigned char* fsm) {
     unsigned* hist = reinterpret_cast<unsigned*>(fsm);
+    __shared__ FuseRange s_fr;
     fuse_init<TPB>(hist);
     wait_prior_grid();
     allow_next_grid();
-    const uint64_t t = __ldcg(&a.ctl->thresh);
+    if (threadIdx.x == 0) s_fr = fuse_range(a);
+    __syncthreads();
+    const uint64_t t = s_fr.g.rhi;
     const uint64_t n = a.n;
     const uintptr_t off = reinterpret_cast<uintptr_t>(a.keys) ^ reinterpret_cast<uintptr_t>(a.keys2);
-    WarpStage ws = warp_stage(fsm + FUSE_BYTES, hist);
+    WarpStage ws = warp_stage(fsm + FUSE_BYTES, hist, &s_fr);
     if ((off & 31) == 0) {
         filter_pass_pair_vec<TPB, 8>(a, t, ws);
     } else if ((off & 15) == 0) {
@@ -740,7 +750,7 @@ __device__ bool filter_pass_bulk(const TopkArgs& a, uint64_t t, unsigned char* s
     const KeyLimit lim = key_limit(t, a.kind, a.desc);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(tile) * stages);
     uint64_t* empty = full + TK_MAX_STAGES;
-    WarpStage ws = warp_stage(reinterpret_cast<unsigned char*>(empty + TK_MAX_STAGES), nullptr);
+    WarpStage ws = warp_stage(reinterpret_cast<unsigned char*>(empty + TK_MAX_STAGES), nullptr, nullptr);
     const uint64_t step = static_cast<uint64_t>(gridDim.x) * tile;       // bytes between my tiles
 
     if (threadIdx.x == 0) {
