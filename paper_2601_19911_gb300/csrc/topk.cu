@@ -14,7 +14,8 @@
 //      keys, run only when there is a sample.  32-byte streaming loads, one
 //      compare per key against the threshold in the key's own bit domain,
 //      and every key that passes is appended (per-warp staging, one global
-//      atomic per flush) to a candidate buffer with its row-id.
+//      atomic per flush) to a candidate buffer with its row-id -- or only
+//      counted, when the sample shows ties that would not fit there.
 //   Phases 2-4 are one cooperative launch (topk_select_kernel) whose CTAs
 //   meet at bounded grid barriers.  Its source is the candidate buffer when
 //   the sample worked (at least K candidates, no overflow) and the full
@@ -65,15 +66,14 @@ __device__ __forceinline__ uint64_t key_bits(const TopkArgs& a, const void* keys
     return a.w4 ? static_cast<uint64_t>(static_cast<const uint32_t*>(keys)[i]) : static_cast<const uint64_t*>(keys)[i];
 }
 
-__device__ __forceinline__ Elem load_input(const TopkArgs& a, uint64_t i) {
-    Elem e;
-    if (a.pair)
-        e.r = pair_rank(static_cast<const uint32_t*>(a.keys)[i], static_cast<const uint32_t*>(a.keys2)[i], a);
-    else
-        e.r = rank_key(key_bits(a, a.keys, i), a.kind, a.desc);
-    e.rid = a.rowids ? a.rowids[i] : static_cast<uint32_t>(i);
-    return e;
+__device__ __forceinline__ uint64_t input_rank(const TopkArgs& a, uint64_t i) {
+    if (a.pair) return pair_rank(static_cast<const uint32_t*>(a.keys)[i], static_cast<const uint32_t*>(a.keys2)[i], a);
+    return rank_key(key_bits(a, a.keys, i), a.kind, a.desc);
 }
+__device__ __forceinline__ uint32_t input_rowid(const TopkArgs& a, uint64_t i) {
+    return a.rowids ? a.rowids[i] : static_cast<uint32_t>(i);
+}
+__device__ __forceinline__ Elem load_input(const TopkArgs& a, uint64_t i) { return Elem{input_rank(a, i), input_rowid(a, i)}; }
 
 __device__ __forceinline__ Elem load_src(const TopkArgs& a, bool cand, uint64_t i) {
     if (cand) return Elem{__ldcg(a.cand_r + i), __ldcg(a.cand_rid + i)};
@@ -187,7 +187,8 @@ __device__ __forceinline__ void fold_reset(unsigned long long* mm) {
 // threshold is the largest of those samples.  With the smallest of them it
 // also fixes the interval of the select's fused first pass (see fuse_range):
 // four times their spread below the threshold, or the threshold alone when
-// they are all equal.
+// they are all equal.  When so many samples tie that the candidates would not
+// fit their buffer, the streaming pass is told to count only (count_pass).
 __device__ void sample_threshold(const TopkArgs& a, unsigned* sh, unsigned long long* sc) {
     uint64_t s[TK_SPT];
 #pragma unroll
@@ -195,7 +196,7 @@ __device__ void sample_threshold(const TopkArgs& a, unsigned* sh, unsigned long 
     const int kb = a.w4 ? 32 : 64;
     const unsigned long long r = a.sample_rank;
     uint64_t prefix = 0, edge = 0;
-    unsigned long long rem = r, cum = 0;
+    unsigned long long rem = r, cum = 0, upto = 0;           // upto: samples up to the edge
     for (int L = 0; L < kb; L += a.digit) {
         const int d = min(a.digit, kb - L);
         for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB) sh[b] = 0;
@@ -211,7 +212,8 @@ __device__ void sample_threshold(const TopkArgs& a, unsigned* sh, unsigned long 
         rem -= pk.below;
         cum += pk.below;
         edge = prefix | ((1ull << (64 - L - d)) - 1ull);
-        if (cum + pk.in_b <= r + 8) break;
+        upto = cum + pk.in_b;
+        if (upto <= r + 8) break;
     }
     // The filter may be launched now (the other CTAs are gone), not before: its
     // first loads, 20 MB over the GPU, keep this CTA's own loads and
@@ -247,6 +249,7 @@ __device__ void sample_threshold(const TopkArgs& a, unsigned* sh, unsigned long 
         const uint64_t t = hi, d = hi - lo;
         a.ctl->thresh = t;
         a.ctl->fbase = d >= t / 4 ? (d ? 0ull : t) : t - 4 * d;
+        a.ctl->count_only = a.fuse && !a.host_keys && upto * a.n > a.cand_cap * TK_SAMPLE;
         a.ctl->ts[1] = gtimer();
     }
 }
@@ -258,10 +261,12 @@ __device__ void sample_threshold(const TopkArgs& a, unsigned* sh, unsigned long 
 struct FuseRange {
     Range g;
     int sh;
+    int count_only;
 };
 __device__ __forceinline__ FuseRange fuse_range(const TopkArgs& a) {
     FuseRange f;
     f.g = Range{__ldcg(&a.ctl->fbase), __ldcg(&a.ctl->thresh), 0u, max_rowid(a)};
+    f.count_only = __ldcg(&a.ctl->count_only);
     f.sh = range_shift(f.g, a.digit);
     return f;
 }
@@ -466,6 +471,48 @@ __device__ __forceinline__ void cta_flush_fused(const TopkArgs& a, const WarpSta
     if (all) stage_write_fused(a, ws, s_base + before);
 }
 
+// The streaming pass when the candidates would not fit (few distinct keys): no
+// entry is stored, but all up to the threshold are counted as above, so the
+// select reads the input with its first refine pass done.  K = 10, 2 * 10^6
+// int64 keys of one value 95 -> 50 us (56 without a sample), of 12 values 101 ->
+// 52 (75); 2^26 keys of one value 3226 -> 1472.
+template <int TPB>
+__device__ void count_pass(const TopkArgs& a, const FuseRange& f, unsigned* hist) {
+    constexpr int U = 4;                       // loads in flight per thread
+    const unsigned lane = threadIdx.x & 31u;
+    const uint64_t stride = static_cast<uint64_t>(TPB) * gridDim.x;
+    const bool ties = f.g.rlo == f.g.rhi;      // the bins are of row-ids
+    unsigned hits = 0;
+    for (uint64_t wb = static_cast<uint64_t>(blockIdx.x) * TPB + (threadIdx.x & ~31u); wb < a.n; wb += U * stride) {
+        uint64_t r[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (wb + lane + u * stride < a.n) r[u] = input_rank(a, wb + lane + u * stride);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint64_t i = wb + lane + u * stride;
+            const bool in = i < a.n && r[u] <= f.g.rhi;
+            unsigned bin = 0xFFFFFFFFu;
+            if (in && r[u] < f.g.rlo) bin = TK_BINS;
+            else if (in) bin = range_bin(f.g, f.sh, r[u], ties ? input_rowid(a, i) : 0u);
+            const unsigned peers = __match_any_sync(0xFFFFFFFFu, bin);
+            if (in && lane == static_cast<unsigned>(__ffs(peers) - 1))
+                atomicAdd(&hist[bin], static_cast<unsigned>(__popc(peers)));
+            hits += in ? 1u : 0u;
+        }
+    }
+    __shared__ unsigned s_hits[TPB / 32];
+    hits = __reduce_add_sync(0xFFFFFFFFu, hits);
+    if (lane == 0) s_hits[threadIdx.x >> 5] = hits;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long all = 0;
+        for (int w = 0; w < TPB / 32; ++w) all += s_hits[w];
+        if (all) atomicAdd(&a.ctl->cand_count, all);
+    }
+    fuse_merge<TPB>(a, hist);
+}
+
 // Phase 1: the single streaming pass.  Appends (rank word, row-id) of every
 // key whose rank word is <= t; counts all of them.  Two 32-byte loads in
 // flight per thread, tested in one comparison per key and one vote per 64
@@ -585,6 +632,7 @@ __device__ __forceinline__ void filter_pass(const TopkArgs& a, unsigned char* fs
     allow_next_grid();
     if (threadIdx.x == 0) s_fr = fuse_range(a);
     __syncthreads();
+    if (!COPY && s_fr.count_only) return count_pass<TPB>(a, s_fr, hist);
     const uint64_t t = s_fr.g.rhi;
     const KeyLimit kl = key_limit(t, a.kind, a.desc);
     uint64_t lim;
@@ -689,6 +737,7 @@ __device__ __forceinline__ void filter_pass_pair(const TopkArgs& a, unsigned cha
     allow_next_grid();
     if (threadIdx.x == 0) s_fr = fuse_range(a);
     __syncthreads();
+    if (s_fr.count_only) return count_pass<TPB>(a, s_fr, hist);
     const uint64_t t = s_fr.g.rhi;
     const uint64_t n = a.n;
     const uintptr_t off = reinterpret_cast<uintptr_t>(a.keys) ^ reinterpret_cast<uintptr_t>(a.keys2);
@@ -1179,8 +1228,10 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
     if (stamp) ctl->ts[2] = gtimer();
     // Source of the selection: the candidates of the streaming pass when the
     // sample judged well (at least k of them, all stored), else the input.
-    bool cand = false;
-    uint64_t src_n = a.n;
+    // Either way, with k or more entries up to the threshold the fused
+    // histogram holds them all.
+    bool cand = false, counted = false;
+    uint64_t src_n = a.n, upto = a.n;                        // entries up to the threshold, or all
     uint64_t low = 0;                                        // candidates below the fused interval
     FuseRange fr{};
     unsigned hv0[TK_BINS / TK_TPB];                          // the thread's bins of the fused pass
@@ -1195,23 +1246,24 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
         const uint64_t i0 = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x;
         if (i0 < a.cand_cap) first = Elem{__ldcg(a.cand_r + i0), __ldcg(a.cand_rid + i0)};
         if (err != 0) return report(a);
-        cand = cnt >= a.k && cnt <= a.cand_cap;
+        counted = a.fuse && cnt >= a.k;
+        cand = cnt >= a.k && cnt <= a.cand_cap && !(a.fuse && fr.count_only);
         if (cand) src_n = cnt;
+        if (cand || counted) upto = cnt;
         if (stamp) ctl->path = cand ? 1 : 2;
     }
     const unsigned long long use_ts3 = stamp ? gtimer() : 0ull;
 
-    // Phase 2: refine the interval that holds the K-th entry.  Candidates are
-    // all at or below the threshold.
-    Range g{0ull, cand ? fr.g.rhi : max_rank(a), 0u, max_rowid(a)};
-    uint64_t krem = a.k, bcnt = src_n;
+    // Phase 2: refine the interval that holds the K-th entry, at or below the
+    // threshold when k entries are.
+    Range g{0ull, cand || counted ? fr.g.rhi : max_rank(a), 0u, max_rowid(a)};
+    uint64_t krem = a.k, bcnt = upto;
     int pass = 0, npass = 0;
-    // With the filter's fused first pass, pass 0's histogram is ready on the
-    // candidate path; on the fallback path it holds the filter's partial
-    // counts, so the passes start at buffer 1 (clean) and pass 2 clears
-    // buffer 0 before pass 3 uses it.
-    bool ready = a.fuse && cand;
-    if (a.fuse && !cand) pass = 1;
+    // With the filter's fused first pass, pass 0's histogram is ready; when
+    // fewer than k entries are counted in it, the passes start at buffer 1
+    // (clean) and pass 2 clears buffer 0 before pass 3 uses it.
+    bool ready = counted;
+    if (a.fuse && !counted) pass = 1;
     if (ready && bcnt > TK_SMALL && krem < bcnt) {
         if (low >= a.k) {
             g.rhi = fr.g.rlo - 1;

@@ -76,7 +76,7 @@ struct TopkCtl {
     int err;                         // olap_status of the device side
     int path;                        // 0 direct, 1 sampled candidates, 2 fallback
     int passes;                      // refine passes run
-    int pad;
+    int count_only;                  // the candidates would not fit: the streaming pass counts only
     // Minimum and maximum rank word, minimum and maximum row-id of the entries
     // a refine pass saw (three slots, by pass), and of the selected entries
     // before the finish partition.
