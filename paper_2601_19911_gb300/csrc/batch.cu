@@ -13,10 +13,10 @@
 //     at or below the threshold to the CTA's own candidate buffer (no global
 //     atomics); the candidates are counted in 4096 equal bins of that
 //     interval, and those of the bins up to the K-th entry's are put in bin
-//     order in shared memory and ranked within their bins.  Small items take
-//     all their keys as candidates.  Ties and outliers that crowd a bin go
-//     through block-local radix passes and a sort instead, a misjudged sample
-//     through radix passes over the item's keys.
+//     order in shared memory and ranked within their bins, or sorted when
+//     ties or outliers crowd one.  Small items take all their keys as
+//     candidates.  More than one sort holds, or a misjudged sample, go through
+//     block-local radix passes first.
 //   * probe: the probe loop of the join kernel over one chunk of at most
 //     BP_CHUNK probe rows of an item, handed to the CTA's warps by a row
 //     queue in shared memory; a large item is many chunks taken by many
@@ -290,12 +290,15 @@ __device__ __forceinline__ void src_get(const Item& it, bool cand, const uint64_
 
 // Select and sort at once: the bins (a histogram of the entries) up to the
 // one that reaches kk are scattered into bin order in shared memory, and
-// every entry finds its place within its bin, which holds a few.  False, with nothing written, when those bins hold more than BT_SMALL
-// entries or one of them more than BT_BIN_MAX (ties, outliers): the caller
-// then refines and sorts.  An item of 482,000 keys with K = 500 leaves about
-// 3,000 candidates, whose bitonic sort over 4096 slots takes 78 steps; with
-// the streaming pass above, the kernel went from 600 to 398 us (512 items,
-// 1.8 GB of keys).
+// every entry finds its place within its bin, which holds a few; when one holds
+// more than BT_BIN_MAX (ties, outliers), what was kept is sorted instead, which
+// is mostly far less than the input.  False, with nothing written, when more
+// than BT_SMALL entries are kept: the caller then refines and sorts.  An item
+// of 482,000 keys with K = 500 leaves about 3,000 candidates, whose bitonic
+// sort over 4096 slots takes 78 steps; with the streaming pass above, the
+// kernel went from 600 to 398 us (512 items, 1.8 GB of keys).  64 items of 1000
+// to 4000 int64 keys of two values, all sorted 98 us, the kept ones 57; 512
+// items of up to 10^6 keys of 1024 values, refined and sorted 296, 228 so.
 constexpr unsigned BT_BIN_MAX = 128;
 __device__ bool cta_bin_select(const Item& it, bool cand, const uint64_t* cand_r, const uint32_t* cand_rid,
                                uint64_t src_n, uint64_t kk, const CtaBins& bin, unsigned char* smem,
@@ -329,21 +332,21 @@ __device__ bool cta_bin_select(const Item& it, bool cand, const uint64_t* cand_r
     }
     unsigned run = static_cast<unsigned>(block_excl_scan<BT_TPB>(local, sc, sc + 16));
     // (the scan ends with a barrier: every bin has been read)
-    bool ok = true;
+    bool crowded = false;
     unsigned total = 0;                                    // through the bin that reaches kk, in one thread
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
         if (run < kk) {                                    // one of the bins that are kept
-            if (v[j] > BT_BIN_MAX) ok = false;
+            if (v[j] > BT_BIN_MAX) crowded = true;
             if (run + v[j] >= kk) total = run + v[j];
         }
         off[threadIdx.x * PER + j] = run;
         run += v[j];
     }
     if (total) sc[20] = total;
-    if (total > BT_SMALL) ok = false;
-    if (!__syncthreads_and(ok)) return false;
+    crowded = __syncthreads_or(crowded) != 0;
     total = static_cast<unsigned>(sc[20]);
+    if (total > BT_SMALL) return false;
     for (uint64_t i0 = threadIdx.x; i0 < src_n; i0 += U * BT_TPB) {
         uint64_t r[U];
         uint32_t rid[U];
@@ -363,6 +366,11 @@ __device__ bool cta_bin_select(const Item& it, bool cand, const uint64_t* cand_r
         }
     }
     __syncthreads();
+    if (crowded) {
+        block_sort<BT_TPB>(sr, srid, static_cast<int>(total));
+        for (unsigned p = threadIdx.x; p < kk; p += BT_TPB) put_result(it, p, sr[p], srid[p]);
+        return true;
+    }
     // off[b] is now the end of bin b, and the start of the next
     for (unsigned p = threadIdx.x; p < total; p += BT_TPB) {
         const uint64_t r = sr[p];
@@ -448,15 +456,6 @@ __device__ void cta_topk(const Item& it, unsigned char* smem, uint64_t* cand_r, 
     const bool small = n <= BT_SMALL || kk > n / 16;
     if (small) g = cta_input_range(it, sc);
     if ((cand || small) && cta_bin_select(it, cand, cand_r, cand_rid, src_n, kk, CtaBins(g), smem, sc)) {
-        if (threadIdx.x == 0) *it.count = kk;
-        return;
-    }
-    if (n <= BT_SMALL) {
-        __syncthreads();
-        for (uint64_t i = threadIdx.x; i < n; i += BT_TPB) sr[i] = item_rank(it, i, &srid[i]);
-        __syncthreads();
-        block_sort<BT_TPB>(sr, srid, static_cast<int>(n));
-        for (uint64_t i = threadIdx.x; i < kk; i += BT_TPB) put_result(it, i, sr[i], srid[i]);
         if (threadIdx.x == 0) *it.count = kk;
         return;
     }
