@@ -175,33 +175,56 @@ __global__ void __launch_bounds__(JS_TPB, 2) join_block_scatter_kernel(const int
 }
 
 // Build, second pass: one block of the table at a time per CTA.  Its entries
-// are taken into registers, inserted in shared memory (first free slot at or
-// after the home bucket, slot 0 before slot 1, wrapping within the block),
-// counted along their chains, and the whole block is written over them: the
-// table is written once, in order, and needs no clearing.  A block keeps a
-// free slot, so every chain in it ends.  Bound by the instructions of the
-// insertion and by the writes.  With the passes before and the Bloom filter,
-// 4 * 10^6 rows take 148 us and 2^24 rows 705 us, where clearing the table, a
-// CAS and a chain walk per row and eight atomics on the filter took 364 and
-// 2352 us.
+// are taken into registers and put in shared memory as linear probing would
+// leave them (first free slot at or after the home bucket, slot 0 before slot
+// 1, wrapping within the block), counted along their chains, and the whole
+// block is written over them: the table is written once, in order, and needs
+// no clearing.  A block keeps a free slot, so every chain in it ends.
+//
+// No entry searches for its slot.  In the order of their home buckets, the
+// entries of bucket b take the slots from max(end of the bucket before, 2 b)
+// on, so the ends follow from a scan over the buckets' counts; what runs past
+// the last slot comes before bucket 0 in a second look at the same scan.  (By
+// CAS from slot to slot, many copies of a key in a block meet at every slot:
+// 100,000 rows, 1200 of one key: BUILD_A; 10^6 rows of 64 copies each: BUILD_B.)
+// Copies of a key lie in their home bucket's run of slots, so only the rest
+// of its own run is compared with an entry.
+// Bound by the instructions of that and by the writes.  With the passes
+// before and the Bloom filter, 4 * 10^6 rows take BUILD_C us and 2^24 rows BUILD_D, where
+// clearing the table, a CAS and a chain walk per row and eight atomics on the
+// filter took 364 and 2352 us.
 constexpr uint64_t JS_PART_MIN_N = 1ull << 22;                // smaller builds go row by row
 constexpr int JT_TPB = 512;
 constexpr int JT_SLOTS = 2 * static_cast<int>(JT_BLOCK);
 constexpr int JT_PER = JT_SLOTS / JT_TPB;
-constexpr int JT_BLOOM_MAX = 256;                             // filter blocks per table block in shared memory
-constexpr int JT_SMEM = JT_SLOTS * 16 + JT_BLOOM_MAX * 32;
+constexpr int JT_BLOOM_MAX = 128;                             // filter blocks per table block, at a load of 0.9
+constexpr int JT_SMEM = JT_SLOTS * 14 + static_cast<int>(JT_BLOCK) * 4 + JT_BLOOM_MAX * 32;
+static_assert(JT_BLOCK == 2 * JT_TPB, "two buckets per thread");
+static_assert(JT_SLOTS <= 2048, "places in 11 bits, ends in 16");
+
+// A stretch of buckets as a function of the slot its entries may start at:
+// they end at max(start + entries, least).
+struct Stretch {
+    unsigned entries, least;
+};
+__device__ __forceinline__ Stretch stretch_join(const Stretch& a, const Stretch& b) {
+    return Stretch{a.entries + b.entries, max(a.least + b.entries, b.least)};
+}
 
 __global__ void __launch_bounds__(JT_TPB, 3) join_block_build_kernel(ulonglong2* slots, uint64_t blocks, int block_log,
                                                                      uint32_t* bloom, int per_log, JoinCtl* ctl) {
     extern __shared__ __align__(16) unsigned char tsmem[];
     uint64_t* sk = reinterpret_cast<uint64_t*>(tsmem);                       // keys of the block's slots
     uint32_t* sr = reinterpret_cast<uint32_t*>(tsmem + JT_SLOTS * 8);        // their row-ids
-    uint32_t* sb = reinterpret_cast<uint32_t*>(tsmem + JT_SLOTS * 12);       // the block's filter words
-    __shared__ int copies;                                                   // some key of the block has several
+    uint16_t* sf = reinterpret_cast<uint16_t*>(tsmem + JT_SLOTS * 12);       // further copies of their keys
+    unsigned* run = reinterpret_cast<unsigned*>(tsmem + JT_SLOTS * 14);      // entries per bucket, then first slot | entries << 16
+    uint32_t* sb = run + JT_BLOCK;                                           // the block's filter words
+    __shared__ Stretch ws[JT_TPB / 32];
     if (ctl->crowded) return;                                                // (set by the pass before)
     const unsigned bm = (1u << block_log) - 1u;
     const unsigned nslots = 2u << block_log;
     const unsigned nwords = bloom ? (BLOOM_WORDS << per_log) : 0u;
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     uint64_t k[JT_PER];
     uint32_t r[JT_PER];
     auto cursor = [&](uint64_t blk) {
@@ -226,25 +249,17 @@ __global__ void __launch_bounds__(JT_TPB, 3) join_block_build_kernel(ulonglong2*
         ulonglong2* mine = slots + blk * nslots;
         for (unsigned i = threadIdx.x; i < nslots / 2; i += JT_TPB)
             reinterpret_cast<ulonglong2*>(sk)[i] = make_ulonglong2(JN_EMPTY, JN_EMPTY);
+        run[threadIdx.x] = 0u;
+        run[threadIdx.x + JT_TPB] = 0u;
         for (unsigned i = threadIdx.x; i < nwords; i += JT_TPB) sb[i] = 0u;
-        if (threadIdx.x == 0) copies = 0;
         __syncthreads();                                     // (every thread has its entries in registers)
-        bool met = false;                                    // a copy of a key of this thread on its way
+        unsigned at[JT_PER];                                 // home bucket | rank among its entries << 10
 #pragma unroll
         for (int j = 0; j < JT_PER; ++j) {
             if (k[j] == JN_EMPTY) continue;
             const uint64_t h = fmix64(k[j]);
-            unsigned at = 2u * (static_cast<unsigned>(h) & bm);
-            while (true) {
-                unsigned long long c = *reinterpret_cast<volatile unsigned long long*>(sk + at);
-                if (c == JN_EMPTY)
-                    c = atomicCAS(reinterpret_cast<unsigned long long*>(sk + at), JN_EMPTY,
-                                  static_cast<unsigned long long>(k[j]));
-                if (c == JN_EMPTY) break;
-                met = met || c == k[j];
-                at = (at + 1u) & (nslots - 1u);              // slot 1, then slot 0 of the next bucket
-            }
-            sr[at] = r[j];
+            const unsigned b = static_cast<unsigned>(h) & bm;
+            at[j] = b | atomicAdd(&run[b], 1u) << 10;
             if (nwords) {
                 // the lanes go through the words of their blocks in different
                 // orders: in the same order they would meet on four banks
@@ -257,34 +272,65 @@ __global__ void __launch_bounds__(JT_TPB, 3) join_block_build_kernel(ulonglong2*
                 }
             }
         }
-        if (met) copies = 1;
-        // the next block's entries, on their way while this block is finished
+        __syncthreads();
+        // Where the entries of the thread's two buckets start.
+        const unsigned b0 = 2u * threadIdx.x;
+        const uint2 c = reinterpret_cast<const uint2*>(run)[threadIdx.x];
+        Stretch incl{0u, 0u};                                // (no bucket there: a table of fewer)
+        if (b0 <= bm) incl = Stretch{c.x, 2u * b0 + c.x};
+        if (b0 < bm) incl = stretch_join(incl, Stretch{c.y, 2u * b0 + 2u + c.y});
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const Stretch before{__shfl_up_sync(0xFFFFFFFFu, incl.entries, o), __shfl_up_sync(0xFFFFFFFFu, incl.least, o)};
+            if (lane >= static_cast<unsigned>(o)) incl = stretch_join(before, incl);
+        }
+        if (lane == 31) ws[warp] = incl;
+        Stretch mine_from{__shfl_up_sync(0xFFFFFFFFu, incl.entries, 1), __shfl_up_sync(0xFFFFFFFFu, incl.least, 1)};
+        if (lane == 0) mine_from = Stretch{0u, 0u};
+        __syncthreads();
+        Stretch from{0u, 0u}, all{0u, 0u};
+#pragma unroll
+        for (unsigned w = 0; w < JT_TPB / 32; ++w) {
+            if (w == warp) from = all;
+            all = stretch_join(all, ws[w]);
+        }
+        from = stretch_join(from, mine_from);
+        const unsigned end = max(all.entries, all.least);    // of the last bucket, from slot 0
+        const unsigned wrapped = end > nslots ? end - nslots : 0u;
+        if (b0 <= bm) {
+            const unsigned f0 = max(max(wrapped + from.entries, from.least), 2u * b0);
+            const unsigned f1 = max(f0 + c.x, 2u * b0 + 2u);
+            reinterpret_cast<uint2*>(run)[threadIdx.x] = make_uint2(f0 | c.x << 16, f1 | c.y << 16);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < JT_PER; ++j) {
+            if (k[j] == JN_EMPTY) continue;
+            const unsigned p = ((run[at[j] & 1023u] & 0xFFFFu) + (at[j] >> 10)) & (nslots - 1u);
+            sk[p] = k[j];
+            sr[p] = r[j];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < JT_PER; ++j) {
+            if (k[j] == JN_EMPTY) continue;
+            const unsigned v = run[at[j] & 1023u];
+            const unsigned p = (v & 0xFFFFu) + (at[j] >> 10), stop = (v & 0xFFFFu) + (v >> 16);
+            unsigned f = 0;
+            for (unsigned q = p + 1u; q < stop; ++q) f += sk[q & (nslots - 1u)] == k[j] ? 1u : 0u;
+            sf[p & (nslots - 1u)] = static_cast<uint16_t>(f);
+        }
+        // the next block's entries, on their way while this block is written
         load(blk + gridDim.x, next_cnt);
         next_cnt = cursor(blk + 2ull * gridDim.x);
         __syncthreads();
-        // Of two copies of a key the one further along passed the other on
-        // its way, so a block where no thread met one has none to count.
-        const bool count = copies != 0;
-        for (unsigned b0 = threadIdx.x; b0 <= bm; b0 += JT_TPB) {            // a bucket at a time
-            const ulonglong2 kk = reinterpret_cast<const ulonglong2*>(sk)[b0];
-            const uint2 rr = reinterpret_cast<const uint2*>(sr)[b0];
-            uint32_t f0 = 0, f1 = 0;                                         // further copies
-            if (count) {
-                f0 = kk.x != JN_EMPTY && kk.y == kk.x ? 1u : 0u;
-                unsigned b = b0;
-                uint64_t k1 = kk.y;
-                while (k1 != JN_EMPTY) {                                     // bucket b full: the chain goes on
-                    b = (b + 1u) & bm;
-                    if (b == b0) break;                                      // (once round: a block keeps a free slot)
-                    const uint64_t k0 = sk[2 * b];
-                    k1 = sk[2 * b + 1];
-                    f0 += (k0 == kk.x) + (k1 == kk.x);
-                    f1 += (k0 == kk.y) + (k1 == kk.y);
-                }
-            }
-            const uint64_t w0 = kk.x == JN_EMPTY ? ~0ull : rr.x | (static_cast<uint64_t>(f0) << 32);
-            const uint64_t w1 = kk.y == JN_EMPTY ? ~0ull : rr.y | (static_cast<uint64_t>(f1) << 32);
-            asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(mine + 2 * b0), "l"(kk.x), "l"(w0), "l"(kk.y),
+        for (unsigned b = threadIdx.x; b <= bm; b += JT_TPB) {               // a bucket at a time
+            const ulonglong2 kk = reinterpret_cast<const ulonglong2*>(sk)[b];
+            const uint2 rr = reinterpret_cast<const uint2*>(sr)[b];
+            const unsigned ff = reinterpret_cast<const unsigned*>(sf)[b];
+            const uint64_t w0 = kk.x == JN_EMPTY ? ~0ull : rr.x | (static_cast<uint64_t>(ff & 0xFFFFu) << 32);
+            const uint64_t w1 = kk.y == JN_EMPTY ? ~0ull : rr.y | (static_cast<uint64_t>(ff >> 16) << 32);
+            asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(mine + 2 * b), "l"(kk.x), "l"(w0), "l"(kk.y),
                          "l"(w1)
                          : "memory");
         }
@@ -1210,12 +1256,11 @@ olap_status olap_join_build(olap_ctx* ctx, const int64_t* keys, const uint32_t* 
         t->bloom = reinterpret_cast<uint32_t*>(static_cast<unsigned char*>(mem) + slot_bytes + 256);
         t->bloom_blocks = bloom_blocks;
     }
-    // Two passes over table blocks; the general build when there are no rows,
-    // when a block's filter does not fit in shared memory, or when a block
-    // turned out crowded.
+    // Two passes over table blocks; the general build when there are no rows or
+    // when a block turned out crowded.
     const int grid = ctx->sm_count * 8;
     const int per_log = bloom_blocks ? log2_of(bloom_blocks) - log2_of(blocks) : 0;
-    bool general = n == 0 || (1 << per_log) > JT_BLOOM_MAX;
+    bool general = n == 0;
     JoinCtl hc{};
     auto read_ctl = [&]() -> olap_status {
         e = cudaMemcpyAsync(ctx->host_status, jc, sizeof(hc), cudaMemcpyDeviceToHost, ctx->stream);
