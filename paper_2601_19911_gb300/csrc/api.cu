@@ -3,9 +3,7 @@
 // come back) and the Top-K entry points.
 #include <algorithm>
 #include <cstring>
-#include <mutex>
 #include <string>
-#include <vector>
 
 #include "ctx.h"
 #include "topk.cuh"
@@ -32,89 +30,6 @@ bool within_budget(const olap_ctx* ctx, size_t extra) {
     const uint64_t held = ctx->scratch_bytes + ctx->dev_in_bytes + ctx->dev_out_bytes + ctx->table_bytes;
     return held + extra <= ctx->opts.mem_budget_bytes;
 }
-
-namespace devmem {
-
-namespace {
-struct Piece {
-    int dev;
-    void* p;
-    size_t cap;
-};
-std::mutex g_lock;
-std::vector<Piece> g_kept;
-int g_contexts[64] = {};
-
-void give_back(int dev) {                                    // with g_lock held, `dev` current
-    size_t w = 0;
-    for (const Piece& x : g_kept) {
-        if (x.dev == dev) cudaFree(x.p);
-        else g_kept[w++] = x;
-    }
-    g_kept.resize(w);
-}
-}  // namespace
-
-cudaError_t alloc(int dev, void** p, size_t bytes) {
-    cudaError_t e = cudaMalloc(p, bytes);
-    if (e != cudaErrorMemoryAllocation) return e;
-    cudaGetLastError();
-    {
-        std::lock_guard<std::mutex> guard(g_lock);
-        give_back(dev);
-    }
-    return cudaMalloc(p, bytes);
-}
-
-cudaError_t take(int dev, void** p, size_t bytes, size_t* cap) {
-    {
-        std::lock_guard<std::mutex> guard(g_lock);
-        size_t best = g_kept.size();
-        for (size_t i = 0; i < g_kept.size(); ++i)
-            if (g_kept[i].dev == dev && g_kept[i].cap >= bytes && g_kept[i].cap <= bytes + bytes / 2 + (1u << 20) &&
-                (best == g_kept.size() || g_kept[i].cap < g_kept[best].cap))
-                best = i;
-        if (best < g_kept.size()) {
-            *p = g_kept[best].p;
-            *cap = g_kept[best].cap;
-            g_kept[best] = g_kept.back();
-            g_kept.pop_back();
-            return cudaSuccess;
-        }
-    }
-    *cap = bytes;
-    return alloc(dev, p, bytes);
-}
-
-void give(int dev, void* p, size_t cap) {
-    {
-        std::lock_guard<std::mutex> guard(g_lock);
-        size_t held = cap;
-        int pieces = 1;
-        for (const Piece& x : g_kept)
-            if (x.dev == dev) {
-                held += x.cap;
-                ++pieces;
-            }
-        if (dev >= 0 && dev < 64 && g_contexts[dev] > 0 && held <= KEEP_TOTAL && pieces <= KEEP_BLOCKS) {
-            g_kept.push_back(Piece{dev, p, cap});
-            return;
-        }
-    }
-    cudaFree(p);
-}
-
-void context_created(int dev) {
-    std::lock_guard<std::mutex> guard(g_lock);
-    if (dev >= 0 && dev < 64) ++g_contexts[dev];
-}
-
-void context_gone(int dev) {
-    std::lock_guard<std::mutex> guard(g_lock);
-    if (dev >= 0 && dev < 64 && --g_contexts[dev] == 0) give_back(dev);
-}
-
-}  // namespace devmem
 
 static olap_status grow(olap_ctx* ctx, void** buf, size_t* have, size_t need, const char* what) {
     if (*have >= need) return OLAP_OK;
@@ -478,7 +393,7 @@ olap_status olap_ctx_create(const olap_opts* opts, olap_ctx** out) {
     }
     ctx->topk_geom = g;
     if ((e = cudaMallocHost(reinterpret_cast<void**>(&ctx->host_status), 64)) != cudaSuccess) return bail(e);
-    if ((e = cudaMalloc(&ctx->aux, OLAP_AUX_BYTES)) != cudaSuccess) return bail(e);
+    if ((e = devmem::alloc(ctx->device, &ctx->aux, OLAP_AUX_BYTES)) != cudaSuccess) return bail(e);
     if ((e = cudaMemset(ctx->aux, 0, OLAP_AUX_BYTES)) != cudaSuccess) return bail(e);
     devmem::context_created(ctx->device);
     ctx->counted = true;

@@ -858,7 +858,7 @@ olap_status olap_batch_create(olap_ctx* ctx, const olap_batch_item* items, uint6
         // [rank words | row-ids | counts], each 256-byte aligned
         const size_t rb = (part_entries * 8 + 255) & ~static_cast<size_t>(255);
         const size_t ib = (part_entries * 4 + 255) & ~static_cast<size_t>(255);
-        e = cudaMalloc(&part_buf, rb + ib + splits.size() * 8);
+        e = devmem::alloc(ctx->device, &part_buf, rb + ib + splits.size() * 8);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return cuda_fail(ctx, e, "batch part results");
@@ -957,12 +957,12 @@ olap_status olap_batch_create(olap_ctx* ctx, const olap_batch_item* items, uint6
         return cuda_fail(ctx, e, "batch streams");
     }
     b->grid_probe = ctx->sm_count * std::max(1, per_p);
-    if ((e = cudaMalloc(&b->d_items, std::max<uint64_t>(1, n_units) * sizeof(Item))) != cudaSuccess ||
-        (e = cudaMalloc(&b->d_merge, std::max<size_t>(1, merges.size()) * sizeof(Item))) != cudaSuccess ||
-        (e = cudaMalloc(&b->d_chunks, std::max<size_t>(1, chunks.size()) * sizeof(ProbeChunk))) != cudaSuccess ||
-        (e = cudaMalloc(reinterpret_cast<void**>(&b->d_next), 256)) != cudaSuccess ||
-        (e = cudaMalloc(&b->cand_r, static_cast<size_t>(b->grid_topk) * BT_CAND * 8)) != cudaSuccess ||
-        (e = cudaMalloc(&b->cand_rid, static_cast<size_t>(b->grid_topk) * BT_CAND * 4)) != cudaSuccess) {
+    if ((e = devmem::alloc(ctx->device, &b->d_items, std::max<uint64_t>(1, n_units) * sizeof(Item))) != cudaSuccess ||
+        (e = devmem::alloc(ctx->device, &b->d_merge, std::max<size_t>(1, merges.size()) * sizeof(Item))) != cudaSuccess ||
+        (e = devmem::alloc(ctx->device, &b->d_chunks, std::max<size_t>(1, chunks.size()) * sizeof(ProbeChunk))) != cudaSuccess ||
+        (e = devmem::alloc(ctx->device, &b->d_next, 256)) != cudaSuccess ||
+        (e = devmem::alloc(ctx->device, &b->cand_r, static_cast<size_t>(b->grid_topk) * BT_CAND * 8)) != cudaSuccess ||
+        (e = devmem::alloc(ctx->device, &b->cand_rid, static_cast<size_t>(b->grid_topk) * BT_CAND * 4)) != cudaSuccess) {
         cudaGetLastError();
         batch_release(b);
         return cuda_fail(ctx, e, "batch allocation");

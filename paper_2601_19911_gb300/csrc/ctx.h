@@ -8,6 +8,7 @@
 #include <set>
 #include <string>
 
+#include "devmem.h"
 #include "hostcopy.h"
 #include "olap.h"
 #include "topk.cuh"
@@ -87,7 +88,7 @@ struct olap_ctx {
     uint64_t table_bytes = 0;
     std::set<olap_join_table*> tables;
 
-    bool counted = false;             // among the device's live contexts (see DeviceMemory)
+    bool counted = false;             // among the device's live contexts (see devmem.h)
 
     std::string last_error;
 };
@@ -106,29 +107,6 @@ olap_status ensure_dev_out(olap_ctx* ctx, size_t bytes);
 olap_status ensure_pinned(olap_ctx* ctx);
 olap_status ensure_part(olap_ctx* ctx, size_t bytes);
 olap_status ensure_build_part(olap_ctx* ctx, size_t bytes);
-
-// Device memory of freed join tables, kept for the next table of about the
-// same size: a table's cudaMalloc and cudaFree take 370 us at 134 MB, twice
-// what building it takes.  Shared by the process's contexts and threads under
-// one lock; at most KEEP_TOTAL per device and KEEP_BLOCKS pieces; given back when
-// the device's last context goes and whenever an allocation of the library
-// fails for want of memory.  Tables of a context with a memory budget take no
-// part.
-namespace devmem {
-constexpr size_t KEEP_TOTAL = 2ull << 30;
-constexpr int KEEP_BLOCKS = 8;
-// cudaMalloc on the current device `dev`; gives the kept memory back and tries
-// again when there is not enough.
-cudaError_t alloc(int dev, void** p, size_t bytes);
-// Memory for a table: a kept piece of bytes to 1.5 * bytes (+ 1 MiB), or a new
-// one; *cap is its size.
-cudaError_t take(int dev, void** p, size_t bytes, size_t* cap);
-// Keep a table's memory (no work may use it any more), or free it.
-void give(int dev, void* p, size_t cap);
-// A context of `dev` was created / is going.
-void context_created(int dev);
-void context_gone(int dev);
-}  // namespace devmem
 
 // Partitions a probe of n rows against table t uses (1 = direct probe), and
 // the partition scratch it needs (0 for a direct probe).

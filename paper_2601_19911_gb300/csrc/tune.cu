@@ -133,8 +133,8 @@ extern "C" olap_status olap_autotune(olap_ctx* ctx, const olap_tune_request* req
         const bool w4 = key_bytes(req->topk_key_type) == 4;
         const size_t w = w4 ? 4 : 8;
         DevBuf keys, ok, orow;
-        if ((e = cudaMalloc(&keys.p, n * w)) != cudaSuccess || (e = cudaMalloc(&ok.p, kk * w)) != cudaSuccess ||
-            (e = cudaMalloc(&orow.p, kk * 4)) != cudaSuccess) {
+        if ((e = devmem::alloc(ctx->device, &keys.p, n * w)) != cudaSuccess || (e = devmem::alloc(ctx->device, &ok.p, kk * w)) != cudaSuccess ||
+            (e = devmem::alloc(ctx->device, &orow.p, kk * 4)) != cudaSuccess) {
             cudaGetLastError();
             return cuda_fail(ctx, e, "tuning allocation");
         }
@@ -187,9 +187,9 @@ extern "C" olap_status olap_autotune(olap_ctx* ctx, const olap_tune_request* req
         const uint64_t cap = std::max<uint64_t>(1, static_cast<uint64_t>(
                                                        std::ceil(static_cast<double>(np) * 1.05 + 4096.0)));
         DevBuf bk, pk, pairs, cnt;
-        if ((e = cudaMalloc(&bk.p, nb * 8)) != cudaSuccess || (e = cudaMalloc(&pk.p, std::max<uint64_t>(np, 1) * 8)) !=
-            cudaSuccess || (e = cudaMalloc(&pairs.p, cap * 8)) != cudaSuccess ||
-            (e = cudaMalloc(&cnt.p, 256)) != cudaSuccess) {
+        if ((e = devmem::alloc(ctx->device, &bk.p, nb * 8)) != cudaSuccess || (e = devmem::alloc(ctx->device, &pk.p, std::max<uint64_t>(np, 1) * 8)) !=
+            cudaSuccess || (e = devmem::alloc(ctx->device, &pairs.p, cap * 8)) != cudaSuccess ||
+            (e = devmem::alloc(ctx->device, &cnt.p, 256)) != cudaSuccess) {
             cudaGetLastError();
             return cuda_fail(ctx, e, "tuning allocation");
         }
