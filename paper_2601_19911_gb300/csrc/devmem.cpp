@@ -67,21 +67,30 @@ cudaError_t take(int dev, void** p, size_t bytes, size_t* cap) {
 }
 
 void give(int dev, void* p, size_t cap) {
-    {
-        std::lock_guard<std::mutex> guard(g_lock);
-        size_t held = cap;
-        int pieces = 1;
-        for (const Piece& x : g_kept)
-            if (x.dev == dev) {
-                held += x.cap;
-                ++pieces;
-            }
-        if (dev >= 0 && dev < 64 && g_contexts[dev] > 0 && held <= KEEP_TOTAL && pieces <= KEEP_BLOCKS) {
-            g_kept.push_back(Piece{dev, p, cap});
-            return;
+    std::lock_guard<std::mutex> guard(g_lock);
+    if (dev < 0 || dev >= 64 || g_contexts[dev] == 0 || cap > KEEP_TOTAL) {
+        cudaFree(p);
+        return;
+    }
+    size_t held = cap;
+    int pieces = 1;
+    for (const Piece& x : g_kept)
+        if (x.dev == dev) {
+            held += x.cap;
+            ++pieces;
+        }
+    size_t w = 0;
+    for (const Piece& x : g_kept) {                          // the oldest make room
+        if (x.dev == dev && (held > KEEP_TOTAL || pieces > KEEP_BLOCKS)) {
+            cudaFree(x.p);
+            held -= x.cap;
+            --pieces;
+        } else {
+            g_kept[w++] = x;
         }
     }
-    cudaFree(p);
+    g_kept.resize(w);
+    g_kept.push_back(Piece{dev, p, cap});
 }
 
 void context_created(int dev) {

@@ -4,9 +4,10 @@
 // A freed join table's memory is kept for the next table of about the same
 // size: a table's cudaMalloc and cudaFree take 370 us at 134 MB, twice what
 // building it takes.  Shared by the process's contexts and threads under one
-// lock; at most KEEP_TOTAL per device and KEEP_BLOCKS pieces; given back when
-// the device's last context goes and when an allocation of the library fails
-// for want of memory.  Contexts with a memory budget take no part.
+// lock; at most KEEP_TOTAL per device and KEEP_BLOCKS pieces, the oldest making
+// room for the newest; given back when the device's last context goes and when
+// an allocation of the library fails for want of memory.  Contexts with a
+// memory budget take no part.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -111,3 +111,23 @@ def test_every_device_allocation_may_get_it():
         text = re.sub(r"//.*", "", open(src).read())
         calls = len(re.findall(r"\bcudaMalloc(?:Async|Managed|Pitch)?\s*\(", text))
         assert calls == (2 if src.endswith("devmem.cpp") else 0), src
+
+
+def test_old_pieces_make_room(mem):
+    """Pieces of a size that is no longer asked for do not stay for good."""
+    _keep(mem, *[4096] * 8)                        # all places taken by small ones
+    p, cap = _take(mem, 100 * MIB)
+    mem.t_give(p, cap)
+    assert _take(mem, 100 * MIB)[0] == p
+    assert mem.t_used() == 7 * 4096 + 100 * MIB
+
+
+def test_kept_memory_is_bounded(mem):
+    _keep(mem, GIB, GIB, 100 * MIB)                # 2 GiB at most: the first one goes
+    assert mem.t_used() == GIB + 100 * MIB
+    _keep(mem, *[(10 + i * 40) * MIB for i in range(12)])
+    assert mem.t_used() <= 2 * GIB
+    p, cap = _take(mem, 3 * GIB)                   # too large to keep, and none goes for it
+    used = mem.t_used() - cap
+    mem.t_give(p, cap)
+    assert mem.t_used() == used
