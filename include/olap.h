@@ -160,6 +160,11 @@ const char* olap_last_error(const olap_ctx* ctx);
 void* olap_ctx_stream(const olap_ctx* ctx);
 /* Wait for all work the context enqueued. */
 olap_status olap_ctx_sync(olap_ctx* ctx);
+/* Free the device memory that the library keeps on `device` (of freed join
+ * tables, at most 2 GiB; see olap_join_free), for other allocators of the
+ * process; the library's own allocations do so by themselves.  *released, if
+ * not NULL, receives the bytes.  OLAP_E_INVALID for a bad device. */
+olap_status olap_device_trim(int device, uint64_t* released);
 /* 1 when the context copies pageable host memory with a kernel that reads it
  * directly (OLAP_HOST_AUTO on a device with host-page-table access), else 0;
  * 0 for NULL. */
@@ -421,7 +426,9 @@ olap_status olap_join_table_info(const olap_join_table* table, uint64_t* n_build
                                  uint64_t* n_side, uint64_t* bloom_bytes);
 
 /* Free a table (NULL is ignored).  Waits for the table's device to finish
- * work that may still read it. */
+ * work that may still read it.  A context without a memory budget keeps the
+ * memory for later builds (at most 2 GiB and 8 pieces per device, the oldest
+ * giving way) until the device's last context goes or olap_device_trim. */
 void olap_join_free(olap_join_table* table);
 
 /* ------------------------------------------------------------------------

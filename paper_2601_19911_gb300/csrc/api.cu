@@ -430,6 +430,24 @@ const char* olap_last_error(const olap_ctx* ctx) { return ctx ? ctx->last_error.
 
 void* olap_ctx_stream(const olap_ctx* ctx) { return ctx ? static_cast<void*>(ctx->stream) : nullptr; }
 
+olap_status olap_device_trim(int device, uint64_t* released) {
+    if (released) *released = 0;
+    int ndev = 0, cur = 0;
+    if (cudaGetDeviceCount(&ndev) != cudaSuccess || cudaGetDevice(&cur) != cudaSuccess) {
+        cudaGetLastError();
+        return OLAP_E_CUDA;
+    }
+    if (device < 0 || device >= ndev) return OLAP_E_INVALID;
+    if (cudaSetDevice(device) != cudaSuccess) {
+        cudaGetLastError();
+        return OLAP_E_CUDA;
+    }
+    const uint64_t bytes = devmem::trim(device);
+    cudaSetDevice(cur);
+    if (released) *released = bytes;
+    return OLAP_OK;
+}
+
 int olap_ctx_host_direct(const olap_ctx* ctx) { return ctx && ctx->host_direct ? 1 : 0; }
 
 olap_status olap_selftest_wait(olap_ctx* ctx, uint64_t limit_cycles, int32_t* out_status) {

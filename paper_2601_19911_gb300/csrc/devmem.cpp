@@ -93,6 +93,11 @@ void give(int dev, void* p, size_t cap) {
     g_kept.push_back(Piece{dev, p, cap});
 }
 
+uint64_t trim(int dev) {
+    std::lock_guard<std::mutex> guard(g_lock);
+    return give_back(dev);
+}
+
 void context_created(int dev) {
     std::lock_guard<std::mutex> guard(g_lock);
     if (dev >= 0 && dev < 64) ++g_contexts[dev];

@@ -5,9 +5,10 @@
 // size: a table's cudaMalloc and cudaFree take 370 us at 134 MB, twice what
 // building it takes.  Shared by the process's contexts and threads under one
 // lock; at most KEEP_TOTAL per device and KEEP_BLOCKS pieces, the oldest making
-// room for the newest; given back when the device's last context goes and when
-// an allocation of the library fails for want of memory.  Contexts with a
-// memory budget take no part.
+// room for the newest; given back when the device's last context goes, when an
+// allocation of the library fails for want of memory, and by olap_device_trim
+// for the process's other allocators.  Contexts with a memory budget take no
+// part.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -31,6 +32,8 @@ cudaError_t alloc(int dev, T** p, size_t bytes) {
 cudaError_t take(int dev, void** p, size_t bytes, size_t* cap);
 // Keep a piece (no work may use it any more), or free it.
 void give(int dev, void* p, size_t cap);
+// Free what is kept on `dev`, `dev` current; returns the bytes.
+uint64_t trim(int dev);
 // A context of `dev` was created / is going.
 void context_created(int dev);
 void context_gone(int dev);

@@ -29,7 +29,7 @@ MEM_HOST, MEM_HOST_PINNED, MEM_DEVICE = 0, 1, 2
 # Every symbol include/olap.h declares, checked by the ABI tests.
 EXPORTS = [
     "olap_ctx_create", "olap_ctx_destroy", "olap_last_error", "olap_ctx_stream", "olap_ctx_sync",
-    "olap_ctx_host_direct", "olap_selftest_wait",
+    "olap_device_trim", "olap_ctx_host_direct", "olap_selftest_wait",
     "olap_topk", "olap_topk_pair", "olap_topk_async", "olap_topk_noalloc", "olap_topk_info_last", "olap_topk_rows",
     "olap_ctx_time_kernels", "olap_kernel_ms_last", "olap_ctx_launches", "olap_autotune",
     "olap_join_build", "olap_join_probe", "olap_join_probe_async", "olap_join_probe_partitions",
@@ -204,6 +204,8 @@ def load(path: str | None = None):
         lib.olap_ctx_stream.argtypes = [vp]
         lib.olap_ctx_sync.restype = i32
         lib.olap_ctx_sync.argtypes = [vp]
+        lib.olap_device_trim.restype = i32
+        lib.olap_device_trim.argtypes = [i32, ctypes.POINTER(u64)]
         lib.olap_ctx_host_direct.restype = i32
         lib.olap_ctx_host_direct.argtypes = [vp]
         lib.olap_selftest_wait.restype = i32
@@ -707,6 +709,16 @@ class JoinTable:
             self.free()
         except Exception:
             pass
+
+
+def device_trim(device: int = 0) -> int:
+    """olap_device_trim: free the device memory the library keeps for later
+    join builds; returns the bytes."""
+    got = ctypes.c_uint64()
+    st = load().olap_device_trim(int(device), ctypes.byref(got))
+    if st != OK:
+        raise OlapError(st, f"olap_device_trim({device}) failed")
+    return got.value
 
 
 def topk_noalloc(d_keys, k: int, order: int, d_out_keys, d_out_rowids, d_rowids=None, dev_status=None,

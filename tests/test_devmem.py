@@ -8,7 +8,7 @@ import subprocess
 
 import pytest
 
-from paper_2601_19911_gb300 import build
+from paper_2601_19911_gb300 import build, olap
 
 CSRC = build.CSRC
 GIB, MIB = 1 << 30, 1 << 20
@@ -44,6 +44,7 @@ int t_sticky() { return last != cudaSuccess; }
 void* t_alloc(size_t n) { void* p = nullptr; return olap::devmem::alloc(0, &p, n) == cudaSuccess ? p : nullptr; }
 void* t_take(size_t n, size_t* cap) { void* p = nullptr; return olap::devmem::take(0, &p, n, cap) == cudaSuccess ? p : nullptr; }
 void t_give(void* p, size_t cap) { olap::devmem::give(0, p, cap); }
+uint64_t t_trim() { return olap::devmem::trim(0); }
 void t_context(int up) { if (up) olap::devmem::context_created(0); else olap::devmem::context_gone(0); }
 }
 """
@@ -60,6 +61,7 @@ def mem(tmp_path):
     for name in ("t_alloc", "t_take"):
         getattr(lib, name).restype = ctypes.c_void_p
     lib.t_used.restype = ctypes.c_size_t
+    lib.t_trim.restype = ctypes.c_uint64
     lib.t_alloc.argtypes = [ctypes.c_size_t]
     lib.t_take.argtypes = [ctypes.c_size_t, ctypes.POINTER(ctypes.c_size_t)]
     lib.t_give.argtypes = [ctypes.c_void_p, ctypes.c_size_t]
@@ -131,3 +133,17 @@ def test_kept_memory_is_bounded(mem):
     used = mem.t_used() - cap
     mem.t_give(p, cap)
     assert mem.t_used() == used
+
+
+def test_trim(mem):
+    _keep(mem, GIB, 10 * MIB)
+    assert mem.t_trim() == GIB + 10 * MIB
+    assert mem.t_used() == 0 and mem.t_trim() == 0
+    _keep(mem, MIB)                                # and keeping goes on
+    assert mem.t_used() == MIB
+
+
+def test_trim_of_a_bad_device():
+    with pytest.raises(olap.OlapError) as ei:
+        olap.device_trim(-1)
+    assert ei.value.status in (olap.E_INVALID, olap.E_CUDA)
