@@ -161,7 +161,7 @@ void* olap_ctx_stream(const olap_ctx* ctx);
 /* Wait for all work the context enqueued. */
 olap_status olap_ctx_sync(olap_ctx* ctx);
 /* Free the device memory that the library keeps on `device` (of freed join
- * tables, at most 2 GiB; see olap_join_free), for other allocators of the
+ * tables and large builds, at most 2 GiB; see olap_join_free), for other allocators of the
  * process; the library's own allocations do so by themselves.  *released, if
  * not NULL, receives the bytes.  OLAP_E_INVALID for a bad device. */
 olap_status olap_device_trim(int device, uint64_t* released);

@@ -81,10 +81,6 @@ olap_status ensure_part(olap_ctx* ctx, size_t bytes) {
     return grow(ctx, &ctx->part, &ctx->part_bytes, bytes, "probe partition allocation");
 }
 
-olap_status ensure_build_part(olap_ctx* ctx, size_t bytes) {
-    return grow(ctx, &ctx->build_part, &ctx->build_part_bytes, bytes, "build partition allocation");
-}
-
 olap_status ensure_pinned(olap_ctx* ctx) {
     if (ctx->pinned_bytes) return OLAP_OK;
     const size_t b = ctx->opts.staging_bytes ? ctx->opts.staging_bytes : (64ull << 20);
@@ -409,7 +405,6 @@ void olap_ctx_destroy(olap_ctx* ctx) {
     if (ctx->dev_in) cudaFree(ctx->dev_in);
     if (ctx->dev_out) cudaFree(ctx->dev_out);
     if (ctx->part) cudaFree(ctx->part);
-    if (ctx->build_part) cudaFree(ctx->build_part);
     if (ctx->rows_buf) cudaFree(ctx->rows_buf);
     for (int i = 0; i < 2; ++i) {
         if (ctx->pinned[i]) cudaFreeHost(ctx->pinned[i]);

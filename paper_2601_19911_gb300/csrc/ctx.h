@@ -70,10 +70,6 @@ struct olap_ctx {
     // Partitioned-probe scratch (grow-only): partitioned keys and row-ids.
     void* part = nullptr;
     size_t part_bytes = 0;
-    // The same for a large build, which must neither move the probes' scratch
-    // (captured probes hold its address) nor write into a queued probe's rows.
-    void* build_part = nullptr;
-    size_t build_part_bytes = 0;
     uint64_t l2_bytes = 0;            // device L2 size
     bool host_direct = false;         // copy pageable host memory with a kernel (no CPU staging)
 
@@ -106,7 +102,6 @@ olap_status ensure_dev_in(olap_ctx* ctx, size_t bytes);
 olap_status ensure_dev_out(olap_ctx* ctx, size_t bytes);
 olap_status ensure_pinned(olap_ctx* ctx);
 olap_status ensure_part(olap_ctx* ctx, size_t bytes);
-olap_status ensure_build_part(olap_ctx* ctx, size_t bytes);
 
 // Partitions a probe of n rows against table t uses (1 = direct probe), and
 // the partition scratch it needs (0 for a direct probe).

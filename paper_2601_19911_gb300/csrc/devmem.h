@@ -2,8 +2,9 @@
 // for reuse, and the pieces that join builds keep.
 //
 // A freed join table's memory is kept for the next table of about the same
-// size: a table's cudaMalloc and cudaFree take 370 us at 134 MB, twice what
-// building it takes.  Shared by the process's contexts and threads under one
+// size, and the partition scratch of a large build for the next one: a
+// table's cudaMalloc and cudaFree take 370 us at 134 MB, twice what building
+// it takes.  Shared by the process's contexts and threads under one
 // lock; at most KEEP_TOTAL per device and KEEP_BLOCKS pieces, the oldest making
 // room for the newest; given back when the device's last context goes, when an
 // allocation of the library fails for want of memory, and by olap_device_trim

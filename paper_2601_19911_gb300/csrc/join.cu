@@ -1249,9 +1249,20 @@ olap_status olap_join_build(olap_ctx* ctx, const int64_t* keys, const uint32_t* 
     }
     t->slots = static_cast<ulonglong2*>(mem);
     t->bytes = bytes;
+    ctx->table_bytes += bytes;                               // counted from here on: the scratch below is checked beside it
+    // Partition scratch of a large build, for the time of the build.
+    void* part = nullptr;
+    size_t part_cap = 0;
     JoinCtl* jc = reinterpret_cast<JoinCtl*>(static_cast<unsigned char*>(mem) + slot_bytes);
+    auto drop_part = [&]() {                                 // (no work uses it any more)
+        if (part && keep) devmem::give(ctx->device, part, part_cap);
+        else if (part) cudaFree(part);
+        part = nullptr;
+    };
     auto bail = [&](olap_status st) {
         cudaStreamSynchronize(ctx->stream);                  // launched passes may still write it
+        drop_part();
+        ctx->table_bytes -= bytes;
         cudaFree(mem);
         delete t;
         return st;
@@ -1290,19 +1301,25 @@ olap_status olap_join_build(olap_ctx* ctx, const int64_t* keys, const uint32_t* 
         const uint32_t* br = dr;
         if (blocks > static_cast<uint64_t>(JS_BINS) && n >= JS_PART_MIN_N) {
             const PartGrids pg = part_grids(ctx->device, ctx->sm_count);
-            const size_t pb = probe_part_bytes(n, JS_PARTS);
-            if (pg.count && ensure_build_part(ctx, pb + PART_COUNT_BYTES) == OLAP_OK) {
-                void* counts = static_cast<unsigned char*>(ctx->build_part) + pb;
+            const size_t pb = probe_part_bytes(n, JS_PARTS), want = pb + PART_COUNT_BYTES;
+            if (pg.count && within_budget(ctx, want)) {
+                e = keep ? devmem::take(ctx->device, &part, want, &part_cap) : devmem::alloc(ctx->device, &part, want);
+                if (e != cudaSuccess) {
+                    cudaGetLastError();
+                    part = nullptr;
+                }
+            }
+            if (part) {
+                void* counts = static_cast<unsigned char*>(part) + pb;
                 e = cudaMemsetAsync(counts, 0, PART_COUNT_BYTES, ctx->stream);
                 if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "partition counts"));
-                const PartArgs q = part_args(ctx->build_part, counts, dk, dr, n, buckets, JS_PARTS);
+                const PartArgs q = part_args(part, counts, dk, dr, n, buckets, JS_PARTS);
                 launch_after(join_part_count_kernel, pg.count, JQ_TPB, 0, ctx->stream, false, q);
                 launch_after(part_scatter(JS_PARTS), pg.scatter, JQ_TPB, 0, ctx->stream, true, q);
                 ctx->launches += 2;
                 bk = q.out_keys;
                 br = q.out_rowids;
             }
-            ctx->last_error.clear();
         }
         const uint64_t threads = static_cast<uint64_t>(sgrid) * JS_TPB;
         const int per = static_cast<int>(std::min<uint64_t>((n + threads - 1) / threads, JS_PER));
@@ -1316,6 +1333,7 @@ olap_status olap_join_build(olap_ctx* ctx, const int64_t* keys, const uint32_t* 
         ctx->launches += 2;
         olap_status st = read_ctl();
         if (st != OLAP_OK) return bail(st);
+        drop_part();
         t->chain_mask = (1ull << block_log) - 1;
         general = hc.crowded != 0;
     }
@@ -1353,8 +1371,8 @@ olap_status olap_join_build(olap_ctx* ctx, const int64_t* keys, const uint32_t* 
         }
         t->n_side = hc.side_count;
         t->bytes += hc.side_count * 4;
+        ctx->table_bytes += hc.side_count * 4;
     }
-    ctx->table_bytes += t->bytes;
     ctx->tables.insert(t);
     t->owner = ctx;
     *out = t;
