@@ -27,7 +27,8 @@ olap_status cuda_fail(olap_ctx* ctx, cudaError_t e, const char* what) {
 
 bool within_budget(const olap_ctx* ctx, size_t extra) {
     if (ctx->opts.mem_budget_bytes == 0) return true;
-    const uint64_t held = ctx->scratch_bytes + ctx->dev_in_bytes + ctx->dev_out_bytes + ctx->table_bytes;
+    const uint64_t held = ctx->scratch_bytes + ctx->dev_in_bytes + ctx->dev_out_bytes + ctx->rows_buf_bytes +
+                          ctx->part_bytes + ctx->table_bytes;
     return held + extra <= ctx->opts.mem_budget_bytes;
 }
 

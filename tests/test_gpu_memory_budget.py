@@ -65,3 +65,25 @@ def test_scratch_is_kept_and_returned_without_a_budget(sides):
             _check(ctx, t, sides)
             t.free()
         assert TABLE + SCRATCH <= olap.device_trim(0) < TABLE + SCRATCH + 4 * MIB
+
+
+def test_probe_and_row_scratch_count():
+    """What a partitioned probe and a full-row Top-K hold on to is part of the
+    cap that later calls are checked against."""
+    keys = torch.randint(-(1 << 62), 1 << 62, (1 << 20,), device="cuda")
+    table = (1 << 20) * 64                               # bytes of its table, at most
+    out = torch.empty((1 << 20, 2), dtype=torch.int32, device="cuda")
+    rows = torch.randint(0, 255, (1 << 20, 16), dtype=torch.uint8, device="cuda")
+    for use in ("probe", "rows"):
+        with olap.Context(0, mem_budget_bytes=2 * table + 8 * MIB, join_partitions=16) as ctx:
+            t = ctx.join_build(keys)
+            ctx.join_build(keys).free()                  # room for a second one
+            if use == "probe":
+                ctx.join_probe(t, keys, out=out)         # 12 MiB of partitioned rows
+            else:
+                ctx.topk_rows(rows, 16, 0, olap.KEY_I64, 100)    # 8 MiB of keys, and the selection's scratch
+            with pytest.raises(olap.OlapError) as ei:
+                ctx.join_build(keys)
+            assert ei.value.status == olap.E_NOMEM
+            t.free()
+            ctx.join_build(keys).free()                  # one still fits
