@@ -171,10 +171,10 @@ olap_status olap_device_trim(int device, uint64_t* released);
 int olap_ctx_host_direct(const olap_ctx* ctx);
 /* Self-test of the bounded device-side waits (every spin in the library
  * gives up after a limit and reports OLAP_E_TIMEOUT instead of hanging): one
- * thread runs the grid barriers' wait on a device word that nothing writes,
- * for at most limit_cycles (1 .. 2^31) SM clock cycles, then returns.
- * *out_status receives the device status the wait recorded -- OLAP_E_TIMEOUT
- * when the bound works.  Returns OLAP_E_INVALID for a bad limit, else OLAP_OK
+ * CTA runs the grid barriers' wait on a device word that nothing writes, for
+ * at most limit_cycles (1 .. 2^31) SM clock cycles, then returns, beside one
+ * that reports success.  *out_status receives the status as a blocking call
+ * reads it -- OLAP_E_TIMEOUT when the bound works and the host hears of it.  Returns OLAP_E_INVALID for a bad limit, else OLAP_OK
  * (or E_CUDA).  The context stays usable. */
 olap_status olap_selftest_wait(olap_ctx* ctx, uint64_t limit_cycles, int32_t* out_status);
 

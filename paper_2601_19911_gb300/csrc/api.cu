@@ -156,10 +156,25 @@ static olap_status direct_copy(olap_ctx* ctx, void* dst, const void* src, size_t
     return OLAP_OK;
 }
 
-// Self-test of the bounded device waits: one thread waits, with the wait
-// the grid barriers use, on a word that nothing writes.
-__global__ void wait_selftest_kernel(const unsigned* word, int* err, long long limit) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) wait_changed(word, 0u, err, limit);
+// Self-test of the bounded device waits: CTA 1 waits, with the wait the grid
+// barriers use, on a word that nothing writes, after CTA 0 has reported that all
+// is well.
+__global__ void wait_selftest_kernel(const unsigned* word, int* err, long long limit, int32_t* status,
+                                     int32_t* host_err) {
+    if (threadIdx.x != 0) return;
+    if (blockIdx.x == 0) *status = OLAP_OK;
+    else if (!wait_changed(word, 0u, err, limit)) raise_expiry(err, host_err);
+}
+
+// The status of a blocking call in the context's page-locked words: [0] CTA 0's
+// (not OLAP_OK until it has one), [1] any other CTA's error.
+static void status_reset(olap_ctx* ctx) {
+    ctx->host_status[0] = OLAP_E_CUDA;
+    ctx->host_status[1] = OLAP_OK;
+}
+static olap_status status_read(const olap_ctx* ctx) {                 // after the call's work
+    const volatile int32_t* w = ctx->host_status;
+    return static_cast<olap_status>(w[1] != OLAP_OK ? w[1] : w[0]);
 }
 
 olap_status copy_h2d(olap_ctx* ctx, void* dst, const void* src, size_t bytes, olap_mem where) {
@@ -257,7 +272,7 @@ static olap_status topk_enqueue(olap_ctx* ctx, const void* d_keys, olap_key_type
                                 const uint32_t* d_rowids, uint64_t n, uint64_t kk, olap_order order,
                                 void* d_out_keys, uint32_t* d_out_rowids, int32_t* dev_status,
                                 cudaStream_t stream, TopkCtl** ctl_out, const PairSpec* pair = nullptr,
-                                const void* host_keys = nullptr) {
+                                const void* host_keys = nullptr, int32_t* host_err = nullptr) {
     TopkArgs a{};
     a.keys = d_keys;
     a.host_keys = host_keys;
@@ -270,6 +285,7 @@ static olap_status topk_enqueue(olap_ctx* ctx, const void* d_keys, olap_key_type
     a.out_keys = d_out_keys;
     a.out_rowids = d_out_rowids;
     a.dev_status = dev_status;
+    a.host_err = host_err;
     if (pair) {
         a.pair = 1;
         a.w4 = 0;                                           // 64-bit composite rank words
@@ -456,14 +472,13 @@ olap_status olap_selftest_wait(olap_ctx* ctx, uint64_t limit_cycles, int32_t* ou
     unsigned* word = static_cast<unsigned*>(ctx->aux) + 512;
     int* err = reinterpret_cast<int*>(static_cast<unsigned*>(ctx->aux) + 520);
     if ((e = cudaMemsetAsync(word, 0, 64, ctx->stream)) != cudaSuccess) return cuda_fail(ctx, e, "self-test reset");
-    wait_selftest_kernel<<<1, 32, 0, ctx->stream>>>(word, err, static_cast<long long>(limit_cycles));
+    status_reset(ctx);
+    wait_selftest_kernel<<<2, 32, 0, ctx->stream>>>(word, err, static_cast<long long>(limit_cycles), ctx->host_status,
+                                                    ctx->host_status + 1);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "self-test launch");
     ctx->launches += 1;
-    if ((e = cudaMemcpyAsync(ctx->host_status, err, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream)) !=
-            cudaSuccess ||
-        (e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess)
-        return cuda_fail(ctx, e, "self-test wait");
-    *out_status = *ctx->host_status;
+    if ((e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) return cuda_fail(ctx, e, "self-test wait");
+    *out_status = status_read(ctx);
     return OLAP_OK;
 }
 
@@ -651,9 +666,10 @@ olap_status olap_topk(olap_ctx* ctx, const void* keys, olap_key_type type, const
         dok = ctx->dev_out;
         dor = reinterpret_cast<uint32_t*>(static_cast<unsigned char*>(ctx->dev_out) + okb);
     }
-    // the kernels write the status into the context's page-locked word
-    *ctx->host_status = OLAP_E_CUDA;
-    st = topk_enqueue(ctx, dk, type, dr, n, kk, order, dok, dor, ctx->host_status, ctx->stream, nullptr, nullptr, hk);
+    // the kernels write the status into the context's page-locked words
+    status_reset(ctx);
+    st = topk_enqueue(ctx, dk, type, dr, n, kk, order, dok, dor, ctx->host_status, ctx->stream, nullptr, nullptr, hk,
+                      ctx->host_status + 1);
     if (st != OLAP_OK) return st;
     ctx->last_rowids_in_place = rowids_in_place;
     if (copy_out) {
@@ -664,9 +680,9 @@ olap_status olap_topk(olap_ctx* ctx, const void* keys, olap_key_type type, const
     }
     e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "Top-K");
-    if (*ctx->host_status != OLAP_OK) {
+    if ((st = status_read(ctx)) != OLAP_OK) {
         ctx->barrier_dirty = true;
-        return fail(ctx, static_cast<olap_status>(*ctx->host_status), "Top-K device wait expired");
+        return fail(ctx, st, "Top-K device wait expired");
     }
     *out_count = kk;
     return OLAP_OK;
@@ -733,8 +749,9 @@ olap_status olap_topk_pair(olap_ctx* ctx, const void* keys0, olap_key_type type0
         dor = reinterpret_cast<uint32_t*>(m + 2 * ob);
     }
     const PairSpec ps{d1, type1, order1, do1};
-    *ctx->host_status = OLAP_E_CUDA;
-    if ((st = topk_enqueue(ctx, d0, type0, dr, n, kk, order0, do0, dor, ctx->host_status, ctx->stream, nullptr, &ps)) !=
+    status_reset(ctx);
+    if ((st = topk_enqueue(ctx, d0, type0, dr, n, kk, order0, do0, dor, ctx->host_status, ctx->stream, nullptr, &ps,
+                           nullptr, ctx->host_status + 1)) !=
         OLAP_OK)
         return st;
     ctx->last_rowids_in_place = rowids_in_place;
@@ -745,9 +762,9 @@ olap_status olap_topk_pair(olap_ctx* ctx, const void* keys0, olap_key_type type0
     }
     e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "Top-K");
-    if (*ctx->host_status != OLAP_OK) {
+    if ((st = status_read(ctx)) != OLAP_OK) {
         ctx->barrier_dirty = true;
-        return fail(ctx, static_cast<olap_status>(*ctx->host_status), "Top-K device wait expired");
+        return fail(ctx, st, "Top-K device wait expired");
     }
     *out_count = kk;
     return OLAP_OK;

@@ -162,6 +162,13 @@ __device__ __forceinline__ bool wait_changed(const unsigned* word, unsigned old,
     return true;
 }
 
+// A CTA that gives up says so where the host looks (NULL: nowhere).  CTA 0's
+// status alone would not do: it may have passed the last barrier and reported
+// that all is well before another CTA's wait ran out.
+__device__ __forceinline__ void raise_expiry(const int* err, int32_t* host_err) {
+    if (host_err) *host_err = ld_volatile_i32(err);
+}
+
 __device__ __forceinline__ bool grid_sync(GridBar* bar, int* err, unsigned& target) {
     target += gridDim.x;
     __syncthreads();

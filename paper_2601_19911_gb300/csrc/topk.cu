@@ -1110,9 +1110,12 @@ __device__ __forceinline__ uint64_t merge_path(const uint64_t* ar, const uint32_
     return lo;
 }
 
-// Early exit after an expired wait: CTA 0 publishes the device status.
+// Early exit after an expired wait: CTA 0 publishes the device status, and a
+// blocking call hears of every CTA.
 __device__ __forceinline__ void report(const TopkArgs& a) {
-    if (blockIdx.x == 0 && threadIdx.x == 0 && a.dev_status) *a.dev_status = ld_volatile_i32(&a.ctl->err);
+    if (threadIdx.x != 0) return;
+    raise_expiry(&a.ctl->err, a.host_err);
+    if (blockIdx.x == 0 && a.dev_status) *a.dev_status = ld_volatile_i32(&a.ctl->err);
 }
 
 }  // namespace

@@ -128,7 +128,8 @@ struct TopkArgs {
     int desc2;
     const void* keys2;
     void* out_keys2;
-    int32_t* dev_status;             // optional device status word
+    int32_t* dev_status;             // optional status word, written by CTA 0
+    int32_t* host_err;               // optional, zero before the call: the error of any CTA that gave up
 };
 
 // Plan of one Top-K call: which path and how much scratch it needs.
