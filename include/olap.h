@@ -442,7 +442,10 @@ void olap_join_free(olap_join_table* table);
  * capacity).  All pointers are device pointers; count is a device uint64;
  * status (device int32, may be NULL) receives OLAP_OK or OLAP_E_DEVICE when
  * the device-side check of the descriptor rejects it.  The items' buffers
- * must outlive the batch; their contents may change between runs.
+ * must outlive the batch; their contents may change between runs.  Items run
+ * at the same time and in no order, except that all probes come before all
+ * Top-K items where one of each share memory that either writes (without
+ * batch_overlap).
  * ------------------------------------------------------------------------ */
 typedef struct olap_batch olap_batch;
 

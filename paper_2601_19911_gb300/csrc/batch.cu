@@ -686,6 +686,7 @@ struct olap_batch {
     // Overlap: the probe branch runs on a second stream forked from the
     // launch stream inside the graph (the two kernels are independent).
     bool overlap = false;
+    bool probe_first = false;             // probe and Top-K items share memory: see items_share
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int digit = 12;                       // radix digit width of the per-CTA Top-K
@@ -695,6 +696,45 @@ struct olap_batch {
 };
 
 namespace {
+
+// Whether a Top-K item and a probe item share memory that one of them writes.
+// The probe kernel runs beside the Top-K kernel's last items, so such batches
+// keep the order in which every probe comes first.
+bool items_share(const std::vector<Item>& items) {
+    struct Span {
+        uintptr_t lo, hi;
+        int who;                              // 0 Top-K, 1 probe
+        bool write;
+    };
+    std::vector<Span> v;
+    for (const Item& d : items) {
+        const int who = d.op == OLAP_OP_PROBE ? 1 : 0;
+        auto add = [&](const void* p, uint64_t bytes, bool write) {
+            const uintptr_t lo = reinterpret_cast<uintptr_t>(p);
+            if (p && bytes) v.push_back({lo, lo + bytes, who, write});
+        };
+        const uint64_t w = who == 0 && d.w4 ? 4 : 8, kk = std::min<uint64_t>(d.k, d.n);
+        add(d.keys, d.n * w, false);
+        add(d.rowids, d.n * 4, false);
+        if (who == 0) {
+            add(d.out_keys, kk * w, true);
+            add(d.out_rowids, kk * 4, true);
+        } else {
+            add(d.out_pairs, std::min<uint64_t>(d.cap, 1ull << 48) * 8, true);
+        }
+        add(d.count, 8, true);
+        add(d.status, 4, true);
+    }
+    std::sort(v.begin(), v.end(), [](const Span& a, const Span& b) { return a.lo < b.lo; });
+    uintptr_t read_to[2] = {0, 0}, written_to[2] = {0, 0};   // ends of the ranges so far, by kind of item
+    for (const Span& x : v) {
+        const int other = 1 - x.who;
+        if (x.lo < written_to[other] || (x.write && x.lo < read_to[other])) return true;
+        uintptr_t& to = x.write ? written_to[x.who] : read_to[x.who];
+        to = std::max(to, x.hi);
+    }
+    return false;
+}
 
 olap_status enqueue_batch(olap_batch* b, cudaStream_t s) {
     // queue heads and the error count live in one 256-byte block
@@ -714,20 +754,24 @@ olap_status enqueue_batch(olap_batch* b, cudaStream_t s) {
             probe_items, b->n_probe, b->d_errors);
         ++b->graph_kernels;
     }
+    auto probes = [&](bool after) {
+        if (!b->n_chunks) return;
+        launch_after(batch_probe_kernel, static_cast<unsigned>(b->grid_probe), JP_TPB, JP_SMEM, ps, after, probe_items,
+                     static_cast<const ProbeChunk*>(b->d_chunks), b->n_chunks, b->d_next + 1);
+        ++b->graph_kernels;
+    };
+    if (b->probe_first) probes(false);
     if (b->n_topk) {
         batch_topk_kernel<<<b->grid_topk, BT_TPB, BT_SMEM, s>>>(b->d_items, b->n_topk, b->d_next, b->cand_r,
                                                                 b->cand_rid, b->d_errors, b->digit);
         ++b->graph_kernels;
     }
-    if (b->n_chunks) {
+    if (!b->probe_first) {
         // Behind the Top-K kernel, whose last items leave CTAs idle one by
         // one: the probe's (independent, and in far shorter chunks) take their
         // places.  512 + 128 items 638 -> 565 us; with the probe first, or two
         // branches that share the memory from the start, the idle time stays.
-        launch_after(batch_probe_kernel, static_cast<unsigned>(b->grid_probe), JP_TPB, JP_SMEM, ps,
-                     b->n_topk > 0 && !b->overlap, probe_items, static_cast<const ProbeChunk*>(b->d_chunks), b->n_chunks,
-                     b->d_next + 1);
-        ++b->graph_kernels;
+        probes(b->n_topk > 0 && !b->overlap);
     }
     if (b->n_merge) {          // after every part: the merges of split items
         const unsigned mg = static_cast<unsigned>(std::min<uint64_t>(b->n_merge, b->grid_topk));
@@ -811,6 +855,7 @@ olap_status olap_batch_create(olap_ctx* ctx, const olap_batch_item* items, uint6
         if (!x.count) return fail(ctx, OLAP_E_INVALID, "batch item: NULL count");
         if (x.n >= (1ull << 32)) return fail(ctx, OLAP_E_INVALID, "batch item: n must be below 2^32");
     }
+    const bool mixed = items_share(dev);
     // Top-K items first, then probe items; each group largest first, so the
     // long items start early and short ones fill in.
     std::vector<uint64_t> order(n_items);
@@ -948,6 +993,7 @@ olap_status olap_batch_create(olap_ctx* ctx, const olap_batch_item* items, uint6
     const int topk_per_sm = ctx->opts.batch_topk_ctas_per_sm > 0 ? ctx->opts.batch_topk_ctas_per_sm : 2;
     b->grid_topk = ctx->sm_count * std::max(1, std::min(per_t, topk_per_sm));
     b->overlap = ctx->opts.batch_overlap == 1 && n_topk > 0 && n_units > n_topk;
+    b->probe_first = mixed && !b->overlap;
     if (b->overlap &&
         ((e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking)) != cudaSuccess ||
          (e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming)) != cudaSuccess ||
