@@ -14,6 +14,9 @@ between steps.
 K, single thread) on a bounded sample of the same workload instead.
 Under torchrun each rank runs an independent replica on its own GPU ("replicas
 only": the selection needs no exchange); rank 0 prints the max-over-ranks time.
+
+Standard output gets one short JSON line; the report with every leg's sweeps
+and rooflines goes to standard error, as one JSON line too.
 """
 from __future__ import annotations
 
@@ -122,6 +125,33 @@ class ClockSampler:
             return {"sm_mhz": None, "sm_max_mhz": None, "reasons": ["unavailable"], "samples": 0}
         return {"sm_mhz": float(np.median(sm)), "sm_max_mhz": mx, "mem_mhz": float(np.median(mem)),
                 "mem_mhz_min": float(np.min(mem)), "reasons": sorted(reasons), "samples": len(sm)}
+
+
+# What the one line on standard output keeps of each part of the report, which
+# goes to standard error whole (its sweeps are some tens of kilobytes).
+HEADLINE_PARTS = {
+    "config": None,
+    "roofline": ("bound", "achieved", "peak", "unit", "frac", "traffic", "peak_kind", "kernel",
+                 "algorithmic_bytes_per_launch", "kernel_ms", "call_ms"),
+    "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "rowid_bytes_read_in_place", "ms_per_step"),
+    "clocks": None,
+    "cpu_baseline": ("value", "unit", "cores", "kind"),
+}
+
+
+def headline(report: dict) -> dict:
+    """The report without its sweeps: every scalar, the parts above, and of
+    each further leg its value, unit and time per step."""
+    line = {}
+    for key, v in report.items():
+        if not isinstance(v, dict):
+            line[key] = v
+            continue
+        keep = HEADLINE_PARTS.get(key, ("value", "unit", "ms_per_step"))
+        part = dict(v) if keep is None else {k: v[k] for k in keep if k in v}
+        if part:
+            line[key] = part
+    return line
 
 
 def _dist():
@@ -265,7 +295,8 @@ def join_leg(args, ctx, torch, world):
         "metric": "join probes/s", "unit": "Gprobes/s", "value": world * npr / (ms * 1e-3) / 1e9,
         "ms_per_step": ms, "steps": steps, "ms_median": _median_p95(per)[0], "ms_p95": _median_p95(per)[1],
         "cell": {"build_rows": nb, "build": mult, "probe_rows": npr, "dist": dist, "hit_rate": hit,
-                 "pairs": need, "pairs_per_probe": m, "buckets": info["n_buckets"], "load": 0.5,
+                 "pairs": need, "pairs_per_probe": m, "buckets": info["n_buckets"],
+                 "load": nb / (2 * info["n_buckets"]),
                  "rowids": "implicit", "probe_partitions": parts, "prefiltered": pinfo["prefiltered"],
                  "rows_probed_after_prefilter": pinfo["rows_probed"]},
         "build": {"ms": build_s * 1e3, "Grows_per_s": nb / build_s / 1e9},
@@ -1266,7 +1297,8 @@ def run_ours(args):
         line["cpu_baseline"] = cpu_baseline(n, k)
         line["cpu_baseline"]["host"] = _host_info()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     ctx.close()
     if world > 1:
         import torch.distributed as dist
