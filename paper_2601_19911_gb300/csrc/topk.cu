@@ -1562,25 +1562,14 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
             }
             __syncthreads();
         }
-        if (stamp) ctl->ts[7] = gtimer();
-        if (a.k <= TK_SMALL) {
-            const int cnt = static_cast<int>(a.k);
-            for (int i = threadIdx.x; i < cnt; i += TK_TPB) {
-                sr[i] = __ldcg(a.out_r0 + i);
-                srid[i] = __ldcg(a.out_rid0 + i);
-            }
-            __syncthreads();
-            block_sort<TK_TPB>(sr, srid, cnt);
-            if (stamp) ctl->ts[8] = gtimer();
-            for (int i = threadIdx.x; i < cnt; i += TK_TPB) write_result(a, i, sr[i], srid[i]);
-            if (threadIdx.x == 0 && a.dev_status) *a.dev_status = ld_volatile_i32(&ctl->err);
-            if (threadIdx.x == 0) ctl->ts[6] = gtimer();
+        if (stamp) {
+            ctl->ts[7] = gtimer();
+            ctl->ts[8] = ctl->ts[7];
         }
     }
-    if (a.k <= TK_SMALL) return;
     if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
 
-    // K > 4096: sort tiles of TK_SMALL, then merge-path rounds.
+    // Tiles of TK_SMALL sorted, then merge-path rounds.
     const uint64_t k = a.k;
     const uint64_t ntiles = (k + TK_SMALL - 1) / TK_SMALL;
     for (uint64_t tIdx = blockIdx.x; tIdx < ntiles; tIdx += gridDim.x) {
@@ -2037,7 +2026,7 @@ cudaError_t topk_launch(const TopkArgs& args, const TopkGeom& geom, cudaStream_t
         size_t smem = static_cast<size_t>(regs_smem(geom.regs_tpb));
         if (a.host_keys) {
             fn = a.w4 ? topk_filter_host_kernel<true> : topk_filter_host_kernel<false>;
-            grid = TK_HOST_CTAS;
+            grid = static_cast<unsigned>(geom.grid_small);   // one CTA per SM
             block = TKR_TPB;
             smem = static_cast<size_t>(regs_smem(TKR_TPB));
         } else if (a.pair) {

@@ -55,7 +55,6 @@ constexpr int TK_SMEM_MAX = 227 * 1024;   // opt-in shared memory per CTA
 // the register-load flavour uses CTAs of 256, 512 (default) or 1024 threads.
 constexpr int TKF_TPB = 256;
 constexpr int TKR_TPB = 512;
-constexpr unsigned TK_HOST_CTAS = 152;    // CTAs of the pass over a column in host memory
 constexpr int TK_TILE_DEFAULT = 16384;
 constexpr int TK_STAGES_DEFAULT = 3;
 constexpr int TK_CTAS_PER_SM_DEFAULT = 4;
