@@ -227,13 +227,20 @@ __device__ void sample_threshold(const TopkArgs& a, unsigned* sh, unsigned long 
     }
     __syncthreads();
     uint64_t mn = ~0ull, mx = 0;
+    if (upto <= 64) {
 #pragma unroll
-    for (int j = 0; j < TK_SPT; ++j)
-        if (s[j] <= edge) {
-            mn = min(mn, s[j]);
-            mx = max(mx, s[j]);
-        }
-    if (__any_sync(0xFFFFFFFFu, mn <= mx)) {
+        for (int j = 0; j < TK_SPT; ++j)
+            if (s[j] <= edge) {
+                atomicMin(&lo, static_cast<unsigned long long>(s[j]));
+                atomicMax(&hi, static_cast<unsigned long long>(s[j]));
+            }
+    } else {                                                 // ties: lane by lane they would wait for each other
+#pragma unroll
+        for (int j = 0; j < TK_SPT; ++j)
+            if (s[j] <= edge) {
+                mn = min(mn, s[j]);
+                mx = max(mx, s[j]);
+            }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             mn = min(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, o));
@@ -280,10 +287,28 @@ struct WarpStage {
     const FuseRange* fr;  // its interval (shared)
 };
 constexpr int WS_BYTES = WS_CAP * 12;
-// Rank word of a staged word.  (Ranked as they leave the stage, in one loop, not
-// as they enter it, in one of the filter's 16 unrolled places.)
-__device__ __forceinline__ uint64_t staged_rank(const TopkArgs& a, uint64_t w) {
-    return a.pair ? w : rank_key(w, a.kind, a.desc);
+// Rank word of a staged word, as three masks: the map of rank_key without
+// branches (floats flip the magnitude of negatives, signed types the sign bit,
+// DESC complements; 4-byte keys lie in the upper half; two-column words are
+// ranks already).  Ranked as they leave the stage, in one loop, not as they
+// enter it, in one of the filter's 16 unrolled places.
+struct RankMask {
+    uint64_t flip, fixed;
+    int up;
+};
+__device__ __forceinline__ RankMask rank_mask(const TopkArgs& a) {
+    RankMask m{0ull, 0ull, 0};
+    if (a.pair) return m;
+    const uint64_t all = a.w4 ? 0xFFFFFFFF00000000ull : ~0ull;
+    if (a.kind == OLAP_KEY_F32 || a.kind == OLAP_KEY_F64) m.flip = all & ~SIGN64;
+    if (a.kind != OLAP_KEY_U32 && a.kind != OLAP_KEY_U64) m.fixed = SIGN64;
+    if (a.desc) m.fixed ^= all;
+    m.up = a.w4 ? 32 : 0;
+    return m;
+}
+__device__ __forceinline__ uint64_t staged_rank(const RankMask& m, uint64_t w) {
+    const uint64_t v = w << m.up;
+    return v ^ (static_cast<uint64_t>(static_cast<int64_t>(v) >> 63) & m.flip) ^ m.fixed;
 }
 constexpr int FUSE_BYTES = (TK_BINS + 4) * 4;     // the histogram, its count of entries below, 16-byte units
 
@@ -334,11 +359,12 @@ __device__ __forceinline__ void stage_flush_plain(const TopkArgs& a, WarpStage& 
     unsigned long long base = 0;
     if (lane == 0) base = atomicAdd(&a.ctl->cand_count, static_cast<unsigned long long>(ws.count));
     base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    const RankMask m = rank_mask(a);
     for (unsigned j = lane; j < ws.count; j += 32) {
         const unsigned long long pos = base + j;
         if (pos < a.cand_cap) {
             const uint32_t idx = ws.idx[j];
-            a.cand_r[pos] = staged_rank(a, ws.w[j]);
+            a.cand_r[pos] = staged_rank(m, ws.w[j]);
             a.cand_rid[pos] = a.rowids ? a.rowids[idx] : idx;
         }
     }
@@ -349,10 +375,11 @@ __device__ __forceinline__ void stage_flush_plain(const TopkArgs& a, WarpStage& 
 // The same, also counting the hits for the fused first pass.
 __device__ __forceinline__ void stage_write_fused(const TopkArgs& a, const WarpStage& ws, unsigned long long base) {
     const FuseRange f = *ws.fr;
+    const RankMask m = rank_mask(a);
     for (unsigned j = threadIdx.x & 31u; j < ws.count; j += 32) {
         const unsigned long long pos = base + j;
         const uint32_t idx = ws.idx[j];
-        const uint64_t r = staged_rank(a, ws.w[j]);
+        const uint64_t r = staged_rank(m, ws.w[j]);
         const uint32_t rid = a.rowids ? a.rowids[idx] : idx;
         if (pos < a.cand_cap) {
             a.cand_r[pos] = r;
@@ -474,10 +501,12 @@ __device__ __forceinline__ void cta_flush_fused(const TopkArgs& a, const WarpSta
 // The streaming pass when the candidates would not fit (few distinct keys): no
 // entry is stored, but all up to the threshold are counted as above, so the
 // select reads the input with its first refine pass done.  K = 10, 2 * 10^6
-// int64 keys of one value 95 -> 50 us (56 without a sample), of 12 values 101 ->
-// 52 (75); 2^26 keys of one value 3226 -> 1472.
+// int64 keys of one value 95 -> 54 us (56 without a sample), of 12 values 101 ->
+// 55 (75); 2^26 keys of one value 3226 -> 1545.
+// A call: its code would lie in the way of the common path, which every launch
+// fetches anew.
 template <int TPB>
-__device__ void count_pass(const TopkArgs& a, const FuseRange& f, unsigned* hist) {
+__device__ __noinline__ void count_pass(const TopkArgs& a, const FuseRange& f, unsigned* hist) {
     constexpr int U = 4;                       // loads in flight per thread
     const unsigned lane = threadIdx.x & 31u;
     const uint64_t stride = static_cast<uint64_t>(TPB) * gridDim.x;
@@ -1129,6 +1158,9 @@ __global__ void __launch_bounds__(TK_TPB) topk_prepare_kernel(TopkArgs a) {
     __shared__ int last;
     TopkCtl* ctl = a.ctl;
     wait_prior_grid();                    // the call before may still read the control block
+    // (a host column's first loads take the link, not the sample's way: 3 * 10^6
+    // page-locked keys 167 -> 162 us)
+    if (a.host_keys) allow_next_grid();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctl->ts[0] = gtimer();
         a.bar->count = 0;
@@ -1175,7 +1207,7 @@ __global__ void __launch_bounds__(TKF_TPB, 4) topk_filter_bulk_kernel(TopkArgs a
 // Kernel 2 of 3, register-load flavour (TPB threads; dynamic shared memory:
 // the fused pass's histogram and the per-warp stages).
 template <bool W4, int TPB>
-__global__ void __launch_bounds__(TPB, 1024 / TPB) topk_filter_regs_kernel(TopkArgs a) {
+__global__ void __launch_bounds__(TPB, 1024 / TPB) topk_filter_regs_kernel(const __grid_constant__ TopkArgs a) {
     extern __shared__ __align__(16) unsigned char fsm[];
     filter_pass<W4, TPB>(a, fsm);
 }
@@ -1196,172 +1228,19 @@ __global__ void __launch_bounds__(TKR_TPB, 1) topk_filter_host_kernel(TopkArgs a
 
 // Kernel 2 of 3 for a two-column key (register loads of both columns).
 template <int TPB>
-__global__ void __launch_bounds__(TPB, 1024 / TPB) topk_filter_pair_kernel(TopkArgs a) {
+__global__ void __launch_bounds__(TPB, 1024 / TPB) topk_filter_pair_kernel(const __grid_constant__ TopkArgs a) {
     extern __shared__ __align__(16) unsigned char fsm[];
     filter_pass_pair<TPB>(a, fsm);
 }
 
-// Kernel 3 of 3 (cooperative): refine, split, finish and sort.  For inputs of
-// at most TK_DIRECT_N keys with a sample it also makes the streaming pass (a
-// filter kernel of its own costs a launch and its end more than a few
-// megabytes take to read), and a grid barrier stands where the filter kernel
-// ended: 2^20 float64 keys, K = 100, 29 us with refine passes over the input,
-// 23 us so.
-enum SelectFilter { SEL_NONE = 0, SEL_W8 = 1, SEL_W4 = 2, SEL_PAIR = 3 };
-template <int FILTER>
-__global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ unsigned long long sc[24];
+// The select's finish for more survivors than one CTA's shared memory ranks.
+__device__ void finish_large(const TopkArgs& a, unsigned char* smem, unsigned long long* sc,
+                                          unsigned bar_target, int pass, bool take_all, uint64_t krem, uint64_t bcnt) {
     TopkCtl* ctl = a.ctl;
     unsigned* sh = reinterpret_cast<unsigned*>(smem);
     uint64_t* sr = reinterpret_cast<uint64_t*>(smem);
     uint32_t* srid = reinterpret_cast<uint32_t*>(smem + TK_RANK_MAX * 8);
-
-    unsigned bar_target = 0;                                 // of the grid barriers
-    if (FILTER == SEL_NONE) {
-        wait_prior_grid();
-        allow_next_grid();
-    } else {
-        if (FILTER == SEL_W8) filter_pass<false, TK_TPB>(a, smem);
-        if (FILTER == SEL_W4) filter_pass<true, TK_TPB>(a, smem);
-        if (FILTER == SEL_PAIR) filter_pass_pair<TK_TPB>(a, smem);
-        if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
-    }
     const bool stamp = blockIdx.x == 0 && threadIdx.x == 0;
-    if (stamp) ctl->ts[2] = gtimer();
-    // Source of the selection: the candidates of the streaming pass when the
-    // sample judged well (at least k of them, all stored), else the input.
-    // Either way, with k or more entries up to the threshold the fused
-    // histogram holds them all.
-    bool cand = false, counted = false;
-    uint64_t src_n = a.n, upto = a.n;                        // entries up to the threshold, or all
-    uint64_t low = 0;                                        // candidates below the fused interval
-    FuseRange fr{};
-    unsigned hv0[TK_BINS / TK_TPB];                          // the thread's bins of the fused pass
-    Elem first{0, 0};                                        // the thread's first candidate
-    if (a.use_sample) {
-        // all that the first steps need, in one round trip to L2
-        const int err = __ldcg(&ctl->err);
-        const uint64_t cnt = __ldcg(&ctl->cand_count);
-        fr = fuse_range(a);
-        low = __ldcg(&ctl->flow);
-        pick_load_global<TK_TPB>(a.ghist, hv0);
-        const uint64_t i0 = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x;
-        if (i0 < a.cand_cap) first = Elem{__ldcg(a.cand_r + i0), __ldcg(a.cand_rid + i0)};
-        if (err != 0) return report(a);
-        counted = a.fuse && cnt >= a.k;
-        cand = cnt >= a.k && cnt <= a.cand_cap && !(a.fuse && fr.count_only);
-        if (cand) src_n = cnt;
-        if (cand || counted) upto = cnt;
-        if (stamp) ctl->path = cand ? 1 : 2;
-    }
-    const unsigned long long use_ts3 = stamp ? gtimer() : 0ull;
-
-    // Phase 2: refine the interval that holds the K-th entry, at or below the
-    // threshold when k entries are.
-    Range g{0ull, cand || counted ? fr.g.rhi : max_rank(a), 0u, max_rowid(a)};
-    uint64_t krem = a.k, bcnt = upto;
-    int pass = 0, npass = 0;
-    // With the filter's fused first pass, pass 0's histogram is ready; when
-    // fewer than k entries are counted in it, the passes start at buffer 1
-    // (clean) and pass 2 clears buffer 0 before pass 3 uses it.
-    bool ready = counted;
-    if (a.fuse && !counted) pass = 1;
-    if (ready && bcnt > TK_SMALL && krem < bcnt) {
-        if (low >= a.k) {
-            g.rhi = fr.g.rlo - 1;
-            if (a.w4) g.rhi &= 0xFFFFFFFF00000000ull;
-            bcnt = low;
-        } else {
-            const Pick pk = pick_loaded<TK_TPB>(hv0, a.k - low, sc);
-            krem = a.k - low - pk.below;
-            bcnt = pk.in_b;
-            g = range_narrow(a, fr.g, fr.sh, pk.b);
-        }
-        ready = false;
-        ++pass;
-        ++npass;
-    }
-    while (bcnt > TK_SMALL && !range_point(g) && krem < bcnt) {
-        const int shift = range_shift(g, a.digit);
-        unsigned* gh = a.ghist + (pass % 3) * TK_BINS;
-        unsigned* gz = a.ghist + ((pass + 1) % 3) * TK_BINS;
-        unsigned long long* mm = ctl->mm[pass % 3];
-        hist_pass(a, cand, src_n, g, shift, gh, gz, sh, mm, ctl->mm[(pass + 1) % 3]);
-        if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
-        ++npass;
-        unsigned hv[TK_BINS / TK_TPB];
-        pick_load_global<TK_TPB>(gh, hv);
-        const Pick pk = pick_loaded<TK_TPB>(hv, krem, sc);
-        // every entry of the interval in one bin: go on with the interval that
-        // their minima and maxima span
-        const bool whole = pk.below == 0 && pk.in_b == bcnt;
-        krem -= pk.below;
-        bcnt = pk.in_b;
-        g = whole ? range_of(a, mm) : range_narrow(a, g, shift, pk.b);
-        ++pass;
-    }
-    // The buffer at pass % 3 must be clean for the finish: when the fused
-    // pass-0 histogram was never consumed, buffer 1 (zeroed by prepare) is.
-    if (ready) pass = 1;
-    if (stamp) {
-        ctl->passes = npass;
-        ctl->ts[3] = use_ts3;
-        ctl->ts[4] = gtimer();
-    }
-
-    // Phase 3: split around the interval.
-    const bool take_all = (krem == bcnt) || range_point(g);
-    // the larger-K finish wants the span of the entries split writes out
-    const bool large = (take_all ? a.k : a.k - krem) + (take_all ? 0 : bcnt) > TK_RANK_MAX;
-    if (large)
-        split_pass_large(a, cand, src_n, g, take_all, krem, krem == bcnt, smem);
-    else
-        split_pass(a, cand, src_n, g, take_all, krem, first);
-    if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
-    if (stamp) ctl->ts[5] = gtimer();
-
-    // Phase 4, survivors that fit one CTA's shared memory (every K <= 4096):
-    // each warp of the grid takes survivors one at a time and computes its
-    // final position as its rank -- the number of entries of its own set
-    // that order before it (equal entries by position), so ranks are
-    // distinct.  The "below" entries precede every bucket entry;
-    // a bucket entry is kept when its rank within the bucket is below krem.
-    {
-        const uint64_t nb = take_all ? a.k : a.k - krem;     // out_r0[0, nb)
-        const uint64_t ns = take_all ? 0 : bcnt;             // small buffer
-        if (nb + ns <= TK_RANK_MAX) {
-            const int nbi = static_cast<int>(nb), nsi = static_cast<int>(ns);
-            for (int i = threadIdx.x; i < nbi; i += TK_TPB) {
-                sr[i] = __ldcg(a.out_r0 + i);
-                srid[i] = __ldcg(a.out_rid0 + i);
-            }
-            for (int i = threadIdx.x; i < nsi; i += TK_TPB) {
-                sr[nbi + i] = __ldcg(a.small_r + i);
-                srid[nbi + i] = __ldcg(a.small_rid + i);
-            }
-            __syncthreads();
-            if (stamp) ctl->ts[7] = gtimer();
-            const unsigned lane = threadIdx.x & 31u;
-            const int nwarps = static_cast<int>(gridDim.x) * (TK_TPB / 32);
-            const int gw = static_cast<int>(blockIdx.x) * (TK_TPB / 32) + static_cast<int>(threadIdx.x >> 5);
-            for (int e = gw; e < nbi + nsi; e += nwarps) {
-                const bool below = e < nbi;
-                const unsigned c = warp_rank_of(sr, srid, below ? 0 : nbi, below ? nbi : nbi + nsi, e);
-                if (lane == 0) {
-                    if (below) write_result(a, c, sr[e], srid[e]);
-                    else if (c < krem) write_result(a, nb + c, sr[e], srid[e]);
-                }
-            }
-            if (stamp) {
-                ctl->ts[8] = gtimer();
-                ctl->ts[6] = ctl->ts[8];
-                if (a.dev_status) *a.dev_status = ld_volatile_i32(&ctl->err);
-            }
-            return;
-        }
-    }
-
     // Phase 4, larger K.  (a) The bucket entries (ns <= 4096) are ranked by
     // the grid as above and the first krem written at their final positions.
     // (b) The below entries are partitioned into bins -- a histogram, a scan,
@@ -1635,6 +1514,173 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(TopkArgs a) {
     if (gtid == 0) ctl->ts[6] = gtimer();
 }
 
+// Kernel 3 of 3 (cooperative): refine, split, finish and sort.  For inputs of
+// at most TK_DIRECT_N keys with a sample it also makes the streaming pass (a
+// filter kernel of its own costs a launch and its end more than a few
+// megabytes take to read), and a grid barrier stands where the filter kernel
+// ended: 2^20 float64 keys, K = 100, 29 us with refine passes over the input,
+// 23 us so.
+// LARGE: for K above TK_SMALL.  A smaller K always fits the ranked finish, and its
+// kernel goes without the code of the larger one, which each call would fetch
+// past (2^24 int64 keys, K = 1: the call 46 -> 43 us).
+enum SelectFilter { SEL_NONE = 0, SEL_W8 = 1, SEL_W4 = 2, SEL_PAIR = 3 };
+template <int FILTER, bool LARGE>
+__global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(const __grid_constant__ TopkArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ unsigned long long sc[24];
+    TopkCtl* ctl = a.ctl;
+    unsigned* sh = reinterpret_cast<unsigned*>(smem);
+    uint64_t* sr = reinterpret_cast<uint64_t*>(smem);
+    uint32_t* srid = reinterpret_cast<uint32_t*>(smem + TK_RANK_MAX * 8);
+
+    unsigned bar_target = 0;                                 // of the grid barriers
+    if (FILTER == SEL_NONE) {
+        wait_prior_grid();
+        allow_next_grid();
+    } else {
+        if (FILTER == SEL_W8) filter_pass<false, TK_TPB>(a, smem);
+        if (FILTER == SEL_W4) filter_pass<true, TK_TPB>(a, smem);
+        if (FILTER == SEL_PAIR) filter_pass_pair<TK_TPB>(a, smem);
+        if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
+    }
+    const bool stamp = blockIdx.x == 0 && threadIdx.x == 0;
+    if (stamp) ctl->ts[2] = gtimer();
+    // Source of the selection: the candidates of the streaming pass when the
+    // sample judged well (at least k of them, all stored), else the input.
+    // Either way, with k or more entries up to the threshold the fused
+    // histogram holds them all.  (count_only is never set without it.)
+    bool cand = false, counted = false;
+    uint64_t src_n = a.n, upto = a.n;                        // entries up to the threshold, or all
+    uint64_t low = 0;                                        // candidates below the fused interval
+    FuseRange fr{};
+    unsigned hv0[TK_BINS / TK_TPB];                          // the thread's bins of the fused pass
+    Elem first{0, 0};                                        // the thread's first candidate
+    if (a.use_sample) {
+        // all that the first steps need, in one round trip to L2
+        const int err = __ldcg(&ctl->err);
+        const uint64_t cnt = __ldcg(&ctl->cand_count);
+        fr = fuse_range(a);
+        low = __ldcg(&ctl->flow);
+        pick_load_global<TK_TPB>(a.ghist, hv0);
+        const uint64_t i0 = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x;
+        if (i0 < a.cand_cap) first = Elem{__ldcg(a.cand_r + i0), __ldcg(a.cand_rid + i0)};
+        if (err != 0) return report(a);
+        counted = a.fuse && cnt >= a.k;
+        cand = cnt >= a.k && cnt <= a.cand_cap && !fr.count_only;
+        if (cand) src_n = cnt;
+        if (cand || counted) upto = cnt;
+        if (stamp) ctl->path = cand ? 1 : 2;
+    }
+    const unsigned long long use_ts3 = stamp ? gtimer() : 0ull;
+
+    // Phase 2: refine the interval that holds the K-th entry, at or below the
+    // threshold when k entries are.
+    Range g{0ull, cand || counted ? fr.g.rhi : max_rank(a), 0u, max_rowid(a)};
+    uint64_t krem = a.k, bcnt = upto;
+    int pass = 0, npass = 0;
+    // With the filter's fused first pass, pass 0's histogram is ready; when
+    // fewer than k entries are counted in it, the passes start at buffer 1
+    // (clean) and pass 2 clears buffer 0 before pass 3 uses it.
+    bool ready = counted;
+    if (a.fuse && !counted) pass = 1;
+    if (ready && bcnt > TK_SMALL && krem < bcnt) {
+        if (low >= a.k) {
+            g.rhi = fr.g.rlo - 1;
+            if (a.w4) g.rhi &= 0xFFFFFFFF00000000ull;
+            bcnt = low;
+        } else {
+            const Pick pk = pick_loaded<TK_TPB>(hv0, a.k - low, sc);
+            krem = a.k - low - pk.below;
+            bcnt = pk.in_b;
+            g = range_narrow(a, fr.g, fr.sh, pk.b);
+        }
+        ready = false;
+        ++pass;
+        ++npass;
+    }
+    while (bcnt > TK_SMALL && !range_point(g) && krem < bcnt) {
+        const int shift = range_shift(g, a.digit);
+        unsigned* gh = a.ghist + (pass % 3) * TK_BINS;
+        unsigned* gz = a.ghist + ((pass + 1) % 3) * TK_BINS;
+        unsigned long long* mm = ctl->mm[pass % 3];
+        hist_pass(a, cand, src_n, g, shift, gh, gz, sh, mm, ctl->mm[(pass + 1) % 3]);
+        if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
+        ++npass;
+        unsigned hv[TK_BINS / TK_TPB];
+        pick_load_global<TK_TPB>(gh, hv);
+        const Pick pk = pick_loaded<TK_TPB>(hv, krem, sc);
+        // every entry of the interval in one bin: go on with the interval that
+        // their minima and maxima span
+        const bool whole = pk.below == 0 && pk.in_b == bcnt;
+        krem -= pk.below;
+        bcnt = pk.in_b;
+        g = whole ? range_of(a, mm) : range_narrow(a, g, shift, pk.b);
+        ++pass;
+    }
+    // The buffer at pass % 3 must be clean for the finish: when the fused
+    // pass-0 histogram was never consumed, buffer 1 (zeroed by prepare) is.
+    if (ready) pass = 1;
+    if (stamp) {
+        ctl->passes = npass;
+        ctl->ts[3] = use_ts3;
+        ctl->ts[4] = gtimer();
+    }
+
+    // Phase 3: split around the interval.
+    const bool take_all = (krem == bcnt) || range_point(g);
+    // the larger-K finish wants the span of the entries split writes out
+    const bool large = (take_all ? a.k : a.k - krem) + (take_all ? 0 : bcnt) > TK_RANK_MAX;
+    if (LARGE && large)
+        split_pass_large(a, cand, src_n, g, take_all, krem, krem == bcnt, smem);
+    else
+        split_pass(a, cand, src_n, g, take_all, krem, first);
+    if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);
+    if (stamp) ctl->ts[5] = gtimer();
+
+    // Phase 4, survivors that fit one CTA's shared memory (every K <= 4096):
+    // each warp of the grid takes survivors one at a time and computes its
+    // final position as its rank -- the number of entries of its own set
+    // that order before it (equal entries by position), so ranks are
+    // distinct.  The "below" entries precede every bucket entry;
+    // a bucket entry is kept when its rank within the bucket is below krem.
+    {
+        const uint64_t nb = take_all ? a.k : a.k - krem;     // out_r0[0, nb)
+        const uint64_t ns = take_all ? 0 : bcnt;             // small buffer
+        if (!LARGE || nb + ns <= TK_RANK_MAX) {
+            const int nbi = static_cast<int>(nb), nsi = static_cast<int>(ns);
+            for (int i = threadIdx.x; i < nbi; i += TK_TPB) {
+                sr[i] = __ldcg(a.out_r0 + i);
+                srid[i] = __ldcg(a.out_rid0 + i);
+            }
+            for (int i = threadIdx.x; i < nsi; i += TK_TPB) {
+                sr[nbi + i] = __ldcg(a.small_r + i);
+                srid[nbi + i] = __ldcg(a.small_rid + i);
+            }
+            __syncthreads();
+            if (stamp) ctl->ts[7] = gtimer();
+            const unsigned lane = threadIdx.x & 31u;
+            const int nwarps = static_cast<int>(gridDim.x) * (TK_TPB / 32);
+            const int gw = static_cast<int>(blockIdx.x) * (TK_TPB / 32) + static_cast<int>(threadIdx.x >> 5);
+            for (int e = gw; e < nbi + nsi; e += nwarps) {
+                const bool below = e < nbi;
+                const unsigned c = warp_rank_of(sr, srid, below ? 0 : nbi, below ? nbi : nbi + nsi, e);
+                if (lane == 0) {
+                    if (below) write_result(a, c, sr[e], srid[e]);
+                    else if (c < krem) write_result(a, nb + c, sr[e], srid[e]);
+                }
+            }
+            if (stamp) {
+                ctl->ts[8] = gtimer();
+                ctl->ts[6] = ctl->ts[8];
+                if (a.dev_status) *a.dev_status = ld_volatile_i32(&ctl->err);
+            }
+            return;
+        }
+    }
+
+    if (LARGE) finish_large(a, smem, sc, bar_target, pass, take_all, krem, bcnt);
+}
+
 // The whole Top-K of a small input, in one launch without a control block or
 // a grid barrier: every CTA loads all n keys into shared memory, finds the
 // interval of the K-th entry by refine passes of its own over them (the same
@@ -1904,10 +1950,14 @@ static bool set_kernel_attrs(int device) {
     opt_in(topk_filter_host_kernel<false>, regs_smem(TKR_TPB));
     opt_in(topk_filter_host_kernel<true>, regs_smem(TKR_TPB));
     opt_in(topk_local_kernel, TKL_SMEM_MAX);
-    opt_in(topk_select_kernel<SEL_NONE>, TK_SORT_SMEM);
-    opt_in(topk_select_kernel<SEL_W8>, TK_SORT_SMEM);
-    opt_in(topk_select_kernel<SEL_W4>, TK_SORT_SMEM);
-    opt_in(topk_select_kernel<SEL_PAIR>, TK_SORT_SMEM);
+    opt_in(topk_select_kernel<SEL_NONE, false>, TK_SORT_SMEM);
+    opt_in(topk_select_kernel<SEL_NONE, true>, TK_SORT_SMEM);
+    opt_in(topk_select_kernel<SEL_W8, false>, TK_SORT_SMEM);
+    opt_in(topk_select_kernel<SEL_W8, true>, TK_SORT_SMEM);
+    opt_in(topk_select_kernel<SEL_W4, false>, TK_SORT_SMEM);
+    opt_in(topk_select_kernel<SEL_W4, true>, TK_SORT_SMEM);
+    opt_in(topk_select_kernel<SEL_PAIR, false>, TK_SORT_SMEM);
+    opt_in(topk_select_kernel<SEL_PAIR, true>, TK_SORT_SMEM);
     if (!ok) return false;
     g_smem_limit[device].store(lim);
     return true;
@@ -1953,10 +2003,14 @@ bool topk_geometry(int device, int tile_bytes, int stages, int ctas_per_sm, int 
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, TK_TPB, TK_SORT_SMEM) != cudaSuccess) per = 0;
         per_sm = std::min(per_sm, per);
     };
-    fits(topk_select_kernel<SEL_NONE>);
-    fits(topk_select_kernel<SEL_W8>);
-    fits(topk_select_kernel<SEL_W4>);
-    fits(topk_select_kernel<SEL_PAIR>);
+    fits(topk_select_kernel<SEL_NONE, false>);
+    fits(topk_select_kernel<SEL_NONE, true>);
+    fits(topk_select_kernel<SEL_W8, false>);
+    fits(topk_select_kernel<SEL_W8, true>);
+    fits(topk_select_kernel<SEL_W4, false>);
+    fits(topk_select_kernel<SEL_W4, true>);
+    fits(topk_select_kernel<SEL_PAIR, false>);
+    fits(topk_select_kernel<SEL_PAIR, true>);
     // Two CTAs per SM for the select in general; one per SM when it reads a
     // candidate list and finishes a small K: its grid barriers then dominate,
     // and half the arrivals take less time (measured, 2^28 keys, K = 1000:
@@ -1991,6 +2045,16 @@ static cudaError_t launch_kernel(void (*fn)(TopkArgs), unsigned grid, unsigned b
     cfg.attrs = at;
     cfg.numAttrs = na;
     return cudaLaunchKernelEx(&cfg, fn, a);
+}
+
+template <bool LARGE>
+static void (*select_kernel(int filter))(TopkArgs) {
+    switch (filter) {
+        case SEL_W8: return topk_select_kernel<SEL_W8, LARGE>;
+        case SEL_W4: return topk_select_kernel<SEL_W4, LARGE>;
+        case SEL_PAIR: return topk_select_kernel<SEL_PAIR, LARGE>;
+        default: return topk_select_kernel<SEL_NONE, LARGE>;
+    }
 }
 
 cudaError_t topk_launch(const TopkArgs& args, const TopkGeom& geom, cudaStream_t stream, cudaEvent_t* ev) {
@@ -2051,9 +2115,9 @@ cudaError_t topk_launch(const TopkArgs& args, const TopkGeom& geom, cudaStream_t
     if (ev && (e = cudaEventRecord(ev[2], stream)) != cudaSuccess) return e;
     // (the direct path keeps both CTAs per SM: its passes read the input)
     const int sgrid = (a.use_sample && a.k <= static_cast<uint64_t>(TK_SMALL)) ? geom.grid_small : geom.grid;
-    void (*sel)(TopkArgs) = topk_select_kernel<SEL_NONE>;
-    if (a.use_sample == TK_SAMPLE_INLINE)
-        sel = a.pair ? topk_select_kernel<SEL_PAIR> : a.w4 ? topk_select_kernel<SEL_W4> : topk_select_kernel<SEL_W8>;
+    const int which = a.use_sample != TK_SAMPLE_INLINE ? SEL_NONE : a.pair ? SEL_PAIR : a.w4 ? SEL_W4 : SEL_W8;
+    const bool large = a.k > static_cast<uint64_t>(TK_SMALL);
+    void (*const sel)(TopkArgs) = large ? select_kernel<true>(which) : select_kernel<false>(which);
     e = launch_kernel(sel, static_cast<unsigned>(sgrid), TK_TPB, TK_SORT_SMEM, stream, a, true);
     if (e != cudaSuccess || !ev) return e;
     return cudaEventRecord(ev[3], stream);
