@@ -288,12 +288,17 @@ __global__ void __launch_bounds__(JT_TPB, 3) join_block_build_kernel(ulonglong2*
         Stretch mine_from{__shfl_up_sync(0xFFFFFFFFu, incl.entries, 1), __shfl_up_sync(0xFFFFFFFFu, incl.least, 1)};
         if (lane == 0) mine_from = Stretch{0u, 0u};
         __syncthreads();
-        Stretch from{0u, 0u}, all{0u, 0u};
+        Stretch upto = ws[lane & (JT_TPB / 32 - 1)];          // every warp scans the warps' stretches
 #pragma unroll
-        for (unsigned w = 0; w < JT_TPB / 32; ++w) {
-            if (w == warp) from = all;
-            all = stretch_join(all, ws[w]);
+        for (int o = 1; o < JT_TPB / 32; o <<= 1) {
+            const Stretch before{__shfl_up_sync(0xFFFFFFFFu, upto.entries, o), __shfl_up_sync(0xFFFFFFFFu, upto.least, o)};
+            if (lane >= static_cast<unsigned>(o)) upto = stretch_join(before, upto);
         }
+        const Stretch all{__shfl_sync(0xFFFFFFFFu, upto.entries, JT_TPB / 32 - 1),
+                          __shfl_sync(0xFFFFFFFFu, upto.least, JT_TPB / 32 - 1)};
+        Stretch from{__shfl_sync(0xFFFFFFFFu, upto.entries, (warp + 31u) & 31u),
+                     __shfl_sync(0xFFFFFFFFu, upto.least, (warp + 31u) & 31u)};
+        if (warp == 0) from = Stretch{0u, 0u};
         from = stretch_join(from, mine_from);
         const unsigned end = max(all.entries, all.least);    // of the last bucket, from slot 0
         const unsigned wrapped = end > nslots ? end - nslots : 0u;
