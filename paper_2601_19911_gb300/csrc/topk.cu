@@ -256,7 +256,7 @@ __device__ void sample_threshold(const TopkArgs& a, unsigned* sh, unsigned long 
         const uint64_t t = hi, d = hi - lo;
         a.ctl->thresh = t;
         a.ctl->fbase = d >= t / 4 ? (d ? 0ull : t) : t - 4 * d;
-        a.ctl->count_only = a.fuse && !a.host_keys && upto * a.n > a.cand_cap * TK_SAMPLE;
+        a.ctl->count_only = a.fuse && !a.host_keys && 4 * upto * a.n > 5 * a.cand_cap * TK_SAMPLE;
         a.ctl->ts[1] = gtimer();
     }
 }
@@ -1001,7 +1001,7 @@ constexpr int SPLIT_U = 4;
 static_assert(TK_TPB / 32 * SPLIT_CAP * 12 <= TK_SORT_SMEM, "the warps' stages");
 static_assert(SPLIT_U * 32 <= SPLIT_CAP, "a step's entries fit an empty stage");
 __device__ void split_pass_large(const TopkArgs& a, bool cand, uint64_t src_n, const Range& g, bool take_all,
-                                 uint64_t krem, bool whole, unsigned char* smem) {
+                                 uint64_t krem, bool whole, Elem first, unsigned char* smem) {
     TopkCtl* ctl = a.ctl;
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, lt_mask = (1u << lane) - 1u;
     uint64_t* wr = reinterpret_cast<uint64_t*>(smem + warp * (SPLIT_CAP * 12));
@@ -1012,6 +1012,7 @@ __device__ void split_pass_large(const TopkArgs& a, bool cand, uint64_t src_n, c
     const uint64_t eq_base = a.k - krem;
     unsigned long long* eq_ctr = take_all ? &ctl->eq_count : &ctl->small_count;
     const int last = whole ? 0 : -1;                         // range_cmp of the entries that all go to out
+    bool loaded = cand;                                      // `first` is the thread's first candidate
     auto write = [&](unsigned long long base) {
         __syncwarp();
         for (unsigned j = lane; j < cnt; j += 32) {
@@ -1026,8 +1027,10 @@ __device__ void split_pass_large(const TopkArgs& a, bool cand, uint64_t src_n, c
 #pragma unroll
         for (int u = 0; u < SPLIT_U; ++u) {
             const uint64_t i = wb + lane + u * stride;
-            if (i < src_n) e[u] = load_src(a, cand, i);
+            if (u == 0 && loaded) e[u] = first;
+            else if (i < src_n) e[u] = load_src(a, cand, i);
         }
+        loaded = false;
         if (cnt + SPLIT_U * 32 > SPLIT_CAP) {
             unsigned long long base = 0;
             if (lane == 0) base = atomicAdd(&ctl->out_count, static_cast<unsigned long long>(cnt));
@@ -1273,8 +1276,8 @@ __device__ void finish_large(const TopkArgs& a, unsigned char* smem, unsigned lo
         }
         // One partition with the given bins: 1 done, 0 a bin too large, -1 a
         // wait expired.  ph: clean; pc: zeroed here for the cursors; `pure`:
-        // odd bins hold identical entries.
-        auto partition = [&](auto bin, unsigned* ph, unsigned* pc, bool pure) -> int {
+        // odd bins hold identical entries; `most`: entries of a bin.
+        auto partition = [&](auto bin, unsigned* ph, unsigned* pc, bool pure, unsigned most) -> int {
             for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB) sh[b] = 0;
             if (blockIdx.x == 0)
                 for (int b = threadIdx.x; b < TK_BINS; b += TK_TPB) pc[b] = 0;
@@ -1311,7 +1314,7 @@ __device__ void finish_large(const TopkArgs& a, unsigned char* smem, unsigned lo
                 off[threadIdx.x * PER + j] = static_cast<unsigned>(run);
                 run += v[j];
             }
-            if (!__syncthreads_and(mx <= static_cast<unsigned>(TK_BIN_MAX))) return 0;
+            if (!__syncthreads_and(mx <= most)) return 0;
             // Scatter the below entries into bin order (out_r1).
             for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * TK_TPB + threadIdx.x; i < nb; i += gstride) {
                 const uint64_t er = __ldcg(a.out_r0 + i);
@@ -1374,8 +1377,10 @@ __device__ void finish_large(const TopkArgs& a, unsigned char* smem, unsigned lo
         for (int j = 0; j < 3; ++j) hb[j] = a.ghist + ((pass + j) % 3) * TK_BINS;
         const Range pr = range_of(a, ctl->fin);
         const int psh = range_shift(pr, a.digit);
-        int done = partition([&](uint64_t r, uint32_t rid) { return range_bin(pr, psh, r, rid); }, hb[0], hb[1], false);
-        if (done == 0 && nb <= TK_SPLIT_MAX) {
+        const bool splits = nb <= TK_SPLIT_MAX;
+        int done = partition([&](uint64_t r, uint32_t rid) { return range_bin(pr, psh, r, rid); }, hb[0], hb[1], false,
+                             splits ? TK_BIN_EVEN : TK_BIN_MAX);
+        if (done == 0 && splits) {
             uint64_t* pr_r = reinterpret_cast<uint64_t*>(smem + TK_BINS * 4 + TK_SMALL * 12);
             uint32_t* pr_rid = reinterpret_cast<uint32_t*>(smem + TK_BINS * 4 + TK_SMALL * 12 + (TK_SPLITTERS + 1) * 8);
             for (int j = threadIdx.x; j < TK_SPLITTERS; j += TK_TPB) {
@@ -1408,7 +1413,7 @@ __device__ void finish_large(const TopkArgs& a, unsigned char* smem, unsigned lo
                 const bool eq = lo < TK_SPLITTERS && pr_r[lo] == r && pr_rid[lo] == rid;
                 return static_cast<unsigned>(2 * lo + (eq ? 1 : 0));
             };
-            done = partition(gap, hb[1], hb[2], true);
+            done = partition(gap, hb[1], hb[2], true, TK_BIN_MAX);
         }
         if (done < 0) return report(a);
         if (done) {
@@ -1631,7 +1636,7 @@ __global__ void __launch_bounds__(TK_TPB, 2) topk_select_kernel(const __grid_con
     // the larger-K finish wants the span of the entries split writes out
     const bool large = (take_all ? a.k : a.k - krem) + (take_all ? 0 : bcnt) > TK_RANK_MAX;
     if (LARGE && large)
-        split_pass_large(a, cand, src_n, g, take_all, krem, krem == bcnt, smem);
+        split_pass_large(a, cand, src_n, g, take_all, krem, krem == bcnt, first, smem);
     else
         split_pass(a, cand, src_n, g, take_all, krem, first);
     if (!grid_sync(a.bar, &ctl->err, bar_target)) return report(a);

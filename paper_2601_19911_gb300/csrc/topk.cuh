@@ -43,10 +43,12 @@ static_assert(TK_SPLITTERS <= TK_SMALL, "the splitters fit where K > TK_SMALL en
 // (tied int64 keys, K = 250,000: the call 332 us, 452 with tile sorts and merges;
 // 2 * 10^6 tied float32 keys, K = 400,000: 443 us by splitters, 326 by merges).
 constexpr uint64_t TK_SPLIT_MAX = 2048ull * 128;
-// Entries of a bin that the larger-K finish ranks in one CTA; a larger one makes
-// that CTA the last by far (2^26 normal int64 keys, K = 10^6, bins up to 4096:
-// the finish 1100 us, tile sorts and merges instead 370).
-constexpr int TK_BIN_MAX = 2048;
+// Entries of a bin that the larger-K finish ranks in one CTA, all pairs of them:
+// in equal bins where splitters may take their place (2 * 10^6 normal int64
+// keys, K = 200,000: the call 139 us, 203 with splitters past 256; of 1024
+// values, K = 20,000, bins of 1950 615 us, splitters 92), and otherwise.
+constexpr unsigned TK_BIN_EVEN = 512;
+constexpr unsigned TK_BIN_MAX = 1024;
 constexpr int TK_SORT_SMEM = TK_RANK_MAX * 12;  // select kernel shared bytes (ranking / sort tile / histogram)
 constexpr int TK_MAX_STAGES = 16;         // full + empty mbarrier pairs reserved after the ring
 constexpr int TK_SMEM_MAX = 227 * 1024;   // opt-in shared memory per CTA
