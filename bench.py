@@ -148,9 +148,8 @@ def headline(report: dict) -> dict:
             line[key] = v
             continue
         keep = HEADLINE_PARTS.get(key, ("value", "unit", "ms_per_step"))
-        part = dict(v) if keep is None else {k: v[k] for k in keep if k in v}
-        if part:
-            line[key] = part
+        if key in HEADLINE_PARTS or "value" in v:
+            line[key] = dict(v) if keep is None else {k: v[k] for k in keep if k in v}
     return line
 
 

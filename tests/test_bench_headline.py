@@ -18,7 +18,7 @@ def test_line_keeps_the_contract_and_drops_the_sweeps():
                 "keys_only": {"value": 1}},
         "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": []},
         "join": {"value": 90.0, "unit": "Gprobes/s", "ms_per_step": 3.0, "cells": sweep},
-        "gate": {"cells": sweep}, "serving": {"value": 2.0, "unit": "ms", "gated": sweep},
+        "gate": {"unit": "relative error", "cells": sweep}, "serving": {"value": 2.0, "unit": "ms", "gated": sweep},
         "cpu_baseline": {"value": 0.01, "unit": "Gkeys/s", "cores": 1, "kind": "oracle", "host": sweep},
     }
     line = bench.headline(report)

@@ -56,3 +56,14 @@ def test_ties_around_the_splitters_limit(ctx, k):
     keys = (datagen.splitmix64(8, 700_001) % np.uint64(11)).astype(np.int64) << 50
     _check(ctx, keys, k, olap.DESC)
     _check(ctx, keys, k, olap.ASC, (datagen.splitmix64(9, keys.shape[0]) % np.uint64(50_000)).astype(np.uint32))
+
+
+@pytest.mark.parametrize("m", [1023, 1024, 1025])
+def test_bin_sizes_past_the_splitters_limit(ctx, m):
+    """With more entries than splitters take, bins end at 1024."""
+    n = 300_000
+    keys = (np.arange(n, dtype=np.int64) // m) * (1 << 42) + np.arange(n, dtype=np.int64) % m
+    keys[7] = 1 << 62
+    keys = keys[np.random.default_rng(m).permutation(n)]
+    for k in (270_000, n):
+        _check(ctx, keys, k, olap.ASC)
