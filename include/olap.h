@@ -354,8 +354,8 @@ olap_status olap_topk_rows(olap_ctx* ctx, const void* rows, olap_mem in_where, u
  * blocks of 1024 buckets (over the whole table when a block would overflow); a
  * bucket with a free slot ends every chain, and a probe also stops at its
  * key's last copy.
- * Capacity is the power of two of buckets that keeps n / (2 * buckets) at or
- * below the load factor.  Build rows whose key equals the table's empty
+ * Capacity is the smallest power of two of buckets with n / load factor + 2 or
+ * more slots (so 2^k rows at 0.5 take 2^(k+1) buckets, a load of 0.25).  Build rows whose key equals the table's empty
  * marker (all bits set, i.e. -1) are kept in a side list, so every int64 key
  * value joins correctly.  A table far above L2 also carries a blocked Bloom
  * filter for the pre-probe (see olap_prefilter).  The table stays resident on

@@ -14,8 +14,10 @@
 #include "topk.cuh"
 
 // The context's small device area: [0] probe count word, [256] row queue
-// counter, [1024] the probe's plan, [1536] the plan kernel's counters,
-// [2048] the self-test words, [16384] the plan kernel's packed sample.
+// counter, [264] the probe kernel's ticket, [1024] the probe's plan, [1536] the
+// plan kernel's counters, [2048] the self-test words, [4096] the partitions'
+// counts and cursors with their ticket (4352 bytes), [16384] the plan kernel's
+// packed sample.
 constexpr size_t OLAP_AUX_BYTES = 32768;
 
 struct olap_ctx {
@@ -44,10 +46,11 @@ struct olap_ctx {
     cudaEvent_t pinned_ev[2] = {nullptr, nullptr};
     olap::HostCopyPool* copy_pool = nullptr;   // host threads of the staging copies
 
-    // Small pinned words for device status read-back, and a small device
-    // area for counters of blocking calls (4 KiB).
+    // Small pinned words that kernels write: [0], [1] a blocking Top-K's status,
+    // [8] a blocking probe's pair count (64 bits); and the small device area
+    // (OLAP_AUX_BYTES).
     int32_t* host_status = nullptr;
-    void* aux = nullptr;               // small device area (OLAP_AUX_BYTES): counters, the probe's plan and sample
+    void* aux = nullptr;
 
     // Control block of the last Top-K launched (diagnostics).
     void* last_topk_ctl = nullptr;

@@ -259,8 +259,8 @@ __device__ __forceinline__ void probe_step(uint2* ws, unsigned& cnt, ulonglong2*
 // at a time, so no lane waits for another's longer chain.  Bound by the
 // bucket reads: L2-resident tables run at 143 G probes/s (103 G when every
 // lane walked its chains itself, two rows at a time), a 2^24-row table with
-// 30 M partitioned probes in 484 us for the whole call (648 us), with 2^28
-// probes in 3.30 ms (4.26 ms).
+// 30 M partitioned probes in 484 us for the whole call (648 us; 437 with the
+// present partition passes), with 2^28 probes in 3.30 ms (4.26 ms).
 template <bool L2_ONLY>
 __device__ __forceinline__ void probe_rows(const ProbeArgs& a, const RowQueue& q, unsigned char* warp_smem) {
     uint2* ws = reinterpret_cast<uint2*>(warp_smem + JP_PEND * 16);
