@@ -16,6 +16,7 @@ GIB, MIB = 1 << 30, 1 << 20
 FAKE = r"""
 #include <cuda_runtime.h>
 #include <cstdint>
+#include <cstdlib>
 #include <map>
 #include "devmem.h"
 static std::map<uintptr_t, size_t> live;
@@ -33,7 +34,7 @@ cudaError_t cudaMalloc(void** p, size_t n) {
 }
 cudaError_t cudaFree(void* p) {
     auto it = live.find(reinterpret_cast<uintptr_t>(p));
-    if (it == live.end()) __builtin_trap();
+    if (it == live.end()) abort();
     used -= it->second;
     live.erase(it);
     return cudaSuccess;
